@@ -75,8 +75,6 @@ struct Hier {
   bool probe_pending = false;
   double probe_ms = 0.0;
   long long probe_count = 0;
-  // learned-prolongator inference scratch (features and network outputs)
-  DBuf<float> mlp_feats, mlp_out;
   // per-region energies (tile ranges, tile partials, region sums) and accepted regions
   DBuf<int> energy_tiles;
   DBuf<double> energy_part, energy_out;

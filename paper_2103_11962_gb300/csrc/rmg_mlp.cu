@@ -6,8 +6,8 @@
 // one gets 1 - w), so every predicted row of P sums to one and constants are preserved.
 //
 // Forward pass: BF16 tensor-core MMA (mma.sync m16n8k16, FP32 accumulate); a CTA of 8 warps
-// takes 128 samples, each warp 16 rows. Backward pass: FP32 CUDA cores on the same tile, one
-// atomic add per parameter per CTA. Adam updates FP32 master weights.
+// takes 128 samples, each warp 16 rows. Backward pass: FP32 CUDA cores on the same tile, the
+// weight gradients in registers, one atomic add per parameter per CTA. Adam updates FP32 master weights.
 //
 // Features of fine node n (9 per axis, zero along axes where n sits on a coarse index): for
 // the line of three edges between its two coarse neighbours along the axis, log10 of the three
@@ -17,9 +17,12 @@
 #include <cuda_bf16.h>
 
 #include <algorithm>
+#include <new>
+#include <vector>
 
 #include "rmg_hier.cuh"
 #include "rmg_kernels.cuh"
+#include "rmg_launch.cuh"
 
 namespace rmg {
 namespace {
@@ -30,7 +33,10 @@ constexpr int O_W1 = 0, O_B1 = O_W1 + NH * NF, O_W2 = O_B1 + NH, O_B2 = O_W2 + N
               O_W3 = O_B2 + NH, O_B3 = O_W3 + NOUT * NH;
 constexpr int kRows = 128, kThreads = 256;
 // padded shared-memory strides (elements)
-constexpr int SX = NF + 8, SH = NH + 8, SD = NH + 1;
+constexpr int SX = NF + 8, SH = NH + 8;
+
+// The backward pass reads FP32 rows four values at a time: row strides are multiples of four.
+constexpr int SXF = NF + 4, SHF = NH + 4;
 
 struct MlpSmem {
   __nv_bfloat16 Xb[kRows * SX];
@@ -39,14 +45,17 @@ struct MlpSmem {
   __nv_bfloat16 W2b[NH * SH];
   __nv_bfloat16 H2b[kRows * SH];
   __nv_bfloat16 W3b[8 * SH];
+  float Xf[kRows * SXF];                 // the BF16-rounded X and H1 again as FP32
+  float H1f[kRows * SHF];
+  float W2f[NH * NH];
+  float dZ3[kRows * 4];
+  float dZ2[kRows * SHF];
+  float dZ1[kRows * SHF];
+  float W3f[4 * NH];                     // [j][k], row 3 zero
   float O[kRows * 4];
   float Y[kRows * 4];
   float M[kRows * 4];
-  float W2f[NH * NH];
-  float W3f[NOUT * NH];
-  float dZ3[kRows * 4];
-  float dZ2[kRows * SD];
-  float dZ1[kRows * SD];
+  long long idx[kRows];                  // sample of every row, -1 past the last one
   float red[kThreads / 32];
 };
 
@@ -86,12 +95,25 @@ __device__ __forceinline__ unsigned long long mix64(unsigned long long z) {
   return z ^ (z >> 31);
 }
 
-// mode 0: inference (rows = samples base..base+127, outputs written to out[n][3]).
-// mode 1: gradient (rows sampled or taken in order; gradients and loss accumulated).
-__global__ void __launch_bounds__(kThreads)
+__device__ __forceinline__ void red_add4(float* p, float a, float b, float c, float d) {
+  asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};\n" ::"l"(p), "f"(a), "f"(b), "f"(c),
+               "f"(d) : "memory");
+}
+__device__ __forceinline__ void red_add2(float* p, float a, float b) {
+  asm volatile("red.global.add.v2.f32 [%0], {%1, %2};\n" ::"l"(p), "f"(a), "f"(b) : "memory");
+}
+
+// Gradient and loss over rows that are sampled or taken in order, in tiles of 128 samples.
+//
+// Bound by the FP32 pipe in the backward products (1.3M FMAs a tile). One FMA per two shared
+// loads and a set of 6467 atomic adds per tile took 269 us for 65,573 samples; here every
+// thread owns blocks of the outputs (4 x 4 of dW2, 4 x 2 of dW1, 8 x 4 of dZ1), loads its
+// operands four at a time, and keeps the weight gradients of all its CTA's tiles in registers,
+// so the atomic adds run once per CTA: 76 us (the whole call with its copies 313 -> 105 us).
+__global__ void __launch_bounds__(kThreads, 1)
 k_mlp(const float* __restrict__ params, int n, long long ntiles, const float* __restrict__ feats,
-      const float* __restrict__ labels, const float* __restrict__ mask, int mode, int sample,
-      unsigned long long seed, float inv_norm, float* __restrict__ out, float* __restrict__ grads,
+      const float* __restrict__ labels, const float* __restrict__ mask, int sample,
+      unsigned long long seed, float inv_norm, float* __restrict__ grads,
       float* __restrict__ loss) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   MlpSmem& S = *reinterpret_cast<MlpSmem*>(smem_raw);
@@ -110,36 +132,40 @@ k_mlp(const float* __restrict__ params, int n, long long ntiles, const float* __
     const int j = e / NH, k = e % NH;
     const float w = j < NOUT ? params[O_W3 + j * NH + k] : 0.f;
     S.W3b[j * SH + k] = __float2bfloat16_rn(w);
-    if (j < NOUT) S.W3f[j * NH + k] = w;
+    if (j < 4) S.W3f[j * NH + k] = w;
   }
+  // this thread's share of the gradients: dW2[4 mg..][4 kg..], dW1[4 mg..][2 kg..], and over
+  // the rows of its quarter rq (32 rows) column kq of dW3, db2 and db1
+  const int mg = tid >> 4, kg = tid & 15, rq = tid >> 6, kq = tid & 63;
+  float gw2[4][4] = {}, gw1[4][2] = {}, gw3[NOUT] = {}, gb3 = 0.f, gb2 = 0.f, gb1 = 0.f;
+  float lsum = 0.f;
   // persistent loop over tiles of 128 samples; the weights above are staged once per CTA
   for (long long tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
   const long long base = tile * kRows;
   __syncthreads();
+  if (tid < kRows) {
+    long long i = base + tid;
+    if (sample)
+      i = (long long)(mix64(seed + 0x9E3779B97F4A7C15ull * (unsigned long long)(i + 1)) %
+                      (unsigned long long)n);
+    else if (i >= n)
+      i = -1;
+    S.idx[tid] = i;
+  }
+  __syncthreads();
   // ---- stage the samples
   for (int e = tid; e < kRows * NF; e += kThreads) {
     const int r = e / NF, k = e % NF;
-    long long i = base + r;
-    float v = 0.f;
-    bool valid;
-    if (sample) {
-      i = (long long)(mix64(seed + 0x9E3779B97F4A7C15ull * (unsigned long long)(base + r + 1)) %
-                      (unsigned long long)n);
-      valid = true;
-    } else {
-      valid = i < n;
-    }
-    if (valid) v = feats[i * NF + k];
-    S.Xb[r * SX + k] = __float2bfloat16_rn(v);
-    if (k < 4) {
-      float y = 0.f, m = 0.f;
-      if (mode == 1 && valid && k < NOUT) {
-        y = labels[i * NOUT + k];
-        m = mask[i * NOUT + k];
-      }
-      S.Y[r * 4 + k] = y;
-      S.M[r * 4 + k] = m;
-    }
+    const long long i = S.idx[r];
+    const __nv_bfloat16 v = __float2bfloat16_rn(i >= 0 ? feats[i * NF + k] : 0.f);
+    S.Xb[r * SX + k] = v;
+    S.Xf[r * SXF + k] = __bfloat162float(v);
+  }
+  for (int e = tid; e < kRows * NOUT; e += kThreads) {
+    const int r = e / NOUT, j = e % NOUT;
+    const long long i = S.idx[r];
+    S.Y[r * 4 + j] = i >= 0 ? labels[i * NOUT + j] : 0.f;
+    S.M[r * 4 + j] = i >= 0 ? mask[i * NOUT + j] : 0.f;
   }
   __syncthreads();
 
@@ -152,10 +178,16 @@ k_mlp(const float* __restrict__ params, int n, long long ntiles, const float* __
     for (int nt = 0; nt < 8; ++nt) {
       const int c = nt * 8 + 2 * t;
       const float b0 = params[O_B1 + c], b1 = params[O_B1 + c + 1];
-      S.H1b[(r0 + g) * SH + c] = __float2bfloat16_rn(fmaxf(acc[nt][0] + b0, 0.f));
-      S.H1b[(r0 + g) * SH + c + 1] = __float2bfloat16_rn(fmaxf(acc[nt][1] + b1, 0.f));
-      S.H1b[(r0 + g + 8) * SH + c] = __float2bfloat16_rn(fmaxf(acc[nt][2] + b0, 0.f));
-      S.H1b[(r0 + g + 8) * SH + c + 1] = __float2bfloat16_rn(fmaxf(acc[nt][3] + b1, 0.f));
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int r = r0 + g + 8 * h;
+        const __nv_bfloat16 v0 = __float2bfloat16_rn(fmaxf(acc[nt][2 * h] + b0, 0.f));
+        const __nv_bfloat16 v1 = __float2bfloat16_rn(fmaxf(acc[nt][2 * h + 1] + b1, 0.f));
+        S.H1b[r * SH + c] = v0;
+        S.H1b[r * SH + c + 1] = v1;
+        *reinterpret_cast<float2*>(&S.H1f[r * SHF + c]) =
+            make_float2(__bfloat162float(v0), __bfloat162float(v1));
+      }
     }
   }
   __syncwarp();
@@ -191,88 +223,115 @@ k_mlp(const float* __restrict__ params, int n, long long ntiles, const float* __
   }
   __syncthreads();
 
-  if (mode == 0) {
-    for (int e = tid; e < kRows * NOUT; e += kThreads) {
-      const int r = e / NOUT, j = e % NOUT;
-      if (base + r < n) out[(base + r) * NOUT + j] = S.O[r * 4 + j];
-    }
-    continue;
-  }
-
-  // ---- backward (FP32 CUDA cores)
-  float lsum = 0.f;
+  // ---- backward (FP32)
   for (int e = tid; e < kRows * NOUT; e += kThreads) {
     const int r = e / NOUT, j = e % NOUT;
     const float o = S.O[r * 4 + j], m = S.M[r * 4 + j], d = o - S.Y[r * 4 + j];
     lsum += m * d * d;
     S.dZ3[r * 4 + j] = 2.f * m * d * inv_norm * o * (1.f - o);
   }
+  __syncthreads();
+  // dZ2 = (dZ3 W3) * [H2 > 0], and column kq of dW3, db2 over 32 rows
+  {
+    const float w0 = S.W3f[kq], w1 = S.W3f[NH + kq], w2 = S.W3f[2 * NH + kq];
+#pragma unroll 4
+    for (int r = 32 * rq; r < 32 * rq + 32; ++r) {
+      const float d0 = S.dZ3[r * 4], d1 = S.dZ3[r * 4 + 1], d2 = S.dZ3[r * 4 + 2];
+      const float h = __bfloat162float(S.H2b[r * SH + kq]);
+      gw3[0] = fmaf(d0, h, gw3[0]);
+      gw3[1] = fmaf(d1, h, gw3[1]);
+      gw3[2] = fmaf(d2, h, gw3[2]);
+      const float z = h > 0.f ? fmaf(d2, w2, fmaf(d1, w1, d0 * w0)) : 0.f;
+      S.dZ2[r * SHF + kq] = z;
+      gb2 += z;
+    }
+    if (kq < NOUT)
+      for (int r = 32 * rq; r < 32 * rq + 32; ++r) gb3 += S.dZ3[r * 4 + kq];
+  }
+  __syncthreads();
+  // dW2 += dZ2^T H1
+#pragma unroll 4
+  for (int r = 0; r < kRows; ++r) {
+    const float4 z = *reinterpret_cast<const float4*>(&S.dZ2[r * SHF + 4 * mg]);
+    const float4 h = *reinterpret_cast<const float4*>(&S.H1f[r * SHF + 4 * kg]);
+    const float zv[4] = {z.x, z.y, z.z, z.w}, hv[4] = {h.x, h.y, h.z, h.w};
+#pragma unroll
+    for (int a = 0; a < 4; ++a)
+#pragma unroll
+      for (int b = 0; b < 4; ++b) gw2[a][b] = fmaf(zv[a], hv[b], gw2[a][b]);
+  }
+  // dZ1 = (dZ2 W2) * [H1 > 0]: rows 8 mg .. 8 mg + 7, columns 4 kg ..
+  {
+    float acc[8][4] = {};
+#pragma unroll 2
+    for (int m = 0; m < NH; m += 4) {
+      float4 w[4];
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+        w[q] = *reinterpret_cast<const float4*>(&S.W2f[(m + q) * NH + 4 * kg]);
+#pragma unroll
+      for (int a = 0; a < 8; ++a) {
+        const float4 z = *reinterpret_cast<const float4*>(&S.dZ2[(8 * mg + a) * SHF + m]);
+        const float zv[4] = {z.x, z.y, z.z, z.w};
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          acc[a][0] = fmaf(zv[q], w[q].x, acc[a][0]);
+          acc[a][1] = fmaf(zv[q], w[q].y, acc[a][1]);
+          acc[a][2] = fmaf(zv[q], w[q].z, acc[a][2]);
+          acc[a][3] = fmaf(zv[q], w[q].w, acc[a][3]);
+        }
+      }
+    }
+#pragma unroll
+    for (int a = 0; a < 8; ++a) {
+      const int at = (8 * mg + a) * SHF + 4 * kg;
+      const float4 h = *reinterpret_cast<const float4*>(&S.H1f[at]);
+      *reinterpret_cast<float4*>(&S.dZ1[at]) =
+          make_float4(h.x > 0.f ? acc[a][0] : 0.f, h.y > 0.f ? acc[a][1] : 0.f,
+                      h.z > 0.f ? acc[a][2] : 0.f, h.w > 0.f ? acc[a][3] : 0.f);
+    }
+  }
+  __syncthreads();
+  // dW1 += dZ1^T X, db1
+#pragma unroll 4
+  for (int r = 0; r < kRows; ++r) {
+    const float4 z = *reinterpret_cast<const float4*>(&S.dZ1[r * SHF + 4 * mg]);
+    const float2 x = *reinterpret_cast<const float2*>(&S.Xf[r * SXF + 2 * kg]);
+    const float zv[4] = {z.x, z.y, z.z, z.w};
+#pragma unroll
+    for (int a = 0; a < 4; ++a) {
+      gw1[a][0] = fmaf(zv[a], x.x, gw1[a][0]);
+      gw1[a][1] = fmaf(zv[a], x.y, gw1[a][1]);
+    }
+  }
+#pragma unroll 4
+  for (int r = 32 * rq; r < 32 * rq + 32; ++r) gb1 += S.dZ1[r * SHF + kq];
+  }  // tiles
+
+  // ---- this CTA's sums
+#pragma unroll
+  for (int a = 0; a < 4; ++a) {
+    red_add4(&grads[O_W2 + (4 * mg + a) * NH + 4 * kg], gw2[a][0], gw2[a][1], gw2[a][2],
+             gw2[a][3]);
+    red_add2(&grads[O_W1 + (4 * mg + a) * NF + 2 * kg], gw1[a][0], gw1[a][1]);
+  }
+#pragma unroll
+  for (int j = 0; j < NOUT; ++j) atomicAdd(&grads[O_W3 + j * NH + kq], gw3[j]);
+  atomicAdd(&grads[O_B2 + kq], gb2);
+  atomicAdd(&grads[O_B1 + kq], gb1);
+  if (kq < NOUT) atomicAdd(&grads[O_B3 + kq], gb3);
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) lsum += __shfl_xor_sync(0xffffffffu, lsum, o);
   if (lane == 0) S.red[warp] = lsum;
   __syncthreads();
   if (tid == 0) {
-    float s = 0.f;
-    for (int w = 0; w < kThreads / 32; ++w) s += S.red[w];
-    atomicAdd(loss, s * inv_norm);
+    float sum = 0.f;
+    for (int w = 0; w < kThreads / 32; ++w) sum += S.red[w];
+    atomicAdd(loss, sum * inv_norm);
   }
-  // dW3, db3
-  if (tid < NOUT * NH) {
-    const int j = tid / NH, k = tid % NH;
-    float s = 0.f;
-    for (int r = 0; r < kRows; ++r) s += S.dZ3[r * 4 + j] * __bfloat162float(S.H2b[r * SH + k]);
-    atomicAdd(&grads[O_W3 + j * NH + k], s);
-  } else if (tid < NOUT * NH + NOUT) {
-    const int j = tid - NOUT * NH;
-    float s = 0.f;
-    for (int r = 0; r < kRows; ++r) s += S.dZ3[r * 4 + j];
-    atomicAdd(&grads[O_B3 + j], s);
-  }
-  // dZ2 = (dZ3 W3) * [H2 > 0]
-  for (int e = tid; e < kRows * NH; e += kThreads) {
-    const int r = e / NH, k = e % NH;
-    float s = 0.f;
-#pragma unroll
-    for (int j = 0; j < NOUT; ++j) s += S.dZ3[r * 4 + j] * S.W3f[j * NH + k];
-    S.dZ2[r * SD + k] = __bfloat162float(S.H2b[r * SH + k]) > 0.f ? s : 0.f;
-  }
-  __syncthreads();
-  // dW2, db2
-  for (int e = tid; e < NH * NH; e += kThreads) {
-    const int m = e / NH, k = e % NH;
-    float s = 0.f;
-    for (int r = 0; r < kRows; ++r) s += S.dZ2[r * SD + m] * __bfloat162float(S.H1b[r * SH + k]);
-    atomicAdd(&grads[O_W2 + e], s);
-  }
-  if (tid < NH) {
-    float s = 0.f;
-    for (int r = 0; r < kRows; ++r) s += S.dZ2[r * SD + tid];
-    atomicAdd(&grads[O_B2 + tid], s);
-  }
-  // dZ1 = (dZ2 W2) * [H1 > 0]
-  for (int e = tid; e < kRows * NH; e += kThreads) {
-    const int r = e / NH, k = e % NH;
-    float s = 0.f;
-    for (int m = 0; m < NH; ++m) s += S.dZ2[r * SD + m] * S.W2f[m * NH + k];
-    S.dZ1[r * SD + k] = __bfloat162float(S.H1b[r * SH + k]) > 0.f ? s : 0.f;
-  }
-  __syncthreads();
-  // dW1, db1
-  for (int e = tid; e < NH * NF; e += kThreads) {
-    const int m = e / NF, k = e % NF;
-    float s = 0.f;
-    for (int r = 0; r < kRows; ++r) s += S.dZ1[r * SD + m] * __bfloat162float(S.Xb[r * SX + k]);
-    atomicAdd(&grads[O_W1 + e], s);
-  }
-  if (tid < NH) {
-    float s = 0.f;
-    for (int r = 0; r < kRows; ++r) s += S.dZ1[r * SD + tid];
-    atomicAdd(&grads[O_B1 + tid], s);
-  }
-  }  // tiles
 }
 
-// Inference alone: the forward pass of k_mlp (same BF16 roundings, same MMA sequence, same
+// Inference: the forward pass of k_mlp (same BF16 roundings, same MMA sequence, same
 // epilogues, so the same outputs) with each warp working through its own tiles of 16 samples.
 // Without the backward buffers a block needs 44 KB of shared memory instead of k_mlp's, so
 // more blocks share an SM, and no block-wide barrier stands between a warp's tiles.
@@ -374,60 +433,207 @@ __global__ void k_adam(int np, float* __restrict__ p, const float* __restrict__ 
   }
 }
 
-// Features of every regional node of a level (layout described at the top of the file).
+// What the features read of a level: the region stencils and, for nodes with several copies, the
+// composite couplings in comp[0..3] (centre, +x, +y, +z; written at the shared nodes only).
+struct FeatArgs {
+  const double* coef;
+  const uint8_t* mult;
+  double* comp[4];
+};
+
+// Composite coupling number p (0: centre, 1..3: +x, +y, +z) of stencil KIND, or -1.
+template <int KIND>
+__device__ __forceinline__ int feature_slot(int p) {
+  return p == 0 ? Sten<KIND>::CENTER : sten_slot<KIND>(p == 1, p == 2, p == 3);
+}
+
+// The composite couplings of the shared nodes, one thread per copy: sums over the copies in
+// ascending slot order.
+template <int KIND>
+__global__ void __launch_bounds__(256)
+k_shared_couplings(int nslots, int n_r, const int* __restrict__ sgrp,
+                   const int* __restrict__ gptr, const int* __restrict__ gslot, FeatArgs A) {
+  for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < nslots; q += gridDim.x * blockDim.x) {
+    const int grp = sgrp[q], n = gslot[q], a = gptr[grp], e = gptr[grp + 1];
+    double s[4] = {};
+    for (int k = a; k < e; ++k)
+#pragma unroll
+      for (int p = 0; p <= Sten<KIND>::DIM; ++p)
+        s[p] += A.coef[(size_t)feature_slot<KIND>(p) * n_r + gslot[k]];
+#pragma unroll
+    for (int p = 0; p <= Sten<KIND>::DIM; ++p) A.comp[p][n] = s[p];
+  }
+}
+
+// The 27 features of regional node n (layout described at the top of the file) and zeros up to
+// NF. Nearly every warp holds a few nodes of an interface: the copies' couplings come from
+// k_shared_couplings, so that reading a shared node is one load from another array and the warp
+// does not wait for a walk over the copies at each of the 21 values (that walk inside the
+// one-pass kernel took it to 1244 us, slower than the three kernels it replaced).
+template <int KIND>
+__device__ __forceinline__ void node_features(const Grid& G, const FeatArgs& A, const RegionDev& R,
+                                              int n, int li, float (&f)[NF]) {
+  using St = Sten<KIND>;
+  int x[3];
+  decode(li, R, x[0], x[1], x[2]);
+  const int stride[3] = {1, R.nx, R.nx * R.ny};
+  const int len[3] = {R.nx, R.ny, R.nz};
+  auto coupling = [&](int p, int m, bool single) {
+    return single ? A.coef[(size_t)feature_slot<KIND>(p) * G.n_r + m] : A.comp[p][m];
+  };
+  const double dn = coupling(0, n, A.mult[n] == 1);
+  const double dref = dn > 0.0 ? dn : 1.0;
+  const double inv_ref = 1.0 / dref;            // one FP64 division per node, not 21
+#pragma unroll
+  for (int q = 0; q < NF; ++q) f[q] = 0.f;
+#pragma unroll
+  for (int a = 0; a < St::DIM; ++a) {
+    int rem = x[a] % 3;
+    if (rem && x[a] - rem + 3 > len[a] - 1) rem = 0;   // no right coarse node in the region
+    if (!rem) continue;
+    const int p0 = n - rem * stride[a];
+    double k[3], d[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int m = p0 + i * stride[a];
+      const bool single = A.mult[m] == 1;
+      if (i < 3) k[i] = coupling(a + 1, m, single);
+      d[i] = coupling(0, m, single);
+    }
+    // ratios in FP64, logarithms in FP32 (the features are FP32 network inputs)
+#pragma unroll
+    for (int e = 0; e < 3; ++e)
+      f[9 * a + e] = fminf(log10f(fmaxf((float)(-k[e] * inv_ref), 1e-12f)), 2.f);
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+      f[9 * a + 3 + i] = fminf(log10f(fmaxf((float)(d[i] * inv_ref), 1e-12f)), 12.f);
+    f[9 * a + 7] = rem == 1 ? (float)(1.0 / 3.0) : (float)(2.0 / 3.0);
+    f[9 * a + 8] = 1.f;
+  }
+}
+
+// Features of every regional node of a level, one 128-byte row per node (16-byte stores when the
+// caller's array allows them).
 template <int KIND>
 __global__ void __launch_bounds__(kTile)
-k_features(Grid G, const double* __restrict__ coef, const uint8_t* __restrict__ mult,
-           const int* __restrict__ gid, const int* __restrict__ cgrp, const int* __restrict__ gptr,
-           const int* __restrict__ gslot, float* __restrict__ feats) {
-  using St = Sten<KIND>;
+k_features(Grid G, FeatArgs A, float* __restrict__ feats) {
+  const bool aligned = (reinterpret_cast<uintptr_t>(feats) & 15) == 0;
   RMG_FOR_NODES(G)
-    int x[3];
-    decode(li, R, x[0], x[1], x[2]);
-    const int stride[3] = {1, R.nx, R.nx * R.ny};
-    float* f = feats + (size_t)n * NF;
-    const double dn = comp_coupling<KIND>(coef, G.n_r, n, St::CENTER, mult, gid, cgrp, gptr, gslot);
-    const double dref = dn > 0.0 ? dn : 1.0;
-    const double inv_ref = 1.0 / dref;            // one FP64 division per node, not 21
-    const int len[3] = {R.nx, R.ny, R.nz};
-    for (int a = 0; a < 3; ++a) {
-      int rem = a < St::DIM ? x[a] % 3 : 0;
-      if (rem && x[a] - rem + 3 > len[a] - 1) rem = 0;   // no right coarse node in the region
-      const int slot = sten_slot<KIND>(a == 0, a == 1, a == 2);
-      if (!rem || slot < 0) {
-        for (int q = 0; q < 9; ++q) f[9 * a + q] = 0.f;
-        continue;
-      }
-      const int p0 = n - rem * stride[a];
-      // ratios in FP64, logarithms in FP32 (the features are FP32 network inputs)
-      for (int e = 0; e < 3; ++e) {
-        const double k = -comp_coupling<KIND>(coef, G.n_r, p0 + e * stride[a], slot, mult, gid,
-                                              cgrp, gptr, gslot);
-        const float v = log10f(fmaxf((float)(k * inv_ref), 1e-12f));
-        f[9 * a + e] = fminf(v, 2.f);
-      }
-      for (int i = 0; i < 4; ++i) {
-        const double d = comp_coupling<KIND>(coef, G.n_r, p0 + i * stride[a], St::CENTER, mult,
-                                             gid, cgrp, gptr, gslot);
-        const float v = log10f(fmaxf((float)(d * inv_ref), 1e-12f));
-        f[9 * a + 3 + i] = fminf(v, 12.f);
-      }
-      f[9 * a + 7] = (float)(rem / 3.0);
-      f[9 * a + 8] = 1.f;
+    float f[NF];
+    node_features<KIND>(G, A, R, n, li, f);
+    if (!aligned) {
+#pragma unroll
+      for (int q = 0; q < NF; ++q) feats[(size_t)n * NF + q] = f[q];
+      continue;
     }
-    for (int q = 27; q < NF; ++q) f[q] = 0.f;
+    float4* row = reinterpret_cast<float4*>(feats + (size_t)n * NF);
+#pragma unroll
+    for (int q = 0; q < NF / 4; ++q)
+      row[q] = make_float4(f[4 * q], f[4 * q + 1], f[4 * q + 2], f[4 * q + 3]);
   RMG_END_FOR_NODES
 }
 
-// Predicted weights -> per-axis interpolation weights (0 along inactive axes).
-__global__ void k_weights_from_out(int n_r, const float* __restrict__ feats,
-                                   const float* __restrict__ out, float* __restrict__ wr) {
-  for (int n = blockIdx.x * blockDim.x + threadIdx.x; n < n_r; n += gridDim.x * blockDim.x)
-    for (int a = 0; a < 3; ++a)
-      wr[(size_t)a * n_r + n] = feats[(size_t)n * NF + 9 * a + 8] > 0.5f ? out[n * 3 + a] : 0.f;
+// Interpolation weights of a level in one pass: features, network and weights of 32 consecutive
+// nodes at a time per warp, the features going to the MMA through shared memory (the BF16 rows
+// of k_mlp_infer, the same operations in the same order). Nothing but the coefficients is read
+// and nothing but the weights written; as three kernels the features (128 bytes a node) went
+// through memory with 4-byte stores 128 bytes apart, and that was most of the time: 939 us for
+// 2.54M nodes of a 7-point level, 300 us in this form. The FP64 pipe bounds it now (a product
+// and a conversion per ratio, about 28 ratios a node, and one division).
+struct WeightsSmem {
+  __nv_bfloat16 W1b[NH * SX];
+  __nv_bfloat16 W2b[NH * SH];
+  __nv_bfloat16 W3b[8 * SH];
+  __nv_bfloat16 Xb[kTile / 32][32 * SX];
+  __nv_bfloat16 Hb[kTile / 32][16 * SH];   // layer-1 output of 16 nodes, then layer 2's in place
+};
+
+__device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
+  const __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
+  return *reinterpret_cast<const uint32_t*>(&v);
 }
 
-size_t mlp_smem() { return sizeof(MlpSmem); }
+// H = relu(acc + bias) as BF16 rows g and g + 8 of a 16-row tile.
+__device__ __forceinline__ void store_relu(__nv_bfloat16* H, const float (&acc)[8][4],
+                                           const float* __restrict__ bias, int g, int t) {
+#pragma unroll
+  for (int nt = 0; nt < 8; ++nt) {
+    const int c = nt * 8 + 2 * t;
+    const float b0 = bias[c], b1 = bias[c + 1];
+    *reinterpret_cast<uint32_t*>(&H[g * SH + c]) =
+        pack_bf16(fmaxf(acc[nt][0] + b0, 0.f), fmaxf(acc[nt][1] + b1, 0.f));
+    *reinterpret_cast<uint32_t*>(&H[(g + 8) * SH + c]) =
+        pack_bf16(fmaxf(acc[nt][2] + b0, 0.f), fmaxf(acc[nt][3] + b1, 0.f));
+  }
+}
+
+template <int KIND>
+__global__ void __launch_bounds__(kTile)
+k_learned_weights(Grid G, FeatArgs A, const float* __restrict__ params, float* __restrict__ wr) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  WeightsSmem& S = *reinterpret_cast<WeightsSmem*>(smem_raw);
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int g = lane >> 2, t = lane & 3;
+  for (int e = tid; e < NH * NF; e += kTile)
+    S.W1b[(e / NF) * SX + e % NF] = __float2bfloat16_rn(params[O_W1 + e]);
+  for (int e = tid; e < NH * NH; e += kTile)
+    S.W2b[(e / NH) * SH + e % NH] = __float2bfloat16_rn(params[O_W2 + e]);
+  for (int e = tid; e < 8 * NH; e += kTile) {
+    const int j = e / NH, k = e % NH;
+    S.W3b[j * SH + k] = __float2bfloat16_rn(j < NOUT ? params[O_W3 + j * NH + k] : 0.f);
+  }
+  __syncthreads();
+  __nv_bfloat16* X = S.Xb[warp];
+  __nv_bfloat16* H = S.Hb[warp];
+  for (int ti = blockIdx.x; ti < G.ntiles; ti += gridDim.x) {
+    const Tile tile = G.tiles[ti];
+    const RegionDev R = G.regions[tile.region];
+    const int l0 = tile.start + warp * 32;             // first node of the warp in the region
+    const int nodes = min(32, R.nx * R.ny * R.nz - l0);
+    if (nodes <= 0) continue;
+    float f[NF];
+    if (lane < nodes) {
+      node_features<KIND>(G, A, R, R.off + l0 + lane, l0 + lane, f);
+    } else {
+#pragma unroll
+      for (int q = 0; q < NF; ++q) f[q] = 0.f;
+    }
+    __syncwarp();                                      // the previous tile's reads are done
+    uint4* row = reinterpret_cast<uint4*>(&X[lane * SX]);
+#pragma unroll
+    for (int q = 0; q < NF / 8; ++q)
+      row[q] = make_uint4(pack_bf16(f[8 * q], f[8 * q + 1]), pack_bf16(f[8 * q + 2], f[8 * q + 3]),
+                          pack_bf16(f[8 * q + 4], f[8 * q + 5]),
+                          pack_bf16(f[8 * q + 6], f[8 * q + 7]));
+    __syncwarp();
+    for (int r0 = 0; r0 < nodes; r0 += 16) {
+      {
+        float acc[8][4] = {};
+        warp_mma<8, NF>(X, SX, r0, S.W1b, SX, acc);
+        __syncwarp();                                  // the last 16 nodes' layer 2 is read
+        store_relu(H, acc, params + O_B1, g, t);
+      }
+      __syncwarp();
+      {
+        float acc[8][4] = {};
+        warp_mma<8, NH>(H, SH, 0, S.W2b, SH, acc);
+        __syncwarp();                                  // layer 1's values are all read
+        store_relu(H, acc, params + O_B2, g, t);
+      }
+      __syncwarp();
+      float acc[1][4] = {};
+      warp_mma<1, NH>(H, SH, 0, S.W3b, SH, acc);
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const int i = r0 + g + (q >= 2 ? 8 : 0), col = 2 * t + (q & 1);
+        if (col >= NOUT || i >= nodes) continue;
+        const float z = acc[0][q] + params[O_B3 + col];
+        const bool active = __bfloat162float(X[i * SX + 9 * col + 8]) > 0.5f;
+        wr[(size_t)col * G.n_r + R.off + l0 + i] = active ? 1.f / (1.f + __expf(-z)) : 0.f;
+      }
+    }
+  }
+}
 
 }  // namespace
 }  // namespace rmg
@@ -458,34 +664,64 @@ rmg_status mlp_guard(rmg_ctx* ctx, F&& f) {
   }
 }
 
-void mlp_launch(rmg_mlp* net, int n, const float* feats, const float* labels, const float* mask,
-                int mode, int sample, int rows, unsigned long long seed, float inv_norm,
-                float* out, float* loss) {
+void mlp_infer(rmg_mlp* net, int n, const float* feats, float* out) {
   Ctx& c = net->ctx->c;
-  if (mode == 0 && !sample) {                    // inference over samples 0 .. n-1
-    const int smem = (int)sizeof(MlpInferSmem);
-    RMG_CUDA(cudaFuncSetAttribute(k_mlp_infer, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  smem));
-    int per_sm = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_mlp_infer, kThreads, smem) !=
-        cudaSuccess) {
-      cudaGetLastError();
-      per_sm = 1;
-    }
-    const long long warps = ((long long)n + kWarpRows - 1) / kWarpRows;
-    const long long want = (warps + kThreads / 32 - 1) / (kThreads / 32);
-    const int blocks = (int)std::max<long long>(
-        1, std::min<long long>(want, (long long)c.nsm * std::max(1, per_sm)));
-    k_mlp_infer<<<blocks, kThreads, smem, c.stream>>>(net->p.get(), n, feats, out);
-    RMG_LAUNCHED();
-    return;
+  const int smem = (int)sizeof(MlpInferSmem);
+  RMG_CUDA(cudaFuncSetAttribute(k_mlp_infer, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+  int per_sm = 0;
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_mlp_infer, kThreads, smem) !=
+      cudaSuccess) {
+    cudaGetLastError();
+    per_sm = 1;
   }
-  const int smem = (int)mlp_smem();
+  const long long warps = ((long long)n + kWarpRows - 1) / kWarpRows;
+  const long long want = (warps + kThreads / 32 - 1) / (kThreads / 32);
+  const int blocks = (int)std::max<long long>(
+      1, std::min<long long>(want, (long long)c.nsm * std::max(1, per_sm)));
+  k_mlp_infer<<<blocks, kThreads, smem, c.stream>>>(net->p.get(), n, feats, out);
+  RMG_LAUNCHED();
+}
+
+// Gradient (into net->g) and loss over `rows` rows. The shared memory of k_mlp leaves one CTA
+// per SM, so one CTA per SM strides over the tiles.
+void mlp_backward(rmg_mlp* net, int n, const float* feats, const float* labels, const float* mask,
+                  int sample, int rows, unsigned long long seed, float inv_norm, float* loss) {
+  Ctx& c = net->ctx->c;
+  const int smem = (int)sizeof(MlpSmem);
   RMG_CUDA(cudaFuncSetAttribute(k_mlp, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-  const long long tiles = (rows + kRows - 1) / kRows;
-  const int blocks = (int)std::min<long long>(tiles, (long long)c.nsm * 2);
-  k_mlp<<<blocks, kThreads, smem, c.stream>>>(net->p.get(), n, tiles, feats, labels, mask, mode,
-                                             sample, seed, inv_norm, out, net->g.get(), loss);
+  const long long tiles = ((long long)rows + kRows - 1) / kRows;
+  const int blocks = (int)std::min<long long>(tiles, (long long)c.nsm);
+  k_mlp<<<blocks, kThreads, smem, c.stream>>>(net->p.get(), n, tiles, feats, labels, mask, sample,
+                                             seed, inv_norm, net->g.get(), loss);
+  RMG_LAUNCHED();
+}
+
+// The couplings of the level's shared nodes go to four of its FP64 cycle vectors, which hold
+// nothing between calls.
+template <int KIND>
+FeatArgs feat_args(const Hier& h, int level) {
+  const Level& L = *h.lv[level];
+  const LevelVecs<double>& V = h.v64[level];
+  FeatArgs A{L.coef.get(), L.mult.get(), {V.u2.get(), V.r.get(), V.y.get(), V.d.get()}};
+  if (L.nslots) {
+    k_shared_couplings<KIND><<<persistent_grid(*h.c, (L.nslots + 255) / 256), 256, 0,
+                               h.c->stream>>>(L.nslots, L.n_r, L.sgrp.get(), L.gptr.get(),
+                                              L.gslot.get(), A);
+    RMG_LAUNCHED();
+  }
+  return A;
+}
+
+template <int KIND>
+void learned_weights(const rmg_mlp& net, const Hier& h, int level, float* wr) {
+  const Ctx& c = *h.c;
+  const Level& L = *h.lv[level];
+  const FeatArgs A = feat_args<KIND>(h, level);
+  const Grid G = L.grid();
+  const int smem = (int)sizeof(WeightsSmem);
+  const int per_sm = resident_per_sm_smem((const void*)k_learned_weights<KIND>, smem);
+  k_learned_weights<KIND><<<persistent_grid(c, G.ntiles, per_sm), kTile, smem, c.stream>>>(
+      G, A, net.p.get(), wr);
   RMG_LAUNCHED();
 }
 }  // namespace
@@ -502,7 +738,7 @@ rmg_status rmg_mlp_create(rmg_ctx* ctx, const float* init_params, rmg_mlp** out)
   net->ctx = ctx;
   rmg_status st = mlp_guard(ctx, [&] {
     RMG_REQUIRE(init_params, RMG_ERR_ARG, "init_params is NULL");
-    net->p.alloc(NPARAMS); net->g.alloc(NPARAMS); net->m.alloc(NPARAMS); net->v.alloc(NPARAMS);
+    net->p.alloc(NPARAMS); net->g.alloc(NPARAMS + 1); net->m.alloc(NPARAMS); net->v.alloc(NPARAMS);
     RMG_CUDA(cudaMemcpy(net->p.get(), init_params, NPARAMS * sizeof(float), cudaMemcpyHostToDevice));
     RMG_CUDA(cudaMemset(net->m.get(), 0, NPARAMS * sizeof(float)));
     RMG_CUDA(cudaMemset(net->v.get(), 0, NPARAMS * sizeof(float)));
@@ -529,7 +765,7 @@ rmg_status rmg_mlp_forward(rmg_mlp* net, int n, const float* feats, float* out) 
   if (!net) return RMG_ERR_ARG;
   return mlp_guard(net->ctx, [&] {
     RMG_REQUIRE(n > 0 && feats && out, RMG_ERR_ARG, "bad arguments");
-    mlp_launch(net, n, feats, nullptr, nullptr, 0, 0, n, 0, 0.f, out, nullptr);
+    mlp_infer(net, n, feats, out);
   });
 }
 
@@ -539,13 +775,15 @@ rmg_status rmg_mlp_gradient(rmg_mlp* net, int n, const float* feats, const float
   return mlp_guard(net->ctx, [&] {
     RMG_REQUIRE(n > 0 && feats && labels && mask && grad && loss, RMG_ERR_ARG, "bad arguments");
     Ctx& c = net->ctx->c;
-    net->loss.ensure(1);
-    RMG_CUDA(cudaMemsetAsync(net->g.get(), 0, NPARAMS * sizeof(float), c.stream));
-    RMG_CUDA(cudaMemsetAsync(net->loss.get(), 0, sizeof(float), c.stream));
-    mlp_launch(net, n, feats, labels, mask, 1, 0, n, 0, 1.f / (3.f * n), nullptr, net->loss.get());
+    // gradient and loss side by side (g has room for both): one memset and one copy back
+    RMG_CUDA(cudaMemsetAsync(net->g.get(), 0, (NPARAMS + 1) * sizeof(float), c.stream));
+    mlp_backward(net, n, feats, labels, mask, 0, n, 0, 1.f / (3.f * n), net->g.get() + NPARAMS);
+    std::vector<float> host(NPARAMS + 1);
+    RMG_CUDA(cudaMemcpyAsync(host.data(), net->g.get(), (NPARAMS + 1) * sizeof(float),
+                             cudaMemcpyDeviceToHost, c.stream));
     RMG_CUDA(cudaStreamSynchronize(c.stream));
-    RMG_CUDA(cudaMemcpy(grad, net->g.get(), NPARAMS * sizeof(float), cudaMemcpyDeviceToHost));
-    RMG_CUDA(cudaMemcpy(loss, net->loss.get(), sizeof(float), cudaMemcpyDeviceToHost));
+    std::copy(host.begin(), host.begin() + NPARAMS, grad);
+    *loss = host[NPARAMS];
   });
 }
 
@@ -562,9 +800,9 @@ rmg_status rmg_mlp_train(rmg_mlp* net, int n, const float* feats, const float* l
     const float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
     for (int s = 0; s < steps; ++s) {
       RMG_CUDA(cudaMemsetAsync(net->g.get(), 0, NPARAMS * sizeof(float), c.stream));
-      mlp_launch(net, n, feats, labels, mask, 1, 1, batch,
-                 seed * 0x100000001B3ull + (unsigned long long)(net->steps_done + s) * batch,
-                 1.f / (3.f * batch), nullptr, net->loss.get() + s);
+      mlp_backward(net, n, feats, labels, mask, 1, batch,
+                   seed * 0x100000001B3ull + (unsigned long long)(net->steps_done + s) * batch,
+                   1.f / (3.f * batch), net->loss.get() + s);
       const int t = net->steps_done + s + 1;
       const float c1 = 1.f / (1.f - powf(b1, (float)t)), c2 = 1.f / (1.f - powf(b2, (float)t));
       k_adam<<<(NPARAMS + 255) / 256, 256, 0, c.stream>>>(NPARAMS, net->p.get(), net->g.get(),
@@ -588,9 +826,8 @@ rmg_status rmg_hier_mlp_features(rmg_hier* hh, int level, float* feats) {
     Level& L = *h.lv[level];
     const Grid G = L.grid();
     const int gb = persistent_grid(*h.c, G.ntiles);
-#define RMG_FEAT(K)                                                                            \
-  k_features<K><<<gb, kTile, 0, h.c->stream>>>(G, L.coef.get(), L.mult.get(), L.gid.get(),     \
-                                               L.cgrp.get(), L.gptr.get(), L.gslot.get(), feats)
+#define RMG_FEAT(K) \
+  k_features<K><<<gb, kTile, 0, h.c->stream>>>(G, feat_args<K>(h, level), feats)
     switch (L.kind) {
       case 5: RMG_FEAT(5); break;
       case 7: RMG_FEAT(7); break;
@@ -604,22 +841,15 @@ rmg_status rmg_hier_mlp_features(rmg_hier* hh, int level, float* feats) {
 
 rmg_status rmg_hier_mlp_weights(rmg_hier* hh, int level, rmg_mlp* net, float* wr) {
   if (!hh || !net) return RMG_ERR_ARG;
-  Hier& h = hh->h;
-  const int n_r = (level >= 0 && level < h.levels()) ? h.lv[level]->n_r : 0;
-  rmg_status st = mlp_guard(h.layout->ctx, [&] {
-    RMG_REQUIRE(n_r > 0 && wr, RMG_ERR_ARG, "bad arguments");
-    h.mlp_feats.ensure((size_t)h.lv[0]->n_r * NF);       // sized for the finest level, kept
-    h.mlp_out.ensure((size_t)h.lv[0]->n_r * 3);
-  });
-  if (st != RMG_OK) return st;
-  st = rmg_hier_mlp_features(hh, level, h.mlp_feats.get());
-  if (st != RMG_OK) return st;
-  return mlp_guard(h.layout->ctx, [&] {
-    mlp_launch(net, n_r, h.mlp_feats.get(), nullptr, nullptr, 0, 0, n_r, 0, 0.f,
-               h.mlp_out.get(), nullptr);
-    k_weights_from_out<<<persistent_grid(*h.c, (n_r + 255) / 256), 256, 0, h.c->stream>>>(
-        n_r, h.mlp_feats.get(), h.mlp_out.get(), wr);
-    RMG_LAUNCHED();
+  return mlp_guard(hh->h.layout->ctx, [&] {
+    Hier& h = hh->h;
+    RMG_REQUIRE(level >= 0 && level < h.levels() && wr, RMG_ERR_ARG, "bad arguments");
+    switch (h.lv[level]->kind) {
+      case 5: learned_weights<5>(*net, h, level, wr); break;
+      case 7: learned_weights<7>(*net, h, level, wr); break;
+      case 9: learned_weights<9>(*net, h, level, wr); break;
+      default: learned_weights<27>(*net, h, level, wr); break;
+    }
   });
 }
 
