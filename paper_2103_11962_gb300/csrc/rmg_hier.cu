@@ -530,6 +530,45 @@ struct Exec {
     ++launches;
   }
 
+  // Levels l0 .. coarsest in one kernel (rmg_tail.cu); b of level l0 holds the right-hand side.
+  void tail(int l0, bool down, bool solve, bool up) {
+    TailArgs<VT, CT> A{};
+    const int Lv = h.levels();
+    A.nlev = Lv - l0;
+    for (int l = l0; l < Lv; ++l) {
+      const Level& L = *h.lv[l];
+      LevelVecs<VT>& v = V(l);
+      const TailGeometry& g = h.tail_geo[l];
+      A.lev[l - l0] = TailLevel<VT, CT>{
+          L.n_r, L.nslots, g.info.get(), L.regions.get(), L.mask.get(), L.mult.get(),
+          g.coloured.get(), {}, g.slots.get(), L.gslot.get(), coef(l), dinv(l), c1(l, 0),
+          c2(l, 0), h.stored[l] ? pw(l) : nullptr, v.u.get(), v.u2.get(), v.b.get(), v.r.get(),
+          v.y.get(), v.d.get()};
+      std::copy(g.cstart, g.cstart + 9, A.lev[l - l0].cstart);
+    }
+    A.smoother = h.o.smoother;
+    A.nu1 = h.o.nu1;
+    A.nu2 = h.o.nu2;
+    A.degree = h.o.cheb_degree;
+    A.omega = VT(h.o.omega);
+    A.down = down;
+    A.solve = solve;
+    A.up = up;
+    A.nc = h.nc;
+    A.refine = h.coarse_refine;
+    A.cu2slot = h.cu2slot.get();
+    A.cidx = h.cidx.get();
+    A.gid = h.lv[Lv - 1]->gid.get();
+    A.Ainv32 = h.Ainv32.get();
+    A.A = h.X.get();
+    A.Ainv = h.Ainv.get();
+    A.cscale = h.cscale.get();
+    A.xc = h.xc.get();
+    A.cres = h.cres.get();
+    tail_launch<VT, CT>(h.lv[0]->dim, h.lv[0]->B, h.tail_blocks, A, st);
+    ++launches;
+  }
+
   int level0_flips() const {
     if (h.o.smoother == RMG_SMOOTHER_GS) return 0;       // Gauss-Seidel updates u in place
     const int per = (h.o.smoother == RMG_SMOOTHER_JACOBI) ? 1 : h.o.cheb_degree;
@@ -542,13 +581,23 @@ struct Exec {
     oth.assign(Lv, nullptr);
     for (int l = 0; l < Lv; ++l) { cur[l] = V(l).u.get(); oth[l] = V(l).u2.get(); }
     if (Lv > 1 && (level0_flips() & 1)) std::swap(cur[0], oth[0]);
-    for (int l = 0; l < Lv - 1; ++l) {
+    const int l0 = h.tail0 > 0 ? h.tail0 : Lv - 1;     // levels below l0: their own launches
+    for (int l = 0; l < l0; ++l) {
       smooth(l, h.o.nu1, true);
       residual(l);
       restrict_to(l);
     }
-    coarse(Lv - 1);
-    for (int l = Lv - 2; l >= 0; --l) {
+    if (h.tail0 <= 0) {
+      coarse(Lv - 1);
+    } else if (h.tail_solve) {
+      tail(l0, true, true, true);
+    } else {
+      tail(l0, true, false, false);
+      coarse(Lv - 1);
+      tail(l0, false, false, true);
+    }
+    if (h.tail0 > 0 && l0 < Lv - 1 && (level0_flips() & 1)) flip(l0);
+    for (int l = l0 - 1; l >= 0; --l) {
       prolong(l);
       smooth(l, h.o.nu2, false, l == 0, true);
     }
@@ -648,6 +697,8 @@ static void coarsen_level(Hier& h, const Level& F, Level& C) {
   C.coef.alloc((size_t)C.B * C.B * C.kind * C.n_r);
 }
 
+static void tail_levels(Hier& h);
+
 void hier_build(Hier& h) {
   Ctx& c = *h.c;
   RMG_REQUIRE(h.layout->has_operator, RMG_ERR_STATE, "rmg_setup needs an operator on the layout");
@@ -737,7 +788,45 @@ void hier_build(Hier& h) {
   h.cscale.alloc(nd); h.cres.alloc(nd); h.cw32.alloc(nd); h.cnorm.alloc(5); h.cerr.alloc(1);
   h.xc.alloc(nd); h.rc.alloc(nd);
   RMG_CUDA(cudaMemsetAsync(h.xc.get(), 0, h.xc.bytes(), c.stream));
+  tail_levels(h);
   RMG_CUDA(cudaStreamSynchronize(c.stream));
+}
+
+// Levels of the one-kernel coarse end (rmg_tail.cu). The kernel has 16 SMs, so a level belongs in
+// it while the GPU's other SMs would save less than the launches cost. A sweep as two launches
+// takes 6 to 8 us up to about 25k nodes of a 27-point level; inside the kernel its two phases
+// take 5 us for 12k nodes in FP32 (L2 latency and barriers; the second round of 16k threads comes
+// at 16k nodes) and 6 us for 3k nodes in FP64 (64 DFMA/clk for 16 SMs). The lines: 24k nodes of
+// a 27-point level in FP32, 8k in FP64. The dense solve goes inside up to kTailDense unknowns:
+// every refinement step reads the FP64 matrix once, 4.7 MB there, about 3 us on 16 SMs.
+// Measured, launches against one kernel for the coarse end: V-cycle of 1.5M nodes in FP64
+// 646 -> 588 us; solves of 27k nodes 2852 -> 2164 us and of 572k nodes with Gauss-Seidel
+// 13.7 -> 11.3 ms.
+static void tail_levels(Hier& h) {
+  Ctx& c = *h.c;
+  const int Lv = h.levels(), B = h.lv[0]->B, dim = h.lv[0]->dim;
+  h.tail0 = -1;
+  h.tail_geo = std::vector<TailGeometry>(Lv);
+  if (Lv < 2 || h.o.nu1 < 1 || !h.dense_ok) return;
+  const long long most = h.mixed() ? 660000 : 210000;      // coefficients of a sweep
+  int l0 = Lv;
+  while (l0 > 1 && Lv - l0 < kTailLevels) {
+    const Level& L = *h.lv[l0 - 1];
+    bool ok = (long long)L.n_r * (dim == 3 ? 27 : 9) * B * B <= most * (B == 1 ? 1 : 2);
+    for (int d : L.hdims) ok = ok && d < 1024;              // packed positions
+    if (!ok) break;
+    --l0;
+  }
+  h.tail_solve = (long long)h.nc * B <= kTailDense;
+  // two launches around a separate solve pay only with a smoothed level inside
+  if (l0 >= Lv || (!h.tail_solve && l0 >= Lv - 1)) return;
+  h.tail_blocks = !h.mixed() ? tail_cluster<double, double>(dim, B)
+                  : h.o.precision == RMG_PREC_FP32 ? tail_cluster<float, float>(dim, B)
+                                                   : tail_cluster<float, __nv_bfloat16>(dim, B);
+  if (!h.tail_blocks) return;
+  for (int l = l0; l < Lv; ++l)
+    h.tail_geo[l].build(c, *h.lv[l], h.o.smoother == RMG_SMOOTHER_GS && l + 1 < Lv);
+  h.tail0 = l0;
 }
 
 // D~^-1 = (Psi^T Psi diag([[A]]))^-1, per component of a block operator (diagonal of A_cc).
@@ -1122,14 +1211,18 @@ static bool coarse_factor_mixed(Hier& h, int nd) {
   RMG_CUDA(cudaStreamSynchronize(st));
   const double b2 = h.pinned[0], r0 = h.pinned[1], r1 = h.pinned[2], r2 = h.pinned[3];
   if (err || !(b2 > 0.0) || !std::isfinite(r0) || !std::isfinite(r2) || !(r0 > 0.0)) return false;
-  // per-step contraction from the last two steps (the first one also removes the FP32
-  // rounding of the right-hand side), in norms
-  const double rho = std::sqrt(std::max(r2, 1e-300) / std::max(r1, 1e-300));
-  const double rel0 = std::sqrt(r0 / b2);
+  // per-step contraction in norms: of the second step (the first one also removes the FP32
+  // rounding of the right-hand side) unless that step ends at the FP64 floor, where the ratio
+  // says nothing about the contraction
+  const double rel0 = std::sqrt(r0 / b2), rel1 = std::sqrt(r1 / b2), rel2 = std::sqrt(r2 / b2);
+  const double rho = rel2 > 1e-15 ? rel2 / std::max(rel1, 1e-300) : rel1 / rel0;
   if (!(rho < 0.1)) return false;
+  // the steps that bring the relative residual to 1e-15 with two digits to spare, and no fewer
+  // than the test vector took
+  const int seen = rel1 <= 1e-15 ? 1 : rel2 <= 1e-15 ? 2 : 3;
   int steps = 1;
   double rel = rel0 * std::max(rho, 1e-16);
-  while (rel > 1e-15 && steps < 8) {
+  while ((rel > 1e-17 || steps < seen) && steps < 8) {
     rel *= std::max(rho, 1e-16);
     ++steps;
   }

@@ -4,6 +4,7 @@
 #include <memory>
 
 #include "rmg_internal.cuh"
+#include "rmg_tail.cuh"
 
 namespace rmg {
 
@@ -87,6 +88,12 @@ struct Hier {
   // while the device flag Scalars::half_asym is 0
   bool half_on = false;
   DBuf<float> half32;
+  // coarse end of the cycle in one kernel (rmg_tail.cu): first level it takes (-1: none), whether
+  // the dense solve is inside, the cluster's blocks, and geometry per level
+  int tail0 = -1;
+  bool tail_solve = false;
+  int tail_blocks = 0;
+  std::vector<TailGeometry> tail_geo;
 
   ~Hier();
   int levels() const { return (int)lv.size(); }

@@ -571,7 +571,7 @@ __global__ void k_gs_zero(int n, const VT* __restrict__ b, VT* __restrict__ r,
 // parities of i, j, l for 9/27-point ones (4 colours in 2D, 8 in 3D). Nodes of one colour are
 // never coupled by the stencil.
 template <int KIND>
-__device__ __forceinline__ int gs_colour_of(int i, int j, int l) {
+__host__ __device__ __forceinline__ int gs_colour_of(int i, int j, int l) {
   return (KIND == 5 || KIND == 7) ? ((i + j + l) & 1) : ((i & 1) | ((j & 1) << 1) | ((l & 1) << 2));
 }
 
