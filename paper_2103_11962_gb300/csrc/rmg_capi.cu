@@ -114,6 +114,8 @@ rmg_status rmg_create(rmg_ctx** out, int device, void* stream) {
     RMG_CUDA(cudaMemset(ctx->c.d_err.get(), 0, sizeof(int)));
     ctx->c.max_partials = ctx->c.nsm * 8;
     ctx->c.partials.alloc(2 * ctx->c.max_partials);   // room for two fused reductions
+    ctx->c.arrived.alloc(1);
+    RMG_CUDA(cudaMemset(ctx->c.arrived.get(), 0, ctx->c.arrived.bytes()));
   });
   if (st != RMG_OK) {
     delete ctx;

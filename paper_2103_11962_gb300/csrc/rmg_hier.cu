@@ -171,20 +171,91 @@ __global__ void k_coarse_scatter(int n_r, int B, const int* __restrict__ gid,
   }
 }
 
-// PCG scalar updates (single thread)
-__global__ void k_alpha(Scalars* sc) { sc->alpha = sc->rz / sc->pq; }
-__global__ void k_beta(Scalars* sc, int flexible) {
-  // flexible (Polak-Ribiere) form: beta = r.(z - z_old) / rz_old, with r.z_old in sc->beta
-  const double num = flexible ? sc->rz_new - sc->beta : sc->rz_new;
-  sc->beta = num / sc->rz;
-  sc->rz = sc->rz_new;
+// ---- sums over the whole vector that end in the kernel that forms them: every block leaves its
+// partial sums, and the block that arrives last adds them up, in the same order whichever it is,
+// and updates the scalars of the iteration. As separate kernels (partials, total, scalar update)
+// an iteration had seven single-block launches of 2 us more.
+struct Arrive {
+  double* partials;
+  unsigned* count;      // zero between kernels
+};
+
+// True in the block that arrives last; its threads see all partials then.
+__device__ __forceinline__ bool last_block(const Arrive& A) {
+  __shared__ bool last;
+  if (threadIdx.x == 0) {
+    __threadfence();
+    last = atomicAdd(A.count, 1u) == gridDim.x - 1;
+    if (last) *A.count = 0u;
+    __threadfence();
+  }
+  __syncthreads();
+  return last;
 }
 
-// x += alpha p, r -= alpha q, partial sums of r.r (all FP64).
+// Sum of partials[0, np) in the order of k_finalize (valid in thread 0).
+__device__ __forceinline__ double total(const double* partials, int np) {
+  double s = 0.0;
+  for (int k = threadIdx.x; k < np; k += blockDim.x) s += __ldcg(partials + k);
+  return block_sum<256>(s);
+}
+
+// r.z -> beta (and the next rz): the plain form, or the flexible (Polak-Ribiere) one
+// beta = r.(z - z_old) / rz_old.
+__device__ __forceinline__ void set_beta(Scalars* sc, double rz_new, double rz_old_z, bool flexible) {
+  const double num = flexible ? rz_new - rz_old_z : rz_new;
+  sc->beta = num / sc->rz;
+  sc->rz = rz_new;
+}
+
+// What follows a dot product of CG: alpha = rz / (p.q), beta from r.z, or the first rz.
+enum CgDot : int { CG_ALPHA, CG_BETA, CG_RZ };
+__global__ void __launch_bounds__(256)
+k_cg_dot(int n, int n_nodes, const double* __restrict__ x, const double* __restrict__ y,
+         const uint8_t* __restrict__ mult, Arrive A, Scalars* sc, int what) {
+  double s = 0.0;
+  for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x)
+    s = fma(x[k] * inv_mult<double>(mult[k < n_nodes ? k : k % n_nodes]), y[k], s);
+  s = block_sum<256>(s);
+  if (threadIdx.x == 0) A.partials[blockIdx.x] = s;
+  if (!last_block(A)) return;
+  s = total(A.partials, gridDim.x);
+  if (threadIdx.x != 0) return;
+  if (what == CG_ALPHA) sc->alpha = sc->rz / s;
+  else if (what == CG_BETA) set_beta(sc, s, 0.0, false);
+  else sc->rz = s;
+}
+
+// The two products of the flexible form in FP64 (Gauss-Seidel cycle): r.z and r.z_old, then
+// z_old = z and beta.
+__global__ void __launch_bounds__(256)
+k_cg_flex64(int n, int n_nodes, const double* __restrict__ r, const double* __restrict__ z,
+            double* __restrict__ zold, const uint8_t* __restrict__ mult, Arrive A, Scalars* sc) {
+  double s0 = 0.0, s1 = 0.0;
+  for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
+    const double rk = r[k] * inv_mult<double>(mult[k < n_nodes ? k : k % n_nodes]);
+    s0 = fma(rk, z[k], s0);
+    s1 = fma(rk, zold[k], s1);
+    zold[k] = z[k];
+  }
+  s0 = block_sum<256>(s0);
+  s1 = block_sum<256>(s1);
+  if (threadIdx.x == 0) {
+    A.partials[blockIdx.x] = s0;
+    A.partials[gridDim.x + blockIdx.x] = s1;
+  }
+  if (!last_block(A)) return;
+  s0 = total(A.partials, gridDim.x);
+  s1 = total(A.partials + gridDim.x, gridDim.x);
+  if (threadIdx.x == 0) set_beta(sc, s0, s1, true);
+}
+
+// x += alpha p, r -= alpha q; r.r (all FP64) goes to page-locked host memory, where the host
+// reads it after the stream has finished.
 __global__ void __launch_bounds__(256)
 k_cg_update(int n, int n_nodes, const double* __restrict__ p, const double* __restrict__ q,
             const uint8_t* __restrict__ mult, const Scalars* __restrict__ sc,
-            double* __restrict__ x, double* __restrict__ r, double* __restrict__ partials) {
+            double* __restrict__ x, double* __restrict__ r, Arrive A, double* host_rr) {
   const double a = sc->alpha;
   double s = 0.0;
   for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
@@ -194,7 +265,10 @@ k_cg_update(int n, int n_nodes, const double* __restrict__ p, const double* __re
     s = fma(rk * inv_mult<double>(mult[k < n_nodes ? k : k % n_nodes]), rk, s);
   }
   s = block_sum<256>(s);
-  if (threadIdx.x == 0) partials[blockIdx.x] = s;
+  if (threadIdx.x == 0) A.partials[blockIdx.x] = s;
+  if (!last_block(A)) return;
+  s = total(A.partials, gridDim.x);
+  if (threadIdx.x == 0) *host_rr = s;
 }
 
 // Mixed-precision cycle. The FP32 (or BF16-coefficient) V-cycle is the preconditioner of a
@@ -206,12 +280,12 @@ k_cg_update(int n, int n_nodes, const double* __restrict__ p, const double* __re
 // or overflow in FP32 squares and products). zscale = 1 / rscale undoes it (exactly).
 
 // x += alpha p, r -= alpha q (FP64); r32 = FP32(r * rscale), the cycle's right-hand side;
-// partial sums of r.r / mult in FP64.
+// r.r / mult in FP64 to the host.
 __global__ void __launch_bounds__(256)
 k_cg_update_mixed(int n, int n_nodes, const double* __restrict__ p, const double* __restrict__ q,
                   const uint8_t* __restrict__ mult, const Scalars* __restrict__ sc,
                   double rscale, double* __restrict__ x, double* __restrict__ r,
-                  float* __restrict__ r32, double* __restrict__ partials) {
+                  float* __restrict__ r32, Arrive A, double* host_rr) {
   const double a = sc->alpha;
   double s = 0.0;
   for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
@@ -222,7 +296,10 @@ k_cg_update_mixed(int n, int n_nodes, const double* __restrict__ p, const double
     s = fma(rk * inv_mult<double>(mult[k < n_nodes ? k : k % n_nodes]), rk, s);
   }
   s = block_sum<256>(s);
-  if (threadIdx.x == 0) partials[blockIdx.x] = s;
+  if (threadIdx.x == 0) A.partials[blockIdx.x] = s;
+  if (!last_block(A)) return;
+  s = total(A.partials, gridDim.x);
+  if (threadIdx.x == 0) *host_rr = s;
 }
 
 // r32 = FP32(r * rscale): the cycle's right-hand side at a (re)start of the iteration.
@@ -232,14 +309,14 @@ __global__ void k_to_f32_scaled(int n, const double* __restrict__ r, double rsca
     r32[k] = (float)(r[k] * rscale);
 }
 
-// Partial sums of r.z and r.z_old in FP64 (the FP32 values convert exactly), times zscale;
+// r.z and r.z_old in FP64 (the FP32 values convert exactly), times zscale, and beta from them;
 // the FP32 cycle output z then becomes z_old. Partials of r.z go to partials[0, gridDim), those
 // of r.z_old to partials[gridDim, 2 gridDim). Four consecutive FP32 entries per thread step
 // (16-byte loads); the entries past the last multiple of four take a scalar tail.
 __global__ void __launch_bounds__(256)
 k_flex_dots(int n, int n_nodes, const double* __restrict__ r, const float* __restrict__ z,
-            float* __restrict__ zold, const uint8_t* __restrict__ mult, double zscale,
-            double* __restrict__ partials) {
+            float* __restrict__ zold, const uint8_t* __restrict__ mult, double zscale, Arrive A,
+            Scalars* sc) {
   double s0 = 0.0, s1 = 0.0;
   const int n4 = n >> 2;
   const int tid = blockIdx.x * blockDim.x + threadIdx.x, nth = gridDim.x * blockDim.x;
@@ -266,17 +343,20 @@ k_flex_dots(int n, int n_nodes, const double* __restrict__ r, const float* __res
   s0 = block_sum<256>(s0 * zscale);
   s1 = block_sum<256>(s1 * zscale);
   if (threadIdx.x == 0) {
-    partials[blockIdx.x] = s0;
-    partials[gridDim.x + blockIdx.x] = s1;
+    A.partials[blockIdx.x] = s0;
+    A.partials[gridDim.x + blockIdx.x] = s1;
   }
+  if (!last_block(A)) return;
+  s0 = total(A.partials, gridDim.x);
+  s1 = total(A.partials + gridDim.x, gridDim.x);
+  if (threadIdx.x == 0) set_beta(sc, s0, s1, true);
 }
 
-// First direction after a (re)start: partial sums of r.z in FP64, p = z * zscale (FP64),
-// z_old = z.
+// First direction after a (re)start: rz = r.z in FP64, p = z * zscale (FP64), z_old = z.
 __global__ void __launch_bounds__(256)
 k_start_dir(int n, int n_nodes, const double* __restrict__ r, const float* __restrict__ z,
             const uint8_t* __restrict__ mult, double zscale, double* __restrict__ p,
-            float* __restrict__ zold, double* __restrict__ partials) {
+            float* __restrict__ zold, Arrive A, Scalars* sc) {
   double s = 0.0;
   for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
     const float zk = z[k];
@@ -286,7 +366,10 @@ k_start_dir(int n, int n_nodes, const double* __restrict__ r, const float* __res
     zold[k] = zk;
   }
   s = block_sum<256>(s);
-  if (threadIdx.x == 0) partials[blockIdx.x] = s;
+  if (threadIdx.x == 0) A.partials[blockIdx.x] = s;
+  if (!last_block(A)) return;
+  s = total(A.partials, gridDim.x);
+  if (threadIdx.x == 0) sc->rz = s;
 }
 
 __global__ void k_axpy_neg(int n, const double* __restrict__ z, double* __restrict__ e) {
@@ -1764,6 +1847,9 @@ void pcg_solve(Hier& h, const double* b, double* xout, double rtol, int maxit, d
   double* rvec = h.v64[0].b.get();     // the V-cycle reads its right-hand side here
   double* zvec = h.v64[0].u.get();     // and leaves its result here (FP64 cycle)
   double* breg = h.tmp.get();
+  const Arrive arrive{c.partials.get(), c.arrived.get()};
+  double* host_rr = nullptr;           // device address of pinned[2]
+  RMG_CUDA(cudaHostGetDevicePointer((void**)&host_rr, h.pinned + 2, 0));
   const auto t0 = std::chrono::steady_clock::now();
   comp_to_reg(c, L0, b, breg, true);
   comp_to_reg(c, L0, xout, h.x.get(), true);
@@ -1809,12 +1895,11 @@ void pcg_solve(Hier& h, const double* b, double* xout, double rtol, int maxit, d
     ++ncyc;
     if (mixed) {
       k_start_dir<<<dg, 256, 0, st>>>(n, L0.n_r, rvec, z32, L0.mult.get(), zscale, h.p.get(),
-                                      h.zold32.get(), c.partials.get());
-      RMG_LAUNCHED();
-      k_finalize<<<1, 256, 0, st>>>(c.partials.get(), dg, &sc->rz, FIN_STORE);
+                                      h.zold32.get(), arrive, sc);
       RMG_LAUNCHED();
     } else {
-      dot(c, n, L0.n_r, rvec, zvec, L0.mult.get(), &sc->rz, FIN_STORE, st);
+      k_cg_dot<<<dg, 256, 0, st>>>(n, L0.n_r, rvec, zvec, L0.mult.get(), arrive, sc, CG_RZ);
+      RMG_LAUNCHED();
       k_copy<double><<<eg, 256, 0, st>>>(n, zvec, h.p.get());
       RMG_LAUNCHED();
       if (flex64) {
@@ -1826,19 +1911,19 @@ void pcg_solve(Hier& h, const double* b, double* xout, double rtol, int maxit, d
       ++it;
       launch_stencil(c, L0, L0.coef.get(), h.p.get(), h.v64[0].y.get(),
                      EpiStore<double>{h.q.get()}, st, nullptr);
-      dot(c, n, L0.n_r, h.p.get(), h.q.get(), L0.mult.get(), &sc->pq, FIN_STORE, st);
-      k_alpha<<<1, 1, 0, st>>>(sc);
+      k_cg_dot<<<dg, 256, 0, st>>>(n, L0.n_r, h.p.get(), h.q.get(), L0.mult.get(), arrive, sc,
+                                   CG_ALPHA);
       RMG_LAUNCHED();
       if (mixed)
         k_cg_update_mixed<<<dg, 256, 0, st>>>(n, L0.n_r, h.p.get(), h.q.get(), L0.mult.get(), sc,
-                                              rscale, h.x.get(), rvec, r32, c.partials.get());
+                                              rscale, h.x.get(), rvec, r32, arrive, host_rr);
       else
         k_cg_update<<<dg, 256, 0, st>>>(n, L0.n_r, h.p.get(), h.q.get(), L0.mult.get(), sc,
-                                        h.x.get(), rvec, c.partials.get());
+                                        h.x.get(), rvec, arrive, host_rr);
       RMG_LAUNCHED();
-      k_finalize<<<1, 256, 0, st>>>(c.partials.get(), dg, &sc->rr, FIN_STORE);
-      RMG_LAUNCHED();
-      read2(&rr, &bb);
+      RMG_CUDA(cudaStreamSynchronize(st));
+      probe_collect(h);
+      rr = h.pinned[2];
       relres = std::sqrt(rr) / bnorm;
       if (history) history[it] = relres;
       if (relres <= rtol) {
@@ -1861,24 +1946,16 @@ void pcg_solve(Hier& h, const double* b, double* xout, double rtol, int maxit, d
       ++ncyc;
       if (mixed) {
         k_flex_dots<<<dg, 256, 0, st>>>(n, L0.n_r, rvec, z32, h.zold32.get(), L0.mult.get(),
-                                        zscale, c.partials.get());
-        RMG_LAUNCHED();
-        k_finalize<<<1, 256, 0, st>>>(c.partials.get(), dg, &sc->rz_new, FIN_STORE);
-        RMG_LAUNCHED();
-        k_finalize<<<1, 256, 0, st>>>(c.partials.get() + dg, dg, &sc->beta, FIN_STORE);
-        RMG_LAUNCHED();
-        k_beta<<<1, 1, 0, st>>>(sc, 1);
+                                        zscale, arrive, sc);
         RMG_LAUNCHED();
         k_p_update<float><<<eg, 256, 0, st>>>(n, z32, zscale, sc, h.p.get());
         RMG_LAUNCHED();
       } else {
-        dot(c, n, L0.n_r, rvec, zvec, L0.mult.get(), &sc->rz_new, FIN_STORE, st);
-        if (flex64) {
-          dot(c, n, L0.n_r, rvec, h.zold.get(), L0.mult.get(), &sc->beta, FIN_STORE, st);
-          k_copy<double><<<eg, 256, 0, st>>>(n, zvec, h.zold.get());
-          RMG_LAUNCHED();
-        }
-        k_beta<<<1, 1, 0, st>>>(sc, flex64 ? 1 : 0);
+        if (flex64)
+          k_cg_flex64<<<dg, 256, 0, st>>>(n, L0.n_r, rvec, zvec, h.zold.get(), L0.mult.get(),
+                                          arrive, sc);
+        else
+          k_cg_dot<<<dg, 256, 0, st>>>(n, L0.n_r, rvec, zvec, L0.mult.get(), arrive, sc, CG_BETA);
         RMG_LAUNCHED();
         k_p_update<double><<<eg, 256, 0, st>>>(n, zvec, 1.0, sc, h.p.get());
         RMG_LAUNCHED();

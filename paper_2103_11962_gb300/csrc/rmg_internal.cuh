@@ -220,6 +220,7 @@ struct Ctx {
   std::string last_error;
   DBuf<int> d_err;                // device error flag
   DBuf<double> partials;          // block partial sums for reductions
+  DBuf<unsigned> arrived;         // blocks arrived at a reduction in flight (0 between kernels)
   int max_partials = 0;
   void check_device_error(const char* where);
 };
