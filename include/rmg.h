@@ -87,7 +87,7 @@ typedef struct {
   int precision;         /* rmg_precision                                                  */
   int use_graph;         /* capture the V-cycle in a CUDA graph (1) or launch eagerly (0)  */
   int tile_shape;        /* stencil-sweep tiles: -1 autotune (default), else a shape index  */
-  int symmetric_storage; /* FP32 cycle, scalar operator: half planes of level 0 (1, default),
+  int symmetric_storage; /* FP32 cycle: half planes of level 0 (1, default),
                             or the full planes only (0); see rmg_hier_coef_planes           */
 } rmg_options;
 
@@ -420,10 +420,11 @@ rmg_status rmg_hier_galerkin(rmg_hier* hier, int level);
  * ints; fails with RMG_ERR_ARG for a level outside the hierarchy. */
 rmg_status rmg_hier_tile_shape(rmg_hier* hier, int level, int* tx, int* ty, int* tz);
 /* Stencil coefficients per regional node that the cycle's sweeps read on a level, as of the
- * last rmg_setup_numeric: B * B * S for an S-point stencil, or (S + 1) / 2 where the half form
- * is in use. The half form (FP32 cycle, scalar operator, level 0, symmetric_storage 1) rests
- * on the symmetry of the regional operator, a(n, n+e) = a(n+e, n) inside every region (Sec. 4
- * splits a symmetric composite matrix into symmetric region matrices): it keeps the centre and
+ * last rmg_setup_numeric: B * B * S for an S-point stencil, or B * B * (S + 1) / 2 where the half
+ * form is in use. The half form (FP32 cycle, level 0, symmetric_storage 1) rests on the symmetry
+ * of the regional operator, a(n, n+e) = a(n+e, n) inside every region, for block operators
+ * A_cc'(n, n+e) = A_c'c(n+e, n) (Sec. 4 splits a symmetric composite matrix into symmetric
+ * region matrices): it keeps the centre and
  * the (S - 1) / 2 slots after it, and reads a coefficient of the other half at the neighbour
  * that owns its mirror. Each setup compares every mirrored pair of the FP32 coefficients bit
  * for bit; the half form is used only when all agree, so that the sweeps compute exactly the

@@ -428,7 +428,8 @@ rmg_status rmg_hier_coef_planes(rmg_hier* hh, int level, int* planes) {
   if (level < 0 || level >= h.levels()) return fail(h.layout->ctx, RMG_ERR_ARG, "bad level");
   if (h.kind0 == 0) return fail(h.layout->ctx, RMG_ERR_STATE, "no numeric setup yet");
   const Level& L = *h.lv[level];
-  *planes = (h.half(level) && h.hsc.half_asym == 0) ? (L.kind + 1) / 2 : L.B * L.B * L.kind;
+  *planes = (h.half(level) && h.hsc.half_asym == 0) ? L.B * L.B * ((L.kind + 1) / 2)
+                                                       : L.B * L.B * L.kind;
   return RMG_OK;
 }
 

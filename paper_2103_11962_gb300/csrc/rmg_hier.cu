@@ -17,7 +17,9 @@ Hier::~Hier() {
   for (auto e : probe_ev) if (e) cudaEventDestroy(e);
 }
 
-const int* Hier::half_flag() const { return &sc.get()->half_asym; }
+const int* Hier::half_flag() const {
+  return half_regions.get() ? half_regions.get() : &sc.get()->half_asym;
+}
 
 // the mixed-precision dense coarse solve (defined with the coarse factorisation below)
 static int mixed_coarse_solve(Hier& h, cudaStream_t st, int nd, int steps, double* nrm);
@@ -831,8 +833,8 @@ void hier_build(Hier& h) {
       if (o.precision == RMG_PREC_FP32_BF16COEF) L.coef16.ensure((size_t)L.B * L.B * L.kind * L.n_r);
     }
   }
-  // half planes for the FP32 cycle's level-0 sweeps of a scalar operator
-  h.half_on = o.symmetric_storage != 0 && o.precision == RMG_PREC_FP32 && h.lv[0]->B == 1;
+  // half planes for the FP32 cycle's level-0 sweeps
+  h.half_on = o.symmetric_storage != 0 && o.precision == RMG_PREC_FP32;
   if (Lv > 1) h.layout->apbuf.ensure((size_t)(h.lv[0]->dim == 3 ? 27 : 9) * h.lv[0]->n_r);
   h.sc.alloc(1);
   RMG_CUDA(cudaMemsetAsync(h.sc.get(), 0, sizeof(Scalars), c.stream));
@@ -1328,19 +1330,23 @@ static void level0_to_fp32(Hier& h) {
   }
   // with the FP32 cycle's half planes and the flag that says whether they hold the operator,
   // in the same pass
-  h.half32.ensure((size_t)(L.kind + 1) / 2 * L.n_r);
+  h.half32.ensure((size_t)L.B * L.B * ((L.kind + 1) / 2) * L.n_r);
   int* flag = &h.sc.get()->half_asym;
   RMG_CUDA(cudaMemsetAsync(flag, 0, sizeof(int), c.stream));
+  if (L.B > 1) {
+    h.half_regions.ensure(L.nreg);
+    RMG_CUDA(cudaMemsetAsync(h.half_regions.get(), 0, h.half_regions.bytes(), c.stream));
+  }
   const Grid G = L.grid();
   const int gb = persistent_grid(c, G.ntiles);
-#define RMG_L0(K)                                                                              \
-  k_level0_fp32<K><<<gb, kTile, 0, c.stream>>>(G, L.coef.get(), L.coef32.get(), h.half32.get(), \
-                                               flag)
+#define RMG_L0(K, BB)                                                                          \
+  k_level0_fp32<K, BB><<<dim3(gb, BB * BB), kTile, 0, c.stream>>>(                             \
+      G, L.coef.get(), L.coef32.get(), h.half32.get(), flag, h.half_regions.get())
   switch (L.kind) {
-    case 5: RMG_L0(5); break;
-    case 7: RMG_L0(7); break;
-    case 9: RMG_L0(9); break;
-    default: RMG_L0(27); break;
+    case 5: RMG_L0(5, 1); break;
+    case 7: RMG_L0(7, 1); break;
+    case 9: if (L.B == 3) RMG_L0(9, 3); else RMG_L0(9, 1); break;
+    default: if (L.B == 3) RMG_L0(27, 3); else RMG_L0(27, 1); break;
   }
 #undef RMG_L0
   RMG_LAUNCHED();

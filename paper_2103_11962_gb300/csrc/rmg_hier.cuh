@@ -84,10 +84,11 @@ struct Hier {
   DBuf<double> x, r, z, p, q, zold, tmp;
   DBuf<float> zold32;                        // previous FP32 cycle output (flexible CG)
   double* pinned = nullptr;                  // host-mapped residual read-back
-  // FP32 cycle, scalar operator: level 0 also as half planes (k_level0_fp32), read by the sweeps
-  // while the device flag Scalars::half_asym is 0
+  // FP32 cycle: level 0 also as half planes (k_level0_fp32), read by the sweeps while the device
+  // flag Scalars::half_asym is 0 (block operators: in the regions whose flag is 0)
   bool half_on = false;
   DBuf<float> half32;
+  DBuf<int> half_regions;
   // coarse end of the cycle in one kernel (rmg_tail.cu): first level it takes (-1: none), whether
   // the dense solve is inside, the cluster's blocks, and geometry per level
   int tail0 = -1;

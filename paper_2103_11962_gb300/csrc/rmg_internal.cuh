@@ -209,7 +209,7 @@ struct Scalars {
   float cheb_c2f[16][8];
   double pw_norm, pw_inv;  // power method scratch (norm and its reciprocal)
   double pw_num, pw_den;
-  double rz, pq, alpha, beta, rr, bb, rz_new;
+  double rz, pq, alpha, beta, rr, bb;
   int half_asym;           // level-0 FP32 stencil not bitwise symmetric (full planes in use)
 };
 

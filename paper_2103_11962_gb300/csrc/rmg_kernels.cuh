@@ -420,6 +420,74 @@ k_bstencil(Grid G, const CT* __restrict__ coef, const VT* __restrict__ u,
   RMG_END_FOR_NODES
 }
 
+// Half storage of a symmetric FP32 block operator: symmetry pairs block (c, c') at n with block
+// (c', c) at the neighbour, so planes C..S-1 of all blocks hold it,
+// half[((c * B + c') * P + s - C) * n_r + n] with P = S - C, and slot s < C of block (c, c') at n
+// is slot S-1-s of block (c', c) at n + off(s). The centre is stored for both (c, c') and
+// (c', c), so it needs no symmetry. Same products in the same order as k_bstencil, hence the
+// same bits. The sweep is bound by HBM and this form moves 14/27 of the coefficients: 577 instead
+// of 1045 bytes a node; the mirrored ones come from L1 and L2.
+template <bool HALF, int KIND, int B>
+__device__ __forceinline__ void bstencil_row32(const float* __restrict__ coef,
+                                               const float* __restrict__ u, int n, int n_r, int i,
+                                               int j, int l, const RegionDev& R, float (&au)[B]) {
+  using S = Sten<KIND>;
+  static_assert(mirrored_slots<KIND>(), "half storage needs mirrored stencil slots");
+  constexpr int C = S::CENTER, P = HALF ? S::S - C : S::S;   // planes stored per block
+  const int sy = R.nx, sz = R.nx * R.ny;
+#pragma unroll
+  for (int c = 0; c < B; ++c) au[c] = 0.f;
+#pragma unroll
+  for (int s = 0; s < S::S; ++s) {
+    const int dx = S::dx(s), dy = S::dy(s), dz = S::dz(s);
+    bool ok = true;
+    if (dx < 0) ok &= (i > 0);
+    if (dx > 0) ok &= (i < R.nx - 1);
+    if (dy < 0) ok &= (j > 0);
+    if (dy > 0) ok &= (j < R.ny - 1);
+    if (dz < 0) ok &= (l > 0);
+    if (dz > 0) ok &= (l < R.nz - 1);
+    if (!ok) continue;
+    const int nb = n + dx + dy * sy + dz * sz;
+    float uv[B];
+#pragma unroll
+    for (int c2 = 0; c2 < B; ++c2) uv[c2] = u[(size_t)c2 * n_r + nb];
+    const bool mirrored = HALF && s < C;
+    const int plane = !HALF ? s : s < C ? S::S - 1 - s - C : s - C;
+    const int at = mirrored ? nb : n;
+#pragma unroll
+    for (int c = 0; c < B; ++c)
+#pragma unroll
+      for (int c2 = 0; c2 < B; ++c2) {
+        const int blk = mirrored ? c2 * B + c : c * B + c2;
+        au[c] = fmaf(coef[((size_t)blk * P + plane) * n_r + at], uv[c2], au[c]);
+      }
+  }
+}
+
+// asym[region] != 0: the region's full planes (an assembled block matrix can differ from its
+// transpose in the last bit of a few entries, and only their regions then lose the half form).
+template <int KIND, int B, class Epi>
+__global__ void __launch_bounds__(kTile)
+k_bstencil_half(Grid G, const float* __restrict__ coef, const float* __restrict__ half,
+                const int* __restrict__ asym, const float* __restrict__ u,
+                const uint8_t* __restrict__ mult, float* __restrict__ y, Epi epi) {
+  RMG_FOR_NODES(G)
+    int i, j, l;
+    RMG_DECODE(i, j, l);
+    float au[B];
+    if (asym[tile_.region]) bstencil_row32<false, KIND, B>(coef, u, n, G.n_r, i, j, l, R, au);
+    else bstencil_row32<true, KIND, B>(half, u, n, G.n_r, i, j, l, R, au);
+    if (mult[n] > 1) {
+#pragma unroll
+      for (int c = 0; c < B; ++c) y[(size_t)c * G.n_r + n] = au[c];
+    } else {
+#pragma unroll
+      for (int c = 0; c < B; ++c) epi(c * G.n_r + n, au[c], 1);
+    }
+  RMG_END_FOR_NODES
+}
+
 template <typename AT, class Epi>
 __global__ void __launch_bounds__(256)
 k_groups_b(int ngroups, int B, int n_r, const int* __restrict__ gptr,

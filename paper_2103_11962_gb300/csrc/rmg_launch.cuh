@@ -112,6 +112,15 @@ void launch_stencil(Ctx& c, const Level& L, const CT* coef, const VT* u, AT* y, 
         default: launch_resident(c, k_stencil_half<27, Epi>, nt, st, G, coef, half, asym, u, mu, y, epi); break;
       }
       done = true;
+    } else if (half) {
+      RMG_REQUIRE(asym != nullptr && L.B == 3 && (L.kind == 27 || L.kind == 9), RMG_ERR_STATE,
+                  "half planes of a block operator need 3 dofs and a 27- or 9-point stencil");
+      const uint8_t* mu = L.mult.get();
+      if (L.kind == 27)
+        launch_resident(c, k_bstencil_half<27, 3, Epi>, G.ntiles, st, G, coef, half, asym, u, mu, y, epi);
+      else
+        launch_resident(c, k_bstencil_half<9, 3, Epi>, G.ntiles, st, G, coef, half, asym, u, mu, y, epi);
+      done = true;
     }
   }
   RMG_REQUIRE(done || G.lx != -3, RMG_ERR_STATE, "staged tiles outside a half-plane sweep");

@@ -278,13 +278,20 @@ k_ap_tensor27(Grid Gf, const RegionDev* __restrict__ cregs, const float* __restr
 // stencil_row_half (planes C..S-1). *asym becomes 1 when a mirrored pair of the FP32 copy
 // inside a region differs in any bit (the sweeps then keep reading the full planes); the pair's
 // far value is rounded here from its FP64 value, the same rounding that made the copy.
-template <int KIND>
+// With B > 1 (blockIdx.y = block c * B + c') the mirror of block (c, c') is block (c', c), and
+// region_asym (zeroed before) says it for every region.
+template <int KIND, int B>
 __global__ void __launch_bounds__(kTile)
 k_level0_fp32(Grid G, const double* __restrict__ coef, float* __restrict__ coef32,
-              float* __restrict__ half, int* __restrict__ asym) {
+              float* __restrict__ half, int* __restrict__ asym, int* __restrict__ region_asym) {
   using S = Sten<KIND>;
   static_assert(mirrored_slots<KIND>(), "half storage needs mirrored stencil slots");
   constexpr int C = S::CENTER;
+  const int blk = B == 1 ? 0 : blockIdx.y, mirror = B == 1 ? 0 : (blk % B) * B + blk / B;
+  const double* own = coef + (size_t)blk * S::S * G.n_r;
+  const double* far = coef + (size_t)mirror * S::S * G.n_r;
+  float* own32 = coef32 + (size_t)blk * S::S * G.n_r;
+  float* ownh = half + (size_t)blk * (S::S - C) * G.n_r;
   bool bad = false;
   RMG_FOR_NODES(G)
     int i, j, l;
@@ -292,10 +299,10 @@ k_level0_fp32(Grid G, const double* __restrict__ coef, float* __restrict__ coef3
     const int sy = R.nx, sz = R.nx * R.ny;
 #pragma unroll
     for (int s = 0; s < S::S; ++s) {
-      const float cv = static_cast<float>(coef[(size_t)s * G.n_r + n]);
-      coef32[(size_t)s * G.n_r + n] = cv;
+      const float cv = static_cast<float>(own[(size_t)s * G.n_r + n]);
+      own32[(size_t)s * G.n_r + n] = cv;
       if (s < C) continue;
-      half[(size_t)(s - C) * G.n_r + n] = cv;
+      ownh[(size_t)(s - C) * G.n_r + n] = cv;
       const int dx = S::dx(s), dy = S::dy(s), dz = S::dz(s);
       bool ok = s > C;
       if (dx < 0) ok &= (i > 0);
@@ -306,8 +313,10 @@ k_level0_fp32(Grid G, const double* __restrict__ coef, float* __restrict__ coef3
       if (dz > 0) ok &= (l < R.nz - 1);
       if (ok) {
         const float mv = static_cast<float>(
-            coef[(size_t)(S::S - 1 - s) * G.n_r + n + dx + dy * sy + dz * sz]);
-        bad |= __float_as_uint(cv) != __float_as_uint(mv);
+            far[(size_t)(S::S - 1 - s) * G.n_r + n + dx + dy * sy + dz * sz]);
+        const bool differ = __float_as_uint(cv) != __float_as_uint(mv);
+        if (B > 1 && differ) region_asym[tile_.region] = 1;   // every writer stores 1
+        bad |= differ;
       }
     }
   RMG_END_FOR_NODES
