@@ -783,6 +783,7 @@ static void coarsen_level(Hier& h, const Level& F, Level& C) {
 }
 
 static void tail_levels(Hier& h);
+static void coarsen_axes(const Level& F, const Level& C, int axes, AxisGrid& A);
 
 void hier_build(Hier& h) {
   Ctx& c = *h.c;
@@ -810,6 +811,12 @@ void hier_build(Hier& h) {
     h.lv.push_back(h.own.back().get());
   }
   const int Lv = h.levels();
+  h.rap_x = std::vector<AxisGrid>(Lv);
+  h.rap_xy = std::vector<AxisGrid>(Lv);
+  for (int l = 0; l + 1 < Lv; ++l) {
+    coarsen_axes(*h.lv[l], *h.lv[l + 1], 1, h.rap_x[l]);
+    if (h.lv[l]->dim == 3) coarsen_axes(*h.lv[l], *h.lv[l + 1], 2, h.rap_xy[l]);
+  }
   h.stored.assign(Lv, 0);
   h.pw.resize(Lv);
   h.shape.assign(Lv, -1);
@@ -937,66 +944,99 @@ static void compute_dinv(Hier& h, Level& L) {
   }
 }
 
-template <typename T>
-static void galerkin_t(Hier& h, int l, const Level& F, Level& C, const T* fcoef, T* ccoef) {
+// Node grid of level F coarsened along x (axes = 1), or along x and y (axes = 2).
+static void coarsen_axes(const Level& F, const Level& C, int axes, AxisGrid& A) {
+  std::vector<RegionDev> regs(F.nreg);
+  std::vector<Tile> tiles;
+  A.n = 0;
+  for (int r = 0; r < F.nreg; ++r) {
+    const int nx = C.hdims[3 * r], ny = (axes > 1 ? C : F).hdims[3 * r + 1], nz = F.hdims[3 * r + 2];
+    regs[r] = make_region(nx, ny, nz, A.n);
+    for (int s = 0; s < nx * ny * nz; s += kTile) tiles.push_back(Tile{r, s, 0, 0, 0, 0});
+    A.n += nx * ny * nz;
+  }
+  A.ntiles = (int)tiles.size();
+  A.regions.alloc(regs.size());
+  A.tiles.alloc(tiles.size());
+  RMG_CUDA(cudaMemcpy(A.regions.get(), regs.data(), A.regions.bytes(), cudaMemcpyHostToDevice));
+  RMG_CUDA(cudaMemcpy(A.tiles.get(), tiles.data(), A.tiles.bytes(), cudaMemcpyHostToDevice));
+}
+
+// One block of the product with linear interpolation, axis by axis (k_rap_*). The two
+// intermediate operators lie one after the other in the scratch array: at most 13.5 n_r and
+// 6.75 n_r values (regions of 4 nodes per axis), within its 27 n_r doubles.
+template <int KIND, typename T>
+static void galerkin_axes(Hier& h, int l, const Level& F, Level& C, const T* fco, T* cco,
+                          double mdiag) {
   Ctx& c = *h.c;
+  using Ln = Lines<KIND>;
+  const Grid G1 = h.rap_x[l].grid(F.nreg), Gc = C.grid();
+  T* x1 = reinterpret_cast<T*>(h.layout->apbuf.get());
+  auto blocks = [&](const Grid& G, int lines) {
+    return dim3(persistent_grid(c, G.ntiles), lines);
+  };
+  k_rap_first<KIND, T><<<blocks(G1, Ln::N), kTile, 0, c.stream>>>(G1, F.regions.get(), F.n_r, fco,
+                                                                  F.mask.get(), x1);
+  RMG_LAUNCHED();
+  if (Ln::DIM == 2) {
+    k_rap_next<KIND, T><<<blocks(Gc, 3), kTile, 0, c.stream>>>(
+        Gc, G1.regions, G1.n_r, x1, cco, C.mask.get(), C.mult.get(), mdiag);
+    RMG_LAUNCHED();
+    return;
+  }
+  const Grid G2 = h.rap_xy[l].grid(F.nreg);
+  T* y2 = x1 + (size_t)3 * Ln::N * G1.n_r;
+  k_rap_next<KIND, T><<<blocks(G2, 9), kTile, 0, c.stream>>>(G2, G1.regions, G1.n_r, x1, y2,
+                                                             nullptr, nullptr, 0.0);
+  RMG_LAUNCHED();
+  k_rap_last<T><<<blocks(Gc, 9), kTile, 0, c.stream>>>(Gc, G2.regions, G2.n_r, y2, C.mask.get(),
+                                                       C.mult.get(), mdiag, cco);
+  RMG_LAUNCHED();
+}
+
+// The same with stored weights (k_ap_w, k_rtap_w).
+template <int FK, int CK, typename T>
+static void galerkin_stored(Hier& h, int l, const Level& F, Level& C, const T* fco, T* cco,
+                            double mdiag) {
+  Ctx& c = *h.c;
+  constexpr int D = Sten<FK>::DIM;
   T* ap = reinterpret_cast<T*>(h.layout->apbuf.get());
   const Grid Gf = F.grid(), Gc = C.grid();
-  const int gf = persistent_grid(c, Gf.ntiles), gc = persistent_grid(c, Gc.ntiles);
+  const int smem = (D == 3 ? 27 : 9) * kTile * (int)sizeof(T);
+  RMG_CUDA(cudaFuncSetAttribute(k_ap_w<FK, D, T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                smem));
+  k_ap_w<FK, D, T><<<persistent_grid(c, Gf.ntiles), kTile, smem, c.stream>>>(
+      Gf, C.regions.get(), fco, h.pw[l].get(), F.mask.get(), C.mask.get(), ap);
+  RMG_LAUNCHED();
+  k_rtap_w<CK, D, T><<<persistent_grid(c, Gc.ntiles), kTile, 0, c.stream>>>(
+      Gc, F.regions.get(), ap, F.n_r, h.pw[l].get(), C.mask.get(), C.mult.get(), mdiag, cco);
+  RMG_LAUNCHED();
+}
+
+template <typename T>
+static void galerkin_t(Hier& h, int l, const Level& F, Level& C, const T* fcoef, T* ccoef) {
   // (P x I)^T A (P x I) of a B x B block operator is the scalar product on every block; a
   // masked coarse row is the identity row in the diagonal blocks and zero elsewhere
   for (int blk = 0; blk < F.B * F.B; ++blk) {
-  const T* fco = fcoef + (size_t)blk * F.kind * F.n_r;
-  T* cco = ccoef + (size_t)blk * C.kind * C.n_r;
-  const double mdiag = (blk / F.B == blk % F.B) ? 1.0 : 0.0;
-#define RMG_RAP(FK, CK, D)                                                                    \
-  if (sizeof(T) == 4 && FK == 27 && D == 3) {                                                \
-    const int ga = persistent_grid(c, Gf.ntiles, resident_per_sm((const void*)k_ap_tensor27)); \
-    k_ap_tensor27<<<ga, kTile, 0, c.stream>>>(Gf, C.regions.get(), (const float*)fco,          \
-                                              F.mask.get(), C.mask.get(), (float*)ap);        \
-  } else if (sizeof(T) == 4) {                                                                \
-    k_ap_axis32<FK, D><<<gf, kTile, 0, c.stream>>>(Gf, C.regions.get(), (const float*)fco,     \
-                                                   F.mask.get(), C.mask.get(), (float*)ap);   \
-  } else {                                                                                    \
-    const int smem = (D == 3 ? 27 : 9) * kTile * (int)sizeof(T);                              \
-    RMG_CUDA(cudaFuncSetAttribute(k_ap<FK, D, T>, cudaFuncAttributeMaxDynamicSharedMemorySize,    \
-                                  smem));                                                     \
-    k_ap<FK, D, T><<<gf, kTile, smem, c.stream>>>(Gf, C.regions.get(), fco, F.mask.get(),        \
-                                               C.mask.get(), ap);                             \
-  }                                                                                           \
-  RMG_LAUNCHED();                                                                             \
-  k_rtap<CK, D, T><<<gc, kTile, 0, c.stream>>>(Gc, F.regions.get(), ap, F.n_r, C.mask.get(),     \
-                                            C.mult.get(), mdiag, cco)
-#define RMG_RAPW(FK, CK, D)                                                                   \
-  {                                                                                           \
-    const int smem = (D == 3 ? 27 : 9) * kTile * (int)sizeof(T);                         \
-    RMG_CUDA(cudaFuncSetAttribute(k_ap_w<FK, D, T>, cudaFuncAttributeMaxDynamicSharedMemorySize,  \
-                                  smem));                                                     \
-    k_ap_w<FK, D, T><<<gf, kTile, smem, c.stream>>>(Gf, C.regions.get(), fco, h.pw[l].get(),       \
-                                                 F.mask.get(), C.mask.get(), ap);             \
-  }                                                                                           \
-  RMG_LAUNCHED();                                                                             \
-  k_rtap_w<CK, D, T><<<gc, kTile, 0, c.stream>>>(Gc, F.regions.get(), ap, F.n_r, h.pw[l].get(),   \
-                                              C.mask.get(), C.mult.get(), mdiag, cco)
-  if (h.stored[l]) {
-    switch (F.kind) {
-      case 5: RMG_RAPW(5, 9, 2); break;
-      case 9: RMG_RAPW(9, 9, 2); break;
-      case 7: RMG_RAPW(7, 27, 3); break;
-      default: RMG_RAPW(27, 27, 3); break;
-    }
-  } else {
-    switch (F.kind) {
-      case 5: RMG_RAP(5, 9, 2); break;
-      case 9: RMG_RAP(9, 9, 2); break;
-      case 7: RMG_RAP(7, 27, 3); break;
-      default: RMG_RAP(27, 27, 3); break;
+    const T* fco = fcoef + (size_t)blk * F.kind * F.n_r;
+    T* cco = ccoef + (size_t)blk * C.kind * C.n_r;
+    const double mdiag = (blk / F.B == blk % F.B) ? 1.0 : 0.0;
+    if (h.stored[l]) {
+      switch (F.kind) {
+        case 5: galerkin_stored<5, 9, T>(h, l, F, C, fco, cco, mdiag); break;
+        case 9: galerkin_stored<9, 9, T>(h, l, F, C, fco, cco, mdiag); break;
+        case 7: galerkin_stored<7, 27, T>(h, l, F, C, fco, cco, mdiag); break;
+        default: galerkin_stored<27, 27, T>(h, l, F, C, fco, cco, mdiag); break;
+      }
+    } else {
+      switch (F.kind) {
+        case 5: galerkin_axes<5, T>(h, l, F, C, fco, cco, mdiag); break;
+        case 9: galerkin_axes<9, T>(h, l, F, C, fco, cco, mdiag); break;
+        case 7: galerkin_axes<7, T>(h, l, F, C, fco, cco, mdiag); break;
+        default: galerkin_axes<27, T>(h, l, F, C, fco, cco, mdiag); break;
+      }
     }
   }
-  RMG_LAUNCHED();
-  }
-#undef RMG_RAP
-#undef RMG_RAPW
 }
 
 // Level l + 1 = Galerkin product of level l: in FP64 for the plain method; for a mixed

@@ -28,6 +28,14 @@ constexpr int kStagedShape = 9;
 constexpr int kNumTileShapes = (int)(sizeof(kTileShapes) / sizeof(kTileShapes[0]));
 static_assert(kNumTileShapes == RMG_NUM_TILE_SHAPES, "tile shape table and header disagree");
 
+// Node grid of a level coarsened along some axes (intermediate operators of the Galerkin product).
+struct AxisGrid {
+  DBuf<RegionDev> regions;
+  DBuf<Tile> tiles;
+  int ntiles = 0, n = 0;
+  Grid grid(int nreg) const { return Grid{regions.get(), tiles.get(), ntiles, nreg, n, -1, 0}; }
+};
+
 struct Hier {
   rmg_layout* layout = nullptr;
   Ctx* c = nullptr;
@@ -57,6 +65,7 @@ struct Hier {
   cudaGraphExec_t gexec = nullptr;
   cudaStream_t graph_stream = nullptr;
   int launches = 0;
+  std::vector<AxisGrid> rap_x, rap_xy;       // per level: coarsened along x, along x and y
   // stored transfer weights per level (to the next coarser level; linear 3:1 when not
   // stored): pw[l][a * n_r + n] = weight of the right coarse neighbour along axis a (FP32;
   // the entries of P are the FP32 products wz (wy wx) in every precision)

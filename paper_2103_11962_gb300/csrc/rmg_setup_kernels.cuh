@@ -62,214 +62,205 @@ struct EpiRecip {
 };
 
 // ------------------------------------------------------------------ Galerkin product
-// [[Abar]] = [[R]] [[A]] [[P]] (eq. RegionalGalerkinProduct), region by region, in two steps
-// following the product order R (A P):
-//  1. k_ap: for every fine node f, row f of [[A]] [[P]], i.e. sum_s A_s(f) P(f + d_s, C') for
-//     the (at most 3 per axis) coarse nodes C' near f, stored relative to the coarse node
-//     (x - 1) div 3 on each axis: ap[o][f], o = ox + 3 oy + 9 oz.
-//  2. k_rtap: for every coarse node C, sum over the fine nodes f = 3C + (a, b, c) of its
-//     support of P(f, C) ap[.][f]; the weights P(f, C) are compile-time constants.
-// Masked fine nodes have zero rows of P, masked coarse nodes zero columns; a masked coarse
-// row becomes 1/mult on the diagonal so that the composite sum is the identity row.
+// [[Abar]] = [[R]] [[A]] [[P]] (eq. RegionalGalerkinProduct), region by region, with linear 3:1
+// interpolation. The weights are tensor products, and masked fine nodes (zero rows of P) only
+// remove entries of A, so the product factorises into one along each axis: R A P =
+// Rz (Ry (Rx A Px) Py) Pz, each step coarsening one axis of both sides:
+//  1. k_rap_first: along x, from the fine stencil, without the entries of masked nodes, to
+//     (X, y, z) with the stencil's (dy, dz) and the coarse ox;
+//  2. k_rap_next: along y to (X, Y, z) with (ox, oy, dz);
+//  3. k_rap_last: along z to the coarse stencil (in 2D the y step is the last one). Masked coarse
+//     nodes have zero columns of P, and a masked coarse row becomes 1/mult on the diagonal so
+//     that the composite sum is the identity row.
+// A step reads five entries of the axis times up to three offsets and forms three coarse offsets
+// in about 36 FMAs, some 50 a fine node in all for a 7-point stencil, where the two-step form
+// R (A P) took 75 and sent 27 values a fine node through memory twice. The FP64 pipe and memory
+// bound the steps about equally. 3.1M nodes of a 7-point level in FP64: 1034 -> 365 us for the
+// product; 35.9M nodes of a 27-point one in FP32: 7.1 -> 1.7 ms.
 // T is the arithmetic of the product: FP64 for the plain method; FP32 for the hierarchies of
-// the mixed-precision cycle, whose coarse operators only ever enter an FP32 cycle (GB300's
-// FP64 pipe would make these sums the largest part of the setup).
-__device__ __forceinline__ int floor_div3m1(int x) { return (x + 2) / 3 - 1; }   // (x-1) div 3, x >= 0
-
-template <int FK, int DIM, typename T>
-__global__ void __launch_bounds__(kTile)
-k_ap(Grid Gf, const RegionDev* __restrict__ cregs, const T* __restrict__ fcoef,
-     const uint8_t* __restrict__ fmask, const uint8_t* __restrict__ cmask,
-     T* __restrict__ ap) {
-  using FS = Sten<FK>;
-  constexpr int NO = DIM == 3 ? 27 : 9;
-  __shared__ T tab[27 * 8];
-  extern __shared__ __align__(16) unsigned char ap_smem[];   // NO x kTile accumulators
-  T (*acc)[kTile] = reinterpret_cast<T (*)[kTile]>(ap_smem);
-  for (int e = threadIdx.x; e < 27 * 8; e += blockDim.x) {
-    const int r = e >> 3, combo = e & 7;
-    tab[e] = wrem_t<T>(r / 9, combo >> 2) *
-             (wrem_t<T>((r / 3) % 3, (combo >> 1) & 1) * wrem_t<T>(r % 3, combo & 1));
+// the mixed-precision cycle, whose coarse operators only ever enter an FP32 cycle.
+//
+// (dy, dz) of a stencil in the order the steps number them, and whether it has x offsets there.
+template <int KIND>
+struct Lines {
+  static constexpr int DIM = Sten<KIND>::DIM;
+  static constexpr bool BOX = KIND == 9 || KIND == 27;
+  static constexpr int N = KIND == 27 ? 9 : KIND == 7 ? 5 : 3;
+  __host__ __device__ static constexpr int dy(int q) {
+    return DIM == 2 ? q - 1 : BOX ? q % 3 - 1 : q == 1 ? -1 : q == 3 ? 1 : 0;
   }
-  __syncthreads();
-  const int tid = threadIdx.x;
-  RMG_FOR_NODES(Gf)
+  __host__ __device__ static constexpr int dz(int q) {
+    return DIM == 2 ? 0 : BOX ? q / 3 - 1 : q == 0 ? -1 : q == 4 ? 1 : 0;
+  }
+  __host__ __device__ static constexpr bool wide(int q) { return BOX || (dy(q) == 0 && dz(q) == 0); }
+  // number of the line (dy, dz), or -1
+  __host__ __device__ static constexpr int at(int y, int z) {
+    for (int q = 0; q < N; ++q)
+      if (dy(q) == y && dz(q) == z) return q;
+    return -1;
+  }
+};
+
+// out[o + 1] += 9 sum_a w(a) sum_d load(a, d) P(a + d - 3 o): one axis of R A P for one coarse node.
+// `a` is the fine node's offset from the coarse one, `d` the entry's (only 0 when !WIDE). The
+// weights times 3 are 1, 2 and 3, exact in any precision; the 9 of every axis comes off in
+// rap_store. Each fine row is summed against P first: where P is (nearly) in the kernel of A
+// these three terms cancel before anything larger is added. (In one sum with weights rounded to
+// FP32 the row sums, which cancel, lost ten times more over three levels.)
+template <bool WIDE, typename T, class Load>
+__device__ __forceinline__ void rap_axis(Load load, T (&out)[3]) {
 #pragma unroll
-    for (int o = 0; o < NO; ++o) acc[o][tid] = T(0);
-    if (!fmask[n]) {
-      int x, y, z;
-      decode(li, R, x, y, z);
-      const RegionDev C = cregs[tile_.region];
-      const int cx0 = floor_div3m1(x), cy0 = floor_div3m1(y), cz0 = DIM == 3 ? floor_div3m1(z) : 0;
+  for (int a = -2; a <= 2; ++a) {
+    if (!WIDE) {                               // one entry a row: nothing to cancel in it
+      const T v = load(a, 0);
 #pragma unroll
-      for (int s = 0; s < FS::S; ++s) {
-        const int gx = x + FS::dx(s), gy = y + FS::dy(s), gz = z + FS::dz(s);
-        if (gx < 0 || gx >= R.nx || gy < 0 || gy >= R.ny || gz < 0 || gz >= R.nz) continue;
-        const T v = fcoef[(size_t)s * Gf.n_r + n];
-        if (v == T(0)) continue;
-        if (fmask[R.off + gx + R.nx * (gy + R.ny * gz)]) continue;
-        const int x0 = gx / 3, rx = gx - 3 * x0;
-        const int y0 = gy / 3, ry = gy - 3 * y0;
-        const int z0 = DIM == 3 ? gz / 3 : 0, rz = DIM == 3 ? gz - 3 * z0 : 0;
-        const T* t = tab + 8 * (rx + 3 * ry + 9 * rz);
-        for (int c = 0; c < (rz ? 2 : 1); ++c)
-          for (int b = 0; b < (ry ? 2 : 1); ++b)
-            for (int a = 0; a < (rx ? 2 : 1); ++a) {
-              const int X = x0 + a, Y = y0 + b, Z = z0 + c;
-              if (cmask[C.off + X + C.nx * (Y + C.ny * Z)]) continue;
-              const int o = (X - cx0) + 3 * (Y - cy0) + 9 * (Z - cz0);
-              acc[o][tid] = fma(v, t[a + 2 * b + 4 * c], acc[o][tid]);
-            }
+      for (int o = -1; o <= 1; ++o) {
+        const int t = a - 3 * o;
+        if (t < -2 || t > 2) continue;
+        out[o + 1] = fma(v, T((3 - (a < 0 ? -a : a)) * (3 - (t < 0 ? -t : t))), out[o + 1]);
+      }
+      continue;
+    }
+    T row[3] = {T(0), T(0), T(0)};
+#pragma unroll
+    for (int d = -1; d <= 1; ++d) {
+      const T v = load(a, d);
+#pragma unroll
+      for (int o = -1; o <= 1; ++o) {
+        const int t = a + d - 3 * o;
+        if (t < -2 || t > 2) continue;
+        row[o + 1] = fma(v, T(3 - (t < 0 ? -t : t)), row[o + 1]);
       }
     }
 #pragma unroll
-    for (int o = 0; o < NO; ++o) ap[(size_t)o * Gf.n_r + n] = acc[o][tid];
-  RMG_END_FOR_NODES
+    for (int o = -1; o <= 1; ++o)
+      if (a - 3 * o >= -3 && a - 3 * o <= 3)
+        out[o + 1] = fma(row[o + 1], T(3 - (a < 0 ? -a : a)), out[o + 1]);
+  }
 }
 
-// A P for any fine stencil in FP32, for the mixed hierarchies: every output o of the
-// 3 x 3 (x 3) coarse neighbourhood of f (the same ap[o][f] layout as k_ap) is evaluated
-// directly as sum_s A_s(f) wx(g_x - 3 X) wy(g_y - 3 Y) wz(g_z - 3 Z), g = f + d_s, with the
-// linear weights w(t) = 1 - |t|/3 for |t| <= 2. No divergent loops and no shared memory; the
-// 27 x S FMAs are cheap on the FP32 pipe (in FP64 they would not be, so the plain method keeps
-// k_ap). Masked fine neighbours and masked coarse nodes contribute nothing.
-__device__ __forceinline__ float lin_w(int t) {
-  t = t < 0 ? -t : t;
-  return t == 0 ? 1.f : (t == 1 ? 2.f / 3.f : (t == 2 ? 1.f / 3.f : 0.f));
-}
-
-template <int FK, int DIM>
+// Step 1, blockIdx.y = line q: x1[(3 q + ox + 1) * n1 + (X, y, z)].
+template <int KIND, typename T>
 __global__ void __launch_bounds__(kTile)
-k_ap_axis32(Grid Gf, const RegionDev* __restrict__ cregs, const float* __restrict__ fcoef,
-            const uint8_t* __restrict__ fmask, const uint8_t* __restrict__ cmask,
-            float* __restrict__ ap) {
-  using FS = Sten<FK>;
-  constexpr int NO = DIM == 3 ? 27 : 9;
-  constexpr int NZ = DIM == 3 ? 3 : 1;
-  RMG_FOR_NODES(Gf)
-    float out[NO];
+k_rap_first(Grid G1, const RegionDev* __restrict__ fregs, int fn_r, const T* __restrict__ fcoef,
+            const uint8_t* __restrict__ fmask, T* __restrict__ x1) {
+  using Ln = Lines<KIND>;
+  const int q = blockIdx.y;
+  int dy = 0, dz = 0, slot0 = 0;               // slot0: slot of (dx = 0, dy, dz)
 #pragma unroll
-    for (int o = 0; o < NO; ++o) out[o] = 0.f;
-    if (!fmask[n]) {
-      int x, y, z;
-      decode(li, R, x, y, z);
-      const int cx0 = floor_div3m1(x), cy0 = floor_div3m1(y), cz0 = DIM == 3 ? floor_div3m1(z) : 0;
+  for (int k = 0; k < Ln::N; ++k)
+    if (k == q) {
+      dy = Ln::dy(k);
+      dz = Ln::dz(k);
+      slot0 = sten_slot<KIND>(0, Ln::dy(k), Ln::dz(k));
+    }
+  RMG_FOR_NODES(G1)
+    int X, y, z;
+    decode(li, R, X, y, z);
+    const RegionDev F = fregs[tile_.region];
+    T out[3] = {T(0), T(0), T(0)};
+    const int yy = y + dy, zz = z + dz;
+    if (yy >= 0 && yy < F.ny && zz >= 0 && zz < F.nz) {
+      const int row = F.off + F.nx * (y + F.ny * z), far = F.off + F.nx * (yy + F.ny * zz);
+      // nodes 3X - 3 .. 3X + 3 of the two lines that are in the region and not masked
+      unsigned rows = 0, cols = 0;
 #pragma unroll
-      for (int s = 0; s < FS::S; ++s) {
-        const int dx = FS::dx(s), dy = FS::dy(s), dz = FS::dz(s);
-        const int gx = x + dx, gy = y + dy, gz = z + dz;
-        if (gx < 0 || gx >= R.nx || gy < 0 || gy >= R.ny || gz < 0 || gz >= R.nz) continue;
-        if (fmask[R.off + gx + R.nx * (gy + R.ny * gz)]) continue;
-        const float v = fcoef[(size_t)s * Gf.n_r + n];
-        float wx[3], wy[3], wz[NZ];
-#pragma unroll
-        for (int k = 0; k < 3; ++k) {
-          wx[k] = lin_w(gx - 3 * (cx0 + k));
-          wy[k] = lin_w(gy - 3 * (cy0 + k));
-        }
-#pragma unroll
-        for (int k = 0; k < NZ; ++k) wz[k] = DIM == 3 ? lin_w(gz - 3 * (cz0 + k)) : 1.f;
-#pragma unroll
-        for (int kz = 0; kz < NZ; ++kz)
-#pragma unroll
-          for (int ky = 0; ky < 3; ++ky) {
-            const float vyz = v * (wz[kz] * wy[ky]);
-#pragma unroll
-            for (int kx = 0; kx < 3; ++kx) out[kx + 3 * ky + 9 * kz] = fmaf(vyz, wx[kx], out[kx + 3 * ky + 9 * kz]);
-          }
+      for (int t = -3; t <= 3; ++t) {
+        const int x = 3 * X + t;
+        const bool in = x >= 0 && x < F.nx;
+        if (in && t >= -2 && t <= 2 && !fmask[row + x]) rows |= 1u << (t + 3);
+        if (in && !fmask[far + x]) cols |= 1u << (t + 3);
       }
-      const RegionDev C = cregs[tile_.region];
-#pragma unroll
-      for (int kz = 0; kz < NZ; ++kz)
-#pragma unroll
-        for (int ky = 0; ky < 3; ++ky)
-#pragma unroll
-          for (int kx = 0; kx < 3; ++kx) {
-            const int X = cx0 + kx, Y = cy0 + ky, Z = cz0 + kz;
-            const int o = kx + 3 * ky + 9 * kz;
-            if (X < 0 || X >= C.nx || Y < 0 || Y >= C.ny || Z < 0 || Z >= C.nz ||
-                cmask[C.off + X + C.nx * (Y + C.ny * Z)])
-              out[o] = 0.f;
-          }
+      auto load = [&](int a, int d) {
+        const bool use = (rows >> (a + 3) & 1u) && (cols >> (a + d + 3) & 1u);
+        return use ? fcoef[(size_t)(slot0 + d) * fn_r + row + 3 * X + a] : T(0);
+      };
+      if (Ln::BOX || slot0 == Sten<KIND>::CENTER) rap_axis<true>(load, out);
+      else rap_axis<false>(load, out);
     }
 #pragma unroll
-    for (int o = 0; o < NO; ++o) ap[(size_t)o * Gf.n_r + n] = out[o];
+    for (int o = 0; o < 3; ++o) x1[(size_t)(3 * q + o) * G1.n_r + n] = out[o];
   RMG_END_FOR_NODES
 }
 
-// k_ap_axis32 for a 27-point fine stencil in 3D. Its slots and the weights of P are both tensor
-// products, so the contraction factorises axis by axis, sum_dz wz (sum_dy wy (sum_dx wx A_s)):
-// 243 FMAs instead of 729, and 27 weights per node instead of 243 (the sums are in another
-// order than k_ap_axis32's, equal to FP32 rounding). Bound for 3 blocks per SM (80 registers).
-__global__ void __launch_bounds__(kTile, 3)
-k_ap_tensor27(Grid Gf, const RegionDev* __restrict__ cregs, const float* __restrict__ fcoef,
-              const uint8_t* __restrict__ fmask, const uint8_t* __restrict__ cmask,
-              float* __restrict__ ap) {
-  RMG_FOR_NODES(Gf)
-    float out[27];
+// Masks of the coarse level on three finished entries (offsets (ox, oy, oz) + o e of `axis`) of
+// coarse node (I, J, L), and their store.
+template <typename T>
+__device__ __forceinline__ void rap_store(const T (&out)[3], const Grid& Gc, const RegionDev& R,
+                                          int n, int I, int J, int L, int ox, int oy, int oz,
+                                          int axis, int dim, const uint8_t* __restrict__ cmask,
+                                          const uint8_t* __restrict__ cmult, double mdiag,
+                                          T* __restrict__ ccoef) {
+  const bool masked = cmask[n] != 0;
 #pragma unroll
-    for (int o = 0; o < 27; ++o) out[o] = 0.f;
-    if (!fmask[n]) {
-      int x, y, z;
-      decode(li, R, x, y, z);
-      const int cx0 = floor_div3m1(x), cy0 = floor_div3m1(y), cz0 = floor_div3m1(z);
-      float wx[3][3], wy[3][3], wz[3][3];            // [d + 1][k]: weight of fine offset d - 1
-                                                     // towards coarse node c*0 + k
-#pragma unroll
-      for (int d = 0; d < 3; ++d)
-#pragma unroll
-        for (int k = 0; k < 3; ++k) {
-          wx[d][k] = lin_w(x + d - 1 - 3 * (cx0 + k));
-          wy[d][k] = lin_w(y + d - 1 - 3 * (cy0 + k));
-          wz[d][k] = lin_w(z + d - 1 - 3 * (cz0 + k));
-        }
-#pragma unroll
-      for (int dz = 0; dz < 3; ++dz) {
-        float t2[3][3];                                // [ky][kx]
-#pragma unroll
-        for (int k = 0; k < 9; ++k) t2[k / 3][k % 3] = 0.f;
-#pragma unroll
-        for (int dy = 0; dy < 3; ++dy) {
-          float t1[3] = {0.f, 0.f, 0.f};               // [kx]
-#pragma unroll
-          for (int dx = 0; dx < 3; ++dx) {
-            const int gx = x + dx - 1, gy = y + dy - 1, gz = z + dz - 1;
-            if (gx < 0 || gx >= R.nx || gy < 0 || gy >= R.ny || gz < 0 || gz >= R.nz) continue;
-            // the coefficient and the neighbour's mask are loaded independently (no round trip
-            // between them); a masked neighbour contributes a zero product
-            const float cv = fcoef[(size_t)(dx + 3 * dy + 9 * dz) * Gf.n_r + n];
-            const float v = fmask[R.off + gx + R.nx * (gy + R.ny * gz)] ? 0.f : cv;
-#pragma unroll
-            for (int kx = 0; kx < 3; ++kx) t1[kx] = fmaf(v, wx[dx][kx], t1[kx]);
-          }
-#pragma unroll
-          for (int ky = 0; ky < 3; ++ky)
-#pragma unroll
-            for (int kx = 0; kx < 3; ++kx) t2[ky][kx] = fmaf(t1[kx], wy[dy][ky], t2[ky][kx]);
-        }
-#pragma unroll
-        for (int kz = 0; kz < 3; ++kz)
-#pragma unroll
-          for (int ky = 0; ky < 3; ++ky)
-#pragma unroll
-            for (int kx = 0; kx < 3; ++kx)
-              out[kx + 3 * ky + 9 * kz] = fmaf(t2[ky][kx], wz[dz][kz], out[kx + 3 * ky + 9 * kz]);
-      }
-      const RegionDev C = cregs[tile_.region];
-#pragma unroll
-      for (int kz = 0; kz < 3; ++kz)
-#pragma unroll
-        for (int ky = 0; ky < 3; ++ky)
-#pragma unroll
-          for (int kx = 0; kx < 3; ++kx) {
-            const int X = cx0 + kx, Y = cy0 + ky, Z = cz0 + kz;
-            if (X < 0 || X >= C.nx || Y < 0 || Y >= C.ny || Z < 0 || Z >= C.nz ||
-                cmask[C.off + X + C.nx * (Y + C.ny * Z)])
-              out[kx + 3 * ky + 9 * kz] = 0.f;
-          }
+  for (int o = 0; o < 3; ++o) {
+    const int px = ox, py = axis == 1 ? o - 1 : oy, pz = axis == 2 ? o - 1 : oz;
+    const int x = I + px, y = J + py, z = L + pz;
+    const int slot = (px + 1) + 3 * (py + 1) + (dim == 3 ? 9 * (pz + 1) : 0);
+    T v = T(0);
+    if (masked) {
+      if (px == 0 && py == 0 && pz == 0) v = T(mdiag) / T(cmult[n]);
+    } else if (x >= 0 && x < R.nx && y >= 0 && y < R.ny && z >= 0 && z < R.nz &&
+               !cmask[R.off + x + R.nx * (y + R.ny * z)]) {
+      v = out[o] * T(dim == 3 ? 1.0 / 729.0 : 1.0 / 81.0);
     }
+    ccoef[(size_t)slot * Gc.n_r + n] = v;
+  }
+}
+
+// Step 2, blockIdx.y = 3 (dz + 1) + ox + 1 (2D: ox + 1): along y from x1 on (X, y, z) to (X, Y, z);
+// y2[(9 (dz + 1) + 3 (oy + 1) + ox + 1) * n2 + .] in 3D, the coarse stencil itself in 2D.
+template <int KIND, typename T>
+__global__ void __launch_bounds__(kTile)
+k_rap_next(Grid G2, const RegionDev* __restrict__ regs1, int n1, const T* __restrict__ x1,
+           T* __restrict__ y2, const uint8_t* __restrict__ cmask,
+           const uint8_t* __restrict__ cmult, double mdiag) {
+  using Ln = Lines<KIND>;
+  const int ox = (int)blockIdx.y % 3 - 1, dz = Ln::DIM == 3 ? (int)blockIdx.y / 3 - 1 : 0;
+  RMG_FOR_NODES(G2)
+    int X, Y, z;
+    decode(li, R, X, Y, z);
+    const RegionDev F = regs1[tile_.region];
+    const int at = F.off + X + F.nx * (3 * Y + F.ny * z);
+    T out[3] = {T(0), T(0), T(0)};
+    auto load = [&](int b, int d) {
+      const int y = 3 * Y + b;
+      const int line = Ln::DIM == 2 ? d + 1 : Ln::BOX ? 3 * (dz + 1) + d + 1
+                     : dz != 0 ? (dz < 0 ? 0 : 4) : 2 + d;
+      return y >= 0 && y < F.ny ? x1[(size_t)(3 * line + ox + 1) * n1 + at + F.nx * b] : T(0);
+    };
+    if (Ln::BOX || dz == 0) rap_axis<true>(load, out);
+    else rap_axis<false>(load, out);
+    if (Ln::DIM == 2) {
+      rap_store(out, G2, R, n, X, Y, 0, ox, 0, 0, 1, 2, cmask, cmult, mdiag, y2);
+    } else {
 #pragma unroll
-    for (int o = 0; o < 27; ++o) ap[(size_t)o * Gf.n_r + n] = out[o];
+      for (int o = 0; o < 3; ++o)
+        y2[(size_t)(9 * (dz + 1) + 3 * o + ox + 1) * G2.n_r + n] = out[o];
+    }
+  RMG_END_FOR_NODES
+}
+
+// Step 3 (3D), blockIdx.y = 3 (oy + 1) + ox + 1: along z to the coarse stencil.
+template <typename T>
+__global__ void __launch_bounds__(kTile)
+k_rap_last(Grid Gc, const RegionDev* __restrict__ regs2, int n2, const T* __restrict__ y2,
+           const uint8_t* __restrict__ cmask, const uint8_t* __restrict__ cmult, double mdiag,
+           T* __restrict__ ccoef) {
+  const int ox = (int)blockIdx.y % 3 - 1, oy = (int)blockIdx.y / 3 - 1;
+  RMG_FOR_NODES(Gc)
+    int I, J, L;
+    decode(li, R, I, J, L);
+    const RegionDev F = regs2[tile_.region];
+    const int plane = F.nx * F.ny, at = F.off + I + F.nx * J + plane * 3 * L;
+    T out[3] = {T(0), T(0), T(0)};
+    auto load = [&](int c, int d) {
+      const int z = 3 * L + c;
+      return z >= 0 && z < F.nz
+                 ? y2[(size_t)(9 * (d + 1) + 3 * (oy + 1) + ox + 1) * n2 + at + plane * c] : T(0);
+    };
+    rap_axis<true>(load, out);
+    rap_store(out, Gc, R, n, I, J, L, ox, oy, 0, 2, 3, cmask, cmult, mdiag, ccoef);
   RMG_END_FOR_NODES
 }
 
@@ -323,82 +314,14 @@ k_level0_fp32(Grid G, const double* __restrict__ coef, float* __restrict__ coef3
   if (__syncthreads_or(bad) && threadIdx.x == 0) *asym = 1;
 }
 
-template <int DIM, bool CHECK, bool STORED, typename T>
-__device__ __forceinline__ void rtap_sum(const T* __restrict__ ap, int fn_r,
-                                         const RegionDev& F, const float* __restrict__ wr,
-                                         int I, int J, int L, T (&acc)[27]) {
-  constexpr int ZL = DIM == 3 ? -2 : 0, ZH = DIM == 3 ? 2 : 0;
-#pragma unroll
-  for (int c = ZL; c <= ZH; ++c) {
-    const int fz = DIM == 3 ? 3 * L + c : 0;
-    if (CHECK && (fz < 0 || fz >= F.nz)) continue;
-#pragma unroll
-    for (int b = -2; b <= 2; ++b) {
-      const int fy = 3 * J + b;
-      if (CHECK && (fy < 0 || fy >= F.ny)) continue;
-#pragma unroll
-      for (int a = -2; a <= 2; ++a) {
-        const int fx = 3 * I + a;
-        if (CHECK && (fx < 0 || fx >= F.nx)) continue;
-        const int f = F.off + fx + F.nx * (fy + F.ny * fz);
-        T wf;
-        if (STORED) {
-          const float wz = DIM == 3 ? pw_seen_from_coarse<float>(wr, fn_r, f, 2, c) : 1.f;
-          wf = T(wz * (pw_seen_from_coarse<float>(wr, fn_r, f, 1, b) *
-                       pw_seen_from_coarse<float>(wr, fn_r, f, 0, a)));
-        } else {
-          wf = T((DIM == 3 ? w1d(c) : 1.0) * (w1d(b) * w1d(a)));   // compile-time constant
-        }
-        // ap of node f is stored relative to the coarse node (f - 1) div 3 on each axis,
-        // which is C - 1 for offsets a <= 0 and C for a >= 1
-        const int bx = a <= 0 ? 1 : 0, by = b <= 0 ? 1 : 0, bz = DIM == 3 ? (c <= 0 ? 1 : 0) : 0;
-#pragma unroll
-        for (int oz = (DIM == 3 ? -1 : 0); oz <= (DIM == 3 ? 1 : 0); ++oz)
-#pragma unroll
-          for (int oy = -1; oy <= 1; ++oy)
-#pragma unroll
-            for (int ox = -1; ox <= 1; ++ox) {
-              const int ix = ox + bx, iy = oy + by, iz = oz + bz;
-              if (ix < 0 || ix > 2 || iy < 0 || iy > 2 || iz < 0 || iz > 2) continue;
-              // (A P)(f, C + o) vanishes unless |f - 3 (C + o)| <= 3 on every axis (A reaches
-              // one node, P two): skip those structural zeros (compile-time, exact)
-              if (3 * ox - a > 3 || a - 3 * ox > 3 || 3 * oy - b > 3 || b - 3 * oy > 3) continue;
-              if (DIM == 3 && (3 * oz - c > 3 || c - 3 * oz > 3)) continue;
-              const int slot = (ox + 1) + 3 * (oy + 1) + (DIM == 3 ? 9 * (oz + 1) : 0);
-              acc[slot] = fma(wf, ap[(size_t)(ix + 3 * iy + 9 * iz) * fn_r + f], acc[slot]);
-            }
-      }
-    }
-  }
-}
+// Galerkin product with stored per-node weights, in two steps following the product order R (A P):
+//  1. k_ap_w: for every fine node f, row f of [[A]] [[P]], i.e. sum_s A_s(f) P(f + d_s, C') for
+//     the (at most 3 per axis) coarse nodes C' near f, stored relative to the coarse node
+//     (x - 1) div 3 on each axis: ap[o][f], o = ox + 3 oy + 9 oz.
+//  2. k_rtap_w: for every coarse node C, sum over the fine nodes f = 3C + (a, b, c) of its
+//     support of P(f, C) ap[.][f].
+__device__ __forceinline__ int floor_div3m1(int x) { return (x + 2) / 3 - 1; }   // (x-1) div 3, x >= 0
 
-template <int CK, int DIM, typename T>
-__global__ void __launch_bounds__(kTile)
-k_rtap(Grid Gc, const RegionDev* __restrict__ fregs, const T* __restrict__ ap, int fn_r,
-       const uint8_t* __restrict__ cmask, const uint8_t* __restrict__ cmult, double mdiag,
-       T* __restrict__ ccoef) {
-  using CS = Sten<CK>;
-  RMG_FOR_NODES(Gc)
-    T acc[27];
-#pragma unroll
-    for (int o = 0; o < 27; ++o) acc[o] = T(0);
-    if (cmask[n]) {
-      acc[DIM == 3 ? 13 : 4] = T(mdiag) / T(cmult[n]);
-    } else {
-      int I, J, L;
-      decode(li, R, I, J, L);
-      const RegionDev F = fregs[tile_.region];
-      const bool inner = I > 0 && I < R.nx - 1 && J > 0 && J < R.ny - 1 &&
-                         (DIM == 2 || (L > 0 && L < R.nz - 1));
-      if (inner) rtap_sum<DIM, false, false, T>(ap, fn_r, F, nullptr, I, J, L, acc);
-      else rtap_sum<DIM, true, false, T>(ap, fn_r, F, nullptr, I, J, L, acc);
-    }
-#pragma unroll
-    for (int s = 0; s < CS::S; ++s) ccoef[(size_t)s * Gc.n_r + n] = acc[s];
-  RMG_END_FOR_NODES
-}
-
-// Galerkin product with stored per-node weights (same two steps as k_ap / k_rtap).
 template <int FK, int DIM, typename T>
 __global__ void __launch_bounds__(kTile)
 k_ap_w(Grid Gf, const RegionDev* __restrict__ cregs, const T* __restrict__ fcoef,
@@ -447,6 +370,50 @@ k_ap_w(Grid Gf, const RegionDev* __restrict__ cregs, const T* __restrict__ fcoef
   RMG_END_FOR_NODES
 }
 
+template <int DIM, bool CHECK, typename T>
+__device__ __forceinline__ void rtap_sum(const T* __restrict__ ap, int fn_r,
+                                         const RegionDev& F, const float* __restrict__ wr,
+                                         int I, int J, int L, T (&acc)[27]) {
+  constexpr int ZL = DIM == 3 ? -2 : 0, ZH = DIM == 3 ? 2 : 0;
+#pragma unroll
+  for (int c = ZL; c <= ZH; ++c) {
+    const int fz = DIM == 3 ? 3 * L + c : 0;
+    if (CHECK && (fz < 0 || fz >= F.nz)) continue;
+#pragma unroll
+    for (int b = -2; b <= 2; ++b) {
+      const int fy = 3 * J + b;
+      if (CHECK && (fy < 0 || fy >= F.ny)) continue;
+#pragma unroll
+      for (int a = -2; a <= 2; ++a) {
+        const int fx = 3 * I + a;
+        if (CHECK && (fx < 0 || fx >= F.nx)) continue;
+        const int f = F.off + fx + F.nx * (fy + F.ny * fz);
+        const float wz = DIM == 3 ? pw_seen_from_coarse<float>(wr, fn_r, f, 2, c) : 1.f;
+        const T wf = T(wz * (pw_seen_from_coarse<float>(wr, fn_r, f, 1, b) *
+                             pw_seen_from_coarse<float>(wr, fn_r, f, 0, a)));
+        // ap of node f is stored relative to the coarse node (f - 1) div 3 on each axis,
+        // which is C - 1 for offsets a <= 0 and C for a >= 1
+        const int bx = a <= 0 ? 1 : 0, by = b <= 0 ? 1 : 0, bz = DIM == 3 ? (c <= 0 ? 1 : 0) : 0;
+#pragma unroll
+        for (int oz = (DIM == 3 ? -1 : 0); oz <= (DIM == 3 ? 1 : 0); ++oz)
+#pragma unroll
+          for (int oy = -1; oy <= 1; ++oy)
+#pragma unroll
+            for (int ox = -1; ox <= 1; ++ox) {
+              const int ix = ox + bx, iy = oy + by, iz = oz + bz;
+              if (ix < 0 || ix > 2 || iy < 0 || iy > 2 || iz < 0 || iz > 2) continue;
+              // (A P)(f, C + o) vanishes unless |f - 3 (C + o)| <= 3 on every axis (A reaches
+              // one node, P two): skip those structural zeros (compile-time, exact)
+              if (3 * ox - a > 3 || a - 3 * ox > 3 || 3 * oy - b > 3 || b - 3 * oy > 3) continue;
+              if (DIM == 3 && (3 * oz - c > 3 || c - 3 * oz > 3)) continue;
+              const int slot = (ox + 1) + 3 * (oy + 1) + (DIM == 3 ? 9 * (oz + 1) : 0);
+              acc[slot] = fma(wf, ap[(size_t)(ix + 3 * iy + 9 * iz) * fn_r + f], acc[slot]);
+            }
+      }
+    }
+  }
+}
+
 template <int CK, int DIM, typename T>
 __global__ void __launch_bounds__(kTile)
 k_rtap_w(Grid Gc, const RegionDev* __restrict__ fregs, const T* __restrict__ ap, int fn_r,
@@ -465,8 +432,8 @@ k_rtap_w(Grid Gc, const RegionDev* __restrict__ fregs, const T* __restrict__ ap,
       const RegionDev F = fregs[tile_.region];
       const bool inner = I > 0 && I < R.nx - 1 && J > 0 && J < R.ny - 1 &&
                          (DIM == 2 || (L > 0 && L < R.nz - 1));
-      if (inner) rtap_sum<DIM, false, true, T>(ap, fn_r, F, wr, I, J, L, acc);
-      else rtap_sum<DIM, true, true, T>(ap, fn_r, F, wr, I, J, L, acc);
+      if (inner) rtap_sum<DIM, false, T>(ap, fn_r, F, wr, I, J, L, acc);
+      else rtap_sum<DIM, true, T>(ap, fn_r, F, wr, I, J, L, acc);
     }
 #pragma unroll
     for (int s = 0; s < CS::S; ++s) ccoef[(size_t)s * Gc.n_r + n] = acc[s];
