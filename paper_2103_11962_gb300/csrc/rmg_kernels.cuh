@@ -55,8 +55,11 @@ __device__ __forceinline__ int region_of(const RegionDev* R, int nreg, int n) {
   return lo;
 }
 
-#define RMG_FOR_NODES(G)                                                       \
+#define RMG_FOR_NODES(G) RMG_FOR_NODES_AHEAD(G, )
+// The same with a statement that every thread runs before its node, with the block's tile t_.
+#define RMG_FOR_NODES_AHEAD(G, AHEAD)                                          \
   for (int t_ = blockIdx.x; t_ < (G).ntiles; t_ += gridDim.x) {                \
+    AHEAD;                                                                     \
     const Tile tile_ = (G).tiles[t_];                                          \
     const RegionDev R = (G).regions[tile_.region];                             \
     int li, bi_ = -1, bj_ = 0, bl_ = 0;                                        \
@@ -168,6 +171,37 @@ __device__ __forceinline__ float stencil_row_half(const float* __restrict__ half
   return au;
 }
 
+// L2 prefetch of what a block's next run tile reads first-hand: its `planes` coefficient planes of
+// stride n_r, the epilogue's arrays, and u one z-plane ahead (the rest of u is in L2 from earlier
+// tiles). One thread per array asks for the tile's piece of it (up to 1 KB) with one bulk
+// instruction, so that the loads of the next tile find their lines in L2. The ends are cut to
+// 16-byte boundaries inside the array. For the 7-point half planes only (8 arrays a tile): a
+// Chebyshev sweep of 6M nodes 69 -> 58 us (41 bytes a node, 0.53 -> 0.64 of the measured HBM
+// rate); the 27-point ones (18 arrays a tile) got slower, 857 -> 1035 us for 36M nodes.
+template <class Epi>
+__device__ __forceinline__ void prefetch_tile(const Grid& G, int t, const float* coef, int planes,
+                                              const float* u, const Epi& epi) {
+  const int q = threadIdx.x;
+  if (t >= G.ntiles || q > planes + Epi::kReads || G.lx >= 0) return;
+  const Tile tile = G.tiles[t];
+  const RegionDev R = G.regions[tile.region];
+  const int nodes = R.nx * R.ny * R.nz;
+  int a = tile.start, e = min(tile.start + kTile, nodes);
+  const float* base = coef + (size_t)q * G.n_r;
+  if (q == planes) {
+    base = u;
+    a = min(a + R.nx * R.ny, nodes);
+    e = min(e + R.nx * R.ny, nodes);
+  } else if (q > planes) {
+    base = epi.reads(q - planes - 1);
+  }
+  const uintptr_t lo = (reinterpret_cast<uintptr_t>(base + R.off + a) + 15) & ~(uintptr_t)15;
+  const uintptr_t hi = reinterpret_cast<uintptr_t>(base + R.off + e) & ~(uintptr_t)15;
+  if (hi > lo)
+    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;\n" ::"l"(lo), "r"((unsigned)(hi - lo))
+                 : "memory");
+}
+
 // Phase A of the FP32 cycle on a level with half planes: the half form when the pack found the
 // operator symmetric (*asym == 0), else the full planes as k_stencil.
 template <bool HALF, int KIND, class Epi>
@@ -175,7 +209,7 @@ __device__ __forceinline__ void stencil_pass(const Grid& G, const float* __restr
                                              const float* __restrict__ u,
                                              const uint8_t* __restrict__ mult,
                                              float* __restrict__ y, const Epi& epi) {
-  RMG_FOR_NODES(G)
+  RMG_FOR_NODES_AHEAD(G, if (HALF && KIND == 7) prefetch_tile(G, t_ + (int)gridDim.x, coef, 4, u, epi))
     int i, j, l;
     RMG_DECODE(i, j, l);
     const float au = HALF ? stencil_row_half<KIND>(coef, u, n, G.n_r, i, j, l, R)
@@ -521,30 +555,40 @@ __device__ __forceinline__ T inv_mult(int m) {
 template <typename T>
 struct EpiStore {                 // out = A u
   T* out;
+  static constexpr int kReads = 0;
+  __device__ const T* reads(int) const { return nullptr; }
   __device__ void operator()(int n, T au, int) const { out[n] = au; }
 };
 
 template <typename T>
 struct EpiScaled {                // out = D~^-1 A u (power method)
   const T* dinv; T* out;
+  static constexpr int kReads = 1;   // arrays read at the node (prefetch_tile)
+  __device__ const T* reads(int k) const { return dinv; }
   __device__ void operator()(int n, T au, int) const { out[n] = dinv[n] * au; }
 };
 
 template <typename T>
 struct EpiResid {                 // r = b - A u
   const T* b; T* r;
+  static constexpr int kReads = 1;   // arrays read at the node (prefetch_tile)
+  __device__ const T* reads(int k) const { return b; }
   __device__ void operator()(int n, T au, int) const { r[n] = b[n] - au; }
 };
 
 template <typename T>
 struct EpiResidScaled {           // r = (b - A u) / mult: the [[Psi Psi^T]]^-1 of restriction
   const T* b; T* r;
+  static constexpr int kReads = 1;   // arrays read at the node (prefetch_tile)
+  __device__ const T* reads(int k) const { return b; }
   __device__ void operator()(int n, T au, int m) const { r[n] = (b[n] - au) * inv_mult<T>(m); }
 };
 
 template <typename T>
 struct EpiJacobi {                // u_out = u + omega D~^-1 (b - A u)
   const T* u; const T* b; const T* dinv; T omega; T* uo;
+  static constexpr int kReads = 2;   // arrays read at the node (prefetch_tile)
+  __device__ const T* reads(int k) const { return k == 0 ? b : dinv; }
   __device__ void operator()(int n, T au, int) const {
     const T r = b[n] - au;
     uo[n] = fma(omega * dinv[n], r, u[n]);
@@ -556,6 +600,8 @@ struct EpiJacobi {                // u_out = u + omega D~^-1 (b - A u)
 template <typename T>
 struct EpiCheb0 {                 // first Chebyshev step: d = D~^-1 r / theta, u_out = u + d
   const T* u; const T* b; const T* dinv; const T* c2; T* d; T* uo;
+  static constexpr int kReads = 2;   // arrays read at the node (prefetch_tile)
+  __device__ const T* reads(int k) const { return k == 0 ? b : dinv; }
   __device__ void operator()(int n, T au, int) const {
     const T r = b[n] - au;
     const T dn = (dinv[n] * r) * (*c2);
@@ -567,6 +613,8 @@ struct EpiCheb0 {                 // first Chebyshev step: d = D~^-1 r / theta, 
 template <typename T>
 struct EpiCheb {                  // d = c1 d + c2 D~^-1 r, u_out = u + d
   const T* u; const T* b; const T* dinv; const T* c1; const T* c2; T* d; T* uo;
+  static constexpr int kReads = 3;   // arrays read at the node (prefetch_tile)
+  __device__ const T* reads(int k) const { return k == 0 ? b : k == 1 ? dinv : d; }
   __device__ void operator()(int n, T au, int) const {
     const T r = b[n] - au;
     const T dn = (*c1) * d[n] + ((*c2) * dinv[n]) * r;
@@ -602,6 +650,8 @@ __global__ void k_cheb0_zero(int n, const T* __restrict__ b, const T* __restrict
 template <typename T>
 struct EpiResidZero {              // r = b - A u, delta = 0
   const T* b; T* r; T* delta;
+  static constexpr int kReads = 1;   // arrays read at the node (prefetch_tile)
+  __device__ const T* reads(int k) const { return b; }
   __device__ void operator()(int n, T au, int) const {
     r[n] = b[n] - au;
     delta[n] = T(0);
