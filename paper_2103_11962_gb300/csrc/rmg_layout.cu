@@ -580,15 +580,132 @@ __device__ __forceinline__ void cp_async8(void* smem, const void* gmem) {
 // keeps the lanes' reads of their own rows free of bank conflicts).
 constexpr int kSplitChunk = 9;
 
-// Single-copy rows (the rows of shared nodes are left to k_split_shared, so that a warp of
-// single-copy rows does not wait on the longer path of the interface rows among them). A warp
-// takes 32 consecutive nodes of a tile. Their CSR rows are staged through shared memory nine
-// entries at a time, the lanes copying the 32 rows' entries together (the rows of consecutive
-// nodes lie side by side in the CSR, so each pass reads whole sectors once); then every lane
-// handles its own row's entries in order.
+// Rows a warp stages at a time in the direct pass.
+constexpr int kDirectRows = 16;
+
+// The direct pass over 32 consecutive nodes of an affine region: rows that hold the full stencil
+// in column order, with every column where the region's map puts it. Their values go to the slots
+// by position, without a look at any entry but the comparison of its column: the lanes copy the
+// entries of 16 rows to shared memory side by side (whole sectors, all copies in flight
+// together), and store them a slot at a time, 16 nodes side by side. Returns the rows of `cand`
+// that were of that form; the others are left to the general pass, which writes all their slots.
+template <int KIND, int B>
+__device__ __forceinline__ unsigned split_direct(unsigned cand, int g, int64_t e0, const int4& af,
+                                                 const int64_t* __restrict__ col,
+                                                 const double* __restrict__ val, int64_t* bc,
+                                                 double* bv, double* cbase, int n_r) {
+  using S = Sten<KIND>;
+  constexpr int RP = 32 / S::S;                  // rows of one copy
+  const int lane = threadIdx.x & 31;
+  const int sub = lane / S::S, k = lane - sub * S::S;
+  unsigned bad = 0;
+  for (int half = 0; half < 2; ++half) {
+    if (!((cand >> (16 * half)) & 0xffffu)) continue;
+    for (int t = 0; t < B; ++t) {                // entries t S .. t S + S - 1 of the rows
+      const int e = t * S::S + k, slot = e / B, comp = e - slot * B;
+#pragma unroll 4
+      for (int r0 = 0; r0 < kDirectRows; r0 += RP) {
+        const int r = r0 + sub, from = 16 * half + (r & 15);
+        const int64_t er = __shfl_sync(0xffffffffu, (long long)e0, from);
+        if (sub < RP && r < kDirectRows && ((cand >> from) & 1u)) {
+          cp_async8(bc + r * S::S + k, col + er + e);
+          cp_async8(bv + r * S::S + k, val + er + e);
+        }
+      }
+      asm volatile("cp.async.wait_all;\n" ::: "memory");
+      __syncwarp();
+      const int64_t off =
+          (int64_t)(S::dx(slot) + af.y * S::dy(slot) + (S::DIM == 3 ? af.z * S::dz(slot) : 0)) * B +
+          comp;
+#pragma unroll 4
+      for (int r0 = 0; r0 < kDirectRows; r0 += RP) {
+        const int r = r0 + sub, from = 16 * half + (r & 15);
+        const int gr = __shfl_sync(0xffffffffu, g, from);
+        if (sub < RP && r < kDirectRows && ((cand >> from) & 1u) &&
+            bc[r * S::S + k] != (int64_t)gr * B + off)
+          bad |= 1u << from;
+      }
+      const int row = lane & 15, q = 16 * half + row;
+      if ((cand >> q) & 1u) {
+#pragma unroll
+        for (int k0 = 0; k0 < S::S; k0 += 2) {
+          const int k2 = k0 + (lane >> 4), e2 = t * S::S + k2, s2 = e2 / B;
+          if (k2 < S::S)
+            cbase[((size_t)(e2 - s2 * B) * S::S + s2) * n_r + q] = bv[row * S::S + k2];
+        }
+      }
+      __syncwarp();
+    }
+  }
+  return cand & ~__reduce_or_sync(0xffffffffu, bad);
+}
+
+// The direct pass over single-copy rows in regions with an affine map; a warp takes 32
+// consecutive nodes of a tile. The single-copy rows that are left (cut by the domain boundary or
+// by a mask, out of order, or of a region without an affine map) go to a list, {node, region},
+// for k_split_rows. One kernel for both forms held this pass to two blocks per SM, and a warp
+// with one row left waited for it as long as for 32 (477 us for them in a kernel of their own
+// over the tiles, 170 us from the list). 10.6M nodes of a 27-point stencil: the single-copy rows
+// 2571 -> 1716 us; the direct pass moves its 6.3 GB at 4.1 TB/s, 0.61 of the measured rate,
+// bound by the latency of its copies.
+template <int KIND, int B>
+__global__ void __launch_bounds__(kTile / 2, 8)
+k_split_direct(Grid G, const int* __restrict__ gid, const uint8_t* __restrict__ mult,
+               const int4* __restrict__ affine, const int64_t* __restrict__ rowptr,
+               const int64_t* __restrict__ col, const double* __restrict__ val,
+               double* __restrict__ coef, int2* __restrict__ left, int* __restrict__ nleft) {
+  constexpr int kWarps = kTile / 32, kOwn = kWarps / 2;   // warps of a tile, of this block
+  using S = Sten<KIND>;
+  __shared__ __align__(16) int64_t s_col[kOwn][kDirectRows * S::S];
+  __shared__ __align__(16) double s_val[kOwn][kDirectRows * S::S];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int c_row = blockIdx.y;
+  const int tasks = G.ntiles * kWarps;
+  for (int task = blockIdx.x * kOwn + warp; task < tasks; task += gridDim.x * kOwn) {
+    const Tile tile = G.tiles[task / kWarps];
+    const RegionDev R = G.regions[tile.region];
+    const int li = tile.start + (task % kWarps) * 32 + lane;
+    const int n = R.off + li;
+    const int4 af = affine[tile.region];
+    const bool single = li < R.nx * R.ny * R.nz && mult[n] == 1;
+    unsigned ok = 0;
+    if (af.w) {
+      int i, j, l;
+      decode(single ? li : 0, R, i, j, l);
+      bool cand = single && i > 0 && i < R.nx - 1 && j > 0 && j < R.ny - 1 &&
+                  (S::DIM == 2 || (l > 0 && l < R.nz - 1));
+      int64_t e0 = 0;
+      int g = 0;
+      if (cand) {
+        g = gid[n];
+        const int64_t row = (int64_t)g * B + c_row;
+        e0 = rowptr[row];
+        cand = rowptr[row + 1] - e0 == B * S::S;
+      }
+      const unsigned rows = __ballot_sync(0xffffffffu, cand);
+      if (rows)
+        ok = split_direct<KIND, B>(rows, g, e0, af, col, val, s_col[warp], s_val[warp],
+                                   coef + (size_t)c_row * B * S::S * G.n_r + (n - lane), G.n_r);
+    }
+    const unsigned rest = __ballot_sync(0xffffffffu, single) & ~ok;
+    if (!rest) continue;
+    int at = 0;
+    if (lane == 0) at = atomicAdd(nleft + c_row, __popc(rest));
+    at = __shfl_sync(0xffffffffu, at, 0);
+    if ((rest >> lane) & 1u)
+      left[(size_t)c_row * G.n_r + at + __popc(rest & ((1u << lane) - 1u))] =
+          make_int2(n, tile.region);
+  }
+}
+
+// The listed rows, a warp for 32 of them (their order in the list is of no consequence: every row
+// writes its own slots). The CSR rows are staged through shared memory nine entries at a time,
+// the lanes copying the 32 rows' entries together (mostly rows that lie side by side in the CSR);
+// then every lane handles its own row's entries in order.
 template <int KIND, int B>
 __global__ void __launch_bounds__(kTile)
-k_split_csr(Grid G, RMG_SPLIT_PARAMS) {
+k_split_rows(const int2* __restrict__ left, const int* __restrict__ nleft,
+             const RegionDev* __restrict__ regions, int n_r, RMG_SPLIT_PARAMS) {
   constexpr int kWarps = kTile / 32;
   __shared__ __align__(16) int64_t s_col[kWarps][32 * kSplitChunk];
   __shared__ __align__(16) double s_val[kWarps][32 * kSplitChunk];
@@ -597,19 +714,17 @@ k_split_csr(Grid G, RMG_SPLIT_PARAMS) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   int64_t* wc = s_col[warp];
   double* wv = s_val[warp];
-  const int c_row = blockIdx.y;
-  const int tasks = G.ntiles * kWarps;
-  for (int task = blockIdx.x * kWarps + warp; task < tasks; task += gridDim.x * kWarps) {
-    const Tile tile = G.tiles[task / kWarps];
-    const RegionDev R = G.regions[tile.region];
-    const int li = tile.start + (task % kWarps) * 32 + lane;
-    const int n = R.off + li;
-    const bool active = li < R.nx * R.ny * R.nz && mult[n] == 1;
+  const int c_row = blockIdx.y, count = nleft[c_row];
+  for (int first = 32 * (blockIdx.x * kWarps + warp); first < count;
+       first += 32 * gridDim.x * kWarps) {
+    const bool active = first + lane < count;
     RowSplit<KIND, B> rs;
     int64_t e0 = 0;
     int len = 0;
     if (active) {
-      rs.begin(n, li, tile.region, R, c_row, G.n_r, gid, mult, affine, coef);
+      const int2 node = left[(size_t)c_row * n_r + first + lane];
+      const RegionDev R = regions[node.y];
+      rs.begin(node.x, node.x - R.off, node.y, R, c_row, n_r, gid, mult, affine, coef);
       const int64_t row = (int64_t)rs.g * B + c_row;
       e0 = rowptr[row];
       len = (int)(rowptr[row + 1] - e0);
@@ -736,16 +851,27 @@ void split_from_csr(Ctx& c, Level& L, int kind, int B, const int64_t* rowptr, co
     RMG_LAUNCHED();
   }
   if (L.affine.n < (size_t)L.nreg) build_affine(c, L);
-  // single-copy rows over the tiles, then the rows of shared nodes over the group slots; both
-  // grids are one resident wave
+  L.split_left.ensure((size_t)B * L.n_r);
+  L.split_nleft.ensure(B);
+  RMG_CUDA(cudaMemsetAsync(L.split_nleft.get(), 0, L.split_nleft.bytes(), c.stream));
+  // single-copy rows over the tiles, the rows that this left, then the rows of shared nodes over
+  // the group slots; all grids are one resident wave
 #define RMG_SPLIT_ARGS                                                                     \
   L.gid.get(), L.mult.get(), L.c2r.get(), L.cgrp.get(), L.gptr.get(), L.gslot.get(),        \
       L.rid.get(), L.affine.get(), rowptr, col, val, L.ncomp, L.coef.get(), c.d_err.get()
 #define RMG_SPLIT(K, BB)                                                                    \
   do {                                                                                      \
-    const dim3 gb(persistent_grid(c, G.ntiles, resident_per_sm((const void*)k_split_csr<K, BB>)), \
+    /* blocks of half a tile; eight fit an SM with 27 KB of shared memory each */           \
+    const dim3 gd(persistent_grid(c, 2 * G.ntiles), B);                                     \
+    k_split_direct<K, BB><<<gd, kTile / 2, 0, c.stream>>>(                                  \
+        G, L.gid.get(), L.mult.get(), L.affine.get(), rowptr, col, val, L.coef.get(),       \
+        L.split_left.get(), L.split_nleft.get());                                           \
+    RMG_LAUNCHED();                                                                         \
+    const dim3 gb(persistent_grid(c, G.ntiles, resident_per_sm((const void*)k_split_rows<K, BB>)), \
                   B);                                                                       \
-    k_split_csr<K, BB><<<gb, kTile, 0, c.stream>>>(G, RMG_SPLIT_ARGS);                      \
+    k_split_rows<K, BB><<<gb, kTile, 0, c.stream>>>(L.split_left.get(), L.split_nleft.get(), \
+                                                    L.regions.get(), L.n_r, RMG_SPLIT_ARGS); \
+    RMG_LAUNCHED();                                                                         \
     if (L.nslots) {                                                                         \
       const dim3 gs(persistent_grid(c, (L.nslots + kTile - 1) / kTile,                      \
                                     resident_per_sm((const void*)k_split_shared<K, BB>)),   \

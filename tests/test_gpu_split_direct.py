@@ -1,0 +1,77 @@
+"""The split's direct pass: rows in column order go by position, every other form of the same row
+goes entry by entry with the same result."""
+import numpy as np
+import pytest
+
+import workloads as W
+
+torch = pytest.importorskip("torch")
+pytestmark = [pytest.mark.gpu,
+              pytest.mark.filterwarnings("ignore::scipy.sparse.SparseEfficiencyWarning")]
+
+PROBLEMS = {
+    "5-point": (lambda: W.poisson2d_5pt(region_grid=(2, 3), n=10), 5, 1),
+    "9-point": (lambda: W.q1_laplace2d(region_grid=(3, 2), n=10), 9, 1),
+    "7-point": (lambda: W.diffusion3d_7pt(region_grid=(2, 2, 1), choices=(10, 19), seed=2), 7, 1),
+    "27-point": (lambda: W.q1_laplace3d(region_grid=(2, 1, 2), n=10), 27, 1),
+    "27-point blocks": (lambda: W.elasticity3d(region_grid=(2, 1, 1), choices=(10,), seed=2), 27, 3),
+}
+
+
+def _split(ctx, p, kind, B, rowptr, col, val, gids):
+    from paper_2103_11962_gb300 import rmg
+    lay = rmg.Layout(ctx, p.dim, p.region_dims, gids, p.n_nodes, None)
+    t = [torch.from_numpy(np.ascontiguousarray(a)).cuda() for a in (rowptr, col, val)]
+    if B == 1:
+        lay.operator_from_csr(kind, *t)
+    else:
+        lay.operator_from_block_csr(kind, B, *t)
+    h = rmg.Hierarchy(lay, rmg.default_options(levels=1))
+    n = h.level_sizes(0)[0]
+    coef = torch.empty(B * B * kind * n, dtype=torch.float64, device="cuda")
+    h.level_export(0, coef)
+    return coef.view(B, B, kind, n).cpu().numpy()
+
+
+@pytest.mark.parametrize("name", list(PROBLEMS))
+def test_forms_of_a_row(name):
+    from paper_2103_11962_gb300 import rmg
+    make, kind, B = PROBLEMS[name]
+    p = make()
+    A = p.A.tocsr()
+    A.sort_indices()
+    rp, col, val = A.indptr.astype(np.int64), A.indices.astype(np.int64), A.data.copy()
+    # every entry its own value (and the matrix still positive definite)
+    val *= 1.0 + 1e-6 * np.random.default_rng(1).uniform(-1.0, 1.0, val.size)
+    gids = torch.from_numpy(np.asarray(p.region_gids, dtype=np.int64)).cuda()
+    ctx = rmg.Context(0)
+    want = _split(ctx, p, kind, B, rp, col, val, gids)
+    copies = np.bincount(p.region_gids, minlength=p.n_nodes)
+    single = copies[p.region_gids] == 1
+    # the matrix entries themselves at single-copy rows (centre included)
+    full = np.flatnonzero((np.diff(rp).reshape(-1, B).min(1) == B * kind) & (copies == 1))
+    where = {int(g): n for n, g in enumerate(p.region_gids)}
+    for g in full[:: max(1, full.size // 50)]:
+        for c in range(B):
+            row = val[rp[g * B + c]:rp[g * B + c + 1]].reshape(kind, B)
+            assert np.array_equal(want[c, :, :, where[int(g)]].T, row)
+    # entries of every row in another order: the same bits in single-copy rows, sums in another
+    # order in shared ones (a row has at most 81 entries)
+    rng = np.random.default_rng(2)
+    col2, val2 = col.copy(), val.copy()
+    for r in range(rp.size - 1):
+        o = rp[r] + rng.permutation(rp[r + 1] - rp[r])
+        col2[rp[r]:rp[r + 1]], val2[rp[r]:rp[r + 1]] = col[o], val[o]
+    got = _split(ctx, p, kind, B, rp, col2, val2, gids)
+    assert np.array_equal(got[..., single], want[..., single])
+    assert np.abs(got - want).max() <= 81 * 2.0 ** -52 * np.abs(val).max()
+    # one full row whose first column appears twice and whose second is missing
+    g = int(full[full.size // 2])
+    k = rp[g * B]
+    col3 = col.copy()
+    col3[k + B] = col3[k]
+    got = _split(ctx, p, kind, B, rp, col3, val, gids)
+    expect = want.copy()
+    expect[0, 0, 0, where[g]] = val[k] + val[k + B]
+    expect[0, 0, 1, where[g]] = 0.0
+    assert np.array_equal(got, expect)
