@@ -142,7 +142,17 @@ __host__ __device__ constexpr bool mirrored_slots() {
   return true;
 }
 
-template <int KIND>
+// A 4-byte load from a base all threads share and an unsigned 32-bit byte offset of the thread: an
+// addressing form of the load itself, where a 64-bit element address takes two or three more
+// instructions. A 27-point row has 54 loads, and the sweep issued about 500 instructions a node.
+__device__ __forceinline__ float load32(const float* __restrict__ base, unsigned byte) {
+  return __ldg(reinterpret_cast<const float*>(reinterpret_cast<const char*>(base) + byte));
+}
+// Largest level whose byte offsets into one plane fit 32 bits.
+constexpr int kOffset32Nodes = 1 << 30;
+
+// The row of node n from the half planes; OFF32: n_r <= kOffset32Nodes.
+template <int KIND, bool OFF32>
 __device__ __forceinline__ float stencil_row_half(const float* __restrict__ half,
                                                   const float* __restrict__ u, int n, int n_r,
                                                   int i, int j, int l, const RegionDev& R) {
@@ -163,9 +173,11 @@ __device__ __forceinline__ float stencil_row_half(const float* __restrict__ half
     if (dz > 0) ok &= (l < R.nz - 1);
     if (ok) {
       const int nb = n + dx + dy * sy + dz * sz;
-      const float c = s < C ? half[(size_t)(S::S - 1 - s - C) * (size_t)n_r + nb]
-                            : half[(size_t)(s - C) * (size_t)n_r + n];
-      au = fmaf(c, u[nb], au);
+      const float* plane = half + (size_t)(s < C ? S::S - 1 - s - C : s - C) * (size_t)n_r;
+      const int at = s < C ? nb : n;
+      const float c = OFF32 ? load32(plane, 4u * (unsigned)at) : plane[at];
+      const float v = OFF32 ? load32(u, 4u * (unsigned)nb) : u[nb];
+      au = fmaf(c, v, au);
     }
   }
   return au;
@@ -204,7 +216,7 @@ __device__ __forceinline__ void prefetch_tile(const Grid& G, int t, const float*
 
 // Phase A of the FP32 cycle on a level with half planes: the half form when the pack found the
 // operator symmetric (*asym == 0), else the full planes as k_stencil.
-template <bool HALF, int KIND, class Epi>
+template <bool HALF, bool OFF32, int KIND, class Epi>
 __device__ __forceinline__ void stencil_pass(const Grid& G, const float* __restrict__ coef,
                                              const float* __restrict__ u,
                                              const uint8_t* __restrict__ mult,
@@ -212,19 +224,25 @@ __device__ __forceinline__ void stencil_pass(const Grid& G, const float* __restr
   RMG_FOR_NODES_AHEAD(G, if (HALF && KIND == 7) prefetch_tile(G, t_ + (int)gridDim.x, coef, 4, u, epi))
     int i, j, l;
     RMG_DECODE(i, j, l);
-    const float au = HALF ? stencil_row_half<KIND>(coef, u, n, G.n_r, i, j, l, R)
+    const auto v = epi.load(n);
+    const float au = HALF ? stencil_row_half<KIND, OFF32>(coef, u, n, G.n_r, i, j, l, R)
                           : stencil_row<KIND, float, float, float>(coef, u, n, G.n_r, i, j, l, R);
-    if (mult[n] > 1) y[n] = au; else epi(n, au, 1);
+    if (mult[n] > 1) y[n] = au; else epi.apply(n, v, au, 1);
+
   RMG_END_FOR_NODES
 }
 
-template <int KIND, class Epi>
-__global__ void __launch_bounds__(kTile)
+// Bound by load latency: seven blocks per SM (36 registers) against the five that the compiler
+// chose for EpiCheb. With the 32-bit offsets and the early epilogue loads a 27-point sweep of
+// 35.9M nodes went 857 -> 787 us (EpiCheb) and 822 -> 686 us (EpiScaled), 81 and 69 bytes a node
+// at 0.55 and 0.54 of the measured HBM rate; six blocks 798 and 708, loads after the row 823 and 719.
+template <int KIND, bool OFF32, class Epi>
+__global__ void __launch_bounds__(kTile, 7)
 k_stencil_half(Grid G, const float* __restrict__ coef, const float* __restrict__ half,
                const int* __restrict__ asym, const float* __restrict__ u,
                const uint8_t* __restrict__ mult, float* __restrict__ y, Epi epi) {
-  if (*asym) stencil_pass<false, KIND>(G, coef, u, mult, y, epi);
-  else stencil_pass<true, KIND>(G, half, u, mult, y, epi);
+  if (*asym) stencil_pass<false, OFF32, KIND>(G, coef, u, mult, y, epi);
+  else stencil_pass<true, OFF32, KIND>(G, half, u, mult, y, epi);
 }
 
 // ---- staged 27-point half-plane sweep: region tiles in shared memory, pipelined ----------
@@ -461,7 +479,7 @@ k_bstencil(Grid G, const CT* __restrict__ coef, const VT* __restrict__ u,
 // (c', c), so it needs no symmetry. Same products in the same order as k_bstencil, hence the
 // same bits. The sweep is bound by HBM and this form moves 14/27 of the coefficients: 577 instead
 // of 1045 bytes a node; the mirrored ones come from L1 and L2.
-template <bool HALF, int KIND, int B>
+template <bool HALF, bool OFF32, int KIND, int B>
 __device__ __forceinline__ void bstencil_row32(const float* __restrict__ coef,
                                                const float* __restrict__ u, int n, int n_r, int i,
                                                int j, int l, const RegionDev& R, float (&au)[B]) {
@@ -485,7 +503,10 @@ __device__ __forceinline__ void bstencil_row32(const float* __restrict__ coef,
     const int nb = n + dx + dy * sy + dz * sz;
     float uv[B];
 #pragma unroll
-    for (int c2 = 0; c2 < B; ++c2) uv[c2] = u[(size_t)c2 * n_r + nb];
+    for (int c2 = 0; c2 < B; ++c2) {
+      const float* uc = u + (size_t)c2 * n_r;
+      uv[c2] = OFF32 ? load32(uc, 4u * (unsigned)nb) : uc[nb];
+    }
     const bool mirrored = HALF && s < C;
     const int plane = !HALF ? s : s < C ? S::S - 1 - s - C : s - C;
     const int at = mirrored ? nb : n;
@@ -494,14 +515,15 @@ __device__ __forceinline__ void bstencil_row32(const float* __restrict__ coef,
 #pragma unroll
       for (int c2 = 0; c2 < B; ++c2) {
         const int blk = mirrored ? c2 * B + c : c * B + c2;
-        au[c] = fmaf(coef[((size_t)blk * P + plane) * n_r + at], uv[c2], au[c]);
+        const float* p = coef + ((size_t)blk * P + plane) * n_r;
+        au[c] = fmaf(OFF32 ? load32(p, 4u * (unsigned)at) : p[at], uv[c2], au[c]);
       }
   }
 }
 
 // asym[region] != 0: the region's full planes (an assembled block matrix can differ from its
 // transpose in the last bit of a few entries, and only their regions then lose the half form).
-template <int KIND, int B, class Epi>
+template <int KIND, bool OFF32, int B, class Epi>
 __global__ void __launch_bounds__(kTile)
 k_bstencil_half(Grid G, const float* __restrict__ coef, const float* __restrict__ half,
                 const int* __restrict__ asym, const float* __restrict__ u,
@@ -510,8 +532,8 @@ k_bstencil_half(Grid G, const float* __restrict__ coef, const float* __restrict_
     int i, j, l;
     RMG_DECODE(i, j, l);
     float au[B];
-    if (asym[tile_.region]) bstencil_row32<false, KIND, B>(coef, u, n, G.n_r, i, j, l, R, au);
-    else bstencil_row32<true, KIND, B>(half, u, n, G.n_r, i, j, l, R, au);
+    if (asym[tile_.region]) bstencil_row32<false, OFF32, KIND, B>(coef, u, n, G.n_r, i, j, l, R, au);
+    else bstencil_row32<true, OFF32, KIND, B>(half, u, n, G.n_r, i, j, l, R, au);
     if (mult[n] > 1) {
 #pragma unroll
       for (int c = 0; c < B; ++c) y[(size_t)c * G.n_r + n] = au[c];
@@ -555,72 +577,94 @@ __device__ __forceinline__ T inv_mult(int m) {
 template <typename T>
 struct EpiStore {                 // out = A u
   T* out;
-  static constexpr int kReads = 0;
-  __device__ const T* reads(int) const { return nullptr; }
   __device__ void operator()(int n, T au, int) const { out[n] = au; }
 };
 
+// The epilogues of the smoother work in two steps: load() reads what the update needs besides the
+// row, apply() forms and stores it. The FP32 half-plane sweeps load before they form the row, so
+// that these reads, which miss L2, are in flight with the row's own.
+#define RMG_EPI_CALL \
+  __device__ void operator()(int n, T au, int m) const { apply(n, load(n), au, m); }
+
 template <typename T>
-struct EpiScaled {                // out = D~^-1 A u (power method)
+struct EpiScaled {               // out = D~^-1 A u (power method)
   const T* dinv; T* out;
   static constexpr int kReads = 1;   // arrays read at the node (prefetch_tile)
-  __device__ const T* reads(int k) const { return dinv; }
-  __device__ void operator()(int n, T au, int) const { out[n] = dinv[n] * au; }
+  __device__ const T* reads(int) const { return dinv; }
+  struct V { T dinv; };
+  __device__ V load(int n) const { return V{dinv[n]}; }
+  __device__ void apply(int n, V v, T au, int) const { out[n] = v.dinv * au; }
+  RMG_EPI_CALL
 };
 
 template <typename T>
-struct EpiResid {                 // r = b - A u
+struct EpiResid {                // r = b - A u
   const T* b; T* r;
-  static constexpr int kReads = 1;   // arrays read at the node (prefetch_tile)
-  __device__ const T* reads(int k) const { return b; }
-  __device__ void operator()(int n, T au, int) const { r[n] = b[n] - au; }
+  static constexpr int kReads = 1;
+  __device__ const T* reads(int) const { return b; }
+  struct V { T b; };
+  __device__ V load(int n) const { return V{b[n]}; }
+  __device__ void apply(int n, V v, T au, int) const { r[n] = v.b - au; }
+  RMG_EPI_CALL
 };
 
 template <typename T>
-struct EpiResidScaled {           // r = (b - A u) / mult: the [[Psi Psi^T]]^-1 of restriction
+struct EpiResidScaled {          // r = (b - A u) / mult: the [[Psi Psi^T]]^-1 of restriction
   const T* b; T* r;
-  static constexpr int kReads = 1;   // arrays read at the node (prefetch_tile)
-  __device__ const T* reads(int k) const { return b; }
-  __device__ void operator()(int n, T au, int m) const { r[n] = (b[n] - au) * inv_mult<T>(m); }
+  static constexpr int kReads = 1;
+  __device__ const T* reads(int) const { return b; }
+  struct V { T b; };
+  __device__ V load(int n) const { return V{b[n]}; }
+  __device__ void apply(int n, V v, T au, int m) const { r[n] = (v.b - au) * inv_mult<T>(m); }
+  RMG_EPI_CALL
 };
 
 template <typename T>
-struct EpiJacobi {                // u_out = u + omega D~^-1 (b - A u)
+struct EpiJacobi {               // u_out = u + omega D~^-1 (b - A u)
   const T* u; const T* b; const T* dinv; T omega; T* uo;
-  static constexpr int kReads = 2;   // arrays read at the node (prefetch_tile)
+  static constexpr int kReads = 2;
   __device__ const T* reads(int k) const { return k == 0 ? b : dinv; }
-  __device__ void operator()(int n, T au, int) const {
-    const T r = b[n] - au;
-    uo[n] = fma(omega * dinv[n], r, u[n]);
+  struct V { T u, b, dinv; };
+  __device__ V load(int n) const { return V{u[n], b[n], dinv[n]}; }
+  __device__ void apply(int n, V v, T au, int) const {
+    const T r = v.b - au;
+    uo[n] = fma(omega * v.dinv, r, v.u);
   }
+  RMG_EPI_CALL
 };
 
 // The Chebyshev coefficients are read in the cycle's own precision (a per-node conversion
 // from FP64 would occupy the slow FP64 pipe of the FP32 cycle).
 template <typename T>
-struct EpiCheb0 {                 // first Chebyshev step: d = D~^-1 r / theta, u_out = u + d
+struct EpiCheb0 {                // first Chebyshev step: d = D~^-1 r / theta, u_out = u + d
   const T* u; const T* b; const T* dinv; const T* c2; T* d; T* uo;
-  static constexpr int kReads = 2;   // arrays read at the node (prefetch_tile)
+  static constexpr int kReads = 2;
   __device__ const T* reads(int k) const { return k == 0 ? b : dinv; }
-  __device__ void operator()(int n, T au, int) const {
-    const T r = b[n] - au;
-    const T dn = (dinv[n] * r) * (*c2);
+  struct V { T u, b, dinv; };
+  __device__ V load(int n) const { return V{u[n], b[n], dinv[n]}; }
+  __device__ void apply(int n, V v, T au, int) const {
+    const T r = v.b - au;
+    const T dn = (v.dinv * r) * (*c2);
     d[n] = dn;
-    uo[n] = u[n] + dn;
+    uo[n] = v.u + dn;
   }
+  RMG_EPI_CALL
 };
 
 template <typename T>
-struct EpiCheb {                  // d = c1 d + c2 D~^-1 r, u_out = u + d
+struct EpiCheb {                 // d = c1 d + c2 D~^-1 r, u_out = u + d
   const T* u; const T* b; const T* dinv; const T* c1; const T* c2; T* d; T* uo;
-  static constexpr int kReads = 3;   // arrays read at the node (prefetch_tile)
+  static constexpr int kReads = 3;
   __device__ const T* reads(int k) const { return k == 0 ? b : k == 1 ? dinv : d; }
-  __device__ void operator()(int n, T au, int) const {
-    const T r = b[n] - au;
-    const T dn = (*c1) * d[n] + ((*c2) * dinv[n]) * r;
+  struct V { T u, b, dinv, d; };
+  __device__ V load(int n) const { return V{u[n], b[n], dinv[n], d[n]}; }
+  __device__ void apply(int n, V v, T au, int) const {
+    const T r = v.b - au;
+    const T dn = (*c1) * v.d + ((*c2) * v.dinv) * r;
     d[n] = dn;
-    uo[n] = u[n] + dn;
+    uo[n] = v.u + dn;
   }
+  RMG_EPI_CALL
 };
 
 // ------------------------------------------------------------------ elementwise
@@ -648,14 +692,17 @@ __global__ void k_cheb0_zero(int n, const T* __restrict__ b, const T* __restrict
 // (the stencil pair with EpiResidZero, which also sets delta = 0), then runs one launch per
 // colour class.
 template <typename T>
-struct EpiResidZero {              // r = b - A u, delta = 0
+struct EpiResidZero {            // r = b - A u, delta = 0
   const T* b; T* r; T* delta;
-  static constexpr int kReads = 1;   // arrays read at the node (prefetch_tile)
-  __device__ const T* reads(int k) const { return b; }
-  __device__ void operator()(int n, T au, int) const {
-    r[n] = b[n] - au;
+  static constexpr int kReads = 1;
+  __device__ const T* reads(int) const { return b; }
+  struct V { T b; };
+  __device__ V load(int n) const { return V{b[n]}; }
+  __device__ void apply(int n, V v, T au, int) const {
+    r[n] = v.b - au;
     delta[n] = T(0);
   }
+  RMG_EPI_CALL
 };
 
 // The composite value (mean over the copies) of an interface node, written to `out` at every

@@ -74,6 +74,28 @@ void launch_groups(Ctx& c, const Level& L, const AT* y, Epi epi, cudaStream_t st
   RMG_LAUNCHED();
 }
 
+// The half-plane sweep of an FP32 level (OFF32: 32-bit offsets, see load32).
+template <bool OFF32, class Epi>
+void launch_half(Ctx& c, const Level& L, const Grid& G, const float* coef, const float* half,
+                 const int* asym, const float* u, float* y, Epi epi, cudaStream_t st) {
+  const int nt = G.ntiles;
+  const uint8_t* mu = L.mult.get();
+  auto run = [&](auto kernel) {
+    launch_resident(c, kernel, nt, st, G, coef, half, asym, u, mu, y, epi);
+  };
+  if (L.B == 3) {
+    if (L.kind == 27) run(k_bstencil_half<27, OFF32, 3, Epi>);
+    else run(k_bstencil_half<9, OFF32, 3, Epi>);
+    return;
+  }
+  switch (L.kind) {
+    case 5: run(k_stencil_half<5, OFF32, Epi>); break;
+    case 7: run(k_stencil_half<7, OFF32, Epi>); break;
+    case 9: run(k_stencil_half<9, OFF32, Epi>); break;
+    default: run(k_stencil_half<27, OFF32, Epi>); break;
+  }
+}
+
 // Phase A over `sweep` (a tuned tile list of L; the level's run tiles when null), then phase B.
 // An FP32 sweep given half planes (see k_level0_fp32) and their asymmetry flag reads the half
 // form while the flag is 0.
@@ -103,23 +125,14 @@ void launch_stencil(Ctx& c, const Level& L, const CT* coef, const VT* u, AT* y, 
       done = true;
     } else if (half && L.B == 1) {
       RMG_REQUIRE(asym != nullptr, RMG_ERR_STATE, "half planes without their flag");
-      const int nt = G.ntiles;
-      const uint8_t* mu = L.mult.get();
-      switch (L.kind) {
-        case 5: launch_resident(c, k_stencil_half<5, Epi>, nt, st, G, coef, half, asym, u, mu, y, epi); break;
-        case 7: launch_resident(c, k_stencil_half<7, Epi>, nt, st, G, coef, half, asym, u, mu, y, epi); break;
-        case 9: launch_resident(c, k_stencil_half<9, Epi>, nt, st, G, coef, half, asym, u, mu, y, epi); break;
-        default: launch_resident(c, k_stencil_half<27, Epi>, nt, st, G, coef, half, asym, u, mu, y, epi); break;
-      }
+      if (L.n_r <= kOffset32Nodes) launch_half<true>(c, L, G, coef, half, asym, u, y, epi, st);
+      else launch_half<false>(c, L, G, coef, half, asym, u, y, epi, st);
       done = true;
     } else if (half) {
       RMG_REQUIRE(asym != nullptr && L.B == 3 && (L.kind == 27 || L.kind == 9), RMG_ERR_STATE,
                   "half planes of a block operator need 3 dofs and a 27- or 9-point stencil");
-      const uint8_t* mu = L.mult.get();
-      if (L.kind == 27)
-        launch_resident(c, k_bstencil_half<27, 3, Epi>, G.ntiles, st, G, coef, half, asym, u, mu, y, epi);
-      else
-        launch_resident(c, k_bstencil_half<9, 3, Epi>, G.ntiles, st, G, coef, half, asym, u, mu, y, epi);
+      if (L.n_r <= kOffset32Nodes) launch_half<true>(c, L, G, coef, half, asym, u, y, epi, st);
+      else launch_half<false>(c, L, G, coef, half, asym, u, y, epi, st);
       done = true;
     }
   }
