@@ -215,6 +215,7 @@ enum CgDot : int { CG_ALPHA, CG_BETA, CG_RZ };
 __global__ void __launch_bounds__(256)
 k_cg_dot(int n, int n_nodes, const double* __restrict__ x, const double* __restrict__ y,
          const uint8_t* __restrict__ mult, Arrive A, Scalars* sc, int what) {
+  follow();
   double s = 0.0;
   for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x)
     s = fma(x[k] * inv_mult<double>(mult[k < n_nodes ? k : k % n_nodes]), y[k], s);
@@ -233,6 +234,7 @@ k_cg_dot(int n, int n_nodes, const double* __restrict__ x, const double* __restr
 __global__ void __launch_bounds__(256)
 k_cg_flex64(int n, int n_nodes, const double* __restrict__ r, const double* __restrict__ z,
             double* __restrict__ zold, const uint8_t* __restrict__ mult, Arrive A, Scalars* sc) {
+  follow();
   double s0 = 0.0, s1 = 0.0;
   for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
     const double rk = r[k] * inv_mult<double>(mult[k < n_nodes ? k : k % n_nodes]);
@@ -258,6 +260,7 @@ __global__ void __launch_bounds__(256)
 k_cg_update(int n, int n_nodes, const double* __restrict__ p, const double* __restrict__ q,
             const uint8_t* __restrict__ mult, const Scalars* __restrict__ sc,
             double* __restrict__ x, double* __restrict__ r, Arrive A, double* host_rr) {
+  follow();
   const double a = sc->alpha;
   double s = 0.0;
   for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
@@ -288,6 +291,7 @@ k_cg_update_mixed(int n, int n_nodes, const double* __restrict__ p, const double
                   const uint8_t* __restrict__ mult, const Scalars* __restrict__ sc,
                   double rscale, double* __restrict__ x, double* __restrict__ r,
                   float* __restrict__ r32, Arrive A, double* host_rr) {
+  follow();
   const double a = sc->alpha;
   double s = 0.0;
   for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
@@ -307,6 +311,7 @@ k_cg_update_mixed(int n, int n_nodes, const double* __restrict__ p, const double
 // r32 = FP32(r * rscale): the cycle's right-hand side at a (re)start of the iteration.
 __global__ void k_to_f32_scaled(int n, const double* __restrict__ r, double rscale,
                                 float* __restrict__ r32) {
+  follow();
   for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x)
     r32[k] = (float)(r[k] * rscale);
 }
@@ -319,6 +324,7 @@ __global__ void __launch_bounds__(256)
 k_flex_dots(int n, int n_nodes, const double* __restrict__ r, const float* __restrict__ z,
             float* __restrict__ zold, const uint8_t* __restrict__ mult, double zscale, Arrive A,
             Scalars* sc) {
+  follow();
   double s0 = 0.0, s1 = 0.0;
   const int n4 = n >> 2;
   const int tid = blockIdx.x * blockDim.x + threadIdx.x, nth = gridDim.x * blockDim.x;
@@ -359,6 +365,7 @@ __global__ void __launch_bounds__(256)
 k_start_dir(int n, int n_nodes, const double* __restrict__ r, const float* __restrict__ z,
             const uint8_t* __restrict__ mult, double zscale, double* __restrict__ p,
             float* __restrict__ zold, Arrive A, Scalars* sc) {
+  follow();
   double s = 0.0;
   for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
     const float zk = z[k];
@@ -383,6 +390,7 @@ __global__ void k_axpy_neg(int n, const double* __restrict__ z, double* __restri
 template <typename ZT>
 __global__ void k_p_update(int n, const ZT* __restrict__ z, double zscale,
                            const Scalars* __restrict__ sc, double* __restrict__ p) {
+  follow();
   const double b = sc->beta;
   for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x)
     p[k] = fma(double(z[k]), zscale, b * p[k]);
@@ -446,7 +454,7 @@ struct Exec {
     const int gb = persistent_grid(c(), G.ntiles);
     VT* u = cur[l];
 #define RMG_GS(K)                                                                             \
-  k_gs_colour<K, CT, VT><<<gb, kTile, 0, st>>>(G, coef(l), V(l).r.get(), dinv(l),               \
+  launch_next(k_gs_colour<K, CT, VT>, dim3(gb), kTile, 0, st, G, coef(l), V(l).r.get(), dinv(l),               \
                                                V(l).d.get(), u, colour, omega)
     switch (L.kind) {
       case 5: RMG_GS(5); break;
@@ -467,7 +475,7 @@ struct Exec {
       const int ncol = (L.kind == 5 || L.kind == 7) ? 2 : (L.dim == 3 ? 8 : 4);
       for (int s = 0; s < nu; ++s) {
         if (s == 0 && from_zero) {
-          k_gs_zero<VT><<<elementwise_grid(n), 256, 0, st>>>(n, V(l).b.get(), V(l).r.get(),
+          launch_next(k_gs_zero<VT>, dim3(elementwise_grid(n)), 256, 0, st, n, V(l).b.get(), V(l).r.get(),
                                                              V(l).d.get(), cur[l]);
           RMG_LAUNCHED();
           ++launches;
@@ -482,7 +490,7 @@ struct Exec {
     if (h.o.smoother == RMG_SMOOTHER_JACOBI) {
       for (int s = 0; s < nu; ++s) {
         if (s == 0 && from_zero) {
-          k_jacobi_zero<VT><<<elementwise_grid(n), 256, 0, st>>>(n, V(l).b.get(), dinv(l), omega,
+          launch_next(k_jacobi_zero<VT>, dim3(elementwise_grid(n)), 256, 0, st, n, V(l).b.get(), dinv(l), omega,
                                                                  oth[l]);
           RMG_LAUNCHED();
           ++launches;
@@ -495,7 +503,7 @@ struct Exec {
     } else {
       for (int a = 0; a < nu; ++a) {
         if (a == 0 && from_zero) {
-          k_cheb0_zero<VT><<<elementwise_grid(n), 256, 0, st>>>(n, V(l).b.get(), dinv(l),
+          launch_next(k_cheb0_zero<VT>, dim3(elementwise_grid(n)), 256, 0, st, n, V(l).b.get(), dinv(l),
                                                                 c2(l, 0), V(l).d.get(), oth[l]);
           RMG_LAUNCHED();
           ++launches;
@@ -526,7 +534,7 @@ struct Exec {
         VT* wb = V(l + 1).b.get() + (size_t)b * C.n_r;
         VT* yb = V(l + 1).y.get() + (size_t)b * C.n_r;
         const VT* rb = V(l).r.get() + (size_t)b * F.n_r;
-        k_restrict<3, VT><<<gb, kTile, 0, st>>>(Gc, F.regions.get(), rb, C.mask.get(),
+        launch_next(k_restrict<3, VT>, dim3(gb), kTile, 0, st, Gc, F.regions.get(), rb, C.mask.get(),
                                                 C.mult.get(), wb, yb);
         RMG_LAUNCHED();
         ++launches;
@@ -541,18 +549,18 @@ struct Exec {
     const int gb = persistent_grid(c(), Gc.ntiles);
     if (h.stored[l]) {
       if (F.dim == 3)
-        k_restrict_w<3, VT><<<gb, kTile, 0, st>>>(Gc, F.regions.get(), F.n_r, pw(l), V(l).r.get(),
+        launch_next(k_restrict_w<3, VT>, dim3(gb), kTile, 0, st, Gc, F.regions.get(), F.n_r, pw(l), V(l).r.get(),
                                                   C.mask.get(), C.mult.get(), V(l + 1).b.get(),
                                                   V(l + 1).y.get());
       else
-        k_restrict_w<2, VT><<<gb, kTile, 0, st>>>(Gc, F.regions.get(), F.n_r, pw(l), V(l).r.get(),
+        launch_next(k_restrict_w<2, VT>, dim3(gb), kTile, 0, st, Gc, F.regions.get(), F.n_r, pw(l), V(l).r.get(),
                                                   C.mask.get(), C.mult.get(), V(l + 1).b.get(),
                                                   V(l + 1).y.get());
     } else if (F.dim == 3)
-      k_restrict<3, VT><<<gb, kTile, 0, st>>>(Gc, F.regions.get(), V(l).r.get(), C.mask.get(),
+      launch_next(k_restrict<3, VT>, dim3(gb), kTile, 0, st, Gc, F.regions.get(), V(l).r.get(), C.mask.get(),
                                               C.mult.get(), V(l + 1).b.get(), V(l + 1).y.get());
     else
-      k_restrict<2, VT><<<gb, kTile, 0, st>>>(Gc, F.regions.get(), V(l).r.get(), C.mask.get(),
+      launch_next(k_restrict<2, VT>, dim3(gb), kTile, 0, st, Gc, F.regions.get(), V(l).r.get(), C.mask.get(),
                                               C.mult.get(), V(l + 1).b.get(), V(l + 1).y.get());
     RMG_LAUNCHED();
     ++launches;
@@ -569,7 +577,7 @@ struct Exec {
     const int gb = persistent_grid(c(), Gf.ntiles);
     if (F.B > 1) {
       for (int b = 0; b < F.B; ++b) {
-        k_prolong<3, VT><<<gb, kTile, 0, st>>>(Gf, C.regions.get(), F.mask.get(),
+        launch_next(k_prolong<3, VT>, dim3(gb), kTile, 0, st, Gf, C.regions.get(), F.mask.get(),
                                                cur[l + 1] + (size_t)b * C.n_r,
                                                cur[l] + (size_t)b * F.n_r);
         RMG_LAUNCHED();
@@ -579,15 +587,15 @@ struct Exec {
     }
     if (h.stored[l]) {
       if (F.dim == 3)
-        k_prolong_w<3, VT><<<gb, kTile, 0, st>>>(Gf, C.regions.get(), pw(l), F.mask.get(),
+        launch_next(k_prolong_w<3, VT>, dim3(gb), kTile, 0, st, Gf, C.regions.get(), pw(l), F.mask.get(),
                                                  cur[l + 1], cur[l]);
       else
-        k_prolong_w<2, VT><<<gb, kTile, 0, st>>>(Gf, C.regions.get(), pw(l), F.mask.get(),
+        launch_next(k_prolong_w<2, VT>, dim3(gb), kTile, 0, st, Gf, C.regions.get(), pw(l), F.mask.get(),
                                                  cur[l + 1], cur[l]);
     } else if (F.dim == 3)
-      k_prolong<3, VT><<<gb, kTile, 0, st>>>(Gf, C.regions.get(), F.mask.get(), cur[l + 1], cur[l]);
+      launch_next(k_prolong<3, VT>, dim3(gb), kTile, 0, st, Gf, C.regions.get(), F.mask.get(), cur[l + 1], cur[l]);
     else
-      k_prolong<2, VT><<<gb, kTile, 0, st>>>(Gf, C.regions.get(), F.mask.get(), cur[l + 1], cur[l]);
+      launch_next(k_prolong<2, VT>, dim3(gb), kTile, 0, st, Gf, C.regions.get(), F.mask.get(), cur[l + 1], cur[l]);
     RMG_LAUNCHED();
     ++launches;
   }
@@ -696,7 +704,7 @@ struct Exec {
     if (!L.ngroups) return;
     launch_groups(c(), L, (const VT*)cur[0], EpiMean<VT>{V(0).y.get()}, st);
     ++launches;
-    k_copy_slots<VT><<<persistent_grid(c(), (L.nslots + 255) / 256), 256, 0, st>>>(
+    launch_next(k_copy_slots<VT>, dim3(persistent_grid(c(), (L.nslots + 255) / 256)), 256, 0, st, 
         L.nslots, L.gslot.get(), V(0).y.get(), cur[0]);
     RMG_LAUNCHED();
     ++launches;
@@ -1934,17 +1942,17 @@ void pcg_solve(Hier& h, const double* b, double* xout, double rtol, int maxit, d
   while (!converged && it < maxit) {
     // (re)start: z = M^-1 r, p = z
     if (mixed) {
-      k_to_f32_scaled<<<eg, 256, 0, st>>>(n, rvec, rscale, r32);
+      launch_next(k_to_f32_scaled, dim3(eg), 256, 0, st, n, rvec, rscale, r32);
       RMG_LAUNCHED();
     }
     vcycle(h);
     ++ncyc;
     if (mixed) {
-      k_start_dir<<<dg, 256, 0, st>>>(n, L0.n_r, rvec, z32, L0.mult.get(), zscale, h.p.get(),
+      launch_next(k_start_dir, dim3(dg), 256, 0, st, n, L0.n_r, rvec, z32, L0.mult.get(), zscale, h.p.get(),
                                       h.zold32.get(), arrive, sc);
       RMG_LAUNCHED();
     } else {
-      k_cg_dot<<<dg, 256, 0, st>>>(n, L0.n_r, rvec, zvec, L0.mult.get(), arrive, sc, CG_RZ);
+      launch_next(k_cg_dot, dim3(dg), 256, 0, st, n, L0.n_r, rvec, zvec, L0.mult.get(), arrive, sc, CG_RZ);
       RMG_LAUNCHED();
       k_copy<double><<<eg, 256, 0, st>>>(n, zvec, h.p.get());
       RMG_LAUNCHED();
@@ -1957,14 +1965,14 @@ void pcg_solve(Hier& h, const double* b, double* xout, double rtol, int maxit, d
       ++it;
       launch_stencil(c, L0, L0.coef.get(), h.p.get(), h.v64[0].y.get(),
                      EpiStore<double>{h.q.get()}, st, nullptr);
-      k_cg_dot<<<dg, 256, 0, st>>>(n, L0.n_r, h.p.get(), h.q.get(), L0.mult.get(), arrive, sc,
+      launch_next(k_cg_dot, dim3(dg), 256, 0, st, n, L0.n_r, h.p.get(), h.q.get(), L0.mult.get(), arrive, sc,
                                    CG_ALPHA);
       RMG_LAUNCHED();
       if (mixed)
-        k_cg_update_mixed<<<dg, 256, 0, st>>>(n, L0.n_r, h.p.get(), h.q.get(), L0.mult.get(), sc,
+        launch_next(k_cg_update_mixed, dim3(dg), 256, 0, st, n, L0.n_r, h.p.get(), h.q.get(), L0.mult.get(), sc,
                                               rscale, h.x.get(), rvec, r32, arrive, host_rr);
       else
-        k_cg_update<<<dg, 256, 0, st>>>(n, L0.n_r, h.p.get(), h.q.get(), L0.mult.get(), sc,
+        launch_next(k_cg_update, dim3(dg), 256, 0, st, n, L0.n_r, h.p.get(), h.q.get(), L0.mult.get(), sc,
                                         h.x.get(), rvec, arrive, host_rr);
       RMG_LAUNCHED();
       RMG_CUDA(cudaStreamSynchronize(st));
@@ -1991,19 +1999,19 @@ void pcg_solve(Hier& h, const double* b, double* xout, double rtol, int maxit, d
       vcycle(h);
       ++ncyc;
       if (mixed) {
-        k_flex_dots<<<dg, 256, 0, st>>>(n, L0.n_r, rvec, z32, h.zold32.get(), L0.mult.get(),
+        launch_next(k_flex_dots, dim3(dg), 256, 0, st, n, L0.n_r, rvec, z32, h.zold32.get(), L0.mult.get(),
                                         zscale, arrive, sc);
         RMG_LAUNCHED();
-        k_p_update<float><<<eg, 256, 0, st>>>(n, z32, zscale, sc, h.p.get());
+        launch_next(k_p_update<float>, dim3(eg), 256, 0, st, n, z32, zscale, sc, h.p.get());
         RMG_LAUNCHED();
       } else {
         if (flex64)
-          k_cg_flex64<<<dg, 256, 0, st>>>(n, L0.n_r, rvec, zvec, h.zold.get(), L0.mult.get(),
+          launch_next(k_cg_flex64, dim3(dg), 256, 0, st, n, L0.n_r, rvec, zvec, h.zold.get(), L0.mult.get(),
                                           arrive, sc);
         else
-          k_cg_dot<<<dg, 256, 0, st>>>(n, L0.n_r, rvec, zvec, L0.mult.get(), arrive, sc, CG_BETA);
+          launch_next(k_cg_dot, dim3(dg), 256, 0, st, n, L0.n_r, rvec, zvec, L0.mult.get(), arrive, sc, CG_BETA);
         RMG_LAUNCHED();
-        k_p_update<double><<<eg, 256, 0, st>>>(n, zvec, 1.0, sc, h.p.get());
+        launch_next(k_p_update<double>, dim3(eg), 256, 0, st, n, zvec, 1.0, sc, h.p.get());
         RMG_LAUNCHED();
       }
     }

@@ -188,6 +188,7 @@ struct Level {
   DBuf<int> gslot;               // regional slots of every group, ascending
   DBuf<int> rid;                 // region of every regional node (built for the split)
   DBuf<int> sgrp;                // group of every group slot (nslots)
+  DBuf<int4> slots;              // slot records of phase B (k_slot_records)
   DBuf<int2> split_left;         // rows the split's direct pass left, and their number, per
   DBuf<int> split_nleft;         // row component (B * n_r, B)
   DBuf<int4> affine;             // per region {g0, gy, gz, ok}: gid = g0 + i + gy j + gz l

@@ -17,6 +17,13 @@
 
 namespace rmg {
 
+// Start of a kernel that is launched with launch_next(): the next kernel may be set up now (its
+// blocks wait in turn), and nothing is touched before the previous one has finished.
+__device__ __forceinline__ void follow() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
 // a / d for 0 <= a < 2^22 from the float reciprocal rd of d: the truncated product is within
 // one of the quotient (relative error below 2^-22 on a value below 2^22), and one correction
 // step makes it exact.
@@ -116,6 +123,7 @@ template <int KIND, typename CT, typename VT, typename AT, class Epi>
 __global__ void __launch_bounds__(kTile)
 k_stencil(Grid G, const CT* __restrict__ coef, const VT* __restrict__ u,
           const uint8_t* __restrict__ mult, AT* __restrict__ y, Epi epi) {
+  follow();
   RMG_FOR_NODES(G)
     int i, j, l;
     RMG_DECODE(i, j, l);
@@ -241,6 +249,7 @@ __global__ void __launch_bounds__(kTile, 7)
 k_stencil_half(Grid G, const float* __restrict__ coef, const float* __restrict__ half,
                const int* __restrict__ asym, const float* __restrict__ u,
                const uint8_t* __restrict__ mult, float* __restrict__ y, Epi epi) {
+  follow();
   if (*asym) stencil_pass<false, OFF32, KIND>(G, coef, u, mult, y, epi);
   else stencil_pass<true, OFF32, KIND>(G, half, u, mult, y, epi);
 }
@@ -317,6 +326,7 @@ __global__ void __launch_bounds__(kStX * kStY)
 k_stencil_half27_staged(Grid G, const float* __restrict__ coef, const float* __restrict__ half,
                         const int* __restrict__ asym, const float* __restrict__ u,
                         const uint8_t* __restrict__ mult, float* __restrict__ y, Epi epi) {
+  follow();
   extern __shared__ __align__(16) float st_smem[];
   float* CS = st_smem;                                // [kStCoef][14][kStPlane]
   float* US = st_smem + kStCoef * 14 * kStPlane;      // [kStU][kStPlane]
@@ -410,19 +420,37 @@ k_stencil_half27_staged(Grid G, const float* __restrict__ coef, const float* __r
   }
 }
 
+// Sum of y over the copies of slot record t = {node, start in gslot, copies, other copy of two},
+// in ascending slot order. Most groups are pairs on a face: their sum needs no further index.
+template <typename AT>
+__device__ __forceinline__ AT group_sum(const int4& t, const int* __restrict__ gslot,
+                                        const AT* __restrict__ y) {
+  if (t.z == 2) return y[min(t.x, t.w)] + y[max(t.x, t.w)];
+  AT s = AT(0);
+  for (int k = 0; k < t.z; k += 4) {
+    AT v[4];
+#pragma unroll
+    for (int m = 0; m < 4; ++m) v[m] = k + m < t.z ? y[gslot[t.y + k + m]] : AT(0);
+#pragma unroll
+    for (int m = 0; m < 4; ++m)
+      if (k + m < t.z) s += v[m];
+  }
+  return s;
+}
+
 // Phase B: interface groups. y holds the partial row results of every copy. One thread per
 // copy: it sums the partial results of its group in ascending slot order (every copy of a group
-// forms the identical sum) and applies the epilogue to its own copy.
+// forms the identical sum) and applies the epilogue to its own copy. Bound by the latency of its
+// chain of loads, which the slot records cut from four (slot, group, copies, values) to two.
 template <typename AT, class Epi>
 __global__ void __launch_bounds__(256)
-k_groups(int nslots, const int* __restrict__ sgrp, const int* __restrict__ gptr,
-         const int* __restrict__ gslot, const AT* __restrict__ y, Epi epi) {
+k_groups(int nslots, const int4* __restrict__ slots, const int* __restrict__ gslot,
+         const AT* __restrict__ y, Epi epi) {
+  follow();
   for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < nslots; q += gridDim.x * blockDim.x) {
-    const int g = sgrp[q];
-    const int a = gptr[g], e = gptr[g + 1];
-    AT s = AT(0);
-    for (int k = a; k < e; ++k) s += y[gslot[k]];
-    epi(gslot[q], s, e - a);
+    const int4 t = slots[q];
+    const auto v = epi.load(t.x);
+    epi.apply(t.x, v, group_sum<AT>(t, gslot, y), t.z);
   }
 }
 
@@ -433,6 +461,7 @@ template <int KIND, int B, typename CT, typename VT, typename AT, class Epi>
 __global__ void __launch_bounds__(kTile)
 k_bstencil(Grid G, const CT* __restrict__ coef, const VT* __restrict__ u,
            const uint8_t* __restrict__ mult, AT* __restrict__ y, Epi epi) {
+  follow();
   using S = Sten<KIND>;
   RMG_FOR_NODES(G)
     int i, j, l;
@@ -528,6 +557,7 @@ __global__ void __launch_bounds__(kTile)
 k_bstencil_half(Grid G, const float* __restrict__ coef, const float* __restrict__ half,
                 const int* __restrict__ asym, const float* __restrict__ u,
                 const uint8_t* __restrict__ mult, float* __restrict__ y, Epi epi) {
+  follow();
   RMG_FOR_NODES(G)
     int i, j, l;
     RMG_DECODE(i, j, l);
@@ -546,14 +576,14 @@ k_bstencil_half(Grid G, const float* __restrict__ coef, const float* __restrict_
 
 template <typename AT, class Epi>
 __global__ void __launch_bounds__(256)
-k_groups_b(int ngroups, int B, int n_r, const int* __restrict__ gptr,
+k_groups_b(int nslots, int B, int n_r, const int4* __restrict__ slots,
            const int* __restrict__ gslot, const AT* __restrict__ y, Epi epi) {
-  for (int g = blockIdx.x * blockDim.x + threadIdx.x; g < ngroups; g += gridDim.x * blockDim.x) {
-    const int a = gptr[g], e = gptr[g + 1];
+  follow();
+  for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < nslots; q += gridDim.x * blockDim.x) {
+    const int4 t = slots[q];
     for (int c = 0; c < B; ++c) {
-      AT s = AT(0);
-      for (int k = a; k < e; ++k) s += y[(size_t)c * n_r + gslot[k]];
-      for (int k = a; k < e; ++k) epi(c * n_r + gslot[k], s, e - a);
+      const auto v = epi.load(c * n_r + t.x);
+      epi.apply(c * n_r + t.x, v, group_sum<AT>(t, gslot, y + (size_t)c * n_r), t.z);
     }
   }
 }
@@ -574,17 +604,20 @@ __device__ __forceinline__ T inv_mult(int m) {
   }
 }
 
+// The epilogues of the smoother work in two steps: load() reads what the update needs besides the
+// row, apply() forms and stores it. The FP32 half-plane sweeps load before they form the row, so
+// that these reads, which miss L2, are in flight with the row's own; so does phase B.
+#define RMG_EPI_CALL \
+  __device__ void operator()(int n, T au, int m) const { apply(n, load(n), au, m); }
+
 template <typename T>
 struct EpiStore {                 // out = A u
   T* out;
-  __device__ void operator()(int n, T au, int) const { out[n] = au; }
+  struct V {};
+  __device__ V load(int) const { return V{}; }
+  __device__ void apply(int n, V, T au, int) const { out[n] = au; }
+  RMG_EPI_CALL
 };
-
-// The epilogues of the smoother work in two steps: load() reads what the update needs besides the
-// row, apply() forms and stores it. The FP32 half-plane sweeps load before they form the row, so
-// that these reads, which miss L2, are in flight with the row's own.
-#define RMG_EPI_CALL \
-  __device__ void operator()(int n, T au, int m) const { apply(n, load(n), au, m); }
 
 template <typename T>
 struct EpiScaled {               // out = D~^-1 A u (power method)
@@ -671,6 +704,7 @@ struct EpiCheb {                 // d = c1 d + c2 D~^-1 r, u_out = u + d
 template <typename T>
 __global__ void k_jacobi_zero(int n, const T* __restrict__ b, const T* __restrict__ dinv,
                               T omega, T* __restrict__ uo) {
+  follow();
   for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x)
     uo[k] = (omega * dinv[k]) * b[k];
 }
@@ -679,6 +713,7 @@ template <typename T>
 __global__ void k_cheb0_zero(int n, const T* __restrict__ b, const T* __restrict__ dinv,
                              const T* __restrict__ c2, T* __restrict__ d,
                              T* __restrict__ uo) {
+  follow();
   const T c = *c2;
   for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
     const T dn = (dinv[k] * b[k]) * c;
@@ -710,13 +745,16 @@ struct EpiResidZero {            // r = b - A u, delta = 0
 template <typename T>
 struct EpiMean {
   T* out;
-  __device__ void operator()(int n, T s, int m) const { out[n] = s * inv_mult<T>(m); }
+  struct V {};
+  __device__ V load(int) const { return V{}; }
+  __device__ void apply(int n, V, T s, int m) const { out[n] = s * inv_mult<T>(m); }
 };
 
 // dst[gslot[q]] = src[gslot[q]] for every copy of every interface node.
 template <typename T>
 __global__ void k_copy_slots(int nslots, const int* __restrict__ gslot, const T* __restrict__ src,
                              T* __restrict__ dst) {
+  follow();
   for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < nslots; q += gridDim.x * blockDim.x)
     dst[gslot[q]] = src[gslot[q]];
 }
@@ -725,6 +763,7 @@ __global__ void k_copy_slots(int nslots, const int* __restrict__ gslot, const T*
 template <typename VT>
 __global__ void k_gs_zero(int n, const VT* __restrict__ b, VT* __restrict__ r,
                           VT* __restrict__ delta, VT* __restrict__ u) {
+  follow();
   for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
     r[k] = b[k];
     delta[k] = VT(0);
@@ -748,6 +787,7 @@ template <int KIND, typename CT, typename VT>
 __global__ void __launch_bounds__(kTile)
 k_gs_colour(Grid G, const CT* __restrict__ coef, const VT* __restrict__ r,
             const VT* __restrict__ dinv, VT* delta, VT* __restrict__ u, int colour, VT omega) {
+  follow();
   RMG_FOR_NODES(G)
     int i, j, l;
     RMG_DECODE(i, j, l);
@@ -830,6 +870,7 @@ __global__ void __launch_bounds__(kTile)
 k_restrict(Grid Gc, const RegionDev* __restrict__ fregions, const VT* __restrict__ rs,
            const uint8_t* __restrict__ cmask, const uint8_t* __restrict__ cmult,
            VT* __restrict__ w, VT* __restrict__ yc) {
+  follow();
   RMG_FOR_NODES(Gc)
     int I, J, L;
     decode(li, R, I, J, L);
@@ -860,6 +901,7 @@ template <int DIM, typename VT>
 __global__ void __launch_bounds__(kTile)
 k_prolong(Grid Gf, const RegionDev* __restrict__ cregions, const uint8_t* __restrict__ fmask,
           const VT* __restrict__ ubar, VT* __restrict__ u) {
+  follow();
   RMG_FOR_NODES(Gf)
     if (fmask[n]) continue;
     int i, j, l;
@@ -904,6 +946,7 @@ __global__ void __launch_bounds__(kTile)
 k_restrict_w(Grid Gc, const RegionDev* __restrict__ fregions, int fn_r, const float* __restrict__ wr,
              const VT* __restrict__ rs, const uint8_t* __restrict__ cmask,
              const uint8_t* __restrict__ cmult, VT* __restrict__ w, VT* __restrict__ yc) {
+  follow();
   RMG_FOR_NODES(Gc)
     int I, J, L;
     decode(li, R, I, J, L);
@@ -923,6 +966,7 @@ template <int DIM, typename VT>
 __global__ void __launch_bounds__(kTile)
 k_prolong_w(Grid Gf, const RegionDev* __restrict__ cregions, const float* __restrict__ wr,
             const uint8_t* __restrict__ fmask, const VT* __restrict__ ubar, VT* __restrict__ u) {
+  follow();
   RMG_FOR_NODES(Gf)
     if (fmask[n]) continue;
     int i, j, l;

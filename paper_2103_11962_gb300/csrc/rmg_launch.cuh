@@ -57,31 +57,58 @@ inline int resident_per_sm_smem(const void* kernel, int smem) {
   return b;
 }
 
-// kernel<<<one resident wave of blocks over `work` tiles, kTile>>>(args...) on st.
+// kernel<<<grid, block, smem, st>>>(args...) for a kernel that starts with follow(): where the work
+// before it on the stream is a kernel too, it is set up while that one finishes (programmatic
+// dependent launch), which takes about 1 us off each of the short kernels of a small problem.
+// launch_after with next = false is the plain launch (beside an event record).
 template <typename... P, typename... A>
-void launch_resident(const Ctx& c, void (*kernel)(P...), int work, cudaStream_t st,
+void launch_after(bool next, void (*kernel)(P...), dim3 grid, int block, int smem,
+                  cudaStream_t st, A&&... args) {
+  cudaLaunchAttribute attr;
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(block);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cfg.attrs = &attr;
+  cfg.numAttrs = next ? 1 : 0;
+  RMG_CUDA(cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...));
+}
+template <typename... P, typename... A>
+void launch_next(void (*kernel)(P...), dim3 grid, int block, int smem, cudaStream_t st,
+                 A&&... args) {
+  launch_after(true, kernel, grid, block, smem, st, std::forward<A>(args)...);
+}
+
+// launch_after with one resident wave of blocks over `work` tiles.
+template <typename... P, typename... A>
+void launch_resident(const Ctx& c, bool next, void (*kernel)(P...), int work, cudaStream_t st,
                      A&&... args) {
   const int g = persistent_grid(c, work, resident_per_sm((const void*)kernel));
-  kernel<<<g, kTile, 0, st>>>(std::forward<A>(args)...);
+  launch_after(next, kernel, dim3(g), kTile, 0, st, std::forward<A>(args)...);
 }
 
 // Phase B alone (scalar levels): one thread per copy of every interface group.
 template <typename AT, class Epi>
-void launch_groups(Ctx& c, const Level& L, const AT* y, Epi epi, cudaStream_t st) {
+void launch_groups(Ctx& c, const Level& L, const AT* y, Epi epi, cudaStream_t st,
+                   bool next = true) {
   if (!L.ngroups) return;
   const int gs = persistent_grid(c, (L.nslots + 255) / 256);
-  k_groups<AT><<<gs, 256, 0, st>>>(L.nslots, L.sgrp.get(), L.gptr.get(), L.gslot.get(), y, epi);
+  launch_after(next, k_groups<AT, Epi>, dim3(gs), 256, 0, st, L.nslots, L.slots.get(), L.gslot.get(), y,
+              epi);
   RMG_LAUNCHED();
 }
 
 // The half-plane sweep of an FP32 level (OFF32: 32-bit offsets, see load32).
 template <bool OFF32, class Epi>
 void launch_half(Ctx& c, const Level& L, const Grid& G, const float* coef, const float* half,
-                 const int* asym, const float* u, float* y, Epi epi, cudaStream_t st) {
+                 const int* asym, const float* u, float* y, Epi epi, cudaStream_t st, bool next) {
   const int nt = G.ntiles;
   const uint8_t* mu = L.mult.get();
   auto run = [&](auto kernel) {
-    launch_resident(c, kernel, nt, st, G, coef, half, asym, u, mu, y, epi);
+    launch_resident(c, next, kernel, nt, st, G, coef, half, asym, u, mu, y, epi);
   };
   if (L.B == 3) {
     if (L.kind == 27) run(k_bstencil_half<27, OFF32, 3, Epi>);
@@ -121,47 +148,51 @@ void launch_stencil(Ctx& c, const Level& L, const CT* coef, const VT* u, AT* y, 
       const int smem = kStSmemFloats * (int)sizeof(float);
       const auto kern = k_stencil_half27_staged<Epi>;
       const int g = persistent_grid(c, G.ntiles, resident_per_sm_smem((const void*)kern, smem));
-      kern<<<g, kStX * kStY, smem, st>>>(G, coef, half, asym, u, L.mult.get(), y, epi);
+      launch_after(!ev0, kern, dim3(g), kStX * kStY, smem, st, G, coef, half, asym, u, L.mult.get(), y, epi);
       done = true;
     } else if (half && L.B == 1) {
       RMG_REQUIRE(asym != nullptr, RMG_ERR_STATE, "half planes without their flag");
-      if (L.n_r <= kOffset32Nodes) launch_half<true>(c, L, G, coef, half, asym, u, y, epi, st);
-      else launch_half<false>(c, L, G, coef, half, asym, u, y, epi, st);
+      if (L.n_r <= kOffset32Nodes) launch_half<true>(c, L, G, coef, half, asym, u, y, epi, st, !ev0);
+      else launch_half<false>(c, L, G, coef, half, asym, u, y, epi, st, !ev0);
       done = true;
     } else if (half) {
       RMG_REQUIRE(asym != nullptr && L.B == 3 && (L.kind == 27 || L.kind == 9), RMG_ERR_STATE,
                   "half planes of a block operator need 3 dofs and a 27- or 9-point stencil");
-      if (L.n_r <= kOffset32Nodes) launch_half<true>(c, L, G, coef, half, asym, u, y, epi, st);
-      else launch_half<false>(c, L, G, coef, half, asym, u, y, epi, st);
+      if (L.n_r <= kOffset32Nodes) launch_half<true>(c, L, G, coef, half, asym, u, y, epi, st, !ev0);
+      else launch_half<false>(c, L, G, coef, half, asym, u, y, epi, st, !ev0);
       done = true;
     }
   }
   RMG_REQUIRE(done || G.lx != -3, RMG_ERR_STATE, "staged tiles outside a half-plane sweep");
+  auto run = [&](auto kernel) {
+    launch_after(!ev0, kernel, dim3(gb), kTile, 0, st, G, coef, u, L.mult.get(), y, epi);
+  };
   if (done) {
   } else if (L.B == 1) {
     switch (L.kind) {
-      case 5: k_stencil<5, CT, VT, AT><<<gb, kTile, 0, st>>>(G, coef, u, L.mult.get(), y, epi); break;
-      case 7: k_stencil<7, CT, VT, AT><<<gb, kTile, 0, st>>>(G, coef, u, L.mult.get(), y, epi); break;
-      case 9: k_stencil<9, CT, VT, AT><<<gb, kTile, 0, st>>>(G, coef, u, L.mult.get(), y, epi); break;
-      default: k_stencil<27, CT, VT, AT><<<gb, kTile, 0, st>>>(G, coef, u, L.mult.get(), y, epi); break;
+      case 5: run(k_stencil<5, CT, VT, AT, Epi>); break;
+      case 7: run(k_stencil<7, CT, VT, AT, Epi>); break;
+      case 9: run(k_stencil<9, CT, VT, AT, Epi>); break;
+      default: run(k_stencil<27, CT, VT, AT, Epi>); break;
     }
   } else {
     RMG_REQUIRE(L.B == 3 && (L.kind == 27 || L.kind == 9), RMG_ERR_ARG,
                 "block operators need 3 dofs per node and a 27- or 9-point stencil");
     if (L.kind == 27)
-      k_bstencil<27, 3, CT, VT, AT><<<gb, kTile, 0, st>>>(G, coef, u, L.mult.get(), y, epi);
+      run(k_bstencil<27, 3, CT, VT, AT, Epi>);
     else
-      k_bstencil<9, 3, CT, VT, AT><<<gb, kTile, 0, st>>>(G, coef, u, L.mult.get(), y, epi);
+      run(k_bstencil<9, 3, CT, VT, AT, Epi>);
   }
   RMG_LAUNCHED();
   if (ev1) RMG_CUDA(cudaEventRecordWithFlags(ev1, st, g_capturing ? cudaEventRecordExternal : 0));
   if (launches) ++*launches;
   if (L.ngroups) {
     if (L.B == 1) {
-      launch_groups(c, L, y, epi, st);
+      launch_groups(c, L, y, epi, st, !ev1);
     } else {
-      const int gg = persistent_grid(c, (L.ngroups + 255) / 256);
-      k_groups_b<AT><<<gg, 256, 0, st>>>(L.ngroups, L.B, L.n_r, L.gptr.get(), L.gslot.get(), y, epi);
+      const int gg = persistent_grid(c, (L.nslots + 255) / 256);
+      launch_after(!ev1, k_groups_b<AT, Epi>, dim3(gg), 256, 0, st, L.nslots, L.B, L.n_r, L.slots.get(),
+                  L.gslot.get(), (const AT*)y, epi);
       RMG_LAUNCHED();
     }
     if (launches) ++*launches;

@@ -173,6 +173,16 @@ __global__ void k_slot_groups(int ngroups, const int* __restrict__ gptr, int* __
     for (int q = gptr[g]; q < gptr[g + 1]; ++q) sgrp[q] = g;
 }
 
+// Slot records of phase B: {node, start of the group in gslot, copies, the other copy of two}.
+__global__ void k_slot_records(int nslots, const int* __restrict__ sgrp,
+                               const int* __restrict__ gptr, const int* __restrict__ gslot,
+                               int4* __restrict__ slots) {
+  for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < nslots; q += gridDim.x * blockDim.x) {
+    const int a = gptr[sgrp[q]], e = gptr[sgrp[q] + 1];
+    slots[q] = make_int4(gslot[q], a, e - a, gslot[a] == gslot[q] ? gslot[e - 1] : gslot[a]);
+  }
+}
+
 __global__ void k_group_sort(int ngroups, const int* __restrict__ gptr, int* __restrict__ gslot) {
   for (int g = blockIdx.x * blockDim.x + threadIdx.x; g < ngroups; g += gridDim.x * blockDim.x) {
     const int a = gptr[g], e = gptr[g + 1];
@@ -312,6 +322,12 @@ void build_groups(Ctx& c, Level& L, const uint8_t* dir_comp, const uint8_t* rmas
   if (L.ngroups) {
     k_slot_groups<<<persistent_grid(c, (L.ngroups + 255) / 256), 256, 0, c.stream>>>(
         L.ngroups, L.gptr.get(), L.sgrp.get());
+    RMG_LAUNCHED();
+  }
+  L.slots.alloc(std::max(1, L.nslots));
+  if (L.nslots) {
+    k_slot_records<<<persistent_grid(c, (L.nslots + 255) / 256), 256, 0, c.stream>>>(
+        L.nslots, L.sgrp.get(), L.gptr.get(), L.gslot.get(), L.slots.get());
     RMG_LAUNCHED();
   }
   RMG_CUDA(cudaStreamSynchronize(c.stream));

@@ -58,7 +58,9 @@ __global__ void k_diag_local(int n_r, const double* __restrict__ coef,
 
 struct EpiRecip {
   double* dinv;
-  __device__ void operator()(int n, double s, int) const { dinv[n] = 1.0 / s; }
+  struct V {};
+  __device__ V load(int) const { return V{}; }
+  __device__ void apply(int n, V, double s, int) const { dinv[n] = 1.0 / s; }
 };
 
 // ------------------------------------------------------------------ Galerkin product

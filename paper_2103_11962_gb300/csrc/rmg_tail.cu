@@ -500,6 +500,7 @@ struct Tail {
 
 template <int DIM, int B, typename VT, typename CT>
 __global__ void __launch_bounds__(kTailThreads, 1) k_tail(const __grid_constant__ TailArgs<VT, CT> A) {
+  follow();
   // consecutive warps of the index go to different blocks, so that a level smaller than the
   // cluster uses all 16 SMs (the FP64 pipe of one SM takes 16 clocks for a warp's instruction)
   const int tid = (int)(((threadIdx.x >> 5) * gridDim.x + blockIdx.x) * 32 + (threadIdx.x & 31));
@@ -575,8 +576,11 @@ int tail_cluster(int dim, int B) {
 
 template <typename VT, typename CT>
 void tail_launch(int dim, int B, int cluster, const TailArgs<VT, CT>& args, cudaStream_t st) {
-  cudaLaunchAttribute attr;
-  const cudaLaunchConfig_t cfg = tail_config(cluster, &attr, st);
+  cudaLaunchAttribute attr[2];
+  cudaLaunchConfig_t cfg = tail_config(cluster, attr, st);
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;   // as launch_next
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
+  cfg.numAttrs = 2;
   void* p[] = {const_cast<TailArgs<VT, CT>*>(&args)};
   RMG_CUDA(cudaLaunchKernelExC(&cfg, tail_kernel<VT, CT>(dim, B), p));
   RMG_LAUNCHED();
