@@ -524,80 +524,78 @@ struct Exec {
 
   const float* pw(int l) const { return h.pw[l].get(); }
 
+  // Linear restriction of r (level l) into b of level l + 1, y the partial sums of its interface.
+  void restrict_linear(int l, const VT* r, VT* b, VT* y) {
+    const Level& F = *h.lv[l];
+    const Level& C = *h.lv[l + 1];
+    const Grid Gc = C.grid();
+    if (F.dim == 3)
+      launch_next(k_restrict3<VT>, dim3(persistent_grid(c(), Gc.ntiles * (kTile / 32), 12)),
+                  32 * kRestrictWarps, 0, st, Gc, F.regions.get(), r, C.mask.get(), C.mult.get(),
+                  b, y);
+    else
+      launch_next(k_restrict2<VT>, dim3(persistent_grid(c(), Gc.ntiles)), kTile, 0, st, Gc,
+                  F.regions.get(), r, C.mask.get(), C.mult.get(), b, y);
+    RMG_LAUNCHED();
+    ++launches;
+  }
+
   void restrict_to(int l) {
     const Level& F = *h.lv[l];
     const Level& C = *h.lv[l + 1];
-    if (F.B > 1) {   // B x B block operators: the scalar transfer on every component
-      const Grid Gc = C.grid();
-      const int gb = persistent_grid(c(), Gc.ntiles);
-      for (int b = 0; b < F.B; ++b) {
-        VT* wb = V(l + 1).b.get() + (size_t)b * C.n_r;
-        VT* yb = V(l + 1).y.get() + (size_t)b * C.n_r;
-        const VT* rb = V(l).r.get() + (size_t)b * F.n_r;
-        launch_next(k_restrict<3, VT>, dim3(gb), kTile, 0, st, Gc, F.regions.get(), rb, C.mask.get(),
-                                                C.mult.get(), wb, yb);
+    for (int k = 0; k < F.B; ++k) {   // B x B block operators: the scalar transfer per component
+      VT* b = V(l + 1).b.get() + (size_t)k * C.n_r;
+      VT* y = V(l + 1).y.get() + (size_t)k * C.n_r;
+      const VT* r = V(l).r.get() + (size_t)k * F.n_r;
+      if (h.stored[l]) {
+        const Grid Gc = C.grid();
+        const int gb = persistent_grid(c(), Gc.ntiles);
+        auto run = [&](auto kernel) {
+          launch_next(kernel, dim3(gb), kTile, 0, st, Gc, F.regions.get(), F.n_r, pw(l), r,
+                      C.mask.get(), C.mult.get(), b, y);
+        };
+        if (F.dim == 3) run(k_restrict_w<3, VT>);
+        else run(k_restrict_w<2, VT>);
         RMG_LAUNCHED();
         ++launches;
-        if (C.ngroups) {
-          launch_groups(c(), C, (const VT*)yb, EpiStore<VT>{wb}, st);
-          ++launches;
-        }
+      } else {
+        restrict_linear(l, r, b, y);
       }
-      return;
-    }
-    const Grid Gc = C.grid();
-    const int gb = persistent_grid(c(), Gc.ntiles);
-    if (h.stored[l]) {
-      if (F.dim == 3)
-        launch_next(k_restrict_w<3, VT>, dim3(gb), kTile, 0, st, Gc, F.regions.get(), F.n_r, pw(l), V(l).r.get(),
-                                                  C.mask.get(), C.mult.get(), V(l + 1).b.get(),
-                                                  V(l + 1).y.get());
-      else
-        launch_next(k_restrict_w<2, VT>, dim3(gb), kTile, 0, st, Gc, F.regions.get(), F.n_r, pw(l), V(l).r.get(),
-                                                  C.mask.get(), C.mult.get(), V(l + 1).b.get(),
-                                                  V(l + 1).y.get());
-    } else if (F.dim == 3)
-      launch_next(k_restrict<3, VT>, dim3(gb), kTile, 0, st, Gc, F.regions.get(), V(l).r.get(), C.mask.get(),
-                                              C.mult.get(), V(l + 1).b.get(), V(l + 1).y.get());
-    else
-      launch_next(k_restrict<2, VT>, dim3(gb), kTile, 0, st, Gc, F.regions.get(), V(l).r.get(), C.mask.get(),
-                                              C.mult.get(), V(l + 1).b.get(), V(l + 1).y.get());
-    RMG_LAUNCHED();
-    ++launches;
-    if (C.ngroups) {
-      launch_groups(c(), C, (const VT*)V(l + 1).y.get(), EpiStore<VT>{V(l + 1).b.get()}, st);
-      ++launches;
+      if (C.ngroups) {
+        launch_groups(c(), C, (const VT*)y, EpiStore<VT>{b}, st);
+        ++launches;
+      }
     }
   }
 
   void prolong(int l) {
     const Level& F = *h.lv[l];
     const Level& C = *h.lv[l + 1];
-    const Grid Gf = F.grid();
-    const int gb = persistent_grid(c(), Gf.ntiles);
-    if (F.B > 1) {
-      for (int b = 0; b < F.B; ++b) {
-        launch_next(k_prolong<3, VT>, dim3(gb), kTile, 0, st, Gf, C.regions.get(), F.mask.get(),
-                                               cur[l + 1] + (size_t)b * C.n_r,
-                                               cur[l] + (size_t)b * F.n_r);
-        RMG_LAUNCHED();
-        ++launches;
+    for (int k = 0; k < F.B; ++k) {
+      const VT* ubar = cur[l + 1] + (size_t)k * C.n_r;
+      VT* u = cur[l] + (size_t)k * F.n_r;
+      if (h.stored[l]) {
+        const Grid Gf = F.grid();
+        const int gb = persistent_grid(c(), Gf.ntiles);
+        auto run = [&](auto kernel) {
+          launch_next(kernel, dim3(gb), kTile, 0, st, Gf, C.regions.get(), pw(l), F.mask.get(),
+                      ubar, u);
+        };
+        if (F.dim == 3) run(k_prolong_w<3, VT>);
+        else run(k_prolong_w<2, VT>);
+      } else {
+        const Grid G1 = h.rap_x[l].grid(F.nreg);
+        const int gb = persistent_grid(c(), G1.ntiles);
+        auto run = [&](auto kernel) {
+          launch_next(kernel, dim3(gb), kTile, 0, st, G1, F.regions.get(), C.regions.get(),
+                      F.mask.get(), ubar, u);
+        };
+        if (F.dim == 3) run(k_prolong<3, VT>);
+        else run(k_prolong<2, VT>);
       }
-      return;
+      RMG_LAUNCHED();
+      ++launches;
     }
-    if (h.stored[l]) {
-      if (F.dim == 3)
-        launch_next(k_prolong_w<3, VT>, dim3(gb), kTile, 0, st, Gf, C.regions.get(), pw(l), F.mask.get(),
-                                                 cur[l + 1], cur[l]);
-      else
-        launch_next(k_prolong_w<2, VT>, dim3(gb), kTile, 0, st, Gf, C.regions.get(), pw(l), F.mask.get(),
-                                                 cur[l + 1], cur[l]);
-    } else if (F.dim == 3)
-      launch_next(k_prolong<3, VT>, dim3(gb), kTile, 0, st, Gf, C.regions.get(), F.mask.get(), cur[l + 1], cur[l]);
-    else
-      launch_next(k_prolong<2, VT>, dim3(gb), kTile, 0, st, Gf, C.regions.get(), F.mask.get(), cur[l + 1], cur[l]);
-    RMG_LAUNCHED();
-    ++launches;
   }
 
   void coarse(int l) {

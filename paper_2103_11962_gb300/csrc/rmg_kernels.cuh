@@ -865,11 +865,12 @@ __device__ __forceinline__ VT restrict_sum(const VT* __restrict__ rs, const Regi
   return acc;
 }
 
-template <int DIM, typename VT>
+// 2D: a thread per coarse node and its 25 fine nodes.
+template <typename VT>
 __global__ void __launch_bounds__(kTile)
-k_restrict(Grid Gc, const RegionDev* __restrict__ fregions, const VT* __restrict__ rs,
-           const uint8_t* __restrict__ cmask, const uint8_t* __restrict__ cmult,
-           VT* __restrict__ w, VT* __restrict__ yc) {
+k_restrict2(Grid Gc, const RegionDev* __restrict__ fregions, const VT* __restrict__ rs,
+            const uint8_t* __restrict__ cmask, const uint8_t* __restrict__ cmult,
+            VT* __restrict__ w, VT* __restrict__ yc) {
   follow();
   RMG_FOR_NODES(Gc)
     int I, J, L;
@@ -877,13 +878,58 @@ k_restrict(Grid Gc, const RegionDev* __restrict__ fregions, const VT* __restrict
     VT acc = VT(0);
     if (!cmask[n]) {
       const RegionDev F = fregions[tile_.region];
-      const bool inner = I > 0 && I < R.nx - 1 && J > 0 && J < R.ny - 1 &&
-                         (DIM == 2 || (L > 0 && L < R.nz - 1));
-      acc = inner ? restrict_sum<DIM, false, false, VT>(rs, F, nullptr, 0, I, J, L)
-                  : restrict_sum<DIM, true, false, VT>(rs, F, nullptr, 0, I, J, L);
+      const bool inner = I > 0 && I < R.nx - 1 && J > 0 && J < R.ny - 1;
+      acc = inner ? restrict_sum<2, false, false, VT>(rs, F, nullptr, 0, I, J, 0)
+                  : restrict_sum<2, true, false, VT>(rs, F, nullptr, 0, I, J, 0);
     }
     if (cmult[n] > 1) yc[n] = acc; else w[n] = acc;
   RMG_END_FOR_NODES
+}
+
+// 3D: five warps for 32 consecutive coarse nodes, a warp for each z-plane of their support (25
+// fine nodes); the first warp adds the planes. With a thread for all 125 the coarse level had too
+// few threads to hide their latency: RESTRICT_TIMES.
+constexpr int kRestrictWarps = 5;
+template <typename VT>
+__global__ void __launch_bounds__(32 * kRestrictWarps)
+k_restrict3(Grid Gc, const RegionDev* __restrict__ fregions, const VT* __restrict__ rs,
+            const uint8_t* __restrict__ cmask, const uint8_t* __restrict__ cmult,
+            VT* __restrict__ w, VT* __restrict__ yc) {
+  follow();
+  __shared__ VT part[kRestrictWarps][32];
+  constexpr int kChunks = kTile / 32;
+  const int lane = threadIdx.x & 31, c = (int)(threadIdx.x >> 5) - 2;
+  const VT wz = c == 0 ? VT(1) : (c == 1 || c == -1 ? VT(w1d(-1)) : VT(w1d(-2)));
+  for (int task = blockIdx.x; task < Gc.ntiles * kChunks; task += gridDim.x) {
+    const Tile tile = Gc.tiles[task / kChunks];
+    const RegionDev R = Gc.regions[tile.region];
+    const int first = tile.start + (task % kChunks) * 32, li = first + lane;
+    if (first >= R.nx * R.ny * R.nz) continue;             // the same for the whole block
+    const bool in = li < R.nx * R.ny * R.nz;
+    const int n = R.off + li;
+    VT acc = VT(0);
+    if (in && !cmask[n]) {
+      int I, J, L;
+      decode(li, R, I, J, L);
+      RegionDev F = fregions[tile.region];
+      const int z = 3 * L + c;
+      if (z >= 0 && z < F.nz) {
+        F.off += F.nx * F.ny * z;                          // the plane as a 2D region
+        const bool inner = I > 0 && I < R.nx - 1 && J > 0 && J < R.ny - 1;
+        acc = wz * (inner ? restrict_sum<2, false, false, VT>(rs, F, nullptr, 0, I, J, 0)
+                          : restrict_sum<2, true, false, VT>(rs, F, nullptr, 0, I, J, 0));
+      }
+    }
+    part[c + 2][lane] = acc;
+    __syncthreads();
+    if (c == -2 && in) {
+      VT s = part[0][lane];
+#pragma unroll
+      for (int k = 1; k < kRestrictWarps; ++k) s += part[k][lane];
+      if (cmult[n] > 1) yc[n] = s; else w[n] = s;
+    }
+    __syncthreads();
+  }
 }
 
 // Weight of the right coarse neighbour of a fine node with remainder rem (the left one takes
@@ -893,21 +939,23 @@ __device__ __forceinline__ VT rem_weight(int rem) {
   return rem == 0 ? VT(0) : (rem == 1 ? VT(1.0 / 3.0) : VT(2.0 / 3.0));
 }
 
-// Region-local interpolation and correction u += [[P]] ubar (no inter-region exchange). Every
-// fine node gathers the 2 x 2 (x 2) coarse nodes around it and combines them axis by axis with
-// the weights (1 - w, w) of its remainders; a right neighbour past the region edge only occurs
-// with remainder 0 (weight 0) and is clamped onto the left one.
+// Region-local interpolation and correction u += [[P]] ubar (no inter-region exchange). A thread
+// takes the three fine nodes of a line between two coarse columns (G1: the level's node grid
+// coarsened along x): it interpolates the two columns along y and z once and mixes them for its
+// nodes, a third of the loads and half of the arithmetic of a thread per node. A right neighbour
+// past the region edge only occurs with weight 0 and is clamped onto the left one. 1.5M nodes in
+// FP64 52 -> PRO64 us, 6M in FP32 37 -> PRO32 us.
 template <int DIM, typename VT>
 __global__ void __launch_bounds__(kTile)
-k_prolong(Grid Gf, const RegionDev* __restrict__ cregions, const uint8_t* __restrict__ fmask,
-          const VT* __restrict__ ubar, VT* __restrict__ u) {
+k_prolong(Grid G1, const RegionDev* __restrict__ fregions, const RegionDev* __restrict__ cregions,
+          const uint8_t* __restrict__ fmask, const VT* __restrict__ ubar, VT* __restrict__ u) {
   follow();
-  RMG_FOR_NODES(Gf)
-    if (fmask[n]) continue;
-    int i, j, l;
-    decode(li, R, i, j, l);
-    const RegionDev C = cregions[tile_.region];
-    const int cx = i / 3, rx = i - 3 * cx;
+  RMG_FOR_NODES(G1)
+    (void)n;
+    int cx, j, l;
+    decode(li, R, cx, j, l);
+    const RegionDev F = fregions[tile_.region], C = cregions[tile_.region];
+    const int f = F.off + 3 * cx + F.nx * (j + F.ny * l);
     const int cy = j / 3, ry = j - 3 * cy;
     const int cz = DIM == 3 ? l / 3 : 0, rz = DIM == 3 ? l - 3 * cz : 0;
     const int sy = C.nx, sz = C.nx * C.ny;
@@ -915,17 +963,22 @@ k_prolong(Grid Gf, const RegionDev* __restrict__ cregions, const uint8_t* __rest
     const int dy = cy + 1 < C.ny ? sy : 0;
     const int dz = (DIM == 3 && cz + 1 < C.nz) ? sz : 0;
     const VT* b0 = ubar + C.off + cx + sy * cy + sz * cz;
-    const VT wx1 = rem_weight<VT>(rx), wx0 = VT(1) - wx1;
     const VT wy1 = rem_weight<VT>(ry), wy0 = VT(1) - wy1;
-    auto xline = [&](const VT* p) { return fma(wx1, p[dx], wx0 * p[0]); };
-    const VT a0 = fma(wy1, xline(b0 + dy), wy0 * xline(b0));
-    VT acc = a0;
-    if (DIM == 3) {
-      const VT wz1 = rem_weight<VT>(rz), wz0 = VT(1) - wz1;
-      const VT a1 = fma(wy1, xline(b0 + dz + dy), wy0 * xline(b0 + dz));
-      acc = fma(wz1, a1, wz0 * a0);
+    const VT wz1 = rem_weight<VT>(rz), wz0 = VT(1) - wz1;
+    auto column = [&](const VT* p) {
+      const VT a0 = fma(wy1, p[dy], wy0 * p[0]);
+      if (DIM == 2) return a0;
+      const VT a1 = fma(wy1, p[dz + dy], wy0 * p[dz]);
+      return fma(wz1, a1, wz0 * a0);
+    };
+    const VT left = column(b0), right = column(b0 + dx);
+    const int nodes = min(3, F.nx - 3 * cx);
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      if (k >= nodes || fmask[f + k]) continue;
+      const VT w1 = rem_weight<VT>(k), w0 = VT(1) - w1;
+      u[f + k] += k == 0 ? left : fma(w1, right, w0 * left);
     }
-    u[n] = u[n] + acc;
   RMG_END_FOR_NODES
 }
 
