@@ -1219,7 +1219,7 @@ static void coarse_factor(Hier& h) {
   if (h.nc == 0 || !h.dense_ok) return;
   const int nc = h.nc * L.B;     // dense dimension: B dofs per free composite node
   RMG_CUDA(cudaMemsetAsync(h.Mfac.get(), 0, (size_t)nc * nc * sizeof(double), st));
-  const dim3 gb(persistent_grid(c, (L.ncomp + 127) / 128), L.B);
+  const dim3 gb(persistent_grid(c, (L.ncomp + 3) / 4), L.B);      // a warp per composite node
 #define RMG_ASM(K)                                                                              \
   k_coarse_assemble<K><<<gb, 128, 0, st>>>(L.ncomp, L.B, L.regions.get(), L.nreg, L.n_r,        \
                                            L.coef.get(), L.gid.get(), h.cidx.get(), L.c2r.get(), \

@@ -598,16 +598,22 @@ __global__ void k_coarse_maps(int ncomp, const int* __restrict__ freeflag, const
 // Abar = Psibar [[Abar]] Psibar^T restricted to unmasked nodes (eq. CoarseCompositeOperator):
 // row of composite node g = sum over its regional copies of their region rows. With B dofs per
 // node the dense matrix has dimension B * nc, dof cidx * B + b (blockIdx.y = row component).
+// A warp per row and a lane per stencil slot: the entries of one copy go to different columns, and
+// the copies are added one after the other, so every sum keeps its order. (With a thread per row
+// its up to 216 entries were one chain of loads: 83 us for a few dozen rows.)
 template <int KIND>
 __global__ void k_coarse_assemble(int ncomp, int B, const RegionDev* __restrict__ regs, int nreg,
                                   int n_r, const double* __restrict__ coef,
                                   const int* __restrict__ gid, const int* __restrict__ cidx,
                                   const int* __restrict__ c2r, const int* __restrict__ cgrp,
                                   const int* __restrict__ gptr, const int* __restrict__ gslot,
-                                  int nd, double* __restrict__ M) {
+                                  int nd, double* M) {
   using S = Sten<KIND>;
   const int b = blockIdx.y;
-  for (int g = blockIdx.x * blockDim.x + threadIdx.x; g < ncomp; g += gridDim.x * blockDim.x) {
+  const int lane = threadIdx.x & 31;
+  const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  const int nwarps = (gridDim.x * blockDim.x) >> 5;
+  for (int g = warp; g < ncomp; g += nwarps) {
     const int rowc = cidx[g];
     if (rowc < 0) continue;
     const size_t row = (size_t)rowc * B + b;
@@ -619,16 +625,17 @@ __global__ void k_coarse_assemble(int ncomp, int B, const RegionDev* __restrict_
       const RegionDev R = regs[region_of(regs, nreg, n)];
       int i, j, l;
       decode(n - R.off, R, i, j, l);
-      for (int s = 0; s < S::S; ++s) {
-        const int x = i + S::dx(s), y = j + S::dy(s), z = l + S::dz(s);
-        if (x < 0 || x >= R.nx || y < 0 || y >= R.ny || z < 0 || z >= R.nz) continue;
-        const int n2 = R.off + x + R.nx * (y + R.ny * z);
-        const int col = cidx[gid[n2]];
-        if (col < 0) continue;
-        for (int b2 = 0; b2 < B; ++b2)
-          M[row * nd + (size_t)col * B + b2] +=
-              coef[((size_t)(b * B + b2) * S::S + s) * n_r + n];
+      if (lane < S::S) {
+        const int x = i + S::dx(lane), y = j + S::dy(lane), z = l + S::dz(lane);
+        if (x >= 0 && x < R.nx && y >= 0 && y < R.ny && z >= 0 && z < R.nz) {
+          const int col = cidx[gid[R.off + x + R.nx * (y + R.ny * z)]];
+          if (col >= 0)
+            for (int b2 = 0; b2 < B; ++b2)
+              M[row * nd + (size_t)col * B + b2] +=
+                  coef[((size_t)(b * B + b2) * S::S + lane) * n_r + n];
+        }
       }
+      __syncwarp();
     }
   }
 }
@@ -643,19 +650,22 @@ __global__ void k_coarse_assemble(int ncomp, int B, const RegionDev* __restrict_
 // A partial last block is padded with the identity inside the kernels.
 constexpr int kNB = 32;
 
+// The lane keeps its row of the block (then its column of the inverse) in registers and gets the
+// others' by shuffles; through shared memory with run-time bounds a block took 36 us, a chain of
+// about a thousand dependent loads (a coarsest level of 1331 unknowns has 42 blocks in a row).
 template <typename F>
 __global__ void __launch_bounds__(32)
 k_chol_diag(F* M, int n, int k0, F* __restrict__ Dblk, int* err) {
-  __shared__ F T[kNB][kNB + 1];
-  __shared__ F X[kNB][kNB + 1];
-  __shared__ F rdiag[kNB];
   const int nb = min(kNB, n - k0);
   const int ln = threadIdx.x;
-  for (int i = 0; i < kNB; ++i)
-    T[i][ln] = (i < nb && ln < nb) ? M[(size_t)(k0 + i) * n + k0 + ln] : F(i == ln ? 1 : 0);
-  __syncwarp();
+  F a[kNB];                                    // row ln of the block, then of its factor
+#pragma unroll
+  for (int c = 0; c < kNB; ++c)
+    a[c] = (ln < nb && c < nb) ? M[(size_t)(k0 + ln) * n + k0 + c] : F(c == ln ? 1 : 0);
+  F rdiag = F(0);
+#pragma unroll
   for (int j = 0; j < kNB; ++j) {
-    F p = T[j][j];
+    F p = __shfl_sync(0xffffffffu, a[j], j);
     if (!(p > F(0))) {
       if (ln == 0) set_err(err, DERR_NOT_SPD);
       p = F(1);
@@ -673,32 +683,35 @@ k_chol_diag(F* M, int n, int k0, F* __restrict__ Dblk, int* err) {
     } else {
       rd = F(1) / sqrt(p);
     }
-    const F d = p * rd;
-    __syncwarp();
-    if (ln == j) { T[j][j] = d; rdiag[j] = rd; }
-    if (ln > j) T[ln][j] *= rd;
-    __syncwarp();
-    if (ln > j) {
-      const F lij = T[ln][j];
-      for (int c = j + 1; c <= ln; ++c) T[ln][c] -= lij * T[c][j];
+    if (ln == j) {
+      a[j] = p * rd;
+      rdiag = rd;
     }
-    __syncwarp();
+    if (ln > j) a[j] *= rd;
+    const F lij = a[j];
+#pragma unroll
+    for (int c = j + 1; c < kNB; ++c) {
+      const F lcj = __shfl_sync(0xffffffffu, lij, c);
+      if (c <= ln) a[c] -= lij * lcj;
+    }
   }
   // column ln of L^-1 by forward substitution (each lane owns one column)
+  F x[kNB];
+#pragma unroll
   for (int i = 0; i < kNB; ++i) {
-    F x = F(0);
-    if (i >= ln) {
-      F s = F(i == ln ? 1 : 0);
-      for (int m = ln; m < i; ++m) s -= T[i][m] * X[m][ln];
-      x = s * rdiag[i];
-    }
-    X[i][ln] = x;
+    F s = F(i == ln ? 1 : 0);
+#pragma unroll
+    for (int m = 0; m < i; ++m) s -= __shfl_sync(0xffffffffu, a[m], i) * x[m];
+    const F rd = __shfl_sync(0xffffffffu, rdiag, i);
+    x[i] = i >= ln ? s * rd : F(0);
   }
-  __syncwarp();
   F* D = Dblk + (size_t)(k0 / kNB) * kNB * kNB;
-  for (int i = 0; i < kNB; ++i) {
-    D[i * kNB + ln] = X[i][ln];
-    if (i < nb && ln < nb) M[(size_t)(k0 + i) * n + k0 + ln] = ln <= i ? T[i][ln] : F(0);
+#pragma unroll
+  for (int i = 0; i < kNB; ++i) D[i * kNB + ln] = x[i];
+  if (ln < nb) {
+#pragma unroll
+    for (int c = 0; c < kNB; ++c)
+      if (c < nb) M[(size_t)(k0 + ln) * n + k0 + c] = c <= ln ? a[c] : F(0);
   }
 }
 
