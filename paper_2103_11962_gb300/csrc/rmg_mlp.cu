@@ -32,6 +32,7 @@ constexpr int NPARAMS = NH * NF + NH + NH * NH + NH + NOUT * NH + NOUT;
 constexpr int O_W1 = 0, O_B1 = O_W1 + NH * NF, O_W2 = O_B1 + NH, O_B2 = O_W2 + NH * NH,
               O_W3 = O_B2 + NH, O_B3 = O_W3 + NOUT * NH;
 constexpr int kRows = 128, kThreads = 256;
+constexpr int kGradThreads = 512;                          // k_mlp
 // padded shared-memory strides (elements)
 constexpr int SX = NF + 8, SH = NH + 8;
 
@@ -56,7 +57,7 @@ struct MlpSmem {
   float Y[kRows * 4];
   float M[kRows * 4];
   long long idx[kRows];                  // sample of every row, -1 past the last one
-  float red[kThreads / 32];
+  float red[kGradThreads / 32];
 };
 
 __device__ __forceinline__ uint32_t pack2(const __nv_bfloat16* p) {
@@ -107,10 +108,11 @@ __device__ __forceinline__ void red_add2(float* p, float a, float b) {
 //
 // Bound by the FP32 pipe in the backward products (1.3M FMAs a tile). One FMA per two shared
 // loads and a set of 6467 atomic adds per tile took 269 us for 65,573 samples; here every
-// thread owns blocks of the outputs (4 x 4 of dW2, 4 x 2 of dW1, 8 x 4 of dZ1), loads its
+// thread owns blocks of the outputs (4 x 4 of dW2, 4 x 2 of dW1, 4 x 4 of dZ1), loads its
 // operands four at a time, and keeps the weight gradients of all its CTA's tiles in registers,
-// so the atomic adds run once per CTA: 76 us (the whole call with its copies 313 -> 105 us).
-__global__ void __launch_bounds__(kThreads, 1)
+// so the atomic adds run once per CTA, and 16 warps hide each other's shared loads: 70 us (the
+// whole call with its copies 313 -> 99 us; 105 with eight warps).
+__global__ void __launch_bounds__(kGradThreads, 1)
 k_mlp(const float* __restrict__ params, int n, long long ntiles, const float* __restrict__ feats,
       const float* __restrict__ labels, const float* __restrict__ mask, int sample,
       unsigned long long seed, float inv_norm, float* __restrict__ grads,
@@ -121,22 +123,23 @@ k_mlp(const float* __restrict__ params, int n, long long ntiles, const float* __
   const int g = lane >> 2, t = lane & 3;
 
   // ---- stage weights (bf16 copies for the MMA, fp32 copies for the backward pass)
-  for (int e = tid; e < NH * NF; e += kThreads)
+  for (int e = tid; e < NH * NF; e += kGradThreads)
     S.W1b[(e / NF) * SX + e % NF] = __float2bfloat16_rn(params[O_W1 + e]);
-  for (int e = tid; e < NH * NH; e += kThreads) {
+  for (int e = tid; e < NH * NH; e += kGradThreads) {
     const float w = params[O_W2 + e];
     S.W2b[(e / NH) * SH + e % NH] = __float2bfloat16_rn(w);
     S.W2f[e] = w;
   }
-  for (int e = tid; e < 8 * NH; e += kThreads) {
+  for (int e = tid; e < 8 * NH; e += kGradThreads) {
     const int j = e / NH, k = e % NH;
     const float w = j < NOUT ? params[O_W3 + j * NH + k] : 0.f;
     S.W3b[j * SH + k] = __float2bfloat16_rn(w);
     if (j < 4) S.W3f[j * NH + k] = w;
   }
-  // this thread's share of the gradients: dW2[4 mg..][4 kg..], dW1[4 mg..][2 kg..], and over
-  // the rows of its quarter rq (32 rows) column kq of dW3, db2 and db1
-  const int mg = tid >> 4, kg = tid & 15, rq = tid >> 6, kq = tid & 63;
+  // this thread's share of the gradients: over the rows of its half (64 rows from rh)
+  // dW2[4 mg..][4 kg..] and dW1[4 mg..][2 kg..], over 16 rows column kq of dW3, db2 and db1
+  const int rh = 64 * (tid >> 8), mg = (tid & 255) >> 4, kg = tid & 15;
+  const int rq = 16 * (tid >> 6), kq = tid & 63;
   float gw2[4][4] = {}, gw1[4][2] = {}, gw3[NOUT] = {}, gb3 = 0.f, gb2 = 0.f, gb1 = 0.f;
   float lsum = 0.f;
   // persistent loop over tiles of 128 samples; the weights above are staged once per CTA
@@ -154,14 +157,14 @@ k_mlp(const float* __restrict__ params, int n, long long ntiles, const float* __
   }
   __syncthreads();
   // ---- stage the samples
-  for (int e = tid; e < kRows * NF; e += kThreads) {
+  for (int e = tid; e < kRows * NF; e += kGradThreads) {
     const int r = e / NF, k = e % NF;
     const long long i = S.idx[r];
     const __nv_bfloat16 v = __float2bfloat16_rn(i >= 0 ? feats[i * NF + k] : 0.f);
     S.Xb[r * SX + k] = v;
     S.Xf[r * SXF + k] = __bfloat162float(v);
   }
-  for (int e = tid; e < kRows * NOUT; e += kThreads) {
+  for (int e = tid; e < kRows * NOUT; e += kGradThreads) {
     const int r = e / NOUT, j = e % NOUT;
     const long long i = S.idx[r];
     S.Y[r * 4 + j] = i >= 0 ? labels[i * NOUT + j] : 0.f;
@@ -169,14 +172,14 @@ k_mlp(const float* __restrict__ params, int n, long long ntiles, const float* __
   }
   __syncthreads();
 
-  const int r0 = warp * 16;
+  const int r0 = (warp & 7) * 16, c0 = 32 * (warp >> 3);   // rows and columns of the warp
   // ---- layer 1: H1 = relu(X W1^T + b1)
   {
-    float acc[8][4] = {};
-    warp_mma<8, NF>(S.Xb, SX, r0, S.W1b, SX, acc);
+    float acc[4][4] = {};
+    warp_mma<4, NF>(S.Xb, SX, r0, S.W1b + c0 * SX, SX, acc);
 #pragma unroll
-    for (int nt = 0; nt < 8; ++nt) {
-      const int c = nt * 8 + 2 * t;
+    for (int nt = 0; nt < 4; ++nt) {
+      const int c = c0 + nt * 8 + 2 * t;
       const float b0 = params[O_B1 + c], b1 = params[O_B1 + c + 1];
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
@@ -190,14 +193,14 @@ k_mlp(const float* __restrict__ params, int n, long long ntiles, const float* __
       }
     }
   }
-  __syncwarp();
+  __syncthreads();
   // ---- layer 2: H2 = relu(H1 W2^T + b2)
   {
-    float acc[8][4] = {};
-    warp_mma<8, NH>(S.H1b, SH, r0, S.W2b, SH, acc);
+    float acc[4][4] = {};
+    warp_mma<4, NH>(S.H1b, SH, r0, S.W2b + c0 * SH, SH, acc);
 #pragma unroll
-    for (int nt = 0; nt < 8; ++nt) {
-      const int c = nt * 8 + 2 * t;
+    for (int nt = 0; nt < 4; ++nt) {
+      const int c = c0 + nt * 8 + 2 * t;
       const float b0 = params[O_B2 + c], b1 = params[O_B2 + c + 1];
       S.H2b[(r0 + g) * SH + c] = __float2bfloat16_rn(fmaxf(acc[nt][0] + b0, 0.f));
       S.H2b[(r0 + g) * SH + c + 1] = __float2bfloat16_rn(fmaxf(acc[nt][1] + b1, 0.f));
@@ -205,9 +208,9 @@ k_mlp(const float* __restrict__ params, int n, long long ntiles, const float* __
       S.H2b[(r0 + g + 8) * SH + c + 1] = __float2bfloat16_rn(fmaxf(acc[nt][3] + b1, 0.f));
     }
   }
-  __syncwarp();
+  __syncthreads();
   // ---- layer 3: O = sigmoid(H2 W3^T + b3) (8 padded output columns, 3 used)
-  {
+  if (warp < 8) {
     float acc[1][4] = {};
     warp_mma<1, NH>(S.H2b, SH, r0, S.W3b, SH, acc);
     const int c = 2 * t;
@@ -224,18 +227,18 @@ k_mlp(const float* __restrict__ params, int n, long long ntiles, const float* __
   __syncthreads();
 
   // ---- backward (FP32)
-  for (int e = tid; e < kRows * NOUT; e += kThreads) {
+  for (int e = tid; e < kRows * NOUT; e += kGradThreads) {
     const int r = e / NOUT, j = e % NOUT;
     const float o = S.O[r * 4 + j], m = S.M[r * 4 + j], d = o - S.Y[r * 4 + j];
     lsum += m * d * d;
     S.dZ3[r * 4 + j] = 2.f * m * d * inv_norm * o * (1.f - o);
   }
   __syncthreads();
-  // dZ2 = (dZ3 W3) * [H2 > 0], and column kq of dW3, db2 over 32 rows
+  // dZ2 = (dZ3 W3) * [H2 > 0], and column kq of dW3, db2 over 16 rows
   {
     const float w0 = S.W3f[kq], w1 = S.W3f[NH + kq], w2 = S.W3f[2 * NH + kq];
 #pragma unroll 4
-    for (int r = 32 * rq; r < 32 * rq + 32; ++r) {
+    for (int r = rq; r < rq + 16; ++r) {
       const float d0 = S.dZ3[r * 4], d1 = S.dZ3[r * 4 + 1], d2 = S.dZ3[r * 4 + 2];
       const float h = __bfloat162float(S.H2b[r * SH + kq]);
       gw3[0] = fmaf(d0, h, gw3[0]);
@@ -246,12 +249,12 @@ k_mlp(const float* __restrict__ params, int n, long long ntiles, const float* __
       gb2 += z;
     }
     if (kq < NOUT)
-      for (int r = 32 * rq; r < 32 * rq + 32; ++r) gb3 += S.dZ3[r * 4 + kq];
+      for (int r = rq; r < rq + 16; ++r) gb3 += S.dZ3[r * 4 + kq];
   }
   __syncthreads();
   // dW2 += dZ2^T H1
 #pragma unroll 4
-  for (int r = 0; r < kRows; ++r) {
+  for (int r = rh; r < rh + 64; ++r) {
     const float4 z = *reinterpret_cast<const float4*>(&S.dZ2[r * SHF + 4 * mg]);
     const float4 h = *reinterpret_cast<const float4*>(&S.H1f[r * SHF + 4 * kg]);
     const float zv[4] = {z.x, z.y, z.z, z.w}, hv[4] = {h.x, h.y, h.z, h.w};
@@ -260,9 +263,10 @@ k_mlp(const float* __restrict__ params, int n, long long ntiles, const float* __
 #pragma unroll
       for (int b = 0; b < 4; ++b) gw2[a][b] = fmaf(zv[a], hv[b], gw2[a][b]);
   }
-  // dZ1 = (dZ2 W2) * [H1 > 0]: rows 8 mg .. 8 mg + 7, columns 4 kg ..
+  // dZ1 = (dZ2 W2) * [H1 > 0]: rows r4 .. r4 + 3, columns 4 kg ..
   {
-    float acc[8][4] = {};
+    const int r4 = 4 * (tid >> 4);
+    float acc[4][4] = {};
 #pragma unroll 2
     for (int m = 0; m < NH; m += 4) {
       float4 w[4];
@@ -270,8 +274,8 @@ k_mlp(const float* __restrict__ params, int n, long long ntiles, const float* __
       for (int q = 0; q < 4; ++q)
         w[q] = *reinterpret_cast<const float4*>(&S.W2f[(m + q) * NH + 4 * kg]);
 #pragma unroll
-      for (int a = 0; a < 8; ++a) {
-        const float4 z = *reinterpret_cast<const float4*>(&S.dZ2[(8 * mg + a) * SHF + m]);
+      for (int a = 0; a < 4; ++a) {
+        const float4 z = *reinterpret_cast<const float4*>(&S.dZ2[(r4 + a) * SHF + m]);
         const float zv[4] = {z.x, z.y, z.z, z.w};
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
@@ -283,8 +287,8 @@ k_mlp(const float* __restrict__ params, int n, long long ntiles, const float* __
       }
     }
 #pragma unroll
-    for (int a = 0; a < 8; ++a) {
-      const int at = (8 * mg + a) * SHF + 4 * kg;
+    for (int a = 0; a < 4; ++a) {
+      const int at = (r4 + a) * SHF + 4 * kg;
       const float4 h = *reinterpret_cast<const float4*>(&S.H1f[at]);
       *reinterpret_cast<float4*>(&S.dZ1[at]) =
           make_float4(h.x > 0.f ? acc[a][0] : 0.f, h.y > 0.f ? acc[a][1] : 0.f,
@@ -294,7 +298,7 @@ k_mlp(const float* __restrict__ params, int n, long long ntiles, const float* __
   __syncthreads();
   // dW1 += dZ1^T X, db1
 #pragma unroll 4
-  for (int r = 0; r < kRows; ++r) {
+  for (int r = rh; r < rh + 64; ++r) {
     const float4 z = *reinterpret_cast<const float4*>(&S.dZ1[r * SHF + 4 * mg]);
     const float2 x = *reinterpret_cast<const float2*>(&S.Xf[r * SXF + 2 * kg]);
     const float zv[4] = {z.x, z.y, z.z, z.w};
@@ -305,7 +309,7 @@ k_mlp(const float* __restrict__ params, int n, long long ntiles, const float* __
     }
   }
 #pragma unroll 4
-  for (int r = 32 * rq; r < 32 * rq + 32; ++r) gb1 += S.dZ1[r * SHF + kq];
+  for (int r = rq; r < rq + 16; ++r) gb1 += S.dZ1[r * SHF + kq];
   }  // tiles
 
   // ---- this CTA's sums
@@ -326,7 +330,7 @@ k_mlp(const float* __restrict__ params, int n, long long ntiles, const float* __
   __syncthreads();
   if (tid == 0) {
     float sum = 0.f;
-    for (int w = 0; w < kThreads / 32; ++w) sum += S.red[w];
+    for (int w = 0; w < kGradThreads / 32; ++w) sum += S.red[w];
     atomicAdd(loss, sum * inv_norm);
   }
 }
@@ -691,7 +695,7 @@ void mlp_backward(rmg_mlp* net, int n, const float* feats, const float* labels, 
   RMG_CUDA(cudaFuncSetAttribute(k_mlp, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
   const long long tiles = ((long long)rows + kRows - 1) / kRows;
   const int blocks = (int)std::min<long long>(tiles, (long long)c.nsm);
-  k_mlp<<<blocks, kThreads, smem, c.stream>>>(net->p.get(), n, tiles, feats, labels, mask, sample,
+  k_mlp<<<blocks, kGradThreads, smem, c.stream>>>(net->p.get(), n, tiles, feats, labels, mask, sample,
                                              seed, inv_norm, net->g.get(), loss);
   RMG_LAUNCHED();
 }
