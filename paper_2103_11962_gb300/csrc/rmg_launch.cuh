@@ -15,9 +15,9 @@
 namespace rmg {
 
 // Blocks of kTile threads of `kernel` that one SM keeps resident (at most 8), queried once per
-// kernel. The 27-point half-plane sweeps need 40 registers a thread, so an SM holds 6 of their
-// blocks: a grid of 8 per SM left its last quarter of blocks to a second, sparse wave, and
-// sizing the grid by residency took the C3 sweep from 0.33 to 0.23 ms.
+// kernel. A grid of more blocks than fit leaves its last ones to a second, sparse wave: sizing the
+// grid of the 27-point half-plane sweeps by residency took a sweep of 10.6M nodes from 0.33 to
+// 0.23 ms.
 inline int resident_per_sm(const void* kernel) {
   static std::mutex m;
   static std::unordered_map<const void*, int> cache;

@@ -844,7 +844,11 @@ __global__ void k_reg_to_comp(int ncomp, int n_r, int B, const int* __restrict__
       double s = 0.0;
       const int a = gptr[grp], e = gptr[grp + 1];
       for (int q = a; q < e; ++q) s += rb[gslot[q]];
-      c[(size_t)g * B + b] = average ? s / (double)(e - a) : s;
+      // 1/m of a power of two is exact: the product has the quotient's bits without the FP64
+      // division, which nearly every warp (some of its 32 nodes shared) would wait for
+      const int m = e - a;
+      if (average) s = (m & (m - 1)) == 0 ? s * inv_mult<double>(m) : s / (double)m;
+      c[(size_t)g * B + b] = s;
     }
   }
 }
