@@ -454,7 +454,7 @@ struct Exec {
     const int gb = persistent_grid(c(), G.ntiles);
     VT* u = cur[l];
 #define RMG_GS(K)                                                                             \
-  launch_next(k_gs_colour<K, CT, VT>, dim3(gb), kTile, 0, st, G, coef(l), V(l).r.get(), dinv(l),               \
+  launch_after(short_kernels(L), k_gs_colour<K, CT, VT>, dim3(gb), kTile, 0, st, G, coef(l), V(l).r.get(), dinv(l),               \
                                                V(l).d.get(), u, colour, omega)
     switch (L.kind) {
       case 5: RMG_GS(5); break;
@@ -475,7 +475,7 @@ struct Exec {
       const int ncol = (L.kind == 5 || L.kind == 7) ? 2 : (L.dim == 3 ? 8 : 4);
       for (int s = 0; s < nu; ++s) {
         if (s == 0 && from_zero) {
-          launch_next(k_gs_zero<VT>, dim3(elementwise_grid(n)), 256, 0, st, n, V(l).b.get(), V(l).r.get(),
+          launch_after(short_kernels(L), k_gs_zero<VT>, dim3(elementwise_grid(n)), 256, 0, st, n, V(l).b.get(), V(l).r.get(),
                                                              V(l).d.get(), cur[l]);
           RMG_LAUNCHED();
           ++launches;
@@ -490,7 +490,7 @@ struct Exec {
     if (h.o.smoother == RMG_SMOOTHER_JACOBI) {
       for (int s = 0; s < nu; ++s) {
         if (s == 0 && from_zero) {
-          launch_next(k_jacobi_zero<VT>, dim3(elementwise_grid(n)), 256, 0, st, n, V(l).b.get(), dinv(l), omega,
+          launch_after(short_kernels(L), k_jacobi_zero<VT>, dim3(elementwise_grid(n)), 256, 0, st, n, V(l).b.get(), dinv(l), omega,
                                                                  oth[l]);
           RMG_LAUNCHED();
           ++launches;
@@ -503,7 +503,7 @@ struct Exec {
     } else {
       for (int a = 0; a < nu; ++a) {
         if (a == 0 && from_zero) {
-          launch_next(k_cheb0_zero<VT>, dim3(elementwise_grid(n)), 256, 0, st, n, V(l).b.get(), dinv(l),
+          launch_after(short_kernels(L), k_cheb0_zero<VT>, dim3(elementwise_grid(n)), 256, 0, st, n, V(l).b.get(), dinv(l),
                                                                 c2(l, 0), V(l).d.get(), oth[l]);
           RMG_LAUNCHED();
           ++launches;
@@ -530,11 +530,11 @@ struct Exec {
     const Level& C = *h.lv[l + 1];
     const Grid Gc = C.grid();
     if (F.dim == 3)
-      launch_next(k_restrict3<VT>, dim3(persistent_grid(c(), Gc.ntiles * (kTile / 32), 12)),
+      launch_after(short_kernels(F), k_restrict3<VT>, dim3(persistent_grid(c(), Gc.ntiles * (kTile / 32), 12)),
                   32 * kRestrictWarps, 0, st, Gc, F.regions.get(), r, C.mask.get(), C.mult.get(),
                   b, y);
     else
-      launch_next(k_restrict2<VT>, dim3(persistent_grid(c(), Gc.ntiles)), kTile, 0, st, Gc,
+      launch_after(short_kernels(F), k_restrict2<VT>, dim3(persistent_grid(c(), Gc.ntiles)), kTile, 0, st, Gc,
                   F.regions.get(), r, C.mask.get(), C.mult.get(), b, y);
     RMG_LAUNCHED();
     ++launches;
@@ -551,7 +551,7 @@ struct Exec {
         const Grid Gc = C.grid();
         const int gb = persistent_grid(c(), Gc.ntiles);
         auto run = [&](auto kernel) {
-          launch_next(kernel, dim3(gb), kTile, 0, st, Gc, F.regions.get(), F.n_r, pw(l), r,
+          launch_after(short_kernels(F), kernel, dim3(gb), kTile, 0, st, Gc, F.regions.get(), F.n_r, pw(l), r,
                       C.mask.get(), C.mult.get(), b, y);
         };
         if (F.dim == 3) run(k_restrict_w<3, VT>);
@@ -578,7 +578,7 @@ struct Exec {
         const Grid Gf = F.grid();
         const int gb = persistent_grid(c(), Gf.ntiles);
         auto run = [&](auto kernel) {
-          launch_next(kernel, dim3(gb), kTile, 0, st, Gf, C.regions.get(), pw(l), F.mask.get(),
+          launch_after(short_kernels(F), kernel, dim3(gb), kTile, 0, st, Gf, C.regions.get(), pw(l), F.mask.get(),
                       ubar, u);
         };
         if (F.dim == 3) run(k_prolong_w<3, VT>);
@@ -587,7 +587,7 @@ struct Exec {
         const Grid G1 = h.rap_x[l].grid(F.nreg);
         const int gb = persistent_grid(c(), G1.ntiles);
         auto run = [&](auto kernel) {
-          launch_next(kernel, dim3(gb), kTile, 0, st, G1, F.regions.get(), C.regions.get(),
+          launch_after(short_kernels(F), kernel, dim3(gb), kTile, 0, st, G1, F.regions.get(), C.regions.get(),
                       F.mask.get(), ubar, u);
         };
         if (F.dim == 3) run(k_prolong<3, VT>);
@@ -656,7 +656,8 @@ struct Exec {
     A.cscale = h.cscale.get();
     A.xc = h.xc.get();
     A.cres = h.cres.get();
-    tail_launch<VT, CT>(h.lv[0]->dim, h.lv[0]->B, h.tail_blocks, A, st);
+    tail_launch<VT, CT>(h.lv[0]->dim, h.lv[0]->B, h.tail_blocks, short_kernels(*h.lv[l0 - 1]), A,
+                        st);
     ++launches;
   }
 
@@ -702,7 +703,7 @@ struct Exec {
     if (!L.ngroups) return;
     launch_groups(c(), L, (const VT*)cur[0], EpiMean<VT>{V(0).y.get()}, st);
     ++launches;
-    launch_next(k_copy_slots<VT>, dim3(persistent_grid(c(), (L.nslots + 255) / 256)), 256, 0, st, 
+    launch_after(short_kernels(L), k_copy_slots<VT>, dim3(persistent_grid(c(), (L.nslots + 255) / 256)), 256, 0, st, 
         L.nslots, L.gslot.get(), V(0).y.get(), cur[0]);
     RMG_LAUNCHED();
     ++launches;
@@ -1940,17 +1941,17 @@ void pcg_solve(Hier& h, const double* b, double* xout, double rtol, int maxit, d
   while (!converged && it < maxit) {
     // (re)start: z = M^-1 r, p = z
     if (mixed) {
-      launch_next(k_to_f32_scaled, dim3(eg), 256, 0, st, n, rvec, rscale, r32);
+      launch_after(short_kernels(L0), k_to_f32_scaled, dim3(eg), 256, 0, st, n, rvec, rscale, r32);
       RMG_LAUNCHED();
     }
     vcycle(h);
     ++ncyc;
     if (mixed) {
-      launch_next(k_start_dir, dim3(dg), 256, 0, st, n, L0.n_r, rvec, z32, L0.mult.get(), zscale, h.p.get(),
+      launch_after(short_kernels(L0), k_start_dir, dim3(dg), 256, 0, st, n, L0.n_r, rvec, z32, L0.mult.get(), zscale, h.p.get(),
                                       h.zold32.get(), arrive, sc);
       RMG_LAUNCHED();
     } else {
-      launch_next(k_cg_dot, dim3(dg), 256, 0, st, n, L0.n_r, rvec, zvec, L0.mult.get(), arrive, sc, CG_RZ);
+      launch_after(short_kernels(L0), k_cg_dot, dim3(dg), 256, 0, st, n, L0.n_r, rvec, zvec, L0.mult.get(), arrive, sc, CG_RZ);
       RMG_LAUNCHED();
       k_copy<double><<<eg, 256, 0, st>>>(n, zvec, h.p.get());
       RMG_LAUNCHED();
@@ -1963,14 +1964,14 @@ void pcg_solve(Hier& h, const double* b, double* xout, double rtol, int maxit, d
       ++it;
       launch_stencil(c, L0, L0.coef.get(), h.p.get(), h.v64[0].y.get(),
                      EpiStore<double>{h.q.get()}, st, nullptr);
-      launch_next(k_cg_dot, dim3(dg), 256, 0, st, n, L0.n_r, h.p.get(), h.q.get(), L0.mult.get(), arrive, sc,
+      launch_after(short_kernels(L0), k_cg_dot, dim3(dg), 256, 0, st, n, L0.n_r, h.p.get(), h.q.get(), L0.mult.get(), arrive, sc,
                                    CG_ALPHA);
       RMG_LAUNCHED();
       if (mixed)
-        launch_next(k_cg_update_mixed, dim3(dg), 256, 0, st, n, L0.n_r, h.p.get(), h.q.get(), L0.mult.get(), sc,
+        launch_after(short_kernels(L0), k_cg_update_mixed, dim3(dg), 256, 0, st, n, L0.n_r, h.p.get(), h.q.get(), L0.mult.get(), sc,
                                               rscale, h.x.get(), rvec, r32, arrive, host_rr);
       else
-        launch_next(k_cg_update, dim3(dg), 256, 0, st, n, L0.n_r, h.p.get(), h.q.get(), L0.mult.get(), sc,
+        launch_after(short_kernels(L0), k_cg_update, dim3(dg), 256, 0, st, n, L0.n_r, h.p.get(), h.q.get(), L0.mult.get(), sc,
                                         h.x.get(), rvec, arrive, host_rr);
       RMG_LAUNCHED();
       RMG_CUDA(cudaStreamSynchronize(st));
@@ -1997,19 +1998,19 @@ void pcg_solve(Hier& h, const double* b, double* xout, double rtol, int maxit, d
       vcycle(h);
       ++ncyc;
       if (mixed) {
-        launch_next(k_flex_dots, dim3(dg), 256, 0, st, n, L0.n_r, rvec, z32, h.zold32.get(), L0.mult.get(),
+        launch_after(short_kernels(L0), k_flex_dots, dim3(dg), 256, 0, st, n, L0.n_r, rvec, z32, h.zold32.get(), L0.mult.get(),
                                         zscale, arrive, sc);
         RMG_LAUNCHED();
-        launch_next(k_p_update<float>, dim3(eg), 256, 0, st, n, z32, zscale, sc, h.p.get());
+        launch_after(short_kernels(L0), k_p_update<float>, dim3(eg), 256, 0, st, n, z32, zscale, sc, h.p.get());
         RMG_LAUNCHED();
       } else {
         if (flex64)
-          launch_next(k_cg_flex64, dim3(dg), 256, 0, st, n, L0.n_r, rvec, zvec, h.zold.get(), L0.mult.get(),
+          launch_after(short_kernels(L0), k_cg_flex64, dim3(dg), 256, 0, st, n, L0.n_r, rvec, zvec, h.zold.get(), L0.mult.get(),
                                           arrive, sc);
         else
-          launch_next(k_cg_dot, dim3(dg), 256, 0, st, n, L0.n_r, rvec, zvec, L0.mult.get(), arrive, sc, CG_BETA);
+          launch_after(short_kernels(L0), k_cg_dot, dim3(dg), 256, 0, st, n, L0.n_r, rvec, zvec, L0.mult.get(), arrive, sc, CG_BETA);
         RMG_LAUNCHED();
-        launch_next(k_p_update<double>, dim3(eg), 256, 0, st, n, zvec, 1.0, sc, h.p.get());
+        launch_after(short_kernels(L0), k_p_update<double>, dim3(eg), 256, 0, st, n, zvec, 1.0, sc, h.p.get());
         RMG_LAUNCHED();
       }
     }

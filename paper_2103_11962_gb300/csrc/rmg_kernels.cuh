@@ -17,7 +17,7 @@
 
 namespace rmg {
 
-// Start of a kernel that is launched with launch_next(): the next kernel may be set up now (its
+// Start of a kernel that is launched with launch_after(): the next kernel may be set up now (its
 // blocks wait in turn), and nothing is touched before the previous one has finished.
 __device__ __forceinline__ void follow() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");

@@ -57,10 +57,18 @@ inline int resident_per_sm_smem(const void* kernel, int smem) {
   return b;
 }
 
-// kernel<<<grid, block, smem, st>>>(args...) for a kernel that starts with follow(): where the work
-// before it on the stream is a kernel too, it is set up while that one finishes (programmatic
-// dependent launch), which takes about 1 us off each of the short kernels of a small problem.
-// launch_after with next = false is the plain launch (beside an event record).
+// Whether the kernels of a level are short enough to be launched with `next` below. Next to long
+// ones the waiting blocks are in the way: with it on every level, steps of 34M unknowns (27-point)
+// and of 6.3M (elasticity) took 125.2 and 71.4 ms against 120.5 and 68.9 without, a step of 5.8M
+// (7-point, 42M coefficients on level 0) the same, and small solves gained 10%.
+inline bool short_kernels(const Level& L) {
+  return (long long)L.n_r * L.kind * L.B * L.B <= 40000000;
+}
+
+// kernel<<<grid, block, smem, st>>>(args...) for a kernel that starts with follow(). With `next`,
+// where the work before it on the stream is a kernel too, it is set up while that one finishes
+// (programmatic dependent launch), which takes about 1 us off each of the short kernels of a small
+// problem; not beside an event record.
 template <typename... P, typename... A>
 void launch_after(bool next, void (*kernel)(P...), dim3 grid, int block, int smem,
                   cudaStream_t st, A&&... args) {
@@ -76,12 +84,6 @@ void launch_after(bool next, void (*kernel)(P...), dim3 grid, int block, int sme
   cfg.numAttrs = next ? 1 : 0;
   RMG_CUDA(cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...));
 }
-template <typename... P, typename... A>
-void launch_next(void (*kernel)(P...), dim3 grid, int block, int smem, cudaStream_t st,
-                 A&&... args) {
-  launch_after(true, kernel, grid, block, smem, st, std::forward<A>(args)...);
-}
-
 // launch_after with one resident wave of blocks over `work` tiles.
 template <typename... P, typename... A>
 void launch_resident(const Ctx& c, bool next, void (*kernel)(P...), int work, cudaStream_t st,
@@ -96,7 +98,7 @@ void launch_groups(Ctx& c, const Level& L, const AT* y, Epi epi, cudaStream_t st
                    bool next = true) {
   if (!L.ngroups) return;
   const int gs = persistent_grid(c, (L.nslots + 255) / 256);
-  launch_after(next, k_groups<AT, Epi>, dim3(gs), 256, 0, st, L.nslots, L.slots.get(), L.gslot.get(), y,
+  launch_after(next && short_kernels(L), k_groups<AT, Epi>, dim3(gs), 256, 0, st, L.nslots, L.slots.get(), L.gslot.get(), y,
               epi);
   RMG_LAUNCHED();
 }
@@ -137,6 +139,7 @@ void launch_stencil(Ctx& c, const Level& L, const CT* coef, const VT* u, AT* y, 
   if (G.lx == -3 && ((reinterpret_cast<uintptr_t>(u) | reinterpret_cast<uintptr_t>(half)) & 15))
     G = L.grid();
   const int gb = persistent_grid(c, G.ntiles);
+  const bool next = !ev0 && short_kernels(L);
   // external record nodes when capturing, so the events can be timed after a graph replay
   if (ev0) RMG_CUDA(cudaEventRecordWithFlags(ev0, st, g_capturing ? cudaEventRecordExternal : 0));
   bool done = false;
@@ -148,24 +151,24 @@ void launch_stencil(Ctx& c, const Level& L, const CT* coef, const VT* u, AT* y, 
       const int smem = kStSmemFloats * (int)sizeof(float);
       const auto kern = k_stencil_half27_staged<Epi>;
       const int g = persistent_grid(c, G.ntiles, resident_per_sm_smem((const void*)kern, smem));
-      launch_after(!ev0, kern, dim3(g), kStX * kStY, smem, st, G, coef, half, asym, u, L.mult.get(), y, epi);
+      launch_after(next, kern, dim3(g), kStX * kStY, smem, st, G, coef, half, asym, u, L.mult.get(), y, epi);
       done = true;
     } else if (half && L.B == 1) {
       RMG_REQUIRE(asym != nullptr, RMG_ERR_STATE, "half planes without their flag");
-      if (L.n_r <= kOffset32Nodes) launch_half<true>(c, L, G, coef, half, asym, u, y, epi, st, !ev0);
-      else launch_half<false>(c, L, G, coef, half, asym, u, y, epi, st, !ev0);
+      if (L.n_r <= kOffset32Nodes) launch_half<true>(c, L, G, coef, half, asym, u, y, epi, st, next);
+      else launch_half<false>(c, L, G, coef, half, asym, u, y, epi, st, next);
       done = true;
     } else if (half) {
       RMG_REQUIRE(asym != nullptr && L.B == 3 && (L.kind == 27 || L.kind == 9), RMG_ERR_STATE,
                   "half planes of a block operator need 3 dofs and a 27- or 9-point stencil");
-      if (L.n_r <= kOffset32Nodes) launch_half<true>(c, L, G, coef, half, asym, u, y, epi, st, !ev0);
-      else launch_half<false>(c, L, G, coef, half, asym, u, y, epi, st, !ev0);
+      if (L.n_r <= kOffset32Nodes) launch_half<true>(c, L, G, coef, half, asym, u, y, epi, st, next);
+      else launch_half<false>(c, L, G, coef, half, asym, u, y, epi, st, next);
       done = true;
     }
   }
   RMG_REQUIRE(done || G.lx != -3, RMG_ERR_STATE, "staged tiles outside a half-plane sweep");
   auto run = [&](auto kernel) {
-    launch_after(!ev0, kernel, dim3(gb), kTile, 0, st, G, coef, u, L.mult.get(), y, epi);
+    launch_after(next, kernel, dim3(gb), kTile, 0, st, G, coef, u, L.mult.get(), y, epi);
   };
   if (done) {
   } else if (L.B == 1) {
@@ -191,7 +194,7 @@ void launch_stencil(Ctx& c, const Level& L, const CT* coef, const VT* u, AT* y, 
       launch_groups(c, L, y, epi, st, !ev1);
     } else {
       const int gg = persistent_grid(c, (L.nslots + 255) / 256);
-      launch_after(!ev1, k_groups_b<AT, Epi>, dim3(gg), 256, 0, st, L.nslots, L.B, L.n_r, L.slots.get(),
+      launch_after(!ev1 && short_kernels(L), k_groups_b<AT, Epi>, dim3(gg), 256, 0, st, L.nslots, L.B, L.n_r, L.slots.get(),
                   L.gslot.get(), (const AT*)y, epi);
       RMG_LAUNCHED();
     }

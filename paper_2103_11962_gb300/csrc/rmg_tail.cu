@@ -575,12 +575,13 @@ int tail_cluster(int dim, int B) {
 }
 
 template <typename VT, typename CT>
-void tail_launch(int dim, int B, int cluster, const TailArgs<VT, CT>& args, cudaStream_t st) {
+void tail_launch(int dim, int B, int cluster, bool next, const TailArgs<VT, CT>& args,
+                 cudaStream_t st) {
   cudaLaunchAttribute attr[2];
   cudaLaunchConfig_t cfg = tail_config(cluster, attr, st);
-  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;   // as launch_next
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;   // as launch_after
   attr[1].val.programmaticStreamSerializationAllowed = 1;
-  cfg.numAttrs = 2;
+  cfg.numAttrs = next ? 2 : 1;
   void* p[] = {const_cast<TailArgs<VT, CT>*>(&args)};
   RMG_CUDA(cudaLaunchKernelExC(&cfg, tail_kernel<VT, CT>(dim, B), p));
   RMG_LAUNCHED();
@@ -588,7 +589,7 @@ void tail_launch(int dim, int B, int cluster, const TailArgs<VT, CT>& args, cuda
 
 #define RMG_TAIL(VT, CT)                          \
   template int tail_cluster<VT, CT>(int, int);    \
-  template void tail_launch<VT, CT>(int, int, int, const TailArgs<VT, CT>&, cudaStream_t)
+  template void tail_launch<VT, CT>(int, int, int, bool, const TailArgs<VT, CT>&, cudaStream_t)
 RMG_TAIL(double, double);
 RMG_TAIL(float, float);
 RMG_TAIL(float, __nv_bfloat16);

@@ -66,6 +66,7 @@ struct TailGeometry {
 template <typename VT, typename CT>
 int tail_cluster(int dim, int B);
 template <typename VT, typename CT>
-void tail_launch(int dim, int B, int cluster, const TailArgs<VT, CT>& args, cudaStream_t st);
+void tail_launch(int dim, int B, int cluster, bool next, const TailArgs<VT, CT>& args,
+                 cudaStream_t st);     // next: as launch_after
 
 }  // namespace rmg
