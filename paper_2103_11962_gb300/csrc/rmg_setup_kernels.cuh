@@ -598,9 +598,11 @@ __global__ void k_coarse_maps(int ncomp, const int* __restrict__ freeflag, const
 // Abar = Psibar [[Abar]] Psibar^T restricted to unmasked nodes (eq. CoarseCompositeOperator):
 // row of composite node g = sum over its regional copies of their region rows. With B dofs per
 // node the dense matrix has dimension B * nc, dof cidx * B + b (blockIdx.y = row component).
-// A warp per row and a lane per stencil slot: the entries of one copy go to different columns, and
-// the copies are added one after the other, so every sum keeps its order. (With a thread per row
-// its up to 216 entries were one chain of loads: 83 us for a few dozen rows.)
+// A warp per row and a lane per stencil slot, the copies added one after the other. The entries of
+// one copy go to different columns unless its region holds a composite node twice (a region that
+// closes on itself); those of equal columns are then added lane by lane, so every sum keeps its
+// order. (With a thread per row its up to 216 entries were one chain of loads: 83 us for a few
+// dozen rows.)
 template <int KIND>
 __global__ void k_coarse_assemble(int ncomp, int B, const RegionDev* __restrict__ regs, int nreg,
                                   int n_r, const double* __restrict__ coef,
@@ -625,17 +627,27 @@ __global__ void k_coarse_assemble(int ncomp, int B, const RegionDev* __restrict_
       const RegionDev R = regs[region_of(regs, nreg, n)];
       int i, j, l;
       decode(n - R.off, R, i, j, l);
+      int col = -1;
       if (lane < S::S) {
         const int x = i + S::dx(lane), y = j + S::dy(lane), z = l + S::dz(lane);
-        if (x >= 0 && x < R.nx && y >= 0 && y < R.ny && z >= 0 && z < R.nz) {
-          const int col = cidx[gid[R.off + x + R.nx * (y + R.ny * z)]];
-          if (col >= 0)
-            for (int b2 = 0; b2 < B; ++b2)
-              M[row * nd + (size_t)col * B + b2] +=
-                  coef[((size_t)(b * B + b2) * S::S + lane) * n_r + n];
+        if (x >= 0 && x < R.nx && y >= 0 && y < R.ny && z >= 0 && z < R.nz)
+          col = cidx[gid[R.off + x + R.nx * (y + R.ny * z)]];
+      }
+      auto add = [&] {
+        for (int b2 = 0; b2 < B; ++b2)
+          M[row * nd + (size_t)col * B + b2] +=
+              coef[((size_t)(b * B + b2) * S::S + lane) * n_r + n];
+      };
+      const unsigned same = __match_any_sync(0xffffffffu, col);
+      if (!__any_sync(0xffffffffu, col >= 0 && (same & (same - 1)))) {
+        if (col >= 0) add();
+        __syncwarp();
+      } else {
+        for (int s = 0; s < S::S; ++s) {
+          if (lane == s && col >= 0) add();
+          __syncwarp();
         }
       }
-      __syncwarp();
     }
   }
 }
