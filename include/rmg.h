@@ -282,7 +282,8 @@ rmg_status rmg_mlp_gradient(rmg_mlp* mlp, int n, const float* feats, const float
 rmg_status rmg_mlp_train(rmg_mlp* mlp, int n, const float* feats, const float* labels,
                          const float* mask, int steps, int batch, float lr,
                          unsigned long long seed, float* loss_history);
-/* Features of every regional node of a hierarchy level (device float[n_r][32]). */
+/* Features of every regional node of a hierarchy level (device float[n_r][32]). This call and the
+ * next use the PCG work vectors of the hierarchy. */
 rmg_status rmg_hier_mlp_features(rmg_hier* hier, int level, float* feats);
 /* Network inference on a level: per-axis weights (device float[3 * n_r]) for
  * rmg_hier_set_transfer_weights (zero along axes where a node sits on a coarse index). */

@@ -700,13 +700,21 @@ void mlp_backward(rmg_mlp* net, int n, const float* feats, const float* labels, 
   RMG_LAUNCHED();
 }
 
-// The couplings of the level's shared nodes go to four of its FP64 cycle vectors, which hold
-// nothing between calls.
+// Room for the couplings of the level's shared nodes in the PCG work vectors: calls that use those
+// synchronise before they return, so that nothing of theirs is in flight on any stream (a cycle's
+// own vectors may be: rmg_vcycle_apply returns once queued). Every level has a place of its own,
+// so that features of different levels may be formed on different streams. The finest level takes
+// four whole vectors; DIM + 1 arrays of each of the others fit one (3D: level l + 1 has at most an
+// eighth of the nodes of level l, and 4 (1/8 + 1/64 + ..) < 1; 2D: 3 (1/4 + 1/16 + ..) < 1).
 template <int KIND>
 FeatArgs feat_args(const Hier& h, int level) {
   const Level& L = *h.lv[level];
-  const LevelVecs<double>& V = h.v64[level];
-  FeatArgs A{L.coef.get(), L.mult.get(), {V.u2.get(), V.r.get(), V.y.get(), V.d.get()}};
+  FeatArgs A{L.coef.get(), L.mult.get(), {h.x.get(), h.p.get(), h.q.get(), h.tmp.get()}};
+  if (level > 0) {
+    double* at = h.zold.get();
+    for (int l = 1; l < level; ++l) at += (size_t)(L.dim + 1) * h.lv[l]->n_r;
+    for (int p = 0; p < 4; ++p) A.comp[p] = at + (size_t)std::min(p, L.dim) * L.n_r;
+  }
   if (L.nslots) {
     k_shared_couplings<KIND><<<persistent_grid(*h.c, (L.nslots + 255) / 256), 256, 0,
                                h.c->stream>>>(L.nslots, L.n_r, L.sgrp.get(), L.gptr.get(),

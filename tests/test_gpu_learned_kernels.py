@@ -72,3 +72,42 @@ def test_gradient_tiles_and_remainders(ctx, n):
     tol = 64 * 2.0 ** -24
     assert abs(loss - loss1 * scale) <= tol * loss1 * scale
     assert np.abs(g - g1 * scale).max() <= tol * np.abs(g1).max() * scale
+
+
+@pytest.mark.parametrize("problem", ["9-point", "7-point"])
+def test_features_beside_a_cycle_on_another_stream(ctx, problem):
+    """Features and weights only read what a cycle reads: formed on another stream while FP64
+    cycles are queued, they change neither the cycles' results nor their own."""
+    from paper_2103_11962_gb300 import learned, rmg, upload
+    p = PROBLEMS[problem]()
+    dp = upload(p)
+    own = rmg.Context(0)
+    lay = rmg.Layout(own, p.dim, p.region_dims, dp.gids, p.n_nodes, dp.dirichlet)
+    lay.operator_from_csr(p.stencil, dp.rowptr, dp.col, dp.val)
+    h = rmg.Hierarchy(lay, rmg.default_options(levels=3, smoother=rmg.CHEBYSHEV, nu1=1, nu2=1,
+                                               precision=rmg.FP64))
+    net = rmg.MLP(own, learned.init_params(5))
+    n = [h.level_sizes(l)[0] for l in range(3)]
+    want_z = torch.empty_like(dp.b)
+    h.vcycle(dp.b, want_z)
+    want = []
+    for l in range(3):
+        want.append((torch.empty(n[l], 32, device="cuda"), torch.empty(3 * n[l], device="cuda")))
+        h.mlp_features(l, want[l][0])
+        h.mlp_weights(l, net, want[l][1])
+    a, b = torch.cuda.Stream(), torch.cuda.Stream()
+    z = [torch.empty_like(dp.b) for _ in range(8)]
+    got = [[torch.empty_like(t) for t in w] for w in want]
+    torch.cuda.synchronize()
+    for k in range(8):
+        own.set_stream(a.cuda_stream)
+        h.vcycle(dp.b, z[k])
+        own.set_stream(b.cuda_stream)
+        for l in range(3):
+            h.mlp_features(l, got[l][0])
+            h.mlp_weights(l, net, got[l][1])
+    torch.cuda.synchronize()
+    for k in range(8):
+        assert torch.equal(z[k], want_z)
+    for w, g in zip(want, got):
+        assert torch.equal(w[0], g[0]) and torch.equal(w[1], g[1])
