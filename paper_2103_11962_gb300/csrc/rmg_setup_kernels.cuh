@@ -103,12 +103,16 @@ struct Lines {
   }
 };
 
-// out[o + 1] += 9 sum_a w(a) sum_d load(a, d) P(a + d - 3 o): one axis of R A P for one coarse node.
-// `a` is the fine node's offset from the coarse one, `d` the entry's (only 0 when !WIDE). The
-// weights times 3 are 1, 2 and 3, exact in any precision; the 9 of every axis comes off in
-// rap_store. Each fine row is summed against P first: where P is (nearly) in the kernel of A
-// these three terms cancel before anything larger is added. (In one sum with weights rounded to
-// FP32 the row sums, which cancel, lost ten times more over three levels.)
+// Factor 9 of every axis in the weights below, over the power of two that keeps the intermediate
+// operators in the range of the result (without it an FP32 product overflowed 729 times earlier).
+constexpr int rap_weight(int t) { return 3 - (t < 0 ? -t : t); }
+
+// out[o + 1] += 9/8 sum_a w(a) sum_d load(a, d) P(a + d - 3 o): one axis of R A P for one coarse
+// node. `a` is the fine node's offset from the coarse one, `d` the entry's (only 0 when !WIDE). The
+// weights times 3 are 1, 2 and 3, here over 4 (P) and 2 (w), exact in any precision; the 9/8 of
+// every axis comes off in rap_store. Each fine row is summed against P first: where P is (nearly)
+// in the kernel of A these three terms cancel before anything larger is added. (In one sum with
+// weights rounded to FP32 the row sums, which cancel, lost ten times more over three levels.)
 template <bool WIDE, typename T, class Load>
 __device__ __forceinline__ void rap_axis(Load load, T (&out)[3]) {
 #pragma unroll
@@ -119,7 +123,7 @@ __device__ __forceinline__ void rap_axis(Load load, T (&out)[3]) {
       for (int o = -1; o <= 1; ++o) {
         const int t = a - 3 * o;
         if (t < -2 || t > 2) continue;
-        out[o + 1] = fma(v, T((3 - (a < 0 ? -a : a)) * (3 - (t < 0 ? -t : t))), out[o + 1]);
+        out[o + 1] = fma(v, T(rap_weight(a) * rap_weight(t)) * T(0.125), out[o + 1]);
       }
       continue;
     }
@@ -131,13 +135,13 @@ __device__ __forceinline__ void rap_axis(Load load, T (&out)[3]) {
       for (int o = -1; o <= 1; ++o) {
         const int t = a + d - 3 * o;
         if (t < -2 || t > 2) continue;
-        row[o + 1] = fma(v, T(3 - (t < 0 ? -t : t)), row[o + 1]);
+        row[o + 1] = fma(v, T(rap_weight(t)) * T(0.25), row[o + 1]);
       }
     }
 #pragma unroll
     for (int o = -1; o <= 1; ++o)
       if (a - 3 * o >= -3 && a - 3 * o <= 3)
-        out[o + 1] = fma(row[o + 1], T(3 - (a < 0 ? -a : a)), out[o + 1]);
+        out[o + 1] = fma(row[o + 1], T(rap_weight(a)) * T(0.5), out[o + 1]);
   }
 }
 
@@ -204,7 +208,7 @@ __device__ __forceinline__ void rap_store(const T (&out)[3], const Grid& Gc, con
       if (px == 0 && py == 0 && pz == 0) v = T(mdiag) / T(cmult[n]);
     } else if (x >= 0 && x < R.nx && y >= 0 && y < R.ny && z >= 0 && z < R.nz &&
                !cmask[R.off + x + R.nx * (y + R.ny * z)]) {
-      v = out[o] * T(dim == 3 ? 1.0 / 729.0 : 1.0 / 81.0);
+      v = out[o] * T(dim == 3 ? 512.0 / 729.0 : 64.0 / 81.0);
     }
     ccoef[(size_t)slot * Gc.n_r + n] = v;
   }
