@@ -44,16 +44,23 @@ SUBRECORDS = ("c1_poisson2d", "c2_diffusion3d", "c4_highcontrast3d", "c5_elastic
 
 
 # Per-node algorithmic bytes and FP64 flops of the timed kernel, the fine-level Chebyshev
-# recurrence sweep (k_stencil_half, k_stencil or k_bstencil with EpiCheb): its coefficient
+# recurrence sweep (k_stencil, k_bstencil or their half forms with EpiCheb): its coefficient
 # streams, u, b, D~^-1, d read; d and u_out written; 1-byte multiplicity read.
 def sweep_bytes(prec, planes, B=1):
     """Algorithmic bytes per regional node of the Chebyshev recurrence sweep: the stencil
-    coefficients the sweep reads per node (`planes`: B*B*S, or (S+1)/2 for the half form of a
-    symmetric FP32 stencil, as rmg_hier_coef_planes reports), u, b, D~^-1 and d read and d,
+    coefficients the sweep reads per node (`planes`, see sweep_planes), u, b, D~^-1 and d read and d,
     u_out written for each of the B components, and the 1-byte multiplicity."""
     cb = {"fp64": 8, "fp32": 4, "bf16": 2}[prec]
     vb = 8 if prec == "fp64" else 4
     return planes * cb + B * 6 * vb + 1
+
+
+def sweep_planes(stencil, B, half_nodes, nodes):
+    """Coefficients the sweep reads per regional node, in the mean: B*B*(S+1)/2 in the regions on
+    the half form of a symmetric FP32 stencil (`half_nodes` nodes, as rmg_hier_half_regions
+    reports), B*B*S in the others."""
+    full, half = B * B * stencil, B * B * ((stencil + 1) // 2)
+    return full if not half_nodes else full - (full - half) * half_nodes / nodes
 
 
 def sweep_flops(stencil, B=1):
@@ -561,15 +568,15 @@ class Workload:
         pk = peaks()
         n_r0 = p.n_regional_nodes
         Bd = p.dofs_per_node
-        planes0 = h.coef_planes(0)
-        bytes_launch = sweep_bytes(prec, planes0, Bd) * n_r0
+        half_nodes = h.half_regions(0)[1]
+        planes0 = sweep_planes(p.stencil, Bd, half_nodes, n_r0)
+        bytes_launch = round(sweep_bytes(prec, planes0, Bd) * n_r0)
         flops_launch = sweep_flops(p.stencil, Bd) * n_r0
         gbs = bytes_launch / (kern_ms / 1e3) / 1e9
         tfl = flops_launch / (kern_ms / 1e3) / 1e12
         hbm_frac = gbs / pk["hbm_gbs"]
-        kname = (f"k_bstencil<{p.stencil},{Bd}>" if Bd > 1 else
-                 f"k_stencil_half<{p.stencil}>" if planes0 < p.stencil else
-                 f"k_stencil<{p.stencil}>")
+        kname = ("k_bstencil" if Bd > 1 else "k_stencil") + ("_half" if half_nodes else "") + \
+            (f"<{p.stencil},{Bd}>" if Bd > 1 else f"<{p.stencil}>")
         epi = "EpiJacobi" if self.cfg["smoother"] == "jacobi" else "EpiCheb"
         r = dict(bound="hbm", achieved=round(gbs, 1), peak=pk["hbm_gbs"], unit="GB/s",
                  frac=round(hbm_frac, 4), peak_src=pk["src"] + " (MEASURED_PEAKS.json hbm_gbs)",
@@ -581,10 +588,11 @@ class Workload:
                      hbm=dict(achieved=round(gbs, 1), peak=pk["hbm_gbs"], unit="GB/s",
                               frac=round(hbm_frac, 4)))
         tpn, cap = profiled_traffic(f"{kname} {epi}", prec)
-        r.update(kernel=f"{kname[:-1]}, {epi}> level 0 ({prec}, {planes0} coefficients per node)",
+        r.update(kernel=f"{kname[:-1]}, {epi}> level 0 ({prec}, {planes0:.4g} coefficients per node)",
                  ms_per_launch=round(kern_ms, 4), launches_timed=probe_n,
                  bytes_per_launch=bytes_launch, flops_per_launch=flops_launch,
-                 bytes_per_node=sweep_bytes(prec, planes0, Bd), regional_nodes=n_r0,
+                 bytes_per_node=round(sweep_bytes(prec, planes0, Bd), 2), regional_nodes=n_r0,
+                 half_form_nodes=half_nodes,
                  traffic=(round(tpn * n_r0) if tpn else None),
                  traffic_src=(f"ncu dram__bytes_read.sum + dram__bytes_write.sum per node ({cap}) "
                               "x regional nodes" if tpn else None))

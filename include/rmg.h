@@ -421,17 +421,22 @@ rmg_status rmg_hier_galerkin(rmg_hier* hier, int level);
  * ints; fails with RMG_ERR_ARG for a level outside the hierarchy. */
 rmg_status rmg_hier_tile_shape(rmg_hier* hier, int level, int* tx, int* ty, int* tz);
 /* Stencil coefficients per regional node that the cycle's sweeps read on a level, as of the
- * last rmg_setup_numeric: B * B * S for an S-point stencil, or B * B * (S + 1) / 2 where the half
- * form is in use. The half form (FP32 cycle, level 0, symmetric_storage 1) rests on the symmetry
- * of the regional operator, a(n, n+e) = a(n+e, n) inside every region, for block operators
- * A_cc'(n, n+e) = A_c'c(n+e, n) (Sec. 4 splits a symmetric composite matrix into symmetric
- * region matrices): it keeps the centre and
- * the (S - 1) / 2 slots after it, and reads a coefficient of the other half at the neighbour
- * that owns its mirror. Each setup compares every mirrored pair of the FP32 coefficients bit
- * for bit; the half form is used only when all agree, so that the sweeps compute exactly the
- * rows of the full form and no result changes. Host int; RMG_ERR_ARG for a level outside the
- * hierarchy, RMG_ERR_STATE before the first numeric setup. */
+ * last rmg_setup_numeric, in the regions that read most: B * B * S for an S-point stencil, or
+ * B * B * (S + 1) / 2 where every region is on the half form. The half form (FP32 cycle, level 0,
+ * symmetric_storage 1) rests on the symmetry of the regional operator, a(n, n+e) = a(n+e, n)
+ * inside every region, for block operators A_cc'(n, n+e) = A_c'c(n+e, n) (Sec. 4 splits a
+ * symmetric composite matrix into symmetric region matrices): it keeps the centre and the
+ * (S - 1) / 2 slots after it, and reads a coefficient of the other half at the neighbour that
+ * owns its mirror. Each setup compares every mirrored pair of the FP32 coefficients bit for bit;
+ * a scalar operator takes the half form only when all agree, a block operator in the regions
+ * whose pairs all agree (rmg_hier_half_regions), so that the sweeps compute exactly the rows of
+ * the full form and no result changes. Host int; RMG_ERR_ARG for a level outside the hierarchy,
+ * RMG_ERR_STATE before the first numeric setup. */
 rmg_status rmg_hier_coef_planes(rmg_hier* hier, int level, int* planes);
+/* Regions of a level whose sweeps read the half form (see rmg_hier_coef_planes), and their
+ * regional nodes: 0 except on level 0 of an FP32 cycle. Either pointer may be NULL. Errors as
+ * rmg_hier_coef_planes. */
+rmg_status rmg_hier_half_regions(rmg_hier* hier, int level, int* regions, int64_t* nodes);
 /* Coarsest composite matrix restricted to unmasked nodes (dense, row-major, host double
  * [(B*nc)^2], dof cu * B + c) and the composite ids of those nodes (host int64[nc]). Pass NULL
  * to query nc (the number of unmasked composite nodes). */

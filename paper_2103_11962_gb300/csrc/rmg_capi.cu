@@ -433,6 +433,16 @@ rmg_status rmg_hier_coef_planes(rmg_hier* hh, int level, int* planes) {
   return RMG_OK;
 }
 
+rmg_status rmg_hier_half_regions(rmg_hier* hh, int level, int* regions, int64_t* nodes) {
+  if (!hh) return RMG_ERR_ARG;
+  Hier& h = hh->h;
+  if (level < 0 || level >= h.levels()) return fail(h.layout->ctx, RMG_ERR_ARG, "bad level");
+  if (h.kind0 == 0) return fail(h.layout->ctx, RMG_ERR_STATE, "no numeric setup yet");
+  if (regions) *regions = h.half(level) ? h.half_count : 0;
+  if (nodes) *nodes = h.half(level) ? h.half_nodes : 0;
+  return RMG_OK;
+}
+
 rmg_status rmg_hier_coarse_matrix(rmg_hier* hh, int64_t* nc, double* dense, int64_t* ids) {
   if (!hh || !nc) return RMG_ERR_ARG;
   return guarded(hh->h.layout->ctx, [&] {

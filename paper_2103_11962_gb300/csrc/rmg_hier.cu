@@ -18,7 +18,7 @@ Hier::~Hier() {
 }
 
 const int* Hier::half_flag() const {
-  return half_regions.get() ? half_regions.get() : &sc.get()->half_asym;
+  return lv[0]->B > 1 ? half_regions.get() : &sc.get()->half_asym;
 }
 
 // the mixed-precision dense coarse solve (defined with the coarse factorisation below)
@@ -1399,6 +1399,24 @@ static void level0_to_fp32(Hier& h) {
   RMG_LAUNCHED();
 }
 
+// Regions whose flags of the last level0_to_fp32 are clear (synchronises for a block operator).
+static void count_half_regions(Hier& h) {
+  const Level& L = *h.lv[0];
+  std::vector<int> asym(L.nreg, h.hsc.half_asym);
+  if (L.B > 1) {
+    RMG_CUDA(cudaMemcpyAsync(asym.data(), h.half_regions.get(), L.nreg * sizeof(int),
+                             cudaMemcpyDeviceToHost, h.c->stream));
+    RMG_CUDA(cudaStreamSynchronize(h.c->stream));
+  }
+  h.half_count = 0;
+  h.half_nodes = 0;
+  for (int r = 0; r < L.nreg; ++r)
+    if (!asym[r]) {
+      ++h.half_count;
+      h.half_nodes += L.hoff[r + 1] - L.hoff[r];
+    }
+}
+
 // The mixed cycle's remaining copies: FP32 D~^-1 on every level and, for the BF16 variant, the
 // BF16 coefficients (from the FP32 ones).
 static void make_low_precision(Hier& h) {
@@ -1571,6 +1589,7 @@ void hier_numeric(Hier& h) {
   coarse_factor(h);
   RMG_CUDA(cudaMemcpyAsync(&h.hsc, h.sc.get(), sizeof(Scalars), cudaMemcpyDeviceToHost, c.stream));
   RMG_CUDA(cudaStreamSynchronize(c.stream));
+  if (h.half_on) count_half_regions(h);
   const std::vector<char>& stored = h.stored;
   if (h.gexec && (stored != h.graph_stored || h.coarse_refine != h.graph_refine)) {
     cudaGraphExecDestroy(h.gexec);

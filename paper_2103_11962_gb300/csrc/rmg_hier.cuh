@@ -98,6 +98,8 @@ struct Hier {
   bool half_on = false;
   DBuf<float> half32;
   DBuf<int> half_regions;
+  int half_count = 0;                        // regions on the half form, and their nodes
+  long long half_nodes = 0;
   // coarse end of the cycle in one kernel (rmg_tail.cu): first level it takes (-1: none), whether
   // the dense solve is inside, the cluster's blocks, and geometry per level
   int tail0 = -1;

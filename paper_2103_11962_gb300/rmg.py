@@ -93,6 +93,8 @@ def lib():
                                                ctypes.POINTER(ctypes.c_int),
                                                ctypes.POINTER(ctypes.c_int)]),
         "rmg_hier_coef_planes": (ctypes.c_int, [P, ctypes.c_int, ctypes.POINTER(ctypes.c_int)]),
+        "rmg_hier_half_regions": (ctypes.c_int, [P, ctypes.c_int, ctypes.POINTER(ctypes.c_int),
+                                                 I64P]),
         "rmg_hier_coarse_matrix": (ctypes.c_int, [P, I64P, P, P]),
         "rmg_hier_vcycle_launches": (ctypes.c_int, [P, ctypes.POINTER(ctypes.c_int)]),
         "rmg_launch_count": (ctypes.c_ulonglong, []),
@@ -142,7 +144,8 @@ def exported_symbols():
             "rmg_hier_dofs_per_node",
             "rmg_hier_opdep_weights", "rmg_hier_constant_weights", "rmg_hier_convergence_factor",
             "rmg_hier_region_energies", "rmg_hier_blend_weights", "rmg_hier_region_colours",
-            "rmg_hier_tile_shape", "rmg_hier_coef_planes", "rmg_hier_galerkin",
+            "rmg_hier_tile_shape", "rmg_hier_coef_planes", "rmg_hier_half_regions",
+            "rmg_hier_galerkin",
             "rmg_mlp_num_params", "rmg_mlp_create",
             "rmg_mlp_destroy", "rmg_mlp_get_params", "rmg_mlp_forward", "rmg_mlp_gradient",
             "rmg_mlp_train", "rmg_hier_mlp_features", "rmg_hier_mlp_weights"]
@@ -349,10 +352,18 @@ class Hierarchy:
         return a.value, b.value, c.value
 
     def coef_planes(self, level):
-        """Stencil coefficients per node the cycle's sweeps read on a level (half form: fewer)."""
+        """Stencil coefficients per node the cycle's sweeps read on a level, in the regions that
+        read most (half form: fewer; see half_regions)."""
         v = ctypes.c_int()
         self.ctx.check(lib().rmg_hier_coef_planes(self.h, level, ctypes.byref(v)))
         return v.value
+
+    def half_regions(self, level):
+        """(regions, regional nodes) whose sweeps read the half form on a level."""
+        r, n = ctypes.c_int(), ctypes.c_int64()
+        self.ctx.check(lib().rmg_hier_half_regions(self.h, level, ctypes.byref(r),
+                                                   ctypes.byref(n)))
+        return r.value, n.value
 
     def lam(self, level):
         v = ctypes.c_double()

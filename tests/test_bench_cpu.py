@@ -24,6 +24,15 @@ def test_sweep_bytes(prec, planes, B, expect):
     assert bench.sweep_bytes(prec, planes, B) == expect
 
 
+@pytest.mark.parametrize("stencil, B, half_nodes, expect", [
+    (27, 1, 0, 27), (27, 1, 1000, 14), (7, 1, 1000, 4), (9, 3, 1000, 45),
+    (27, 3, 0, 243), (27, 3, 1000, 126),
+    (27, 3, 900, 137.7),       # a tenth of the nodes in regions on the full planes
+])
+def test_sweep_planes(stencil, B, half_nodes, expect):
+    assert bench.sweep_planes(stencil, B, half_nodes, 1000) == pytest.approx(expect)
+
+
 def test_sweep_flops():
     assert bench.sweep_flops(7) == 20
     assert bench.sweep_flops(27, 3) == 2 * 9 * 27 + 18

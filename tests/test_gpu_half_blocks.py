@@ -40,3 +40,33 @@ def test_block_half_planes(grid, choices, symmetric, tile_shape):
         lam.append(h.lam(0))
     assert lam[0] == lam[1]
     assert torch.equal(z[0], z[1])
+
+
+def test_half_regions_are_counted_one_by_one():
+    """One region with a coupling of its own: the others stay on the half form, and are counted."""
+    import numpy as np
+    from paper_2103_11962_gb300 import rmg, upload
+    p = W.elasticity3d(region_grid=(2, 1, 1), choices=(7, 10), seed=5)
+    dp = upload(p)
+    sizes = np.prod(np.asarray(p.region_dims), axis=1)
+    inner = np.bincount(p.region_gids, minlength=p.n_nodes) == 1
+    last = p.region_gids[sizes[0]:]
+    ctx = rmg.Context(0)
+    lay = rmg.Layout(ctx, 3, p.region_dims, dp.gids, p.n_nodes, dp.dirichlet)
+
+    def numbers(val, precision=rmg.FP32):
+        lay.operator_from_block_csr(27, 3, dp.rowptr, dp.col, val)
+        h = rmg.Hierarchy(lay, rmg.default_options(levels=2, precision=precision))
+        return h.half_regions(0), h.half_regions(1), h.coef_planes(0)
+
+    assert numbers(dp.val) == ((2, int(sizes.sum())), (0, 0), 126)
+    val = dp.val.clone()
+    rp = dp.rowptr.cpu().numpy()
+    for g in last[inner[last]]:                # a row of the second region alone
+        cols = dp.col[int(rp[3 * g]):int(rp[3 * g + 1])].cpu().numpy()
+        k = np.flatnonzero(inner[cols // 3] & (cols // 3 != g))
+        if k.size:
+            val[int(rp[3 * g]) + int(k[0])] *= 1.0 + 2.0 ** -20
+            break
+    assert numbers(val) == ((1, int(sizes[0])), (0, 0), 243)
+    assert numbers(dp.val, rmg.FP64) == ((0, 0), (0, 0), 243)
