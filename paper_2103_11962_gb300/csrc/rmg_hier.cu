@@ -892,39 +892,46 @@ void hier_build(Hier& h) {
 }
 
 // Levels of the one-kernel coarse end (rmg_tail.cu). The kernel has 16 SMs, so a level belongs in
-// it while the GPU's other SMs would save less than the launches cost. A sweep as two launches
-// takes 6 to 8 us up to about 25k nodes of a 27-point level; inside the kernel its two phases
-// take 5 us for 12k nodes in FP32 (L2 latency and barriers; the second round of 16k threads comes
-// at 16k nodes) and 6 us for 3k nodes in FP64 (64 DFMA/clk for 16 SMs). The lines: 24k nodes of
-// a 27-point level in FP32, 8k in FP64. The dense solve goes inside up to kTailDense unknowns:
-// every refinement step reads the FP64 matrix once, 4.7 MB there, about 3 us on 16 SMs.
-// Measured, launches against one kernel for the coarse end: V-cycle of 1.5M nodes in FP64
-// 646 -> 588 us; solves of 27k nodes 2852 -> 2164 us and of 572k nodes with Gauss-Seidel
-// 13.7 -> 11.3 ms.
+// it while the GPU's other SMs would save less than the launches cost. In FP32 that is as long as
+// its 16k threads take a node each; in FP64 half of it (32 DFMA/clk on 16 SMs), with blocks of 3
+// again half (three rows a node), and with Gauss-Seidel, whose colours are a launch each, twice.
+// The dense solve goes inside up to kTailDense unknowns (every refinement step reads the FP64
+// matrix once, 1.2 MB there), and the coarsest level alone only up to kTailAlone.
+// Measured V-cycles, us, with the level inside against outside:
+//   FP32, 27 points: 16.0k nodes 151 / 157, 24.0k 191 / 175; 9 points: 9.4k 134 / 137,
+//     18.8k 159 / 158, 37.6k 188 / 175, 70.6k 284 / 234; blocks of 3: 4.0k 308 / 358, 6.0k 346 / 379
+//   FP64, 27 points: 8.0k 169 / 180, 12.0k 193 / 184, 16.0k 241 / 219; 9 points: 9.4k 168 / 168,
+//     18.8k 213 / 188; blocks of 3: 4.0k 680 / 730, 5.0k 707 / 706, 6.0k 826 / 804
+//   Gauss-Seidel, 27 points: 24.0k FP32 302 / 330, FP64 502 / 529; 9 points: 18.8k FP32 237 / 249,
+//     FP64 327 / 325, 70.6k FP32 426 / 367
+//   solve inside against outside: 288 unknowns 263 / 266, 391 188 / 188, 504 315 / 308,
+//     720 356 / 323; coarsest level alone: 176 145 / 147, 275 158 / 157, 440 180 / 175.
 static void tail_levels(Hier& h) {
   Ctx& c = *h.c;
   const int Lv = h.levels(), B = h.lv[0]->B, dim = h.lv[0]->dim;
   h.tail0 = -1;
   h.tail_geo = std::vector<TailGeometry>(Lv);
   if (Lv < 2 || h.o.nu1 < 1 || !h.dense_ok) return;
-  const long long most = h.mixed() ? 660000 : 210000;      // coefficients of a sweep
+  const bool gs = h.o.smoother == RMG_SMOOTHER_GS;
+  const int most = (h.mixed() ? 16384 : 8192) * (gs ? 2 : 1) / (B == 1 ? 1 : 2);
   int l0 = Lv;
   while (l0 > 1 && Lv - l0 < kTailLevels) {
     const Level& L = *h.lv[l0 - 1];
-    bool ok = (long long)L.n_r * (dim == 3 ? 27 : 9) * B * B <= most * (B == 1 ? 1 : 2);
+    bool ok = L.n_r <= most;
     for (int d : L.hdims) ok = ok && d < 1024;              // packed positions
     if (!ok) break;
     --l0;
   }
-  h.tail_solve = (long long)h.nc * B <= kTailDense;
+  const long long nd = (long long)h.nc * B;
+  h.tail_solve = nd <= kTailDense;
   // two launches around a separate solve pay only with a smoothed level inside
-  if (l0 >= Lv || (!h.tail_solve && l0 >= Lv - 1)) return;
+  if (l0 >= Lv || (l0 >= Lv - 1 && nd > kTailAlone)) return;
   h.tail_blocks = !h.mixed() ? tail_cluster<double, double>(dim, B)
                   : h.o.precision == RMG_PREC_FP32 ? tail_cluster<float, float>(dim, B)
                                                    : tail_cluster<float, __nv_bfloat16>(dim, B);
   if (!h.tail_blocks) return;
   for (int l = l0; l < Lv; ++l)
-    h.tail_geo[l].build(c, *h.lv[l], h.o.smoother == RMG_SMOOTHER_GS && l + 1 < Lv);
+    h.tail_geo[l].build(c, *h.lv[l], gs && l + 1 < Lv);
   h.tail0 = l0;
 }
 

@@ -7,7 +7,8 @@ namespace rmg {
 
 constexpr int kTailThreads = 1024;
 constexpr int kTailLevels = 6;           // levels one launch takes
-constexpr int kTailDense = 768;          // unknowns of the coarse solve done inside
+constexpr int kTailDense = 384;          // unknowns of the coarse solve done inside,
+constexpr int kTailAlone = 256;          // and of one that is all there is inside
 constexpr int kTailDenseBlock = 48;      // up to here every block solves alone
 
 // Node of a small level: region, position and region sizes (10 bits each) and the node, one
