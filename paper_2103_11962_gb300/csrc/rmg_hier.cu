@@ -213,7 +213,7 @@ __device__ __forceinline__ void set_beta(Scalars* sc, double rz_new, double rz_o
 // What follows a dot product of CG: alpha = rz / (p.q), beta from r.z, or the first rz.
 enum CgDot : int { CG_ALPHA, CG_BETA, CG_RZ };
 __global__ void __launch_bounds__(256)
-k_cg_dot(int n, int n_nodes, const double* __restrict__ x, const double* __restrict__ y,
+k_cg_dot(int n, int n_nodes, const double* x, const double* y,
          const uint8_t* __restrict__ mult, Arrive A, Scalars* sc, int what) {
   follow();
   double s = 0.0;
@@ -232,9 +232,9 @@ k_cg_dot(int n, int n_nodes, const double* __restrict__ x, const double* __restr
 // The two products of the flexible form in FP64 (Gauss-Seidel cycle): r.z and r.z_old, then
 // z_old = z and beta.
 __global__ void __launch_bounds__(256)
-k_cg_flex64(int n, int n_nodes, const double* __restrict__ r, const double* __restrict__ z,
-            double* __restrict__ zold, const uint8_t* __restrict__ mult, Arrive A, Scalars* sc) {
-  follow();
+k_cg_flex64(int n, int n_nodes, const double* r, const double* z, double* __restrict__ zold,
+            const uint8_t* __restrict__ mult, Arrive A, Scalars* sc) {
+  follow(zold);
   double s0 = 0.0, s1 = 0.0;
   for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
     const double rk = r[k] * inv_mult<double>(mult[k < n_nodes ? k : k % n_nodes]);
@@ -257,10 +257,10 @@ k_cg_flex64(int n, int n_nodes, const double* __restrict__ r, const double* __re
 // x += alpha p, r -= alpha q; r.r (all FP64) goes to page-locked host memory, where the host
 // reads it after the stream has finished.
 __global__ void __launch_bounds__(256)
-k_cg_update(int n, int n_nodes, const double* __restrict__ p, const double* __restrict__ q,
-            const uint8_t* __restrict__ mult, const Scalars* __restrict__ sc,
+k_cg_update(int n, int n_nodes, const double* p, const double* q,
+            const uint8_t* __restrict__ mult, const Scalars* sc,
             double* __restrict__ x, double* __restrict__ r, Arrive A, double* host_rr) {
-  follow();
+  follow(x, r);
   const double a = sc->alpha;
   double s = 0.0;
   for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
@@ -287,11 +287,11 @@ k_cg_update(int n, int n_nodes, const double* __restrict__ p, const double* __re
 // x += alpha p, r -= alpha q (FP64); r32 = FP32(r * rscale), the cycle's right-hand side;
 // r.r / mult in FP64 to the host.
 __global__ void __launch_bounds__(256)
-k_cg_update_mixed(int n, int n_nodes, const double* __restrict__ p, const double* __restrict__ q,
-                  const uint8_t* __restrict__ mult, const Scalars* __restrict__ sc,
+k_cg_update_mixed(int n, int n_nodes, const double* p, const double* q,
+                  const uint8_t* __restrict__ mult, const Scalars* sc,
                   double rscale, double* __restrict__ x, double* __restrict__ r,
                   float* __restrict__ r32, Arrive A, double* host_rr) {
-  follow();
+  follow(x, r);
   const double a = sc->alpha;
   double s = 0.0;
   for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
@@ -309,7 +309,7 @@ k_cg_update_mixed(int n, int n_nodes, const double* __restrict__ p, const double
 }
 
 // r32 = FP32(r * rscale): the cycle's right-hand side at a (re)start of the iteration.
-__global__ void k_to_f32_scaled(int n, const double* __restrict__ r, double rscale,
+__global__ void k_to_f32_scaled(int n, const double* r, double rscale,
                                 float* __restrict__ r32) {
   follow();
   for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x)
@@ -321,10 +321,9 @@ __global__ void k_to_f32_scaled(int n, const double* __restrict__ r, double rsca
 // of r.z_old to partials[gridDim, 2 gridDim). Four consecutive FP32 entries per thread step
 // (16-byte loads); the entries past the last multiple of four take a scalar tail.
 __global__ void __launch_bounds__(256)
-k_flex_dots(int n, int n_nodes, const double* __restrict__ r, const float* __restrict__ z,
-            float* __restrict__ zold, const uint8_t* __restrict__ mult, double zscale, Arrive A,
-            Scalars* sc) {
-  follow();
+k_flex_dots(int n, int n_nodes, const double* r, const float* z, float* __restrict__ zold,
+            const uint8_t* __restrict__ mult, double zscale, Arrive A, Scalars* sc) {
+  follow(zold);
   double s0 = 0.0, s1 = 0.0;
   const int n4 = n >> 2;
   const int tid = blockIdx.x * blockDim.x + threadIdx.x, nth = gridDim.x * blockDim.x;
@@ -362,7 +361,7 @@ k_flex_dots(int n, int n_nodes, const double* __restrict__ r, const float* __res
 
 // First direction after a (re)start: rz = r.z in FP64, p = z * zscale (FP64), z_old = z.
 __global__ void __launch_bounds__(256)
-k_start_dir(int n, int n_nodes, const double* __restrict__ r, const float* __restrict__ z,
+k_start_dir(int n, int n_nodes, const double* r, const float* z,
             const uint8_t* __restrict__ mult, double zscale, double* __restrict__ p,
             float* __restrict__ zold, Arrive A, Scalars* sc) {
   follow();
@@ -388,9 +387,9 @@ __global__ void k_axpy_neg(int n, const double* __restrict__ z, double* __restri
 
 // p = z * zscale + beta p (zscale = 1 for the FP64 cycle).
 template <typename ZT>
-__global__ void k_p_update(int n, const ZT* __restrict__ z, double zscale,
-                           const Scalars* __restrict__ sc, double* __restrict__ p) {
-  follow();
+__global__ void k_p_update(int n, const ZT* z, double zscale, const Scalars* sc,
+                           double* __restrict__ p) {
+  follow(p);
   const double b = sc->beta;
   for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x)
     p[k] = fma(double(z[k]), zscale, b * p[k]);

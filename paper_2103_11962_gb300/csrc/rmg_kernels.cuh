@@ -19,9 +19,21 @@ namespace rmg {
 
 // Start of a kernel that is launched with launch_after(): the next kernel may be set up now (its
 // blocks wait in turn), and nothing is touched before the previous one has finished.
-__device__ __forceinline__ void follow() {
+//
+// What an earlier kernel of the stream writes must not be read through a const __restrict__
+// parameter: the compiler takes such data for constant over the whole kernel and may load it
+// before the wait (a counter read on entry was: it came out as the call before had left it).
+// Those parameters are plain const pointers, and a __restrict__ one that is read and written is
+// handed to follow(), so that the compiler sees its data change here. Coefficients, masks and
+// index arrays, which no kernel launched this way writes, keep __restrict__.
+__device__ __forceinline__ void data_changed(const void* p) {
+  asm volatile("" ::"l"(p) : "memory");
+}
+template <typename... T>
+__device__ __forceinline__ void follow(T*... changed) {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   asm volatile("griddepcontrol.wait;" ::: "memory");
+  (data_changed(changed), ...);
 }
 
 // a / d for 0 <= a < 2^22 from the float reciprocal rd of d: the truncated product is within
@@ -91,7 +103,7 @@ __device__ __forceinline__ int region_of(const RegionDev* R, int nreg, int n) {
 // ------------------------------------------------------------------ stencil application
 // au = sum_s coef[s][n] * u[n + off(s)] over the neighbours inside the region.
 template <int KIND, typename CT, typename VT, typename AT>
-__device__ __forceinline__ AT stencil_row(const CT* __restrict__ coef, const VT* __restrict__ u,
+__device__ __forceinline__ AT stencil_row(const CT* __restrict__ coef, const VT* u,
                                           int n, int n_r, int i, int j, int l,
                                           const RegionDev& R) {
   using S = Sten<KIND>;
@@ -121,7 +133,7 @@ template <typename T> __device__ __forceinline__ T to_acc(T v) { return v; }
 // Phase A: stencil at every node; single-copy nodes finish through the epilogue.
 template <int KIND, typename CT, typename VT, typename AT, class Epi>
 __global__ void __launch_bounds__(kTile)
-k_stencil(Grid G, const CT* __restrict__ coef, const VT* __restrict__ u,
+k_stencil(Grid G, const CT* __restrict__ coef, const VT* u,
           const uint8_t* __restrict__ mult, AT* __restrict__ y, Epi epi) {
   follow();
   RMG_FOR_NODES(G)
@@ -153,8 +165,11 @@ __host__ __device__ constexpr bool mirrored_slots() {
 // A 4-byte load from a base all threads share and an unsigned 32-bit byte offset of the thread: an
 // addressing form of the load itself, where a 64-bit element address takes two or three more
 // instructions. A 27-point row has 54 loads, and the sweep issued about 500 instructions a node.
-__device__ __forceinline__ float load32(const float* __restrict__ base, unsigned byte) {
-  return __ldg(reinterpret_cast<const float*>(reinterpret_cast<const char*>(base) + byte));
+// CONST: data that no kernel of the cycle writes (see follow).
+template <bool CONST>
+__device__ __forceinline__ float load32(const float* base, unsigned byte) {
+  const float* p = reinterpret_cast<const float*>(reinterpret_cast<const char*>(base) + byte);
+  return CONST ? __ldg(p) : *p;
 }
 // Largest level whose byte offsets into one plane fit 32 bits.
 constexpr int kOffset32Nodes = 1 << 30;
@@ -162,7 +177,7 @@ constexpr int kOffset32Nodes = 1 << 30;
 // The row of node n from the half planes; OFF32: n_r <= kOffset32Nodes.
 template <int KIND, bool OFF32>
 __device__ __forceinline__ float stencil_row_half(const float* __restrict__ half,
-                                                  const float* __restrict__ u, int n, int n_r,
+                                                  const float* u, int n, int n_r,
                                                   int i, int j, int l, const RegionDev& R) {
   using S = Sten<KIND>;
   static_assert(mirrored_slots<KIND>(), "half storage needs mirrored stencil slots");
@@ -183,8 +198,8 @@ __device__ __forceinline__ float stencil_row_half(const float* __restrict__ half
       const int nb = n + dx + dy * sy + dz * sz;
       const float* plane = half + (size_t)(s < C ? S::S - 1 - s - C : s - C) * (size_t)n_r;
       const int at = s < C ? nb : n;
-      const float c = OFF32 ? load32(plane, 4u * (unsigned)at) : plane[at];
-      const float v = OFF32 ? load32(u, 4u * (unsigned)nb) : u[nb];
+      const float c = OFF32 ? load32<true>(plane, 4u * (unsigned)at) : plane[at];
+      const float v = OFF32 ? load32<false>(u, 4u * (unsigned)nb) : u[nb];
       au = fmaf(c, v, au);
     }
   }
@@ -226,8 +241,7 @@ __device__ __forceinline__ void prefetch_tile(const Grid& G, int t, const float*
 // operator symmetric (*asym == 0), else the full planes as k_stencil.
 template <bool HALF, bool OFF32, int KIND, class Epi>
 __device__ __forceinline__ void stencil_pass(const Grid& G, const float* __restrict__ coef,
-                                             const float* __restrict__ u,
-                                             const uint8_t* __restrict__ mult,
+                                             const float* u, const uint8_t* __restrict__ mult,
                                              float* __restrict__ y, const Epi& epi) {
   RMG_FOR_NODES_AHEAD(G, if (HALF && KIND == 7) prefetch_tile(G, t_ + (int)gridDim.x, coef, 4, u, epi))
     int i, j, l;
@@ -247,8 +261,8 @@ __device__ __forceinline__ void stencil_pass(const Grid& G, const float* __restr
 template <int KIND, bool OFF32, class Epi>
 __global__ void __launch_bounds__(kTile, 7)
 k_stencil_half(Grid G, const float* __restrict__ coef, const float* __restrict__ half,
-               const int* __restrict__ asym, const float* __restrict__ u,
-               const uint8_t* __restrict__ mult, float* __restrict__ y, Epi epi) {
+               const int* __restrict__ asym, const float* u, const uint8_t* __restrict__ mult,
+               float* __restrict__ y, Epi epi) {
   follow();
   if (*asym) stencil_pass<false, OFF32, KIND>(G, coef, u, mult, y, epi);
   else stencil_pass<true, OFF32, KIND>(G, half, u, mult, y, epi);
@@ -297,7 +311,7 @@ __device__ __forceinline__ void cp_async_wait() {
 // floats long) at z-plane l of region R, tile corner (x0, y0), into dst[p][row][0..40). Only
 // 16-byte chunks that hold a node of the region are copied; a chunk that would end past the
 // array goes element by element. Other shared words keep stale values and are never read.
-__device__ __forceinline__ void stage_windows(float* dst, const float* __restrict__ src, int np,
+__device__ __forceinline__ void stage_windows(float* dst, const float* src, int np,
                                               long long n_r, long long total,
                                               const RegionDev& R, int x0, int y0, int l) {
   constexpr int kChunks = kStRow / 4;
@@ -324,7 +338,7 @@ __device__ __forceinline__ void stage_windows(float* dst, const float* __restric
 template <class Epi>
 __global__ void __launch_bounds__(kStX * kStY)
 k_stencil_half27_staged(Grid G, const float* __restrict__ coef, const float* __restrict__ half,
-                        const int* __restrict__ asym, const float* __restrict__ u,
+                        const int* __restrict__ asym, const float* u,
                         const uint8_t* __restrict__ mult, float* __restrict__ y, Epi epi) {
   follow();
   extern __shared__ __align__(16) float st_smem[];
@@ -424,7 +438,7 @@ k_stencil_half27_staged(Grid G, const float* __restrict__ coef, const float* __r
 // in ascending slot order. Most groups are pairs on a face: their sum needs no further index.
 template <typename AT>
 __device__ __forceinline__ AT group_sum(const int4& t, const int* __restrict__ gslot,
-                                        const AT* __restrict__ y) {
+                                        const AT* y) {
   if (t.z == 2) return y[min(t.x, t.w)] + y[max(t.x, t.w)];
   AT s = AT(0);
   for (int k = 0; k < t.z; k += 4) {
@@ -445,7 +459,7 @@ __device__ __forceinline__ AT group_sum(const int4& t, const int* __restrict__ g
 template <typename AT, class Epi>
 __global__ void __launch_bounds__(256)
 k_groups(int nslots, const int4* __restrict__ slots, const int* __restrict__ gslot,
-         const AT* __restrict__ y, Epi epi) {
+         const AT* y, Epi epi) {
   follow();
   for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < nslots; q += gridDim.x * blockDim.x) {
     const int4 t = slots[q];
@@ -459,7 +473,7 @@ k_groups(int nslots, const int4* __restrict__ slots, const int* __restrict__ gsl
 // vectors are component-major: v[c * n_r + n]. The epilogues receive the flat index c * n_r + n.
 template <int KIND, int B, typename CT, typename VT, typename AT, class Epi>
 __global__ void __launch_bounds__(kTile)
-k_bstencil(Grid G, const CT* __restrict__ coef, const VT* __restrict__ u,
+k_bstencil(Grid G, const CT* __restrict__ coef, const VT* u,
            const uint8_t* __restrict__ mult, AT* __restrict__ y, Epi epi) {
   follow();
   using S = Sten<KIND>;
@@ -510,7 +524,7 @@ k_bstencil(Grid G, const CT* __restrict__ coef, const VT* __restrict__ u,
 // of 1045 bytes a node; the mirrored ones come from L1 and L2.
 template <bool HALF, bool OFF32, int KIND, int B>
 __device__ __forceinline__ void bstencil_row32(const float* __restrict__ coef,
-                                               const float* __restrict__ u, int n, int n_r, int i,
+                                               const float* u, int n, int n_r, int i,
                                                int j, int l, const RegionDev& R, float (&au)[B]) {
   using S = Sten<KIND>;
   static_assert(mirrored_slots<KIND>(), "half storage needs mirrored stencil slots");
@@ -534,7 +548,7 @@ __device__ __forceinline__ void bstencil_row32(const float* __restrict__ coef,
 #pragma unroll
     for (int c2 = 0; c2 < B; ++c2) {
       const float* uc = u + (size_t)c2 * n_r;
-      uv[c2] = OFF32 ? load32(uc, 4u * (unsigned)nb) : uc[nb];
+      uv[c2] = OFF32 ? load32<false>(uc, 4u * (unsigned)nb) : uc[nb];
     }
     const bool mirrored = HALF && s < C;
     const int plane = !HALF ? s : s < C ? S::S - 1 - s - C : s - C;
@@ -545,7 +559,7 @@ __device__ __forceinline__ void bstencil_row32(const float* __restrict__ coef,
       for (int c2 = 0; c2 < B; ++c2) {
         const int blk = mirrored ? c2 * B + c : c * B + c2;
         const float* p = coef + ((size_t)blk * P + plane) * n_r;
-        au[c] = fmaf(OFF32 ? load32(p, 4u * (unsigned)at) : p[at], uv[c2], au[c]);
+        au[c] = fmaf(OFF32 ? load32<true>(p, 4u * (unsigned)at) : p[at], uv[c2], au[c]);
       }
   }
 }
@@ -555,8 +569,8 @@ __device__ __forceinline__ void bstencil_row32(const float* __restrict__ coef,
 template <int KIND, bool OFF32, int B, class Epi>
 __global__ void __launch_bounds__(kTile)
 k_bstencil_half(Grid G, const float* __restrict__ coef, const float* __restrict__ half,
-                const int* __restrict__ asym, const float* __restrict__ u,
-                const uint8_t* __restrict__ mult, float* __restrict__ y, Epi epi) {
+                const int* __restrict__ asym, const float* u, const uint8_t* __restrict__ mult,
+                float* __restrict__ y, Epi epi) {
   follow();
   RMG_FOR_NODES(G)
     int i, j, l;
@@ -577,7 +591,7 @@ k_bstencil_half(Grid G, const float* __restrict__ coef, const float* __restrict_
 template <typename AT, class Epi>
 __global__ void __launch_bounds__(256)
 k_groups_b(int nslots, int B, int n_r, const int4* __restrict__ slots,
-           const int* __restrict__ gslot, const AT* __restrict__ y, Epi epi) {
+           const int* __restrict__ gslot, const AT* y, Epi epi) {
   follow();
   for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < nslots; q += gridDim.x * blockDim.x) {
     const int4 t = slots[q];
@@ -702,7 +716,7 @@ struct EpiCheb {                 // d = c1 d + c2 D~^-1 r, u_out = u + d
 
 // ------------------------------------------------------------------ elementwise
 template <typename T>
-__global__ void k_jacobi_zero(int n, const T* __restrict__ b, const T* __restrict__ dinv,
+__global__ void k_jacobi_zero(int n, const T* b, const T* __restrict__ dinv,
                               T omega, T* __restrict__ uo) {
   follow();
   for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x)
@@ -710,7 +724,7 @@ __global__ void k_jacobi_zero(int n, const T* __restrict__ b, const T* __restric
 }
 
 template <typename T>
-__global__ void k_cheb0_zero(int n, const T* __restrict__ b, const T* __restrict__ dinv,
+__global__ void k_cheb0_zero(int n, const T* b, const T* __restrict__ dinv,
                              const T* __restrict__ c2, T* __restrict__ d,
                              T* __restrict__ uo) {
   follow();
@@ -752,7 +766,7 @@ struct EpiMean {
 
 // dst[gslot[q]] = src[gslot[q]] for every copy of every interface node.
 template <typename T>
-__global__ void k_copy_slots(int nslots, const int* __restrict__ gslot, const T* __restrict__ src,
+__global__ void k_copy_slots(int nslots, const int* __restrict__ gslot, const T* src,
                              T* __restrict__ dst) {
   follow();
   for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < nslots; q += gridDim.x * blockDim.x)
@@ -761,7 +775,7 @@ __global__ void k_copy_slots(int nslots, const int* __restrict__ gslot, const T*
 
 // A sweep from u = 0: r = b, delta = 0, u = 0.
 template <typename VT>
-__global__ void k_gs_zero(int n, const VT* __restrict__ b, VT* __restrict__ r,
+__global__ void k_gs_zero(int n, const VT* b, VT* __restrict__ r,
                           VT* __restrict__ delta, VT* __restrict__ u) {
   follow();
   for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
@@ -785,9 +799,9 @@ __host__ __device__ __forceinline__ int gs_colour_of(int i, int j, int l) {
 // included) and u_i += delta_i.
 template <int KIND, typename CT, typename VT>
 __global__ void __launch_bounds__(kTile)
-k_gs_colour(Grid G, const CT* __restrict__ coef, const VT* __restrict__ r,
+k_gs_colour(Grid G, const CT* __restrict__ coef, const VT* r,
             const VT* __restrict__ dinv, VT* delta, VT* __restrict__ u, int colour, VT omega) {
-  follow();
+  follow(u);
   RMG_FOR_NODES(G)
     int i, j, l;
     RMG_DECODE(i, j, l);
@@ -831,7 +845,7 @@ __device__ __forceinline__ T pw_seen_from_coarse(const W* __restrict__ wr, int n
 // P(f, C) is a compile-time constant for linear interpolation (STORED = false) or the FP32
 // product of the stored per-axis weights of f.
 template <int DIM, bool CHECK, bool STORED, typename VT>
-__device__ __forceinline__ VT restrict_sum(const VT* __restrict__ rs, const RegionDev& F,
+__device__ __forceinline__ VT restrict_sum(const VT* rs, const RegionDev& F,
                                            const float* __restrict__ wr, int fn_r,
                                            int I, int J, int L) {
   VT acc = VT(0);
@@ -868,7 +882,7 @@ __device__ __forceinline__ VT restrict_sum(const VT* __restrict__ rs, const Regi
 // 2D: a thread per coarse node and its 25 fine nodes.
 template <typename VT>
 __global__ void __launch_bounds__(kTile)
-k_restrict2(Grid Gc, const RegionDev* __restrict__ fregions, const VT* __restrict__ rs,
+k_restrict2(Grid Gc, const RegionDev* __restrict__ fregions, const VT* rs,
             const uint8_t* __restrict__ cmask, const uint8_t* __restrict__ cmult,
             VT* __restrict__ w, VT* __restrict__ yc) {
   follow();
@@ -892,7 +906,7 @@ k_restrict2(Grid Gc, const RegionDev* __restrict__ fregions, const VT* __restric
 constexpr int kRestrictWarps = 5;
 template <typename VT>
 __global__ void __launch_bounds__(32 * kRestrictWarps)
-k_restrict3(Grid Gc, const RegionDev* __restrict__ fregions, const VT* __restrict__ rs,
+k_restrict3(Grid Gc, const RegionDev* __restrict__ fregions, const VT* rs,
             const uint8_t* __restrict__ cmask, const uint8_t* __restrict__ cmult,
             VT* __restrict__ w, VT* __restrict__ yc) {
   follow();
@@ -948,8 +962,8 @@ __device__ __forceinline__ VT rem_weight(int rem) {
 template <int DIM, typename VT>
 __global__ void __launch_bounds__(kTile)
 k_prolong(Grid G1, const RegionDev* __restrict__ fregions, const RegionDev* __restrict__ cregions,
-          const uint8_t* __restrict__ fmask, const VT* __restrict__ ubar, VT* __restrict__ u) {
-  follow();
+          const uint8_t* __restrict__ fmask, const VT* ubar, VT* __restrict__ u) {
+  follow(u);
   RMG_FOR_NODES(G1)
     (void)n;
     int cx, j, l;
@@ -997,7 +1011,7 @@ __device__ __forceinline__ T pw_seen_from_coarse(const W* __restrict__ wr, int n
 template <int DIM, typename VT>
 __global__ void __launch_bounds__(kTile)
 k_restrict_w(Grid Gc, const RegionDev* __restrict__ fregions, int fn_r, const float* __restrict__ wr,
-             const VT* __restrict__ rs, const uint8_t* __restrict__ cmask,
+             const VT* rs, const uint8_t* __restrict__ cmask,
              const uint8_t* __restrict__ cmult, VT* __restrict__ w, VT* __restrict__ yc) {
   follow();
   RMG_FOR_NODES(Gc)
@@ -1018,8 +1032,8 @@ k_restrict_w(Grid Gc, const RegionDev* __restrict__ fregions, int fn_r, const fl
 template <int DIM, typename VT>
 __global__ void __launch_bounds__(kTile)
 k_prolong_w(Grid Gf, const RegionDev* __restrict__ cregions, const float* __restrict__ wr,
-            const uint8_t* __restrict__ fmask, const VT* __restrict__ ubar, VT* __restrict__ u) {
-  follow();
+            const uint8_t* __restrict__ fmask, const VT* ubar, VT* __restrict__ u) {
+  follow(u);
   RMG_FOR_NODES(Gf)
     if (fmask[n]) continue;
     int i, j, l;
