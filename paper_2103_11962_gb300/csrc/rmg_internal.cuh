@@ -189,8 +189,11 @@ struct Level {
   DBuf<int> rid;                 // region of every regional node (built for the split)
   DBuf<int> sgrp;                // group of every group slot (nslots)
   DBuf<int4> slots;              // slot records of phase B (k_slot_records)
-  DBuf<int2> split_left;         // rows the split's direct pass left, and their number, per
-  DBuf<int> split_nleft;         // row component (B * n_r, B)
+  DBuf<uint8_t> split_direct;    // regions the split's direct pass takes (k_split_forms)
+  DBuf<int> split_any;           // last calls in which a region was taken and was not
+  int split_call = 0;
+  DBuf<int2> split_left;         // rows it left there, and their number, per row component
+  DBuf<int> split_nleft;         // (B * n_r, B)
   DBuf<int4> affine;             // per region {g0, gy, gz, ok}: gid = g0 + i + gy j + gz l
   // operator
   DBuf<double> coef;             // kind * n_r, slot-major

@@ -599,6 +599,15 @@ constexpr int kSplitChunk = 9;
 // Rows a warp stages at a time in the direct pass.
 constexpr int kDirectRows = 16;
 
+// Column of entry e of a full row of composite node g in column order (a: the affine map).
+template <int KIND, int B>
+__device__ __forceinline__ int64_t direct_column(int g, int e, const int4& a) {
+  using S = Sten<KIND>;
+  const int slot = e / B;
+  const int off = S::dx(slot) + a.y * S::dy(slot) + (S::DIM == 3 ? a.z * S::dz(slot) : 0);
+  return (int64_t)(g + off) * B + (e - slot * B);
+}
+
 // The direct pass over 32 consecutive nodes of an affine region: rows that hold the full stencil
 // in column order, with every column where the region's map puts it. Their values go to the slots
 // by position, without a look at any entry but the comparison of its column: the lanes copy the
@@ -618,7 +627,7 @@ __device__ __forceinline__ unsigned split_direct(unsigned cand, int g, int64_t e
   for (int half = 0; half < 2; ++half) {
     if (!((cand >> (16 * half)) & 0xffffu)) continue;
     for (int t = 0; t < B; ++t) {                // entries t S .. t S + S - 1 of the rows
-      const int e = t * S::S + k, slot = e / B, comp = e - slot * B;
+      const int e = t * S::S + k;
 #pragma unroll 4
       for (int r0 = 0; r0 < kDirectRows; r0 += RP) {
         const int r = r0 + sub, from = 16 * half + (r & 15);
@@ -630,9 +639,7 @@ __device__ __forceinline__ unsigned split_direct(unsigned cand, int g, int64_t e
       }
       asm volatile("cp.async.wait_all;\n" ::: "memory");
       __syncwarp();
-      const int64_t off =
-          (int64_t)(S::dx(slot) + af.y * S::dy(slot) + (S::DIM == 3 ? af.z * S::dz(slot) : 0)) * B +
-          comp;
+      const int64_t off = direct_column<KIND, B>(0, e, af);
 #pragma unroll 4
       for (int r0 = 0; r0 < kDirectRows; r0 += RP) {
         const int r = r0 + sub, from = 16 * half + (r & 15);
@@ -656,53 +663,91 @@ __device__ __forceinline__ unsigned split_direct(unsigned cand, int g, int64_t e
   return cand & ~__reduce_or_sync(0xffffffffu, bad);
 }
 
-// The direct pass over single-copy rows in regions with an affine map; a warp takes 32
-// consecutive nodes of a tile. The single-copy rows that are left (cut by the domain boundary or
-// by a mask, out of order, or of a region without an affine map) go to a list, {node, region},
-// for k_split_rows. One kernel for both forms held this pass to two blocks per SM, and a warp
-// with one row left waited for it as long as for 32 (477 us for them in a kernel of their own
-// over the tiles, 170 us from the list). 10.6M nodes of a 27-point stencil: the single-copy rows
-// 2571 -> 1716 us; the direct pass moves its 6.3 GB at 4.1 TB/s, 0.61 of the measured rate,
-// bound by the latency of its copies.
+// Which regions the direct pass takes, a warp each: those with an affine map whose middle node has
+// a row of the direct form. Programs that write rows in another order (diagonal first, descending)
+// or leave entries out do so in all rows: without this look the direct pass copied such rows for
+// nothing and the list below took them all: diagonal first, 4.9M nodes of a 7-point stencil 539 us
+// and 3M of a 27-point one 1380 us, now 350 and 905 (the general pass alone 330 and 946). For rows
+// in column order the look costs 2 to 4 us of 282 and 704.
+// any[0] and any[1] become `call` when there is a region that is taken and one that is not, a
+// number that earlier calls did not use. Also clears the lengths of the lists.
+template <int KIND, int B>
+__global__ void __launch_bounds__(256)
+k_split_forms(int nreg, const RegionDev* __restrict__ regions, const int* __restrict__ gid,
+              const uint8_t* __restrict__ mult, const int4* __restrict__ affine,
+              const int64_t* __restrict__ rowptr, const int64_t* __restrict__ col,
+              uint8_t* __restrict__ direct, int* __restrict__ any, int call,
+              int* __restrict__ nleft) {
+  using S = Sten<KIND>;
+  if (blockIdx.x == 0 && threadIdx.x < B) nleft[threadIdx.x] = 0;
+  const int lane = threadIdx.x & 31, nwarps = (int)(gridDim.x * blockDim.x) >> 5;
+  for (int r = (int)(blockIdx.x * blockDim.x + threadIdx.x) >> 5; r < nreg; r += nwarps) {
+    const RegionDev R = regions[r];
+    const int4 af = affine[r];
+    const int i = R.nx / 2, j = R.ny / 2, l = R.nz / 2;
+    bool ok = af.w && i > 0 && i < R.nx - 1 && j > 0 && j < R.ny - 1 &&
+              (S::DIM == 2 || (l > 0 && l < R.nz - 1));
+    if (ok) {
+      const int n = R.off + i + R.nx * (j + R.ny * l);
+      const int64_t row = (int64_t)gid[n] * B, e0 = rowptr[row];
+      ok = mult[n] == 1 && rowptr[row + 1] - e0 == B * S::S;
+      for (int e = lane; ok && e < B * S::S; e += 32)
+        ok = col[e0 + e] == direct_column<KIND, B>(gid[n], e, af);
+    }
+    ok = __all_sync(0xffffffffu, ok);
+    if (lane == 0) {
+      direct[r] = ok;
+      any[ok ? 0 : 1] = call;                  // every writer stores the same
+    }
+  }
+}
+
+// The direct pass over single-copy rows in the regions that k_split_forms chose; a warp takes 32
+// consecutive nodes of a tile. The single-copy rows that are left there (cut by the domain
+// boundary or by a mask, out of order) go to a list, {node, region}, for k_split_rows. One kernel
+// for both forms held this pass to two blocks per SM, and a warp with one row left waited for it
+// as long as for 32 (477 us for them in a kernel of their own over the tiles, 170 us from the
+// list). 10.6M nodes of a 27-point stencil: the single-copy rows 2571 -> 1716 us; the direct pass
+// moves its 6.3 GB at 4.1 TB/s, 0.61 of the measured rate, bound by the latency of its copies.
 template <int KIND, int B>
 __global__ void __launch_bounds__(kTile / 2, 8)
 k_split_direct(Grid G, const int* __restrict__ gid, const uint8_t* __restrict__ mult,
-               const int4* __restrict__ affine, const int64_t* __restrict__ rowptr,
-               const int64_t* __restrict__ col, const double* __restrict__ val,
-               double* __restrict__ coef, int2* __restrict__ left, int* __restrict__ nleft) {
+               const int4* __restrict__ affine, const uint8_t* __restrict__ direct,
+               const int64_t* __restrict__ rowptr, const int64_t* __restrict__ col,
+               const double* __restrict__ val, double* __restrict__ coef, int2* __restrict__ left,
+               int* __restrict__ nleft, const int* __restrict__ any, int call) {
   constexpr int kWarps = kTile / 32, kOwn = kWarps / 2;   // warps of a tile, of this block
   using S = Sten<KIND>;
   __shared__ __align__(16) int64_t s_col[kOwn][kDirectRows * S::S];
   __shared__ __align__(16) double s_val[kOwn][kDirectRows * S::S];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int c_row = blockIdx.y;
-  const int tasks = G.ntiles * kWarps;
+  const int tasks = any[0] == call ? G.ntiles * kWarps : 0;
   for (int task = blockIdx.x * kOwn + warp; task < tasks; task += gridDim.x * kOwn) {
     const Tile tile = G.tiles[task / kWarps];
+    if (!direct[tile.region]) continue;
     const RegionDev R = G.regions[tile.region];
     const int li = tile.start + (task % kWarps) * 32 + lane;
     const int n = R.off + li;
     const int4 af = affine[tile.region];
     const bool single = li < R.nx * R.ny * R.nz && mult[n] == 1;
     unsigned ok = 0;
-    if (af.w) {
-      int i, j, l;
-      decode(single ? li : 0, R, i, j, l);
-      bool cand = single && i > 0 && i < R.nx - 1 && j > 0 && j < R.ny - 1 &&
-                  (S::DIM == 2 || (l > 0 && l < R.nz - 1));
-      int64_t e0 = 0;
-      int g = 0;
-      if (cand) {
-        g = gid[n];
-        const int64_t row = (int64_t)g * B + c_row;
-        e0 = rowptr[row];
-        cand = rowptr[row + 1] - e0 == B * S::S;
-      }
-      const unsigned rows = __ballot_sync(0xffffffffu, cand);
-      if (rows)
-        ok = split_direct<KIND, B>(rows, g, e0, af, col, val, s_col[warp], s_val[warp],
-                                   coef + (size_t)c_row * B * S::S * G.n_r + (n - lane), G.n_r);
+    int i, j, l;
+    decode(single ? li : 0, R, i, j, l);
+    bool cand = single && i > 0 && i < R.nx - 1 && j > 0 && j < R.ny - 1 &&
+                (S::DIM == 2 || (l > 0 && l < R.nz - 1));
+    int64_t e0 = 0;
+    int g = 0;
+    if (cand) {
+      g = gid[n];
+      const int64_t row = (int64_t)g * B + c_row;
+      e0 = rowptr[row];
+      cand = rowptr[row + 1] - e0 == B * S::S;
     }
+    const unsigned rows = __ballot_sync(0xffffffffu, cand);
+    if (rows)
+      ok = split_direct<KIND, B>(rows, g, e0, af, col, val, s_col[warp], s_val[warp],
+                                 coef + (size_t)c_row * B * S::S * G.n_r + (n - lane), G.n_r);
     const unsigned rest = __ballot_sync(0xffffffffu, single) & ~ok;
     if (!rest) continue;
     int at = 0;
@@ -714,39 +759,51 @@ k_split_direct(Grid G, const int* __restrict__ gid, const uint8_t* __restrict__ 
   }
 }
 
-// The listed rows, a warp for 32 of them (their order in the list is of no consequence: every row
-// writes its own slots). The CSR rows are staged through shared memory nine entries at a time,
-// the lanes copying the 32 rows' entries together (mostly rows that lie side by side in the CSR);
-// then every lane handles its own row's entries in order.
-template <int KIND, int B>
-__global__ void __launch_bounds__(kTile)
-k_split_rows(const int2* __restrict__ left, const int* __restrict__ nleft,
-             const RegionDev* __restrict__ regions, int n_r, RMG_SPLIT_PARAMS) {
+// The other single-copy rows, a warp for 32 of them: those that the direct pass listed (LISTED,
+// blockIdx.z = 0; their order in the list is of no consequence: every row writes its own slots),
+// and all of the regions that it did not take, by tiles (blockIdx.z = 1). (One loop over both took
+// 329 us instead of 299 for 4.9M nodes with 7 points, 10% more for blocks.) The CSR rows are staged
+// through shared memory nine entries at a time, the lanes copying the 32 rows' entries together
+// (mostly rows that lie side by side in the CSR); then every lane handles its own row's entries in
+// order.
+template <int KIND, int B, bool LISTED>
+__device__ __forceinline__ void split_rows(const Grid& G, const uint8_t* __restrict__ direct,
+                                           const int2* __restrict__ left,
+                                           const int* __restrict__ nleft, bool others,
+                                           int64_t* wc, double* wv, int64_t* s_e0, int* s_len,
+                                           RMG_SPLIT_PARAMS) {
   constexpr int kWarps = kTile / 32;
-  __shared__ __align__(16) int64_t s_col[kWarps][32 * kSplitChunk];
-  __shared__ __align__(16) double s_val[kWarps][32 * kSplitChunk];
-  __shared__ int64_t s_e0[kWarps][32];           // first entry and length of every lane's row
-  __shared__ int s_len[kWarps][32];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  int64_t* wc = s_col[warp];
-  double* wv = s_val[warp];
-  const int c_row = blockIdx.y, count = nleft[c_row];
-  for (int first = 32 * (blockIdx.x * kWarps + warp); first < count;
-       first += 32 * gridDim.x * kWarps) {
-    const bool active = first + lane < count;
+  const int c_row = blockIdx.y;
+  const int tasks = LISTED ? (nleft[c_row] + 31) / 32 : others ? G.ntiles * kWarps : 0;
+  for (int task = blockIdx.x * kWarps + warp; task < tasks; task += gridDim.x * kWarps) {
     RowSplit<KIND, B> rs;
     int64_t e0 = 0;
     int len = 0;
+    bool active;
+    if constexpr (LISTED) {
+      active = 32 * task + lane < nleft[c_row];
+      if (active) {
+        const int2 node = left[(size_t)c_row * G.n_r + 32 * task + lane];
+        const RegionDev R = G.regions[node.y];
+        rs.begin(node.x, node.x - R.off, node.y, R, c_row, G.n_r, gid, mult, affine, coef);
+      }
+    } else {
+      const Tile tile = G.tiles[task / kWarps];
+      const RegionDev R = G.regions[tile.region];
+      if (direct[tile.region]) continue;
+      const int li = tile.start + (task % kWarps) * 32 + lane;
+      const int n = R.off + li;
+      active = li < R.nx * R.ny * R.nz && mult[n] == 1;
+      if (active) rs.begin(n, li, tile.region, R, c_row, G.n_r, gid, mult, affine, coef);
+    }
     if (active) {
-      const int2 node = left[(size_t)c_row * n_r + first + lane];
-      const RegionDev R = regions[node.y];
-      rs.begin(node.x, node.x - R.off, node.y, R, c_row, n_r, gid, mult, affine, coef);
       const int64_t row = (int64_t)rs.g * B + c_row;
       e0 = rowptr[row];
       len = (int)(rowptr[row + 1] - e0);
     }
-    s_e0[warp][lane] = e0;
-    s_len[warp][lane] = len;
+    s_e0[lane] = e0;
+    s_len[lane] = len;
     __syncwarp();
     const int passes = ((int)__reduce_max_sync(0xffffffffu, (unsigned)len) + kSplitChunk - 1) /
                        kSplitChunk;
@@ -757,8 +814,8 @@ k_split_rows(const int2* __restrict__ left, const int* __restrict__ nleft,
         const int idx = lane + 32 * m;
         const int r = idx / kSplitChunk, k = idx - r * kSplitChunk;
         const int e = h * kSplitChunk + k;
-        if (e < s_len[warp][r]) {
-          const int64_t at = s_e0[warp][r] + e;
+        if (e < s_len[r]) {
+          const int64_t at = s_e0[r] + e;
           cp_async8(wc + idx, col + at);
           cp_async8(wv + idx, val + at);
         }
@@ -779,6 +836,27 @@ k_split_rows(const int2* __restrict__ left, const int* __restrict__ nleft,
     }
     if (active) rs.end(mult);
   }
+}
+
+template <int KIND, int B>
+__global__ void __launch_bounds__(kTile)
+k_split_rows(Grid G, const uint8_t* __restrict__ direct, const int2* __restrict__ left,
+             const int* __restrict__ nleft, const int* __restrict__ any, int call,
+             RMG_SPLIT_PARAMS) {
+  constexpr int kWarps = kTile / 32;
+  __shared__ __align__(16) int64_t s_col[kWarps][32 * kSplitChunk];
+  __shared__ __align__(16) double s_val[kWarps][32 * kSplitChunk];
+  __shared__ int64_t s_e0[kWarps][32];           // first entry and length of every lane's row
+  __shared__ int s_len[kWarps][32];
+  const int w = threadIdx.x >> 5;
+  if (blockIdx.z == 0)
+    split_rows<KIND, B, true>(G, direct, left, nleft, false, s_col[w], s_val[w], s_e0[w], s_len[w],
+                              gid, mult, c2r, cgrp, gptr, gslot, rid, affine, rowptr, col, val,
+                              ncomp, coef, err);
+  else
+    split_rows<KIND, B, false>(G, direct, left, nleft, any[1] == call, s_col[w], s_val[w], s_e0[w],
+                               s_len[w], gid, mult, c2r, cgrp, gptr, gslot, rid, affine, rowptr,
+                               col, val, ncomp, coef, err);
 }
 
 // Rows of shared nodes, one thread per regional copy, in group-slot order (the copies of one
@@ -873,24 +951,36 @@ void split_from_csr(Ctx& c, Level& L, int kind, int B, const int64_t* rowptr, co
   if (L.affine.n < (size_t)L.nreg) build_affine(c, L);
   L.split_left.ensure((size_t)B * L.n_r);
   L.split_nleft.ensure(B);
-  RMG_CUDA(cudaMemsetAsync(L.split_nleft.get(), 0, L.split_nleft.bytes(), c.stream));
-  // single-copy rows over the tiles, the rows that this left, then the rows of shared nodes over
-  // the group slots; all grids are one resident wave
+  L.split_direct.ensure(L.nreg);
+  if (!L.split_any.get()) {
+    L.split_any.alloc(2);
+    RMG_CUDA(cudaMemsetAsync(L.split_any.get(), 0, L.split_any.bytes(), c.stream));
+  }
+  const int call = ++L.split_call;
+  // the form of the regions, single-copy rows over the tiles, the rows that this left and the
+  // regions that it did not take, then the rows of shared nodes over the group slots; all grids
+  // are one resident wave (the second half of the rows' blocks mostly has nothing to do)
+  const int gf = persistent_grid(c, (L.nreg + 7) / 8);
 #define RMG_SPLIT_ARGS                                                                     \
   L.gid.get(), L.mult.get(), L.c2r.get(), L.cgrp.get(), L.gptr.get(), L.gslot.get(),        \
       L.rid.get(), L.affine.get(), rowptr, col, val, L.ncomp, L.coef.get(), c.d_err.get()
 #define RMG_SPLIT(K, BB)                                                                    \
   do {                                                                                      \
+    k_split_forms<K, BB><<<gf, 256, 0, c.stream>>>(                                         \
+        L.nreg, L.regions.get(), L.gid.get(), L.mult.get(), L.affine.get(), rowptr, col,    \
+        L.split_direct.get(), L.split_any.get(), call, L.split_nleft.get());                \
+    RMG_LAUNCHED();                                                                         \
     /* blocks of half a tile; eight fit an SM with 27 KB of shared memory each */           \
     const dim3 gd(persistent_grid(c, 2 * G.ntiles), B);                                     \
     k_split_direct<K, BB><<<gd, kTile / 2, 0, c.stream>>>(                                  \
-        G, L.gid.get(), L.mult.get(), L.affine.get(), rowptr, col, val, L.coef.get(),       \
-        L.split_left.get(), L.split_nleft.get());                                           \
+        G, L.gid.get(), L.mult.get(), L.affine.get(), L.split_direct.get(), rowptr, col,    \
+        val, L.coef.get(), L.split_left.get(), L.split_nleft.get(), L.split_any.get(), call); \
     RMG_LAUNCHED();                                                                         \
-    const dim3 gb(persistent_grid(c, G.ntiles, resident_per_sm((const void*)k_split_rows<K, BB>)), \
-                  B);                                                                       \
-    k_split_rows<K, BB><<<gb, kTile, 0, c.stream>>>(L.split_left.get(), L.split_nleft.get(), \
-                                                    L.regions.get(), L.n_r, RMG_SPLIT_ARGS); \
+    const void* rows = (const void*)k_split_rows<K, BB>;                                    \
+    const dim3 gb(persistent_grid(c, G.ntiles, resident_per_sm(rows)), B, 2);               \
+    k_split_rows<K, BB><<<gb, kTile, 0, c.stream>>>(                                        \
+        G, L.split_direct.get(), L.split_left.get(), L.split_nleft.get(), L.split_any.get(), \
+        call, RMG_SPLIT_ARGS);                                                              \
     RMG_LAUNCHED();                                                                         \
     if (L.nslots) {                                                                         \
       const dim3 gs(persistent_grid(c, (L.nslots + kTile - 1) / kTile,                      \
@@ -898,6 +988,7 @@ void split_from_csr(Ctx& c, Level& L, int kind, int B, const int64_t* rowptr, co
                     B);                                                                     \
       k_split_shared<K, BB><<<gs, kTile, 0, c.stream>>>(L.nslots, L.regions.get(), L.n_r,   \
                                                         RMG_SPLIT_ARGS);                    \
+      RMG_LAUNCHED();                                                                       \
     }                                                                                       \
   } while (0)
   switch (kind) {
@@ -908,7 +999,6 @@ void split_from_csr(Ctx& c, Level& L, int kind, int B, const int64_t* rowptr, co
   }
 #undef RMG_SPLIT
 #undef RMG_SPLIT_ARGS
-  RMG_LAUNCHED();
   c.check_device_error("rmg_operator_from_csr");
 }
 

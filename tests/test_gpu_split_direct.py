@@ -75,3 +75,30 @@ def test_forms_of_a_row(name):
     expect[0, 0, 0, where[g]] = val[k] + val[k + B]
     expect[0, 0, 1, where[g]] = 0.0
     assert np.array_equal(got, expect)
+
+
+@pytest.mark.parametrize("name", list(PROBLEMS))
+def test_orders_of_a_row(name):
+    """Orders that programs write rows in: the same bits in single-copy rows, whose entries each
+    have a slot of their own, and sums in another order in shared ones."""
+    from paper_2103_11962_gb300 import rmg
+    make, kind, B = PROBLEMS[name]
+    p = make()
+    A = p.A.tocsr()
+    A.sort_indices()
+    rp, col, val = A.indptr.astype(np.int64), A.indices.astype(np.int64), A.data.copy()
+    val *= 1.0 + 1e-6 * np.random.default_rng(3).uniform(-1.0, 1.0, val.size)
+    gids = torch.from_numpy(np.asarray(p.region_gids, dtype=np.int64)).cuda()
+    ctx = rmg.Context(0)
+    want = _split(ctx, p, kind, B, rp, col, val, gids)
+    single = np.bincount(p.region_gids, minlength=p.n_nodes)[p.region_gids] == 1
+    row = np.repeat(np.arange(rp.size - 1), np.diff(rp))
+    swap = col.copy()                          # the last two entries of a row change places
+    swap[rp[1:] - 1], swap[rp[1:] - 2] = col[rp[1:] - 2], col[rp[1:] - 1]
+    orders = {"diagonal first": col != row, "diagonal last": col == row, "descending": -col,
+              "by component": col % B, "last two": swap}
+    for order, key in orders.items():
+        o = np.lexsort((col, key, row)) if order != "last two" else np.lexsort((swap, row))
+        got = _split(ctx, p, kind, B, rp, np.ascontiguousarray(col[o]), val[o], gids)
+        assert np.array_equal(got[..., single], want[..., single]), order
+        assert np.abs(got - want).max() <= 81 * 2.0 ** -52 * np.abs(val).max(), order
