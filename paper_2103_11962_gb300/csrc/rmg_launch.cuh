@@ -57,12 +57,25 @@ inline int resident_per_sm_smem(const void* kernel, int smem) {
   return b;
 }
 
-// Whether the kernels of a level are short enough to be launched with `next` below. Next to long
-// ones the waiting blocks are in the way: with it on every level, steps of 34M unknowns (27-point)
-// and of 6.3M (elasticity) took 125.2 and 71.4 ms against 120.5 and 68.9 without, a step of 5.8M
-// (7-point, 42M coefficients on level 0) the same, and small solves gained 10%.
-inline bool short_kernels(const Level& L) {
-  return (long long)L.n_r * L.kind * L.B * L.B <= 40000000;
+// Whether the kernels of a level are launched with `next` below.
+// In a graph, where the gaps between kernels are short already, up to 1.5M coefficients (a read of
+// 12 MB in FP64, 3 to 6 us): next to longer kernels the waiting blocks are in the way. FP64 V-cycles
+// with and without it on level 0, us: 672k nodes of 5 points (3.4M) 352 and 320, 1.33M of 7 (9.3M)
+// 507 and 483, 256k of 27 (6.9M) 332 and 269.
+// In a stream up to 40M: the power method of 3.1M nodes with 7 points gains 4 us a sweep, at 42M a
+// solve with 7 points is level, at 970M one with 27 loses 4%. Except, for a product over run tiles,
+// where its grid is smaller than a wave and its rows are long, because the blocks are placed where
+// those of the running kernel end first, and some SMs then get more of them than others. Products,
+// us, with and without: 27 points, 74k nodes (2.0M, two blocks an SM) 8.7 and 12.4, 81k 15.5 and
+// 12.4, 166k (0.53 of a wave) 15.6 and 12.5, 216k (0.69) 17.5 and 18.6, 678k 44.2 and 47.6; 7 points,
+// 333k nodes 8.1 and 12.4, 1.33M 26.1 and 29.4; blocks of 3 on 27 points, 8k nodes (1.9M) 21.6 and
+// 24.7, 22k 22.8 and 20.6, 44k 40.2 and 39.1, 169k 108 and 97, 333k 162 and 156.
+inline bool short_kernels(const Level& L, bool product = false) {
+  const int row = L.kind * L.B * L.B;
+  const long long coefs = (long long)L.n_r * row;
+  if (g_capturing) return coefs <= 1500000;
+  if (!product || coefs <= 2000000) return coefs <= 40000000;
+  return coefs <= 40000000 && (row < 27 || (row == 27 && L.n_r >= 200000));
 }
 
 // kernel<<<grid, block, smem, st>>>(args...) for a kernel that starts with follow(). With `next`,
@@ -95,11 +108,11 @@ void launch_resident(const Ctx& c, bool next, void (*kernel)(P...), int work, cu
 // Phase B alone (scalar levels): one thread per copy of every interface group.
 template <typename AT, class Epi>
 void launch_groups(Ctx& c, const Level& L, const AT* y, Epi epi, cudaStream_t st,
-                   bool next = true) {
+                   bool next = true, bool product = false) {
   if (!L.ngroups) return;
   const int gs = persistent_grid(c, (L.nslots + 255) / 256);
-  launch_after(next && short_kernels(L), k_groups<AT, Epi>, dim3(gs), 256, 0, st, L.nslots, L.slots.get(), L.gslot.get(), y,
-              epi);
+  launch_after(next && short_kernels(L, product), k_groups<AT, Epi>, dim3(gs), 256, 0, st,
+               L.nslots, L.slots.get(), L.gslot.get(), y, epi);
   RMG_LAUNCHED();
 }
 
@@ -139,7 +152,7 @@ void launch_stencil(Ctx& c, const Level& L, const CT* coef, const VT* u, AT* y, 
   if (G.lx == -3 && ((reinterpret_cast<uintptr_t>(u) | reinterpret_cast<uintptr_t>(half)) & 15))
     G = L.grid();
   const int gb = persistent_grid(c, G.ntiles);
-  const bool next = !ev0 && short_kernels(L);
+  const bool product = sweep == nullptr, next = !ev0 && short_kernels(L, product);
   // external record nodes when capturing, so the events can be timed after a graph replay
   if (ev0) RMG_CUDA(cudaEventRecordWithFlags(ev0, st, g_capturing ? cudaEventRecordExternal : 0));
   bool done = false;
@@ -151,7 +164,8 @@ void launch_stencil(Ctx& c, const Level& L, const CT* coef, const VT* u, AT* y, 
       const int smem = kStSmemFloats * (int)sizeof(float);
       const auto kern = k_stencil_half27_staged<Epi>;
       const int g = persistent_grid(c, G.ntiles, resident_per_sm_smem((const void*)kern, smem));
-      launch_after(next, kern, dim3(g), kStX * kStY, smem, st, G, coef, half, asym, u, L.mult.get(), y, epi);
+      launch_after(next, kern, dim3(g), kStX * kStY, smem, st, G, coef, half, asym, u,
+                   L.mult.get(), y, epi);
       done = true;
     } else if (half && L.B == 1) {
       RMG_REQUIRE(asym != nullptr, RMG_ERR_STATE, "half planes without their flag");
@@ -191,11 +205,11 @@ void launch_stencil(Ctx& c, const Level& L, const CT* coef, const VT* u, AT* y, 
   if (launches) ++*launches;
   if (L.ngroups) {
     if (L.B == 1) {
-      launch_groups(c, L, y, epi, st, !ev1);
+      launch_groups(c, L, y, epi, st, !ev1, product);
     } else {
       const int gg = persistent_grid(c, (L.nslots + 255) / 256);
-      launch_after(!ev1 && short_kernels(L), k_groups_b<AT, Epi>, dim3(gg), 256, 0, st, L.nslots, L.B, L.n_r, L.slots.get(),
-                  L.gslot.get(), (const AT*)y, epi);
+      launch_after(!ev1 && short_kernels(L, product), k_groups_b<AT, Epi>, dim3(gg), 256, 0, st,
+                   L.nslots, L.B, L.n_r, L.slots.get(), L.gslot.get(), (const AT*)y, epi);
       RMG_LAUNCHED();
     }
     if (launches) ++*launches;
