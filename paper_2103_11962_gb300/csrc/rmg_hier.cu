@@ -1370,20 +1370,45 @@ static bool coarse_factor_mixed(Hier& h, int nd) {
   return true;
 }
 
-// FP32 copy of the level-0 coefficients for the mixed hierarchy's FP32 Galerkin chain.
-static void level0_to_fp32(Hier& h) {
+// Memory for the half planes of level 0, or none (half_on off). Those of a block operator add 504
+// bytes a node of 27 points to about 3500: they are left out where the device would not keep as
+// much memory free as they take, so that what fits without them still does.
+static void half_reserve(Hier& h) {
+  const Level& L = *h.lv[0];
+  const size_t count = (size_t)L.B * L.B * ((L.kind + 1) / 2) * L.n_r;
+  if (h.half32.n == count) return;
+  if (L.B > 1) {
+    size_t free = 0, total = 0;
+    RMG_CUDA(cudaMemGetInfo(&free, &total));
+    h.half_on = free >= 2 * count * sizeof(float);
+    if (!h.half_on) return;
+  }
+  h.half32.alloc(count);
+}
+
+// Regions whose flags of the last level0_pass are clear (synchronises for a block operator).
+static void count_half_regions(Hier& h) {
+  const Level& L = *h.lv[0];
+  std::vector<int> asym(L.nreg, h.hsc.half_asym);
+  if (L.B > 1) {
+    RMG_CUDA(cudaMemcpyAsync(asym.data(), h.half_regions.get(), L.nreg * sizeof(int),
+                             cudaMemcpyDeviceToHost, h.c->stream));
+    RMG_CUDA(cudaStreamSynchronize(h.c->stream));
+  }
+  h.half_count = 0;
+  h.half_nodes = 0;
+  for (int r = 0; r < L.nreg; ++r)
+    if (!asym[r]) {
+      ++h.half_count;
+      h.half_nodes += L.hoff[r + 1] - L.hoff[r];
+    }
+}
+
+// FP32 coefficients of level 0, their half planes (where there is memory for them) and the flags
+// that say where these hold the operator, in one pass.
+static void level0_pass(Hier& h) {
   Ctx& c = *h.c;
   Level& L = *h.lv[0];
-  if (!h.half_on) {
-    const size_t nco = (size_t)L.B * L.B * L.kind * L.n_r;
-    const int g = persistent_grid(c, (int)std::min<size_t>((nco + 255) / 256, 1 << 20));
-    k_convert<double, float><<<g, 256, 0, c.stream>>>(nco, L.coef.get(), L.coef32.get());
-    RMG_LAUNCHED();
-    return;
-  }
-  // with the FP32 cycle's half planes and the flag that says whether they hold the operator,
-  // in the same pass
-  h.half32.ensure((size_t)L.B * L.B * ((L.kind + 1) / 2) * L.n_r);
   int* flag = &h.sc.get()->half_asym;
   RMG_CUDA(cudaMemsetAsync(flag, 0, sizeof(int), c.stream));
   if (L.B > 1) {
@@ -1405,22 +1430,27 @@ static void level0_to_fp32(Hier& h) {
   RMG_LAUNCHED();
 }
 
-// Regions whose flags of the last level0_to_fp32 are clear (synchronises for a block operator).
-static void count_half_regions(Hier& h) {
-  const Level& L = *h.lv[0];
-  std::vector<int> asym(L.nreg, h.hsc.half_asym);
-  if (L.B > 1) {
-    RMG_CUDA(cudaMemcpyAsync(asym.data(), h.half_regions.get(), L.nreg * sizeof(int),
-                             cudaMemcpyDeviceToHost, h.c->stream));
-    RMG_CUDA(cudaStreamSynchronize(h.c->stream));
+// FP32 copy of the level-0 coefficients for the mixed hierarchy's FP32 Galerkin chain, with the
+// half planes of the FP32 cycle beside it.
+static void level0_to_fp32(Hier& h) {
+  Ctx& c = *h.c;
+  Level& L = *h.lv[0];
+  if (h.half_on && !h.half_none) half_reserve(h);
+  if (!h.half_on) {
+    const size_t nco = (size_t)L.B * L.B * L.kind * L.n_r;
+    const int g = persistent_grid(c, (int)std::min<size_t>((nco + 255) / 256, 1 << 20));
+    k_convert<double, float><<<g, 256, 0, c.stream>>>(nco, L.coef.get(), L.coef32.get());
+    RMG_LAUNCHED();
+    return;
   }
-  h.half_count = 0;
-  h.half_nodes = 0;
-  for (int r = 0; r < L.nreg; ++r)
-    if (!asym[r]) {
-      ++h.half_count;
-      h.half_nodes += L.hoff[r + 1] - L.hoff[r];
-    }
+  level0_pass(h);
+  if (!h.half_none) return;
+  // without the planes the pass only compared: fill them when a region now is symmetric
+  count_half_regions(h);
+  if (!h.half_count) return;
+  h.half_none = false;
+  half_reserve(h);
+  if (h.half_on) level0_pass(h);
 }
 
 // The mixed cycle's remaining copies: FP32 D~^-1 on every level and, for the BF16 variant, the
@@ -1595,9 +1625,14 @@ void hier_numeric(Hier& h) {
   coarse_factor(h);
   RMG_CUDA(cudaMemcpyAsync(&h.hsc, h.sc.get(), sizeof(Scalars), cudaMemcpyDeviceToHost, c.stream));
   RMG_CUDA(cudaStreamSynchronize(c.stream));
-  if (h.half_on) count_half_regions(h);
+  if (h.half32.get()) {
+    count_half_regions(h);
+    h.half_none = L0.B > 1 && h.half_count == 0;
+    if (h.half_none) h.half32.release();     // no sweep reads them
+  }
   const std::vector<char>& stored = h.stored;
-  if (h.gexec && (stored != h.graph_stored || h.coarse_refine != h.graph_refine)) {
+  if (h.gexec && (stored != h.graph_stored || h.coarse_refine != h.graph_refine ||
+                  h.half(0) != h.graph_half)) {
     cudaGraphExecDestroy(h.gexec);
     cudaGraphDestroy(h.graph);
     h.gexec = nullptr;
@@ -1605,6 +1640,7 @@ void hier_numeric(Hier& h) {
   }
   h.graph_stored = stored;
   h.graph_refine = h.coarse_refine;
+  h.graph_half = h.half(0);
   if (h.o.use_graph && !h.gexec && h.dense_ok) {
     if (!h.graph_stream) RMG_CUDA(cudaStreamCreateWithFlags(&h.graph_stream, cudaStreamNonBlocking));
     RMG_CUDA(cudaStreamBeginCapture(h.graph_stream, cudaStreamCaptureModeThreadLocal));

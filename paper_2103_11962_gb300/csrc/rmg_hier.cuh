@@ -96,10 +96,12 @@ struct Hier {
   // FP32 cycle: level 0 also as half planes (k_level0_fp32), read by the sweeps while the device
   // flag Scalars::half_asym is 0 (block operators: in the regions whose flag is 0)
   bool half_on = false;
-  DBuf<float> half32;
+  DBuf<float> half32;                        // empty: the full planes only
   DBuf<int> half_regions;
   int half_count = 0;                        // regions on the half form, and their nodes
   long long half_nodes = 0;
+  bool half_none = false;                    // the last block operator had none: planes released
+  const float* graph_half = nullptr;         // half planes the graph was captured with
   // coarse end of the cycle in one kernel (rmg_tail.cu): first level it takes (-1: none), whether
   // the dense solve is inside, the cluster's blocks, and geometry per level
   int tail0 = -1;

@@ -276,7 +276,7 @@ k_rap_last(Grid Gc, const RegionDev* __restrict__ regs2, int n2, const T* __rest
 // inside a region differs in any bit (the sweeps then keep reading the full planes); the pair's
 // far value is rounded here from its FP64 value, the same rounding that made the copy.
 // With B > 1 (blockIdx.y = block c * B + c') the mirror of block (c, c') is block (c', c), and
-// region_asym (zeroed before) says it for every region.
+// region_asym (zeroed before) says it for every region. Without `half` the pass only compares.
 template <int KIND, int B>
 __global__ void __launch_bounds__(kTile)
 k_level0_fp32(Grid G, const double* __restrict__ coef, float* __restrict__ coef32,
@@ -299,7 +299,7 @@ k_level0_fp32(Grid G, const double* __restrict__ coef, float* __restrict__ coef3
       const float cv = static_cast<float>(own[(size_t)s * G.n_r + n]);
       own32[(size_t)s * G.n_r + n] = cv;
       if (s < C) continue;
-      ownh[(size_t)(s - C) * G.n_r + n] = cv;
+      if (half) ownh[(size_t)(s - C) * G.n_r + n] = cv;
       const int dx = S::dx(s), dy = S::dy(s), dz = S::dz(s);
       bool ok = s > C;
       if (dx < 0) ok &= (i > 0);

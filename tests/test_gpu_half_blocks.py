@@ -70,3 +70,89 @@ def test_half_regions_are_counted_one_by_one():
             break
     assert numbers(val) == ((1, int(sizes[0])), (0, 0), 243)
     assert numbers(dp.val, rmg.FP64) == ((0, 0), (0, 0), 243)
+
+
+def _asymmetric(p, dp, regions):
+    """The matrix with one coupling inside each of the regions moved in its last bits."""
+    import numpy as np
+    val = dp.val.clone()
+    rp = dp.rowptr.cpu().numpy()
+    inner = np.bincount(p.region_gids, minlength=p.n_nodes) == 1
+    off = np.concatenate([[0], np.cumsum(np.prod(np.asarray(p.region_dims), axis=1))])
+    for r in regions:
+        own = p.region_gids[off[r]:off[r + 1]]
+        for g in own[inner[own]]:
+            cols = dp.col[int(rp[3 * g]):int(rp[3 * g + 1])].cpu().numpy()
+            k = np.flatnonzero(inner[cols // 3] & (cols // 3 != g))
+            if k.size:
+                val[int(rp[3 * g]) + int(k[0])] *= 1.0 + 2.0 ** -20
+                break
+    return val
+
+
+def test_half_planes_go_when_no_region_uses_them():
+    """A hierarchy whose operator turns asymmetric in every region gives the memory of its half
+    planes back, and takes it again when a region turns symmetric; the cycle stays that of the
+    full planes."""
+    from paper_2103_11962_gb300 import rmg, upload
+    p = W.elasticity3d(region_grid=(2, 1, 1), choices=(28,), seed=5)
+    dp = upload(p)
+    ctx = rmg.Context(0)
+    lay = rmg.Layout(ctx, 3, p.region_dims, dp.gids, p.n_nodes, dp.dirichlet)
+    lay.operator_from_block_csr(27, 3, dp.rowptr, dp.col, dp.val)
+    opts = dict(levels=2, smoother=rmg.CHEBYSHEV, nu1=1, nu2=1, precision=rmg.FP32)
+    h = rmg.Hierarchy(lay, rmg.default_options(symmetric_storage=1, **opts))
+    full = rmg.Hierarchy(lay, rmg.default_options(symmetric_storage=0, **opts))
+    size = 4 * 126 * p.n_regional_nodes
+    steps = [(0, 1), (0, 1), (1,), (), (0, 1)]
+    vals = [_asymmetric(p, dp, moved) for moved in steps]
+    z = [torch.empty_like(dp.b) for _ in range(2)]
+    free = torch.cuda.mem_get_info()[0]        # with the planes, and all tensors of this test
+    for moved, val in zip(steps, vals):
+        lay.operator_from_block_csr(27, 3, dp.rowptr, dp.col, val)
+        h.setup_numeric()
+        full.setup_numeric()
+        assert h.half_regions(0)[0] == 2 - len(moved)
+        # device memory comes in granules of up to 2 MB; the planes take 22
+        gained = torch.cuda.mem_get_info()[0] - free
+        assert abs(gained - (size if len(moved) == 2 else 0)) <= 2 ** 23
+        h.vcycle(dp.b, z[0])
+        full.vcycle(dp.b, z[1])
+        assert torch.equal(z[0], z[1])
+
+
+def test_no_half_planes_where_memory_is_short():
+    """Half planes of a block operator that would not leave as much memory free as they take are
+    not made: what fits without them still does, with the same results."""
+    from paper_2103_11962_gb300 import rmg, upload
+    p = W.elasticity3d(region_grid=(2, 2, 1), choices=(28,), seed=6)
+    dp = upload(p)
+    ctx = rmg.Context(0)
+    lay = rmg.Layout(ctx, 3, p.region_dims, dp.gids, p.n_nodes, dp.dirichlet)
+    lay.operator_from_block_csr(27, 3, dp.rowptr, dp.col, dp.val)
+    opts = rmg.default_options(levels=2, smoother=rmg.CHEBYSHEV, nu1=1, nu2=1, precision=rmg.FP32)
+    size = 4 * 126 * p.n_regional_nodes
+    want, got = torch.empty_like(dp.b), torch.empty_like(dp.b)
+    for _ in range(2):                         # the first time loads kernels as well
+        torch.cuda.synchronize()
+        torch.cuda.empty_cache()
+        before = torch.cuda.mem_get_info()[0]
+        h = rmg.Hierarchy(lay, opts)
+        assert h.half_regions(0)[0] == 4
+        h.vcycle(dp.b, want)
+        torch.cuda.synchronize()
+        took = before - torch.cuda.mem_get_info()[0]
+        h.close()
+    # all but what the hierarchy takes and half of its half planes
+    left = torch.cuda.mem_get_info()[0] - took - size // 2
+    held = torch.empty(left, dtype=torch.uint8, device="cuda")
+    h = rmg.Hierarchy(lay, opts)
+    assert h.half_regions(0) == (0, 0) and h.coef_planes(0) == 243
+    h.vcycle(dp.b, got)
+    assert torch.equal(got, want)
+    h.setup_numeric()                          # decided once: later setups change nothing
+    assert h.half_regions(0) == (0, 0)
+    h.vcycle(dp.b, got)
+    assert torch.equal(got, want)
+    del held
+    torch.cuda.empty_cache()
