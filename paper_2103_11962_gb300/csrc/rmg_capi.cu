@@ -171,7 +171,7 @@ rmg_status rmg_operator_from_csr(rmg_layout* lay, int stencil, const int64_t* ro
                                  const int64_t* col, const double* val) {
   if (!lay) return RMG_ERR_ARG;
   return guarded(lay->ctx, [&] {
-    split_from_csr(lay->ctx->c, lay->L0, stencil, 1, rowptr, col, val);
+    split_from_csr(lay->ctx->c, lay->L0, stencil, 1, rowptr, col, val, lay->ybuf);
     lay->has_operator = true;
   });
 }
@@ -181,8 +181,7 @@ rmg_status rmg_operator_from_block_csr(rmg_layout* lay, int stencil, int dofs_pe
                                        const double* val) {
   if (!lay) return RMG_ERR_ARG;
   return guarded(lay->ctx, [&] {
-    split_from_csr(lay->ctx->c, lay->L0, stencil, dofs_per_node, rowptr, col, val);
-    lay->ybuf.ensure((size_t)dofs_per_node * lay->L0.n_r);
+    split_from_csr(lay->ctx->c, lay->L0, stencil, dofs_per_node, rowptr, col, val, lay->ybuf);
     lay->has_operator = true;
   });
 }
@@ -208,8 +207,7 @@ rmg_status rmg_operator_from_host_csr(rmg_layout* lay, int stencil, int dofs_per
     copy_host_array(lay->csr_col.get(), col, nnz * sizeof(int64_t), st, nsm);
     copy_host_array(lay->csr_val.get(), val, nnz * sizeof(double), st, nsm);
     split_from_csr(lay->ctx->c, lay->L0, stencil, dofs_per_node, lay->csr_rowptr.get(),
-                   lay->csr_col.get(), lay->csr_val.get());
-    lay->ybuf.ensure((size_t)dofs_per_node * lay->L0.n_r);
+                   lay->csr_col.get(), lay->csr_val.get(), lay->ybuf);
     lay->has_operator = true;
   });
 }

@@ -853,7 +853,7 @@ void hier_build(Hier& h) {
   RMG_CUDA(cudaMemsetAsync(h.sc.get(), 0, sizeof(Scalars), c.stream));
   const int n0 = h.lv[0]->B * h.lv[0]->n_r;
   h.x.alloc(n0); h.p.alloc(n0); h.q.alloc(n0); h.tmp.alloc(n0);
-  h.r.alloc(n0); h.z.alloc(n0); h.zold.alloc(n0);
+  h.zold.alloc(n0);
   if (h.mixed()) h.zold32.alloc(n0);
   RMG_CUDA(cudaHostAlloc(&h.pinned, 64 * sizeof(double), cudaHostAllocDefault));
   RMG_CUDA(cudaEventCreate(&h.probe_ev[0]));

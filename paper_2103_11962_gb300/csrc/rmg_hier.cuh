@@ -90,7 +90,7 @@ struct Hier {
   DBuf<double> energy_part, energy_out;
   DBuf<uint8_t> accept;
   // PCG work vectors (regional, FP64)
-  DBuf<double> x, r, z, p, q, zold, tmp;
+  DBuf<double> x, p, q, zold, tmp;
   DBuf<float> zold32;                        // previous FP32 cycle output (flexible CG)
   double* pinned = nullptr;                  // host-mapped residual read-back
   // FP32 cycle: level 0 also as half planes (k_level0_fp32), read by the sweeps while the device

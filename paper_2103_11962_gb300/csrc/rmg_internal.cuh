@@ -192,8 +192,7 @@ struct Level {
   DBuf<uint8_t> split_direct;    // regions the split's direct pass takes (k_split_forms)
   DBuf<int> split_any;           // last calls in which a region was taken and was not
   int split_call = 0;
-  DBuf<int2> split_left;         // rows it left there, and their number, per row component
-  DBuf<int> split_nleft;         // (B * n_r, B)
+  DBuf<int> split_nleft;         // number of the rows it left there, per row component
   DBuf<int4> affine;             // per region {g0, gy, gz, ok}: gid = g0 + i + gy j + gz l
   // operator
   DBuf<double> coef;             // kind * n_r, slot-major
@@ -248,7 +247,7 @@ struct rmg_layout {
   rmg_ctx* ctx = nullptr;
   rmg::Level L0;
   bool has_operator = false;
-  rmg::DBuf<double> ybuf;         // interface partials for rmg_regional_apply
+  rmg::DBuf<double> ybuf;         // interface partials for rmg_regional_apply, rows the split lists
   rmg::DBuf<double> tmp;          // composite temp
   rmg::DBuf<double> apbuf;        // Galerkin-product scratch (rows of [[A]][[P]]), all hierarchies
   // device copies of a host composite CSR (rmg_operator_from_host_csr)

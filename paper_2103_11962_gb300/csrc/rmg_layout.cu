@@ -933,7 +933,7 @@ __global__ void k_reg_to_comp(int ncomp, int n_r, int B, const int* __restrict__
 }  // namespace
 
 void split_from_csr(Ctx& c, Level& L, int kind, int B, const int64_t* rowptr, const int64_t* col,
-                    const double* val) {
+                    const double* val, DBuf<double>& scratch) {
   RMG_REQUIRE(rowptr && col && val, RMG_ERR_ARG, "CSR arrays are required");
   RMG_REQUIRE((L.dim == 2 && (kind == 5 || kind == 9)) || (L.dim == 3 && (kind == 7 || kind == 27)),
               RMG_ERR_ARG, "stencil must be 5/9 in 2D and 7/27 in 3D");
@@ -949,7 +949,9 @@ void split_from_csr(Ctx& c, Level& L, int kind, int B, const int64_t* rowptr, co
     RMG_LAUNCHED();
   }
   if (L.affine.n < (size_t)L.nreg) build_affine(c, L);
-  L.split_left.ensure((size_t)B * L.n_r);
+  static_assert(sizeof(int2) == sizeof(double), "an entry of the list of rows for a double");
+  if (scratch.n < (size_t)B * L.n_r) scratch.alloc((size_t)B * L.n_r);
+  int2* left = reinterpret_cast<int2*>(scratch.get());
   L.split_nleft.ensure(B);
   L.split_direct.ensure(L.nreg);
   if (!L.split_any.get()) {
@@ -974,12 +976,12 @@ void split_from_csr(Ctx& c, Level& L, int kind, int B, const int64_t* rowptr, co
     const dim3 gd(persistent_grid(c, 2 * G.ntiles), B);                                     \
     k_split_direct<K, BB><<<gd, kTile / 2, 0, c.stream>>>(                                  \
         G, L.gid.get(), L.mult.get(), L.affine.get(), L.split_direct.get(), rowptr, col,    \
-        val, L.coef.get(), L.split_left.get(), L.split_nleft.get(), L.split_any.get(), call); \
+        val, L.coef.get(), left, L.split_nleft.get(), L.split_any.get(), call); \
     RMG_LAUNCHED();                                                                         \
     const void* rows = (const void*)k_split_rows<K, BB>;                                    \
     const dim3 gb(persistent_grid(c, G.ntiles, resident_per_sm(rows)), B, 2);               \
     k_split_rows<K, BB><<<gb, kTile, 0, c.stream>>>(                                        \
-        G, L.split_direct.get(), L.split_left.get(), L.split_nleft.get(), L.split_any.get(), \
+        G, L.split_direct.get(), left, L.split_nleft.get(), L.split_any.get(), \
         call, RMG_SPLIT_ARGS);                                                              \
     RMG_LAUNCHED();                                                                         \
     if (L.nslots) {                                                                         \
