@@ -17,6 +17,7 @@
 #include <algorithm>
 #include <vector>
 
+#include "rmg_cluster.h"
 #include "rmg_kernels.cuh"
 #include "rmg_tail.cuh"
 
@@ -560,18 +561,16 @@ void TailGeometry::build(Ctx& c, const Level& L, bool colours) {
 template <typename VT, typename CT>
 int tail_cluster(int dim, int B) {
   const KernelPtr k = tail_kernel<VT, CT>(dim, B);
-  // 16 blocks need the opt-in (an attribute of the function on the current device)
-  const bool wide = cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) ==
-                    cudaSuccess;
-  for (int cluster : {16, 8}) {
-    if (cluster == 16 && !wide) continue;
+  auto allow_wide = [&] {            // an attribute of the function on the current device
+    return cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) ==
+           cudaSuccess;
+  };
+  auto active = [&](int cluster, int* count) {
     cudaLaunchAttribute attr;
     const cudaLaunchConfig_t cfg = tail_config(cluster, &attr, nullptr);
-    int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, k, &cfg) == cudaSuccess && n > 0) return cluster;
-  }
-  cudaGetLastError();
-  return 0;
+    return cudaOccupancyMaxActiveClusters(count, k, &cfg) == cudaSuccess;
+  };
+  return widest_cluster(allow_wide, active, [] { cudaGetLastError(); });
 }
 
 template <typename VT, typename CT>
