@@ -5,9 +5,10 @@
 // are the weights a fine node takes from its right coarse neighbour along x, y and z (the left
 // one gets 1 - w), so every predicted row of P sums to one and constants are preserved.
 //
-// Forward pass: BF16 tensor-core MMA (mma.sync m16n8k16, FP32 accumulate); a CTA of 8 warps
-// takes 128 samples, each warp 16 rows. Backward pass: FP32 CUDA cores on the same tile, the
-// weight gradients in registers, one atomic add per parameter per CTA. Adam updates FP32 master weights.
+// Forward pass: BF16 tensor-core MMA (mma.sync m16n8k16, FP32 accumulate). Inference: each warp
+// takes tiles of 16 samples. Training: a CTA of 16 warps takes 128 samples, a warp 16 rows and half
+// of a layer's columns; backward pass on FP32 CUDA cores over the same tile, the weight gradients
+// in registers, one atomic add per parameter per CTA. Adam updates FP32 master weights.
 //
 // Features of fine node n (9 per axis, zero along axes where n sits on a coarse index): for
 // the line of three edges between its two coarse neighbours along the axis, log10 of the three
@@ -838,8 +839,11 @@ rmg_status rmg_hier_mlp_features(rmg_hier* hh, int level, float* feats) {
     Level& L = *h.lv[level];
     const Grid G = L.grid();
     const int gb = persistent_grid(*h.c, G.ntiles);
-#define RMG_FEAT(K) \
-  k_features<K><<<gb, kTile, 0, h.c->stream>>>(G, feat_args<K>(h, level), feats)
+#define RMG_FEAT(K)                                                                            \
+  {                                                                                            \
+    const FeatArgs A = feat_args<K>(h, level);                                                 \
+    k_features<K><<<gb, kTile, 0, h.c->stream>>>(G, A, feats);                                 \
+  }
     switch (L.kind) {
       case 5: RMG_FEAT(5); break;
       case 7: RMG_FEAT(7); break;
