@@ -847,7 +847,8 @@ void hier_build(Hier& h) {
     }
   }
   // half planes for the FP32 cycle's level-0 sweeps
-  h.half_on = o.symmetric_storage != 0 && o.precision == RMG_PREC_FP32;
+  h.half_on = o.symmetric_storage != 0 && o.precision == RMG_PREC_FP32 &&
+              h.lv[0]->n_r <= kOffset32Nodes;
   if (Lv > 1) h.layout->apbuf.ensure((size_t)(h.lv[0]->dim == 3 ? 27 : 9) * h.lv[0]->n_r);
   h.sc.alloc(1);
   RMG_CUDA(cudaMemsetAsync(h.sc.get(), 0, sizeof(Scalars), c.stream));

@@ -171,11 +171,12 @@ __device__ __forceinline__ float load32(const float* base, unsigned byte) {
   const float* p = reinterpret_cast<const float*>(reinterpret_cast<const char*>(base) + byte);
   return CONST ? __ldg(p) : *p;
 }
-// Largest level whose byte offsets into one plane fit 32 bits.
+// Largest level whose byte offsets into one plane fit 32 bits; larger ones (300 GB and more with
+// their vectors) have no half planes.
 constexpr int kOffset32Nodes = 1 << 30;
 
-// The row of node n from the half planes; OFF32: n_r <= kOffset32Nodes.
-template <int KIND, bool OFF32>
+// The row of node n from the half planes.
+template <int KIND>
 __device__ __forceinline__ float stencil_row_half(const float* __restrict__ half,
                                                   const float* u, int n, int n_r,
                                                   int i, int j, int l, const RegionDev& R) {
@@ -198,9 +199,7 @@ __device__ __forceinline__ float stencil_row_half(const float* __restrict__ half
       const int nb = n + dx + dy * sy + dz * sz;
       const float* plane = half + (size_t)(s < C ? S::S - 1 - s - C : s - C) * (size_t)n_r;
       const int at = s < C ? nb : n;
-      const float c = OFF32 ? load32<true>(plane, 4u * (unsigned)at) : plane[at];
-      const float v = OFF32 ? load32<false>(u, 4u * (unsigned)nb) : u[nb];
-      au = fmaf(c, v, au);
+      au = fmaf(load32<true>(plane, 4u * (unsigned)at), load32<false>(u, 4u * (unsigned)nb), au);
     }
   }
   return au;
@@ -239,7 +238,7 @@ __device__ __forceinline__ void prefetch_tile(const Grid& G, int t, const float*
 
 // Phase A of the FP32 cycle on a level with half planes: the half form when the pack found the
 // operator symmetric (*asym == 0), else the full planes as k_stencil.
-template <bool HALF, bool OFF32, int KIND, class Epi>
+template <bool HALF, int KIND, class Epi>
 __device__ __forceinline__ void stencil_pass(const Grid& G, const float* __restrict__ coef,
                                              const float* u, const uint8_t* __restrict__ mult,
                                              float* __restrict__ y, const Epi& epi) {
@@ -247,7 +246,7 @@ __device__ __forceinline__ void stencil_pass(const Grid& G, const float* __restr
     int i, j, l;
     RMG_DECODE(i, j, l);
     const auto v = epi.load(n);
-    const float au = HALF ? stencil_row_half<KIND, OFF32>(coef, u, n, G.n_r, i, j, l, R)
+    const float au = HALF ? stencil_row_half<KIND>(coef, u, n, G.n_r, i, j, l, R)
                           : stencil_row<KIND, float, float, float>(coef, u, n, G.n_r, i, j, l, R);
     if (mult[n] > 1) y[n] = au; else epi.apply(n, v, au, 1);
 
@@ -258,14 +257,14 @@ __device__ __forceinline__ void stencil_pass(const Grid& G, const float* __restr
 // chose for EpiCheb. With the 32-bit offsets and the early epilogue loads a 27-point sweep of
 // 35.9M nodes went 857 -> 787 us (EpiCheb) and 822 -> 686 us (EpiScaled), 81 and 69 bytes a node
 // at 0.55 and 0.54 of the measured HBM rate; six blocks 798 and 708, loads after the row 823 and 719.
-template <int KIND, bool OFF32, class Epi>
+template <int KIND, class Epi>
 __global__ void __launch_bounds__(kTile, 7)
 k_stencil_half(Grid G, const float* __restrict__ coef, const float* __restrict__ half,
                const int* __restrict__ asym, const float* u, const uint8_t* __restrict__ mult,
                float* __restrict__ y, Epi epi) {
   follow();
-  if (*asym) stencil_pass<false, OFF32, KIND>(G, coef, u, mult, y, epi);
-  else stencil_pass<true, OFF32, KIND>(G, half, u, mult, y, epi);
+  if (*asym) stencil_pass<false, KIND>(G, coef, u, mult, y, epi);
+  else stencil_pass<true, KIND>(G, half, u, mult, y, epi);
 }
 
 // ---- staged 27-point half-plane sweep: region tiles in shared memory, pipelined ----------
@@ -522,7 +521,7 @@ k_bstencil(Grid G, const CT* __restrict__ coef, const VT* u,
 // (c', c), so it needs no symmetry. Same products in the same order as k_bstencil, hence the
 // same bits. The sweep is bound by HBM and this form moves 14/27 of the coefficients: 577 instead
 // of 1045 bytes a node; the mirrored ones come from L1 and L2.
-template <bool HALF, bool OFF32, int KIND, int B>
+template <bool HALF, int KIND, int B>
 __device__ __forceinline__ void bstencil_row32(const float* __restrict__ coef,
                                                const float* u, int n, int n_r, int i,
                                                int j, int l, const RegionDev& R, float (&au)[B]) {
@@ -547,8 +546,7 @@ __device__ __forceinline__ void bstencil_row32(const float* __restrict__ coef,
     float uv[B];
 #pragma unroll
     for (int c2 = 0; c2 < B; ++c2) {
-      const float* uc = u + (size_t)c2 * n_r;
-      uv[c2] = OFF32 ? load32<false>(uc, 4u * (unsigned)nb) : uc[nb];
+      uv[c2] = load32<false>(u + (size_t)c2 * n_r, 4u * (unsigned)nb);
     }
     const bool mirrored = HALF && s < C;
     const int plane = !HALF ? s : s < C ? S::S - 1 - s - C : s - C;
@@ -559,14 +557,14 @@ __device__ __forceinline__ void bstencil_row32(const float* __restrict__ coef,
       for (int c2 = 0; c2 < B; ++c2) {
         const int blk = mirrored ? c2 * B + c : c * B + c2;
         const float* p = coef + ((size_t)blk * P + plane) * n_r;
-        au[c] = fmaf(OFF32 ? load32<true>(p, 4u * (unsigned)at) : p[at], uv[c2], au[c]);
+        au[c] = fmaf(load32<true>(p, 4u * (unsigned)at), uv[c2], au[c]);
       }
   }
 }
 
 // asym[region] != 0: the region's full planes (an assembled block matrix can differ from its
 // transpose in the last bit of a few entries, and only their regions then lose the half form).
-template <int KIND, bool OFF32, int B, class Epi>
+template <int KIND, int B, class Epi>
 __global__ void __launch_bounds__(kTile)
 k_bstencil_half(Grid G, const float* __restrict__ coef, const float* __restrict__ half,
                 const int* __restrict__ asym, const float* u, const uint8_t* __restrict__ mult,
@@ -576,8 +574,8 @@ k_bstencil_half(Grid G, const float* __restrict__ coef, const float* __restrict_
     int i, j, l;
     RMG_DECODE(i, j, l);
     float au[B];
-    if (asym[tile_.region]) bstencil_row32<false, OFF32, KIND, B>(coef, u, n, G.n_r, i, j, l, R, au);
-    else bstencil_row32<true, OFF32, KIND, B>(half, u, n, G.n_r, i, j, l, R, au);
+    if (asym[tile_.region]) bstencil_row32<false, KIND, B>(coef, u, n, G.n_r, i, j, l, R, au);
+    else bstencil_row32<true, KIND, B>(half, u, n, G.n_r, i, j, l, R, au);
     if (mult[n] > 1) {
 #pragma unroll
       for (int c = 0; c < B; ++c) y[(size_t)c * G.n_r + n] = au[c];

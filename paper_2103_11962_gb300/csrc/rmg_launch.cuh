@@ -116,8 +116,8 @@ void launch_groups(Ctx& c, const Level& L, const AT* y, Epi epi, cudaStream_t st
   RMG_LAUNCHED();
 }
 
-// The half-plane sweep of an FP32 level (OFF32: 32-bit offsets, see load32).
-template <bool OFF32, class Epi>
+// The half-plane sweep of an FP32 level.
+template <class Epi>
 void launch_half(Ctx& c, const Level& L, const Grid& G, const float* coef, const float* half,
                  const int* asym, const float* u, float* y, Epi epi, cudaStream_t st, bool next) {
   const int nt = G.ntiles;
@@ -126,15 +126,15 @@ void launch_half(Ctx& c, const Level& L, const Grid& G, const float* coef, const
     launch_resident(c, next, kernel, nt, st, G, coef, half, asym, u, mu, y, epi);
   };
   if (L.B == 3) {
-    if (L.kind == 27) run(k_bstencil_half<27, OFF32, 3, Epi>);
-    else run(k_bstencil_half<9, OFF32, 3, Epi>);
+    if (L.kind == 27) run(k_bstencil_half<27, 3, Epi>);
+    else run(k_bstencil_half<9, 3, Epi>);
     return;
   }
   switch (L.kind) {
-    case 5: run(k_stencil_half<5, OFF32, Epi>); break;
-    case 7: run(k_stencil_half<7, OFF32, Epi>); break;
-    case 9: run(k_stencil_half<9, OFF32, Epi>); break;
-    default: run(k_stencil_half<27, OFF32, Epi>); break;
+    case 5: run(k_stencil_half<5, Epi>); break;
+    case 7: run(k_stencil_half<7, Epi>); break;
+    case 9: run(k_stencil_half<9, Epi>); break;
+    default: run(k_stencil_half<27, Epi>); break;
   }
 }
 
@@ -169,14 +169,12 @@ void launch_stencil(Ctx& c, const Level& L, const CT* coef, const VT* u, AT* y, 
       done = true;
     } else if (half && L.B == 1) {
       RMG_REQUIRE(asym != nullptr, RMG_ERR_STATE, "half planes without their flag");
-      if (L.n_r <= kOffset32Nodes) launch_half<true>(c, L, G, coef, half, asym, u, y, epi, st, next);
-      else launch_half<false>(c, L, G, coef, half, asym, u, y, epi, st, next);
+      launch_half(c, L, G, coef, half, asym, u, y, epi, st, next);
       done = true;
     } else if (half) {
       RMG_REQUIRE(asym != nullptr && L.B == 3 && (L.kind == 27 || L.kind == 9), RMG_ERR_STATE,
                   "half planes of a block operator need 3 dofs and a 27- or 9-point stencil");
-      if (L.n_r <= kOffset32Nodes) launch_half<true>(c, L, G, coef, half, asym, u, y, epi, st, next);
-      else launch_half<false>(c, L, G, coef, half, asym, u, y, epi, st, next);
+      launch_half(c, L, G, coef, half, asym, u, y, epi, st, next);
       done = true;
     }
   }
