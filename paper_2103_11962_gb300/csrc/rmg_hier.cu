@@ -452,9 +452,9 @@ struct Exec {
     const Grid G = h.sweep(l) ? *h.sweep(l) : L.grid();
     const int gb = persistent_grid(c(), G.ntiles);
     VT* u = cur[l];
-#define RMG_GS(K)                                                                             \
-  launch_after(short_kernels(L), k_gs_colour<K, CT, VT>, dim3(gb), kTile, 0, st, G, coef(l), V(l).r.get(), dinv(l),               \
-                                               V(l).d.get(), u, colour, omega)
+#define RMG_GS(K)                                                                              \
+  launch_after(short_kernels(L), k_gs_colour<K, CT, VT>, dim3(gb), kTile, 0, st, G, coef(l),   \
+               V(l).r.get(), dinv(l), V(l).d.get(), u, colour, omega)
     switch (L.kind) {
       case 5: RMG_GS(5); break;
       case 7: RMG_GS(7); break;
@@ -474,8 +474,8 @@ struct Exec {
       const int ncol = (L.kind == 5 || L.kind == 7) ? 2 : (L.dim == 3 ? 8 : 4);
       for (int s = 0; s < nu; ++s) {
         if (s == 0 && from_zero) {
-          launch_after(short_kernels(L), k_gs_zero<VT>, dim3(elementwise_grid(n)), 256, 0, st, n, V(l).b.get(), V(l).r.get(),
-                                                             V(l).d.get(), cur[l]);
+          launch_after(short_kernels(L), k_gs_zero<VT>, dim3(elementwise_grid(n)), 256, 0, st, n,
+                       V(l).b.get(), V(l).r.get(), V(l).d.get(), cur[l]);
           RMG_LAUNCHED();
           ++launches;
         } else {
@@ -489,8 +489,8 @@ struct Exec {
     if (h.o.smoother == RMG_SMOOTHER_JACOBI) {
       for (int s = 0; s < nu; ++s) {
         if (s == 0 && from_zero) {
-          launch_after(short_kernels(L), k_jacobi_zero<VT>, dim3(elementwise_grid(n)), 256, 0, st, n, V(l).b.get(), dinv(l), omega,
-                                                                 oth[l]);
+          launch_after(short_kernels(L), k_jacobi_zero<VT>, dim3(elementwise_grid(n)), 256, 0, st,
+                       n, V(l).b.get(), dinv(l), omega, oth[l]);
           RMG_LAUNCHED();
           ++launches;
         } else {
@@ -502,8 +502,8 @@ struct Exec {
     } else {
       for (int a = 0; a < nu; ++a) {
         if (a == 0 && from_zero) {
-          launch_after(short_kernels(L), k_cheb0_zero<VT>, dim3(elementwise_grid(n)), 256, 0, st, n, V(l).b.get(), dinv(l),
-                                                                c2(l, 0), V(l).d.get(), oth[l]);
+          launch_after(short_kernels(L), k_cheb0_zero<VT>, dim3(elementwise_grid(n)), 256, 0, st, n,
+                       V(l).b.get(), dinv(l), c2(l, 0), V(l).d.get(), oth[l]);
           RMG_LAUNCHED();
           ++launches;
         } else {
@@ -529,12 +529,12 @@ struct Exec {
     const Level& C = *h.lv[l + 1];
     const Grid Gc = C.grid();
     if (F.dim == 3)
-      launch_after(short_kernels(F), k_restrict3<VT>, dim3(persistent_grid(c(), Gc.ntiles * (kTile / 32), 12)),
-                  32 * kRestrictWarps, 0, st, Gc, F.regions.get(), r, C.mask.get(), C.mult.get(),
-                  b, y);
+      launch_after(short_kernels(F), k_restrict3<VT>,
+                   dim3(persistent_grid(c(), Gc.ntiles * (kTile / 32), 12)), 32 * kRestrictWarps, 0,
+                   st, Gc, F.regions.get(), r, C.mask.get(), C.mult.get(), b, y);
     else
-      launch_after(short_kernels(F), k_restrict2<VT>, dim3(persistent_grid(c(), Gc.ntiles)), kTile, 0, st, Gc,
-                  F.regions.get(), r, C.mask.get(), C.mult.get(), b, y);
+      launch_after(short_kernels(F), k_restrict2<VT>, dim3(persistent_grid(c(), Gc.ntiles)), kTile,
+                   0, st, Gc, F.regions.get(), r, C.mask.get(), C.mult.get(), b, y);
     RMG_LAUNCHED();
     ++launches;
   }
@@ -550,8 +550,8 @@ struct Exec {
         const Grid Gc = C.grid();
         const int gb = persistent_grid(c(), Gc.ntiles);
         auto run = [&](auto kernel) {
-          launch_after(short_kernels(F), kernel, dim3(gb), kTile, 0, st, Gc, F.regions.get(), F.n_r, pw(l), r,
-                      C.mask.get(), C.mult.get(), b, y);
+          launch_after(short_kernels(F), kernel, dim3(gb), kTile, 0, st, Gc, F.regions.get(), F.n_r,
+                       pw(l), r, C.mask.get(), C.mult.get(), b, y);
         };
         if (F.dim == 3) run(k_restrict_w<3, VT>);
         else run(k_restrict_w<2, VT>);
@@ -577,8 +577,8 @@ struct Exec {
         const Grid Gf = F.grid();
         const int gb = persistent_grid(c(), Gf.ntiles);
         auto run = [&](auto kernel) {
-          launch_after(short_kernels(F), kernel, dim3(gb), kTile, 0, st, Gf, C.regions.get(), pw(l), F.mask.get(),
-                      ubar, u);
+          launch_after(short_kernels(F), kernel, dim3(gb), kTile, 0, st, Gf, C.regions.get(), pw(l),
+                       F.mask.get(), ubar, u);
         };
         if (F.dim == 3) run(k_prolong_w<3, VT>);
         else run(k_prolong_w<2, VT>);
@@ -586,8 +586,8 @@ struct Exec {
         const Grid G1 = h.rap_x[l].grid(F.nreg);
         const int gb = persistent_grid(c(), G1.ntiles);
         auto run = [&](auto kernel) {
-          launch_after(short_kernels(F), kernel, dim3(gb), kTile, 0, st, G1, F.regions.get(), C.regions.get(),
-                      F.mask.get(), ubar, u);
+          launch_after(short_kernels(F), kernel, dim3(gb), kTile, 0, st, G1, F.regions.get(),
+                       C.regions.get(), F.mask.get(), ubar, u);
         };
         if (F.dim == 3) run(k_prolong<3, VT>);
         else run(k_prolong<2, VT>);
@@ -702,8 +702,9 @@ struct Exec {
     if (!L.ngroups) return;
     launch_groups(c(), L, (const VT*)cur[0], EpiMean<VT>{V(0).y.get()}, st);
     ++launches;
-    launch_after(short_kernels(L), k_copy_slots<VT>, dim3(persistent_grid(c(), (L.nslots + 255) / 256)), 256, 0, st, 
-        L.nslots, L.gslot.get(), V(0).y.get(), cur[0]);
+    launch_after(short_kernels(L), k_copy_slots<VT>,
+                 dim3(persistent_grid(c(), (L.nslots + 255) / 256)), 256, 0, st, L.nslots,
+                 L.gslot.get(), V(0).y.get(), cur[0]);
     RMG_LAUNCHED();
     ++launches;
   }
@@ -2009,11 +2010,12 @@ void pcg_solve(Hier& h, const double* b, double* xout, double rtol, int maxit, d
     vcycle(h);
     ++ncyc;
     if (mixed) {
-      launch_after(short_kernels(L0), k_start_dir, dim3(dg), 256, 0, st, n, L0.n_r, rvec, z32, L0.mult.get(), zscale, h.p.get(),
-                                      h.zold32.get(), arrive, sc);
+      launch_after(short_kernels(L0), k_start_dir, dim3(dg), 256, 0, st, n, L0.n_r, rvec, z32,
+                   L0.mult.get(), zscale, h.p.get(), h.zold32.get(), arrive, sc);
       RMG_LAUNCHED();
     } else {
-      launch_after(short_kernels(L0), k_cg_dot, dim3(dg), 256, 0, st, n, L0.n_r, rvec, zvec, L0.mult.get(), arrive, sc, CG_RZ);
+      launch_after(short_kernels(L0), k_cg_dot, dim3(dg), 256, 0, st, n, L0.n_r, rvec, zvec,
+                   L0.mult.get(), arrive, sc, CG_RZ);
       RMG_LAUNCHED();
       k_copy<double><<<eg, 256, 0, st>>>(n, zvec, h.p.get());
       RMG_LAUNCHED();
@@ -2026,15 +2028,16 @@ void pcg_solve(Hier& h, const double* b, double* xout, double rtol, int maxit, d
       ++it;
       launch_stencil(c, L0, L0.coef.get(), h.p.get(), h.v64[0].y.get(),
                      EpiStore<double>{h.q.get()}, st, nullptr);
-      launch_after(short_kernels(L0), k_cg_dot, dim3(dg), 256, 0, st, n, L0.n_r, h.p.get(), h.q.get(), L0.mult.get(), arrive, sc,
-                                   CG_ALPHA);
+      launch_after(short_kernels(L0), k_cg_dot, dim3(dg), 256, 0, st, n, L0.n_r, h.p.get(),
+                   h.q.get(), L0.mult.get(), arrive, sc, CG_ALPHA);
       RMG_LAUNCHED();
       if (mixed)
-        launch_after(short_kernels(L0), k_cg_update_mixed, dim3(dg), 256, 0, st, n, L0.n_r, h.p.get(), h.q.get(), L0.mult.get(), sc,
-                                              rscale, h.x.get(), rvec, r32, arrive, host_rr);
+        launch_after(short_kernels(L0), k_cg_update_mixed, dim3(dg), 256, 0, st, n, L0.n_r,
+                     h.p.get(), h.q.get(), L0.mult.get(), sc, rscale, h.x.get(), rvec, r32, arrive,
+                     host_rr);
       else
-        launch_after(short_kernels(L0), k_cg_update, dim3(dg), 256, 0, st, n, L0.n_r, h.p.get(), h.q.get(), L0.mult.get(), sc,
-                                        h.x.get(), rvec, arrive, host_rr);
+        launch_after(short_kernels(L0), k_cg_update, dim3(dg), 256, 0, st, n, L0.n_r, h.p.get(),
+                     h.q.get(), L0.mult.get(), sc, h.x.get(), rvec, arrive, host_rr);
       RMG_LAUNCHED();
       RMG_CUDA(cudaStreamSynchronize(st));
       probe_collect(h);
@@ -2060,19 +2063,22 @@ void pcg_solve(Hier& h, const double* b, double* xout, double rtol, int maxit, d
       vcycle(h);
       ++ncyc;
       if (mixed) {
-        launch_after(short_kernels(L0), k_flex_dots, dim3(dg), 256, 0, st, n, L0.n_r, rvec, z32, h.zold32.get(), L0.mult.get(),
-                                        zscale, arrive, sc);
+        launch_after(short_kernels(L0), k_flex_dots, dim3(dg), 256, 0, st, n, L0.n_r, rvec, z32,
+                     h.zold32.get(), L0.mult.get(), zscale, arrive, sc);
         RMG_LAUNCHED();
-        launch_after(short_kernels(L0), k_p_update<float>, dim3(eg), 256, 0, st, n, z32, zscale, sc, h.p.get());
+        launch_after(short_kernels(L0), k_p_update<float>, dim3(eg), 256, 0, st, n, z32, zscale, sc,
+                     h.p.get());
         RMG_LAUNCHED();
       } else {
         if (flex64)
-          launch_after(short_kernels(L0), k_cg_flex64, dim3(dg), 256, 0, st, n, L0.n_r, rvec, zvec, h.zold.get(), L0.mult.get(),
-                                          arrive, sc);
+          launch_after(short_kernels(L0), k_cg_flex64, dim3(dg), 256, 0, st, n, L0.n_r, rvec, zvec,
+                       h.zold.get(), L0.mult.get(), arrive, sc);
         else
-          launch_after(short_kernels(L0), k_cg_dot, dim3(dg), 256, 0, st, n, L0.n_r, rvec, zvec, L0.mult.get(), arrive, sc, CG_BETA);
+          launch_after(short_kernels(L0), k_cg_dot, dim3(dg), 256, 0, st, n, L0.n_r, rvec, zvec,
+                       L0.mult.get(), arrive, sc, CG_BETA);
         RMG_LAUNCHED();
-        launch_after(short_kernels(L0), k_p_update<double>, dim3(eg), 256, 0, st, n, zvec, 1.0, sc, h.p.get());
+        launch_after(short_kernels(L0), k_p_update<double>, dim3(eg), 256, 0, st, n, zvec, 1.0, sc,
+                     h.p.get());
         RMG_LAUNCHED();
       }
     }
