@@ -761,7 +761,8 @@ k_split_direct(Grid G, const int* __restrict__ gid, const uint8_t* __restrict__ 
 
 // The other single-copy rows, a warp for 32 of them: those that the direct pass listed (LISTED,
 // blockIdx.z = 0; their order in the list is of no consequence: every row writes its own slots),
-// and all of the regions that it did not take, by tiles (blockIdx.z = 1). (One loop over both took
+// and all of the regions that it did not take, by tiles (blockIdx.z = 1; without `direct`, of all
+// regions, and no list). (One loop over both took
 // 329 us instead of 299 for 4.9M nodes with 7 points, 10% more for blocks.) The CSR rows are staged
 // through shared memory nine entries at a time, the lanes copying the 32 rows' entries together
 // (mostly rows that lie side by side in the CSR); then every lane handles its own row's entries in
@@ -791,7 +792,7 @@ __device__ __forceinline__ void split_rows(const Grid& G, const uint8_t* __restr
     } else {
       const Tile tile = G.tiles[task / kWarps];
       const RegionDev R = G.regions[tile.region];
-      if (direct[tile.region]) continue;
+      if (direct && direct[tile.region]) continue;
       const int li = tile.start + (task % kWarps) * 32 + lane;
       const int n = R.off + li;
       active = li < R.nx * R.ny * R.nz && mult[n] == 1;
@@ -839,7 +840,7 @@ __device__ __forceinline__ void split_rows(const Grid& G, const uint8_t* __restr
 }
 
 template <int KIND, int B>
-__global__ void __launch_bounds__(kTile)
+__global__ void __launch_bounds__(kTile, B == 1 && KIND < 27 ? 5 : 4)
 k_split_rows(Grid G, const uint8_t* __restrict__ direct, const int2* __restrict__ left,
              const int* __restrict__ nleft, const int* __restrict__ any, int call,
              RMG_SPLIT_PARAMS) {
@@ -849,14 +850,14 @@ k_split_rows(Grid G, const uint8_t* __restrict__ direct, const int2* __restrict_
   __shared__ int64_t s_e0[kWarps][32];           // first entry and length of every lane's row
   __shared__ int s_len[kWarps][32];
   const int w = threadIdx.x >> 5;
-  if (blockIdx.z == 0)
+  if (direct && blockIdx.z == 0)
     split_rows<KIND, B, true>(G, direct, left, nleft, false, s_col[w], s_val[w], s_e0[w], s_len[w],
                               gid, mult, c2r, cgrp, gptr, gslot, rid, affine, rowptr, col, val,
                               ncomp, coef, err);
   else
-    split_rows<KIND, B, false>(G, direct, left, nleft, any[1] == call, s_col[w], s_val[w], s_e0[w],
-                               s_len[w], gid, mult, c2r, cgrp, gptr, gslot, rid, affine, rowptr,
-                               col, val, ncomp, coef, err);
+    split_rows<KIND, B, false>(G, direct, left, nleft, !direct || any[1] == call, s_col[w],
+                               s_val[w], s_e0[w], s_len[w], gid, mult, c2r, cgrp, gptr, gslot, rid,
+                               affine, rowptr, col, val, ncomp, coef, err);
 }
 
 // Rows of shared nodes, one thread per regional copy, in group-slot order (the copies of one
@@ -963,26 +964,35 @@ void split_from_csr(Ctx& c, Level& L, int kind, int B, const int64_t* rowptr, co
   // regions that it did not take, then the rows of shared nodes over the group slots; all grids
   // are one resident wave (the second half of the rows' blocks mostly has nothing to do)
   const int gf = persistent_grid(c, (L.nreg + 7) / 8);
+  // Small matrices: all single-copy rows by tiles in one launch. The direct pass's three launches and
+  // the latency of its short list cost more than it saves up to about 1M nodes of 5 to 9 points, 100k
+  // of 27 and 100k of blocks of 3. Split, us, by tiles and with the direct pass: 7 points, 1.02M nodes
+  // 105 and 109, 4.9M 330 and 282; 5 points, 0.97M 83 and 90; 27 points, 85k 48 and 54, 166k 70 and 68,
+  // 333k 170 and 144; blocks on 27 points, 22k 115 and 136, 379k 1210 and 1046.
+  const int row = kind * B * B;
+  const bool tiles = (long long)L.n_r * row < (B > 1 ? 24000000 : kind == 27 ? 4000000 : 8000000);
+  const uint8_t* direct = tiles ? nullptr : L.split_direct.get();
 #define RMG_SPLIT_ARGS                                                                     \
   L.gid.get(), L.mult.get(), L.c2r.get(), L.cgrp.get(), L.gptr.get(), L.gslot.get(),        \
       L.rid.get(), L.affine.get(), rowptr, col, val, L.ncomp, L.coef.get(), c.d_err.get()
 #define RMG_SPLIT(K, BB)                                                                    \
   do {                                                                                      \
-    k_split_forms<K, BB><<<gf, 256, 0, c.stream>>>(                                         \
-        L.nreg, L.regions.get(), L.gid.get(), L.mult.get(), L.affine.get(), rowptr, col,    \
-        L.split_direct.get(), L.split_any.get(), call, L.split_nleft.get());                \
-    RMG_LAUNCHED();                                                                         \
-    /* blocks of half a tile; eight fit an SM with 27 KB of shared memory each */           \
-    const dim3 gd(persistent_grid(c, 2 * G.ntiles), B);                                     \
-    k_split_direct<K, BB><<<gd, kTile / 2, 0, c.stream>>>(                                  \
-        G, L.gid.get(), L.mult.get(), L.affine.get(), L.split_direct.get(), rowptr, col,    \
-        val, L.coef.get(), left, L.split_nleft.get(), L.split_any.get(), call); \
-    RMG_LAUNCHED();                                                                         \
+    if (!tiles) {                                                                           \
+      k_split_forms<K, BB><<<gf, 256, 0, c.stream>>>(                                       \
+          L.nreg, L.regions.get(), L.gid.get(), L.mult.get(), L.affine.get(), rowptr, col,  \
+          L.split_direct.get(), L.split_any.get(), call, L.split_nleft.get());              \
+      RMG_LAUNCHED();                                                                       \
+      /* blocks of half a tile; eight fit an SM with 27 KB of shared memory each */         \
+      const dim3 gd(persistent_grid(c, 2 * G.ntiles), B);                                   \
+      k_split_direct<K, BB><<<gd, kTile / 2, 0, c.stream>>>(                                \
+          G, L.gid.get(), L.mult.get(), L.affine.get(), direct, rowptr, col, val,           \
+          L.coef.get(), left, L.split_nleft.get(), L.split_any.get(), call);                \
+      RMG_LAUNCHED();                                                                       \
+    }                                                                                       \
     const void* rows = (const void*)k_split_rows<K, BB>;                                    \
-    const dim3 gb(persistent_grid(c, G.ntiles, resident_per_sm(rows)), B, 2);               \
-    k_split_rows<K, BB><<<gb, kTile, 0, c.stream>>>(                                        \
-        G, L.split_direct.get(), left, L.split_nleft.get(), L.split_any.get(), \
-        call, RMG_SPLIT_ARGS);                                                              \
+    const dim3 gb(persistent_grid(c, G.ntiles, resident_per_sm(rows)), B, tiles ? 1 : 2);   \
+    k_split_rows<K, BB><<<gb, kTile, 0, c.stream>>>(G, direct, left, L.split_nleft.get(),    \
+                                                    L.split_any.get(), call, RMG_SPLIT_ARGS); \
     RMG_LAUNCHED();                                                                         \
     if (L.nslots) {                                                                         \
       const dim3 gs(persistent_grid(c, (L.nslots + kTile - 1) / kTile,                      \

@@ -102,3 +102,52 @@ def test_orders_of_a_row(name):
         got = _split(ctx, p, kind, B, rp, np.ascontiguousarray(col[o]), val[o], gids)
         assert np.array_equal(got[..., single], want[..., single]), order
         assert np.abs(got - want).max() <= 81 * 2.0 ** -52 * np.abs(val).max(), order
+
+
+# sizes that the direct pass takes, with the rows it lists and the regions it leaves
+LARGE = {
+    "5-point": (lambda: W.poisson2d_5pt(region_grid=(14, 14), n=91), 5, 1, 8000000),
+    "9-point": (lambda: W.q1_laplace2d(region_grid=(10, 11), n=91), 9, 1, 8000000),
+    "7-point": (lambda: W.diffusion3d_7pt(region_grid=(4, 4, 3), choices=(31,), seed=2), 7, 1,
+                8000000),
+    "27-point": (lambda: W.q1_laplace3d(region_grid=(2, 3, 2), n=25), 27, 1, 4000000),
+    "27-point blocks": (lambda: W.elasticity3d(region_grid=(2, 2, 2), choices=(25,), seed=2), 27, 3,
+                        24000000),
+}
+
+
+@pytest.mark.parametrize("name", list(LARGE))
+def test_direct_pass_against_the_general_one(name):
+    """Rows in column order go by position; with rows the other way round the same regions go entry
+    by entry, and with a few rows of that kind, or with a column twice, those go through the list.
+    The same bits in single-copy rows, sums in another order in shared ones."""
+    from paper_2103_11962_gb300 import rmg
+    make, kind, B, line = LARGE[name]
+    p = make()
+    assert p.n_regional_nodes * kind * B * B >= line
+    A = p.A.tocsr()
+    A.sort_indices()
+    rp, col, val = A.indptr.astype(np.int64), A.indices.astype(np.int64), A.data.copy()
+    rng = np.random.default_rng(5)
+    val *= 1.0 + 1e-6 * rng.uniform(-1.0, 1.0, val.size)
+    gids = torch.from_numpy(np.asarray(p.region_gids, dtype=np.int64)).cuda()
+    ctx = rmg.Context(0)
+    want = _split(ctx, p, kind, B, rp, col, val, gids)
+    copies = np.bincount(p.region_gids, minlength=p.n_nodes)
+    single = copies[p.region_gids] == 1
+    row = np.repeat(np.arange(rp.size - 1), np.diff(rp))
+    at = np.arange(col.size)
+    back = rp[row] + rp[row + 1] - 1 - at      # the entries of every row the other way round
+    for some in (np.ones(rp.size - 1, bool), rng.uniform(size=rp.size - 1) < 0.01):
+        o = np.where(some[row], back, at)
+        got = _split(ctx, p, kind, B, rp, col[o], val[o], gids)
+        assert np.array_equal(got[..., single], want[..., single])
+        assert np.abs(got - want).max() <= 81 * 2.0 ** -52 * np.abs(val).max()
+    full = np.flatnonzero((np.diff(rp).reshape(-1, B).min(1) == B * kind) & (copies == 1))
+    g = int(full[full.size // 3])
+    col[rp[g * B] + B] = col[rp[g * B]]
+    got = _split(ctx, p, kind, B, rp, col, val, gids)
+    n = int(np.flatnonzero(p.region_gids == g)[0])
+    want[0, 0, 0, n] = val[rp[g * B]] + val[rp[g * B] + B]
+    want[0, 0, 1, n] = 0.0
+    assert np.array_equal(got, want)
