@@ -63,19 +63,23 @@ inline int resident_per_sm_smem(const void* kernel, int smem) {
 // with and without it on level 0, us: 672k nodes of 5 points (3.4M) 352 and 320, 1.33M of 7 (9.3M)
 // 507 and 483, 256k of 27 (6.9M) 332 and 269.
 // In a stream up to 40M: the power method of 3.1M nodes with 7 points gains 4 us a sweep, at 42M a
-// solve with 7 points is level, at 970M one with 27 loses 4%. Except, for a product over run tiles,
-// where its grid is smaller than a wave and its rows are long, because the blocks are placed where
-// those of the running kernel end first, and some SMs then get more of them than others. Products,
-// us, with and without: 27 points, 74k nodes (2.0M, two blocks an SM) 8.7 and 12.4, 81k 15.5 and
-// 12.4, 166k (0.53 of a wave) 15.6 and 12.5, 216k (0.69) 17.5 and 18.6, 678k 44.2 and 47.6; 7 points,
-// 333k nodes 8.1 and 12.4, 1.33M 26.1 and 29.4; blocks of 3 on 27 points, 8k nodes (1.9M) 21.6 and
-// 24.7, 22k 22.8 and 20.6, 44k 40.2 and 39.1, 169k 108 and 97, 333k 162 and 156.
-inline bool short_kernels(const Level& L, bool product = false) {
+// solve with 7 points is level, at 970M one with 27 loses 4%.
+inline bool short_kernels(const Level& L) {
+  const long long coefs = (long long)L.n_r * L.kind * L.B * L.B;
+  return coefs <= (g_capturing ? 1500000 : 40000000);
+}
+// The same for phase A of a product over run tiles in a stream. With long rows only up to 2M
+// coefficients (two blocks an SM) and behind a phase B: the blocks are placed where those of the
+// running kernel end first, and some SMs then get more of them than others. Products, us, phase A
+// plain and dependent (phase B dependent in both): 27 points, 333k nodes 22.4 and 23.4, 817k 48.2
+// and 51.5, 1.16M 65.9 and 69.8, 1.39M in uneven regions 76.9 and 86.5; one region of 54k without
+// phase B 8.3 and 11.2; 7 points, 333k 10.4 and 8.8, 0.91M 18.5 and 16.7, 1.9M 34.9 and 33.1. Both
+// plain and both dependent: 27 points, 74k nodes 12.4 and 8.7, 81k 12.4 and 15.5; blocks of 3 on 27
+// points, 8k nodes (1.9M) 24.7 and 21.6, 22k 20.6 and 22.8, 169k 97 and 108.
+inline bool short_product(const Level& L) {
   const int row = L.kind * L.B * L.B;
-  const long long coefs = (long long)L.n_r * row;
-  if (g_capturing) return coefs <= 1500000;
-  if (!product || coefs <= 2000000) return coefs <= 40000000;
-  return coefs <= 40000000 && (row < 27 || (row == 27 && L.n_r >= 200000));
+  return short_kernels(L) &&
+         (g_capturing || row < 27 || (L.ngroups && (long long)L.n_r * row <= 2000000));
 }
 
 // kernel<<<grid, block, smem, st>>>(args...) for a kernel that starts with follow(). With `next`,
@@ -108,10 +112,10 @@ void launch_resident(const Ctx& c, bool next, void (*kernel)(P...), int work, cu
 // Phase B alone (scalar levels): one thread per copy of every interface group.
 template <typename AT, class Epi>
 void launch_groups(Ctx& c, const Level& L, const AT* y, Epi epi, cudaStream_t st,
-                   bool next = true, bool product = false) {
+                   bool next = true) {
   if (!L.ngroups) return;
   const int gs = persistent_grid(c, (L.nslots + 255) / 256);
-  launch_after(next && short_kernels(L, product), k_groups<AT, Epi>, dim3(gs), 256, 0, st,
+  launch_after(next && short_kernels(L), k_groups<AT, Epi>, dim3(gs), 256, 0, st,
                L.nslots, L.slots.get(), L.gslot.get(), y, epi);
   RMG_LAUNCHED();
 }
@@ -152,7 +156,7 @@ void launch_stencil(Ctx& c, const Level& L, const CT* coef, const VT* u, AT* y, 
   if (G.lx == -3 && ((reinterpret_cast<uintptr_t>(u) | reinterpret_cast<uintptr_t>(half)) & 15))
     G = L.grid();
   const int gb = persistent_grid(c, G.ntiles);
-  const bool product = sweep == nullptr, next = !ev0 && short_kernels(L, product);
+  const bool next = !ev0 && (sweep ? short_kernels(L) : short_product(L));
   // external record nodes when capturing, so the events can be timed after a graph replay
   if (ev0) RMG_CUDA(cudaEventRecordWithFlags(ev0, st, g_capturing ? cudaEventRecordExternal : 0));
   bool done = false;
@@ -203,10 +207,10 @@ void launch_stencil(Ctx& c, const Level& L, const CT* coef, const VT* u, AT* y, 
   if (launches) ++*launches;
   if (L.ngroups) {
     if (L.B == 1) {
-      launch_groups(c, L, y, epi, st, !ev1, product);
+      launch_groups(c, L, y, epi, st, !ev1);
     } else {
       const int gg = persistent_grid(c, (L.nslots + 255) / 256);
-      launch_after(!ev1 && short_kernels(L, product), k_groups_b<AT, Epi>, dim3(gg), 256, 0, st,
+      launch_after(!ev1 && short_kernels(L), k_groups_b<AT, Epi>, dim3(gg), 256, 0, st,
                    L.nslots, L.B, L.n_r, L.slots.get(), L.gslot.get(), (const AT*)y, epi);
       RMG_LAUNCHED();
     }
