@@ -519,8 +519,9 @@ k_bstencil(Grid G, const CT* __restrict__ coef, const VT* u,
 // half[((c * B + c') * P + s - C) * n_r + n] with P = S - C, and slot s < C of block (c, c') at n
 // is slot S-1-s of block (c', c) at n + off(s). The centre is stored for both (c, c') and
 // (c', c), so it needs no symmetry. Same products in the same order as k_bstencil, hence the
-// same bits. The sweep is bound by HBM and this form moves 14/27 of the coefficients: 577 instead
-// of 1045 bytes a node; the mirrored ones come from L1 and L2.
+// same bits. The sweep is bound by HBM and this form names 14/27 of the coefficients: 577 instead
+// of 1045 bytes a node. Most mirrored ones come from L1 and L2; 781 bytes a node came from DRAM
+// with 0.6M nodes (ncu).
 template <bool HALF, int KIND, int B>
 __device__ __forceinline__ void bstencil_row32(const float* __restrict__ coef,
                                                const float* u, int n, int n_r, int i,
