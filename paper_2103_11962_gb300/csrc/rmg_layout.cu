@@ -668,7 +668,7 @@ __device__ __forceinline__ unsigned split_direct(unsigned cand, int g, int64_t e
 // or leave entries out do so in all rows: without this look the direct pass copied such rows for
 // nothing and the list below took them all: diagonal first, 4.9M nodes of a 7-point stencil 539 us
 // and 3M of a 27-point one 1380 us, now 350 and 905 (the general pass alone 330 and 946). For rows
-// in column order the look costs 2 to 4 us of 282 and 704.
+// in column order the look costs 2 to 7 us (of 282 and 704; 346 -> 352 with 1.3M nodes of 27 points).
 // any[0] and any[1] become `call` when there is a region that is taken and one that is not, a
 // number that earlier calls did not use. Also clears the lengths of the lists.
 template <int KIND, int B>
@@ -964,11 +964,11 @@ void split_from_csr(Ctx& c, Level& L, int kind, int B, const int64_t* rowptr, co
   // regions that it did not take, then the rows of shared nodes over the group slots; all grids
   // are one resident wave (the second half of the rows' blocks mostly has nothing to do)
   const int gf = persistent_grid(c, (L.nreg + 7) / 8);
-  // Small matrices: all single-copy rows by tiles in one launch. The direct pass's three launches and
-  // the latency of its short list cost more than it saves up to about 1M nodes of 5 to 9 points, 100k
-  // of 27 and 100k of blocks of 3. Split, us, by tiles and with the direct pass: 7 points, 1.02M nodes
-  // 105 and 109, 4.9M 330 and 282; 5 points, 0.97M 83 and 90; 27 points, 85k 48 and 54, 166k 70 and 68,
-  // 333k 170 and 144; blocks on 27 points, 22k 115 and 136, 379k 1210 and 1046.
+  // Small matrices: all single-copy rows by tiles in one launch. The direct pass's three launches
+  // and the latency of its short list cost more than it saves up to about 1M nodes of 5 to 9 points,
+  // 150k of 27 and 100k of blocks of 3. Split, us, by tiles and with the direct pass: 7 points, 1.02M
+  // nodes 105 and 109, 4.9M 330 and 282; 5 points, 0.97M 83 and 90; 27 points, 85k 48 and 54, 166k
+  // 70 and 68, 333k 170 and 145; blocks on 27 points, 22k 115 and 136, 156k 450 and 384.
   const int row = kind * B * B;
   const bool tiles = (long long)L.n_r * row < (B > 1 ? 24000000 : kind == 27 ? 4000000 : 8000000);
   const uint8_t* direct = tiles ? nullptr : L.split_direct.get();
